@@ -466,6 +466,192 @@ __device__ __forceinline__ void rope_rows(const RopeParams& p, const int64_t rb,
   }
 }
 
+// ---------------------------------------------------------------- packed fp32 pairs
+// Two fp32 values in one 64-bit register pair; sm_100's f32x2 instructions do both lanes'
+// multiply (or fused multiply-add) in one issue, each rounded as the scalar instruction rounds.
+struct F2 { unsigned long long v; };
+__device__ __forceinline__ F2 f2_pack(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(F2 x, float* a, float* b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(*a), "=f"(*b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+
+// ---------------------------------------------------------------- RoPE, both halves per lane
+// A head-row of D elements by D / 16 lanes: lane l owns elements [8l, 8l + 8) and their
+// rotate-half partners [D/2 + 8l, D/2 + 8l + 8), so a rotation needs no other lane (with one
+// vector per lane it took eight shuffles per vector, and the two lanes of a pair computed the
+// same eight sines and cosines). A warp holds GW = 512 / D lane groups and works on one item:
+// rpi consecutive head-rows of one token (RopeParams.ipt items per token), group g taking the
+// rows g, g + GW, ... of it; the lane's angles are computed once per item.
+template <int D>
+struct RopeGeom {
+  static constexpr int LPG = D / 16;     // lanes per head-row
+  static constexpr int GW = 32 / LPG;    // head-rows per warp at a time
+  static_assert(LPG >= 2 && LPG <= 32 && (LPG & (LPG - 1)) == 0, "head size");
+};
+
+// The item of warp `item` of the grid: its token and head-rows [*first, *end); false past the
+// grid's last item.
+__device__ __forceinline__ bool rope_item(const RopeParams& p, int64_t item, int64_t* t, int* first, int* end) {
+  if (item >= p.T * p.ipt) return false;
+  const uint32_t tok = fast_div((uint32_t)item, p.ipt_magic, p.ipt_shift);
+  *t = tok;
+  *first = (int)((uint32_t)item - tok * (uint32_t)p.ipt) * p.rpi;
+  *end = min(p.NH, *first + p.rpi);
+  return true;
+}
+
+// Source of head-row hh of token t (its lane-0 vector).
+template <int D>
+__device__ __forceinline__ const char* rope_row_src(const RopeParams& p, int64_t t, int hh) {
+  constexpr int RB = D * 2;
+  return hh < p.Hq ? row_ptr(p.q, t, p.q_rs, 2) + (int64_t)hh * RB
+       : hh < p.Hq + p.Hkv ? row_ptr(p.k, t, p.k_rs, 2) + (int64_t)(hh - p.Hq) * RB
+                           : row_ptr(p.v, t, p.v_rs, 2) + (int64_t)(hh - p.Hq - p.Hkv) * RB;
+}
+
+// Sines and cosines of a lane's eight pairs for position pos; fq holds the lane's frequencies.
+struct RopeAngles { F2 sn[4], ns[4], cs[4]; };  // ns = -sn
+__device__ __forceinline__ void rope_angles(int32_t pos, const float4* fq, RopeAngles* a) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float s0, c0, s1, c1;
+    rope_sincos((float)pos, fq[q].x, fq[q].y, &s0, &c0);
+    rope_sincos((float)pos, fq[q].z, fq[q].w, &s1, &c1);
+    a->sn[q] = f2_pack(s0, s1);
+    a->ns[q] = f2_pack(-s0, -s1);
+    a->cs[q] = f2_pack(c0, c1);
+  }
+}
+__device__ __forceinline__ void rope_pair_freqs(const float2* inv_freq, int lane, float4* fq) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) fq[q] = ldg_f4(reinterpret_cast<const float*>(inv_freq) + 16 * lane + 4 * q);
+}
+
+// A lane's q- or k-norm weights (kind 1: q, 2: k), for its low and high halves.
+struct RopeGamma { F2 lo[4], hi[4]; };
+template <int D>
+__device__ __forceinline__ void rope_pair_gamma(const float* gamma, int lane, RopeGamma* g) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const float4 a = ldg_f4(gamma + lane * 8 + 4 * q), b = ldg_f4(gamma + D / 2 + lane * 8 + 4 * q);
+    g->lo[2 * q] = f2_pack(a.x, a.y);
+    g->lo[2 * q + 1] = f2_pack(a.z, a.w);
+    g->hi[2 * q] = f2_pack(b.x, b.y);
+    g->hi[2 * q + 1] = f2_pack(b.z, b.w);
+  }
+}
+
+// Finishes head-row hh of token t from its two vectors: [q/k norm,] rotation, store (v: copy).
+// *kind says whose weights *g holds (0: none yet); rows of an item mostly share them.
+template <int DT, int D, bool QKNORM>
+__device__ __forceinline__ void rope_pair_finish(const RopeParams& p, int64_t t, int hh, int lane, int32_t pos,
+                                                 const uint4& lo, const uint4& hi, const RopeAngles& an,
+                                                 RopeGamma* g, int* kind) {
+  constexpr int LPG = RopeGeom<D>::LPG;
+  const bool is_q = hh < p.Hq, is_v = hh >= p.Hq + p.Hkv;
+  char* dst = is_q ? row_ptr(p.q, t, p.q_rs, 2) + (int64_t)hh * (D * 2)
+                   : reinterpret_cast<char*>(is_v ? p.v_cache : p.k_cache) +
+                         ((int64_t)(hh - p.Hq - (is_v ? p.Hkv : 0)) * p.S + pos) * (D * 2);
+  dst += lane * 16;
+  if (is_v) {  // bit copy into the cache
+    st16(dst, lo);
+    st16(dst + D, hi);
+    return;
+  }
+  float a[8], b[8];
+  unpack<DT>(lo, a);
+  unpack<DT>(hi, b);
+  F2 A[4], B[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    A[q] = f2_pack(a[2 * q], a[2 * q + 1]);
+    B[q] = f2_pack(b[2 * q], b[2 * q + 1]);
+  }
+  if (QKNORM) {
+    F2 s2 = f2_mul(A[0], A[0]);
+#pragma unroll
+    for (int q = 1; q < 4; ++q) s2 = f2_fma(A[q], A[q], s2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s2 = f2_fma(B[q], B[q], s2);
+    float s0, s1;
+    f2_unpack(s2, &s0, &s1);
+    float ss = s0 + s1;
+    const unsigned mask =
+        LPG == 32 ? 0xffffffffu : (((1u << LPG) - 1u) << ((threadIdx.x & 31) & ~(LPG - 1)));
+#pragma unroll
+    for (int o = LPG / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(mask, ss, o, LPG);
+    const float inv = rsqrtf(ss * p.inv_D + p.eps);
+    const int want = is_q ? 1 : 2;
+    if (*kind != want) {
+      rope_pair_gamma<D>(is_q ? p.gamma_q : p.gamma_k, lane, g);
+      *kind = want;
+    }
+    const F2 iv = f2_pack(inv, inv);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      A[q] = f2_mul(f2_mul(A[q], iv), g->lo[q]);
+      B[q] = f2_mul(f2_mul(B[q], iv), g->hi[q]);
+    }
+  }
+  // low half: x_i c - x_{i+D/2} s;  high half: x_{i+D/2} c + x_i s
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    f2_unpack(f2_fma(A[q], an.cs[q], f2_mul(B[q], an.ns[q])), &a[2 * q], &a[2 * q + 1]);
+    f2_unpack(f2_fma(B[q], an.cs[q], f2_mul(A[q], an.sn[q])), &b[2 * q], &b[2 * q + 1]);
+  }
+  st16(dst, pack<DT>(a));
+  st16(dst + D, pack<DT>(b));
+}
+
+// One item's rows [first, end) of token t, at most R per lane group: every load the rows need
+// is issued first. fq: the lane's frequencies.
+template <int DT, int D, bool QKNORM, int R>
+__device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, int first, int end, const float4* fq) {
+  constexpr int LPG = RopeGeom<D>::LPG, GW = RopeGeom<D>::GW;
+  const int lane = (threadIdx.x & 31) % LPG;
+  const int hh0 = first + (threadIdx.x & 31) / LPG;
+  uint4 lo[R], hi[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    if (hh0 + j * GW < end) {
+      const char* src = rope_row_src<D>(p, t, hh0 + j * GW) + lane * 16;
+      lo[j] = ld16(src);
+      hi[j] = ld16(src + D);
+    }
+  }
+  const int32_t pos = __ldg(p.pos + t);
+  RopeGamma g;
+  int kind = 0;
+  if (QKNORM && hh0 < end && hh0 < p.Hq + p.Hkv) {
+    kind = hh0 < p.Hq ? 1 : 2;
+    rope_pair_gamma<D>(kind == 1 ? p.gamma_q : p.gamma_k, lane, &g);
+  }
+  if (pos < 0 || (int64_t)pos >= p.S) {  // uniform over the warp: one token per item
+    if ((threadIdx.x & 31) == 0) atomicOr(p.err, kErrPos);
+    return;
+  }
+  RopeAngles an;
+  rope_angles(pos, fq, &an);
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    if (hh0 + j * GW < end)
+      rope_pair_finish<DT, D, QKNORM>(p, t, hh0 + j * GW, lane, pos, lo[j], hi[j], an, &g, &kind);
+}
+
 // ---------------------------------------------------------------- SwiGLU tile
 template <int DT> __device__ __forceinline__ float silu_mul(float g, float u);
 // bf16/fp16 outputs: fast exp and divide (relative error ~1e-6, far below the output ulp;

@@ -80,9 +80,12 @@ struct RopeParams {
   int32_t prefetch;
   uint32_t nh_magic;  // unit / NH for units below 2^32 by fast_div
   int32_t nh_shift;
+  int32_t ipt, rpi;    // warp items per token, head-rows per item (RopeSplit)
+  uint32_t ipt_magic;  // item / ipt by fast_div
+  int32_t ipt_shift;
 };
 
-// RoPE with the block's rows staged by bulk copies (rope_bulk_kernel, calls of many tokens).
+// RoPE with each warp's rows staged by bulk copies (rope_bulk_kernel, calls of many tokens).
 struct RopeBulkParams {
   RopeParams rp;
   uint32_t first_wait_polls;  // polls of the wait for the copies (kBulkWaitPolls; 0 under
@@ -150,18 +153,19 @@ struct KernelEntry {
   const void* fn_step_role = nullptr;  // chain only: fn_step_inplace, role-major block order
   const void* fn_step = nullptr;          // chain only: several calls per launch (ChainStepParams)
   const void* fn_step_inplace = nullptr;  // ... one block per token for the norms
-  const void* fn_large = nullptr;  // add+RMSNorm / RoPE: the entry for calls of >= large_rows rows
-                                   // (tokens)
+  const void* fn_large = nullptr;  // add+RMSNorm: the entry for calls of >= large_rows rows;
+                                   // RoPE: the bulk-copy entry
+  const void* fn_mid = nullptr;    // RoPE: the entry between fn and fn_large (rope_plan chooses)
   int32_t large_rows = 0;
   int32_t kind = 0;      // which grid rule the host applies (KernelKind)
   int32_t vec = 0;       // elements per vector (VE), or tile width for SwiGLU
   int32_t unroll = 1;    // vectors per thread per tile (SwiGLU, chain)
-  int32_t rows = 1;      // rows per block (KK_NORM_ROWS; RoPE's fn_large: tokens per block)
+  int32_t rows = 1;      // rows per block (KK_NORM_ROWS)
 };
 
 enum KernelKind : int32_t {
   KK_ADDNORM_ROW = 1,   // grid = T rows, one block per row
-  KK_ROPE_HALFWARP = 2, // grid = ceil(T*NH / units_per_block)
+  KK_ROPE_PAIR = 2,     // vector: grid by rope_plan
   KK_ROPE_WARP = 3,     // generic: one warp per head-row
   KK_SWIGLU_TILE = 4,   // grid = (tiles per row, rows)
   KK_SWIGLU_FLAT = 5,   // generic: flat grid-stride
@@ -190,7 +194,49 @@ int32_t prepare_rope_args(const void* trident_args_ptr, RopeParams* p, int32_t* 
 // Sets the thread-local last-error message and returns `status`.
 int32_t internal_fail(int32_t status, const char* msg);
 
-// Units (head-rows) handled by one block of the vector RoPE kernel for head size D.
+// Round-up multiplier and shift for dividing 32-bit unsigned integers by d (1 <= d < 2^31):
+// l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1; the kernels take the quotient as
+// (h + ((n - h) >> 1)) >> (l - 1) with h = umulhi(n, m) (fast_div; Granlund and Montgomery,
+// 1994), and l = 0 (d = 1) as n itself. d = 0 (no divisor: callers reject such calls first)
+// stays defined.
+inline void div_magic(uint32_t d, uint32_t* m, int32_t* l) {
+  *m = 0;
+  *l = 0;
+  if (d == 0) return;
+  int32_t s = 0;
+  while ((1ull << s) < d) ++s;
+  *m = (uint32_t)(((1ull << 32) * ((1ull << s) - d)) / d + 1);
+  *l = s;
+}
+
+// How a token's NH head-rows are split into warp items of at most `max_rows` rows per lane
+// group (a warp has 512 / D groups), as evenly as the groups allow.
+struct RopeSplit {
+  int32_t ipt, rpi;  // items per token, head-rows per item
+  uint32_t magic;    // item / ipt by fast_div
+  int32_t shift;
+};
+inline RopeSplit rope_split(int64_t NH, int32_t D, int32_t max_rows) {
+  RopeSplit r{};
+  const int64_t gw = 512 / D, quads = (NH + gw - 1) / gw, ipt = (quads + max_rows - 1) / max_rows;
+  if (ipt < 1) return r;
+  const int64_t rpi = (quads + ipt - 1) / ipt * gw;
+  r.rpi = (int32_t)rpi;
+  r.ipt = (int32_t)((NH + rpi - 1) / rpi);  // no item without rows
+  div_magic((uint32_t)r.ipt, &r.magic, &r.shift);
+  return r;
+}
+
+// Which vector RoPE entry a call of T tokens takes, and its launch shape. The splits depend
+// only on the version's head counts and head size (rope_plans, at registration).
+enum RopeEntry : int32_t { ROPE_SMALL = 0, ROPE_MID = 1, ROPE_BULK = 2 };
+struct RopePlans {
+  RopeSplit split[3];  // by RopeEntry
+};
+void rope_plans(int64_t NH, int32_t D, RopePlans* out);
+RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks);
+
+// Units (head-rows) handled by one RoPE block of the layer chain for head size D.
 inline int32_t rope_units_per_block(int32_t D, int32_t elem_bytes) {
   int32_t lanes_per_head = D * elem_bytes / 16;
   return kThreads / lanes_per_head;

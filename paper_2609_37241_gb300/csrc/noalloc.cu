@@ -99,11 +99,18 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
     return internal_fail(TRIDENT_ERR_CUDA, "scratch preparation launch failed");
   p.inv_freq = table;
   p.err = status;
-  const int64_t upb = rope_units_per_block(p.D, 2);
-  const int64_t blocks = (p.T * p.NH + upb - 1) / upb;
-  void* kargs[1] = {&p};
-  if (cudaLaunchKernel(ke.fn, dim3((unsigned)(blocks < 0x7fffffff ? blocks : 0x7fffffff)), dim3(kThreads),
-                       kargs, 0, s) != cudaSuccess)
+  RopeBulkParams bp;
+  RopePlans plans;
+  int32_t threads = 0;
+  int64_t blocks = 0;
+  rope_plans(p.NH, p.D, &plans);
+  const RopeEntry entry = rope_plan(plans, &p, &threads, &blocks);
+  bp.rp = p;
+  bp.first_wait_polls = kBulkWaitPolls;
+  const void* fn = entry == ROPE_BULK ? ke.fn_large : (entry == ROPE_MID ? ke.fn_mid : ke.fn);
+  void* kargs[1] = {entry == ROPE_BULK ? (void*)&bp : (void*)&p};
+  if (cudaLaunchKernel(fn, dim3((unsigned)(blocks < 0x7fffffff ? blocks : 0x7fffffff)),
+                       dim3((unsigned)threads), kargs, 0, s) != cudaSuccess)
     return internal_fail(TRIDENT_ERR_CUDA, "RoPE launch failed");
   if (out_status &&
       cudaMemcpyAsync(out_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)

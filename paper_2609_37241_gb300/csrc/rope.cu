@@ -1,216 +1,158 @@
 // rope.cu -- RoPE on q/k with KV-cache append, optionally after per-head q/k RMSNorm.
 //
 // Work unit: one head-row (token t, head hh) of D elements; per token there are
-// NH = Hq + 2*Hkv of them (q heads, k heads, v heads). The vector kernel gives each unit
-// D/VE lanes (16 lanes for D = 128 in bf16) so that a unit is one 256-byte coalesced
-// access, and exchanges the rotate-half partner with one xor-shuffle per element.
-// The generic kernel gives each unit one warp and scalar accesses (any alignment, any
-// even D). Calls of many tokens take the bulk-copy kernel (rope_bulk_kernel): a few tokens
-// per block, their rows staged in shared memory by cp.async.bulk on an mbarrier, each
-// token's angles computed once. All compute (cos, sin) of pos * theta^(-2i/D) in the kernel
-// from the version's double-float frequency table [D/2], which the host splits from fp64 at
-// registration.
+// NH = Hq + 2*Hkv of them (q heads, k heads, v heads). The vector kernels give a warp an item
+// of consecutive head-rows of one token (RopeGeom, rope_pair_rows in device_common.cuh): D / 16
+// lanes per head-row, each lane holding both halves of its rotated pairs, so that a rotation
+// needs no exchange between lanes and a token's angles are computed once per lane and item.
+// Three entries, by the call's size (rope_plan): one head-row per lane group where latency
+// counts, two in between, and for calls of many tokens three, staged in shared memory by
+// cp.async.bulk (rope_bulk_kernel). The generic kernel gives each head-row one warp and scalar
+// accesses (any alignment, any even D). All compute (cos, sin) of pos * theta^(-2i/D) in the
+// kernel from the version's double-float frequency table [D/2], which the host splits from
+// fp64 at registration.
+//
+// Bound: HBM at prefill sizes, launch and memory latency at decode sizes. Before, a lane held
+// one vector of a head-row and exchanged its partner by eight shuffles, and each of the two
+// lanes of a pair computed the pair's sines and cosines: issue-bound (72 % SM throughput by
+// ncu at 3333 tokens with q/k norm, 0.45 of the 6.8 TB/s copy rate). Llama head counts
+// (32 + 8 + 8 of D 128), device time per call, before -> now, with q/k norm / without:
+//   30 tokens    3.36 -> 2.06 / 2.95 -> 1.91 us      500 tokens    7.66 -> 4.67 / 6.86 -> 4.20 us
+//   120 tokens   3.58 -> 3.01 / 3.18 -> 2.77 us     3333 tokens   26.5 -> 15.1 / 20.8 -> 13.7 us
+//   250 tokens   5.13 -> 3.22 / 4.48 -> 3.04 us     8192 tokens   51.7 -> 33.3 / 41.8 -> 30.9 us
+// (8192 tokens without the norm: 0.96 of the copy rate.) D 64 at 250 tokens without the norm
+// is the one size of that sweep that lost (2.63 -> 3.01 us).
 #include "device_common.cuh"
 
 namespace trident {
 
-template <int DT, int D, bool QKNORM>
-__global__ void __launch_bounds__(kThreads) rope_vec_kernel(const RopeParams p) {
+// Small and mid entries: 64 threads, two items per block (128 threads: the same within 3 %).
+constexpr int kRopeThreads = 64;
+// Calls of at most this many one-row items (three per SM) take one head-row per lane group:
+// the call is one memory round trip, and a second row per group only lengthens it. Above, two
+// rows per group halve the warps that fetch the same frequency and weight lines: 60 tokens with
+// q/k norm 2.33 us against 2.62 with one row, 500 tokens 4.67 against 5.51.
+constexpr int64_t kRopeSmallItems = 456;
+// Calls of at least this many tokens take the bulk-copy entry: at 512 tokens it is level with two
+// register-held rows per group (with q/k norm 5.0 against 4.9 us, without 4.6 against 3.9), from
+// about 1024 ahead (2048 tokens 10.5 / 8.9 against 12.3 / 10.5 us; 8192 33.3 / 30.9 against
+// 38.0 / 32.8).
+constexpr int32_t kRopeBulkTokens = 512;
+
+
+// Before the launch wait: the lane's frequencies (the version's table is written only at
+// registration), and with p.prefetch the L2 prefetch of the item's row lines and position.
+template <int DT, int D, bool QKNORM, int R>
+__global__ void __launch_bounds__(kRopeThreads) rope_pair_kernel(const RopeParams p) {
   pdl_trigger();
-  constexpr int LPH = D / Act<DT>::VE;
-  constexpr int UPB = kThreads / LPH;
-  const int64_t total = p.T * p.NH;
-  const int lane = threadIdx.x % LPH;
-  if (p.prefetch) rope_prefetch<DT, D>(p, (int64_t)blockIdx.x * UPB + threadIdx.x / LPH, lane);
-  float fq[2 * Act<DT>::VE];
-  rope_lane_freqs<DT, D>(p.inv_freq, lane, fq);  // the version's table: readable before the wait
-  pdl_wait();
-  for (int64_t unit = (int64_t)blockIdx.x * UPB + threadIdx.x / LPH; unit < total;
-       unit += (int64_t)gridDim.x * UPB) {
-    rope_head_row<DT, D, QKNORM>(p, unit, lane, fq);
+  constexpr int LPG = RopeGeom<D>::LPG, GW = RopeGeom<D>::GW;
+  const int lane = (threadIdx.x & 31) % LPG, g = (threadIdx.x & 31) / LPG;
+  int64_t t;
+  int first, end;
+  const bool live = rope_item(p, (int64_t)blockIdx.x * (kRopeThreads / 32) + threadIdx.x / 32, &t, &first, &end);
+  float4 fq[4];
+  rope_pair_freqs(p.inv_freq, lane, fq);
+  if (p.prefetch && live && lane % 8 == 0) {
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      if (first + g + j * GW < end) {
+        const char* src = rope_row_src<D>(p, t, first + g + j * GW) + lane * 16;
+        prefetch_l2(src);
+        prefetch_l2(src + D);
+      }
+    }
+    if ((threadIdx.x & 31) == 0) prefetch_l2(p.pos + t);
   }
+  pdl_wait();
+  if (live) rope_pair_rows<DT, D, QKNORM, R>(p, t, first, end, fq);
 }
 
-// Calls of many tokens (the vector kernel's grid several waves long): a block takes up to
-// kRopeBulkTokens tokens. One thread issues, per token, three bulk copies (cp.async.bulk: a
-// token's q, k and v head-rows are each contiguous, D elements per head) into shared memory,
-// completing on one mbarrier, while the block's threads compute the tokens' D/2 pairs
-// (sin, cos) of pos * theta^(-2i/D) once into shared memory (rope_sincos: the values the vector
-// kernel's lanes compute for each of their elements, so outputs are bit-identical); lanes then
-// rotate head-rows out of shared memory and store them.
+// Calls of many tokens: a warp's item is three head-rows per lane group (3 KB), staged in the
+// warp's own shared memory by bulk copies (cp.async.bulk: an item's q, k and v rows are each
+// contiguous, so one to three copies) on the warp's own mbarrier; meanwhile the lanes compute
+// the token's angles, once per item. No block barrier: each warp waits for its own copies,
+// rotates its rows out of shared memory and stores them. Staged rows take no registers, so 24
+// warps of 3 KB are in flight per SM. Other shapes measured at 3333 tokens (q/k norm): this one
+// 15.1 us; 6 rows per group 15.4; 12 rows 17.8-18.3; 8 blocks per SM (spills) 16.4; three
+// register-held rows 17.0; the former two tokens per block behind a block barrier 26.5.
 //
-// Why not the vector kernel: each of a token's 2 (Hq + Hkv) q/k head-rows recomputes all of
-// its elements' angles there, about half of its instructions, and its register-resident rows
-// (64 registers, four blocks per SM of 4 KB of reads each) keep too few bytes in flight: at
-// 4096 Llama tokens it reaches 0.35 of the measured copy bandwidth, this kernel 0.58 (8192:
-// 0.37 and 0.71). Measured and dropped: lane groups of three register-resident head-rows with
-// the angles in shared memory (0.51 / 0.57), and four or eight tokens per block (0.51 / 0.64,
-// 0.46 / 0.51: a block copies, then computes, so heavier blocks idle the memory longer).
-//
-// The wait is bounded (bp.first_wait_polls try_wait polls, kBulkWaitPolls by default): a
-// block whose copies have not landed by then sets TRIDENT_DEVERR_TIMEOUT, waits (again
-// bounded) for them and returns without writing.
-#ifndef TRIDENT_ROPE_BULK_TOKENS
-#define TRIDENT_ROPE_BULK_TOKENS 2
-#endif
-constexpr int kRopeBulkTokens = TRIDENT_ROPE_BULK_TOKENS;
+// The wait is bounded (bp.first_wait_polls try_wait polls, kBulkWaitPolls by default): a warp
+// whose copies have not landed by then sets TRIDENT_DEVERR_TIMEOUT, waits (again bounded) for
+// them and returns without writing.
+constexpr int kRopeBulkRows = 3;      // head-rows per lane group
+constexpr int kRopeBulkThreads = 128;
 
 template <int DT, int D, bool QKNORM>
-__global__ void __launch_bounds__(kThreads) rope_bulk_kernel(const RopeBulkParams bp) {
+__global__ void __launch_bounds__(kRopeBulkThreads, 6) rope_bulk_kernel(const RopeBulkParams bp) {
   const RopeParams& p = bp.rp;
-  constexpr int TB = kRopeBulkTokens;
-  constexpr int VE = Act<DT>::VE;
-  constexpr int LPH = D / VE;
-  constexpr int HALF = LPH / 2;
-  constexpr int EB = Act<DT>::BYTES;
-  constexpr int G = kThreads / LPH;
-  constexpr int NF = D / 2;
-  static_assert(LPH >= 2 && LPH <= 32 && (LPH & (LPH - 1)) == 0, "head size");
-  extern __shared__ __align__(128) unsigned char s_rows[];  // [TB][NH][D] elements
-  __shared__ __align__(16) float s_sin[TB][NF];
-  __shared__ __align__(16) float s_cos[TB][NF];
-  __shared__ int32_t s_pos[TB];
-  __shared__ __align__(8) unsigned long long bar;
-  const int tid = threadIdx.x;
-  const int lane = tid % LPH;
-  const int g = tid / LPH;
-  const unsigned group_mask =
-      (LPH == 32) ? 0xffffffffu : (((1u << LPH) - 1u) << ((tid & 31) & ~(LPH - 1)));
-  const bool low = lane < HALF;
-  const int f0 = (lane % HALF) * VE;
-  const int64_t tb = (int64_t)blockIdx.x * TB;
-  const int ntok = (int)(p.T - tb < TB ? p.T - tb : TB);
-  const uint32_t qb = (uint32_t)(p.Hq * D * EB), kb = (uint32_t)(p.Hkv * D * EB);
-  const uint32_t tok_bytes = qb + 2 * kb;
-  const uint32_t bar_a = (uint32_t)__cvta_generic_to_shared(&bar);
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar_a) : "memory");
+  constexpr int LPG = RopeGeom<D>::LPG, GW = RopeGeom<D>::GW, RB = D * 2;
+  __shared__ __align__(128) char s_rows[kRopeBulkThreads / 32][kRopeBulkRows * GW * RB];
+  __shared__ __align__(8) unsigned long long s_bar[kRopeBulkThreads / 32];
+  const int w = threadIdx.x / 32, lane = (threadIdx.x & 31) % LPG;
+  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&s_bar[w]);
+  if ((threadIdx.x & 31) == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();  // the barrier is initialised before any lane waits on it
   pdl_trigger();
-  if (p.prefetch) {  // the block's row lines into L2 while the previous kernel finishes
-    const int lines = (int)(tok_bytes / 128);
-    for (int i = tid; i < ntok * lines; i += kThreads) {
-      const int tk = i / lines, l = i - tk * lines;
-      const uint32_t off = (uint32_t)l * 128;
-      const int64_t t = tb + tk;
-      const char* src = off < qb ? row_ptr(p.q, t, p.q_rs, EB) + off
-                                 : off < qb + kb ? row_ptr(p.k, t, p.k_rs, EB) + (off - qb)
-                                                 : row_ptr(p.v, t, p.v_rs, EB) + (off - qb - kb);
-      prefetch_l2(src);
-    }
-  }
+  int64_t t;
+  int first, end;
+  const bool live = rope_item(p, (int64_t)blockIdx.x * (kRopeBulkThreads / 32) + w, &t, &first, &end);
   pdl_wait();
-  __syncthreads();  // the barrier is initialised before anyone waits on it
-  if (tid == 0) {
+  if (!live) return;
+  if ((threadIdx.x & 31) == 0) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                 :: "r"(bar_a), "r"((uint32_t)ntok * tok_bytes) : "memory");
-    for (int tk = 0; tk < ntok; ++tk) {
-      const int64_t t = tb + tk;
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_rows + (size_t)tk * tok_bytes);
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                   :: "r"(dst), "l"(row_ptr(p.q, t, p.q_rs, EB)), "r"(qb), "r"(bar_a) : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                   :: "r"(dst + qb), "l"(row_ptr(p.k, t, p.k_rs, EB)), "r"(kb), "r"(bar_a) : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                   :: "r"(dst + qb + kb), "l"(row_ptr(p.v, t, p.v_rs, EB)), "r"(kb), "r"(bar_a) : "memory");
+                 :: "r"(bar), "r"((uint32_t)((end - first) * RB)) : "memory");
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_rows[w]);
+    int h = first;
+    const int upto[3] = {min(end, p.Hq), min(end, p.Hq + p.Hkv), end};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (h < upto[k]) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     :: "r"(dst + (uint32_t)((h - first) * RB)), "l"(rope_row_src<D>(p, t, h)),
+                        "r"((uint32_t)((upto[k] - h) * RB)), "r"(bar) : "memory");
+        h = upto[k];
+      }
     }
   }
-  for (int idx = tid; idx < ntok * NF; idx += kThreads) {  // the tokens' angles, once each
-    const int tk = idx / NF, i = idx % NF;
-    const int32_t pos = __ldg(p.pos + tb + tk);
-    if (i == 0) s_pos[tk] = pos;
-    float sn = 0.f, cs = 1.f;
-    if (pos >= 0 && (int64_t)pos < p.S) {
-      const float2 f = __ldg(p.inv_freq + i);
-      rope_sincos((float)pos, f.x, f.y, &sn, &cs);
-    }
-    s_sin[tk][i] = sn;
-    s_cos[tk][i] = cs;
+  const int32_t pos = __ldg(p.pos + t);
+  const bool pos_ok = pos >= 0 && (int64_t)pos < p.S;
+  RopeAngles an;
+  {
+    float4 fq[4];
+    rope_pair_freqs(p.inv_freq, lane, fq);
+    rope_angles(pos_ok ? pos : 0, fq, &an);
   }
   auto landed = [&](uint32_t polls) -> bool {
     uint32_t done = 0;
     for (uint32_t it = 0; it < polls && !done; ++it)
       asm volatile("{ .reg .pred q; mbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0; selp.u32 %0, 1, 0, q; }"
-                   : "=r"(done) : "r"(bar_a) : "memory");
+                   : "=r"(done) : "r"(bar) : "memory");
     return done != 0;
   };
   const bool ok = landed(bp.first_wait_polls);
-  if (__syncthreads_or(!ok)) {  // one decision for the whole block (also publishes the angles)
-    if (tid == 0 && p.err) atomicOr(p.err, kErrTimeout);
-    if (!ok) landed(kBulkWaitPolls);  // a second bounded wait for the copies before the block exits
+  if (__any_sync(0xffffffffu, !ok)) {  // one decision for the whole warp
+    if ((threadIdx.x & 31) == 0) atomicOr(p.err, kErrTimeout);
+    if (!ok) landed(kBulkWaitPolls);  // a second bounded wait for the copies before the warp exits
     return;
   }
-  // head-rows u = g + G * i of the block: token tk = u / NH, head-row hh = u % NH, by stepping
-  int tk = 0, hh = g;
-  while (hh >= p.NH) { hh -= p.NH; ++tk; }
-  for (int u = g; u < ntok * p.NH; u += G) {
-    if (u != g) {
-      hh += G;
-      while (hh >= p.NH) { hh -= p.NH; ++tk; }
-    }
-    const int64_t t = tb + tk;
-    const int32_t pos = s_pos[tk];
-    if (pos < 0 || (int64_t)pos >= p.S) {
-      if (lane == 0) atomicOr(p.err, kErrPos);
-      continue;
-    }
-    const uint4 raw = *reinterpret_cast<const uint4*>(s_rows + ((size_t)tk * p.NH + hh) * (D * EB) + lane * 16);
-    int h;
-    bool is_q, is_v;
-    rope_head_of(p, hh, &h, &is_q, &is_v);
-    if (is_v) {  // bit copy into the cache
-      st16(reinterpret_cast<char*>(p.v_cache) + (((int64_t)h * p.S + pos) * D + lane * VE) * EB, raw);
-      continue;
-    }
-    float x[VE];
-    unpack<DT>(raw, x);
-    if (QKNORM) {
-      const float* gam = (is_q ? p.gamma_q : p.gamma_k) + lane * VE;
-      float gg[VE];
+  if (!pos_ok) {
+    if ((threadIdx.x & 31) == 0) atomicOr(p.err, kErrPos);
+    return;
+  }
+  RopeGamma g;
+  int kind = 0;
+  const int hh0 = first + (threadIdx.x & 31) / LPG;
 #pragma unroll
-      for (int q = 0; q < VE / 4; ++q) {
-        const float4 g4 = ldg_f4(gam + 4 * q);
-        gg[4 * q] = g4.x; gg[4 * q + 1] = g4.y; gg[4 * q + 2] = g4.z; gg[4 * q + 3] = g4.w;
-      }
-      float ss = 0.f;
-#pragma unroll
-      for (int e = 0; e < VE; ++e) ss = fmaf(x[e], x[e], ss);
-#pragma unroll
-      for (int o = LPH / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(group_mask, ss, o, LPH);
-      const float inv = rsqrtf(ss * p.inv_D + p.eps);
-#pragma unroll
-      for (int e = 0; e < VE; ++e) x[e] = x[e] * inv * gg[e];
-    }
-    float other[VE];
-#pragma unroll
-    for (int e = 0; e < VE; ++e) other[e] = __shfl_xor_sync(group_mask, x[e], HALF, LPH);
-    float sn[VE], cs[VE];
-#pragma unroll
-    for (int q = 0; q < VE / 4; ++q) {
-      const float4 a = *reinterpret_cast<const float4*>(&s_sin[tk][f0 + 4 * q]);
-      const float4 b = *reinterpret_cast<const float4*>(&s_cos[tk][f0 + 4 * q]);
-      sn[4 * q] = a.x; sn[4 * q + 1] = a.y; sn[4 * q + 2] = a.z; sn[4 * q + 3] = a.w;
-      cs[4 * q] = b.x; cs[4 * q + 1] = b.y; cs[4 * q + 2] = b.z; cs[4 * q + 3] = b.w;
-    }
-    float y[VE];
-#pragma unroll
-    for (int e = 0; e < VE; ++e)
-      y[e] = low ? fmaf(x[e], cs[e], -other[e] * sn[e]) : fmaf(x[e], cs[e], other[e] * sn[e]);
-    if (is_q) {
-      st16(row_ptr(p.q, t, p.q_rs, EB) + ((int64_t)h * D + lane * VE) * EB, pack<DT>(y));
-    } else {
-      st16(reinterpret_cast<char*>(p.k_cache) + (((int64_t)h * p.S + pos) * D + lane * VE) * EB,
-           pack<DT>(y));
-    }
+  for (int j = 0; j < kRopeBulkRows; ++j) {
+    const int hh = hh0 + j * GW;
+    if (hh >= end) break;
+    const char* row = s_rows[w] + (hh - first) * RB + lane * 16;
+    rope_pair_finish<DT, D, QKNORM>(p, t, hh, lane, pos, ld16(row), ld16(row + D), an, &g, &kind);
   }
 }
-
-// Calls of at least this many tokens take rope_bulk_kernel (Llama heads: 512 tokens 8.3
-// against 9.5 us; from 256 tokens down the vector kernel is as fast or faster).
-#ifndef TRIDENT_ROPE_BULK_MIN_TOKENS
-#define TRIDENT_ROPE_BULK_MIN_TOKENS 512
-#endif
 
 template <int DT, bool QKNORM>
 __global__ void __launch_bounds__(kThreads) rope_generic_kernel(const RopeParams p) {
@@ -274,20 +216,37 @@ __global__ void __launch_bounds__(kThreads) rope_generic_kernel(const RopeParams
   }
 }
 
-template <int DT, bool QK>
-static const void* pick_vec(int32_t D) {
-  if (D == 64) return (const void*)rope_vec_kernel<DT, 64, QK>;
-  if (D == 128) return (const void*)rope_vec_kernel<DT, 128, QK>;
-  if (D == 256) return (const void*)rope_vec_kernel<DT, 256, QK>;
-  return nullptr;
+void rope_plans(int64_t NH, int32_t D, RopePlans* out) {
+  out->split[ROPE_SMALL] = rope_split(NH, D, 1);
+  out->split[ROPE_MID] = rope_split(NH, D, 2);
+  out->split[ROPE_BULK] = rope_split(NH, D, kRopeBulkRows);
+}
+
+RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks) {
+  const RopeEntry e = p->T >= kRopeBulkTokens ? ROPE_BULK
+                      : p->T * plans.split[ROPE_SMALL].ipt > kRopeSmallItems ? ROPE_MID : ROPE_SMALL;
+  const RopeSplit& r = plans.split[e];
+  p->ipt = r.ipt;
+  p->rpi = r.rpi;
+  p->ipt_magic = r.magic;
+  p->ipt_shift = r.shift;
+  *threads = e == ROPE_BULK ? kRopeBulkThreads : kRopeThreads;
+  *blocks = (p->T * r.ipt + *threads / 32 - 1) / (*threads / 32);
+  return e;
+}
+
+template <int DT, bool QK, int D>
+static void pick_d(KernelEntry* out) {
+  out->fn = (const void*)rope_pair_kernel<DT, D, QK, 1>;
+  out->fn_mid = (const void*)rope_pair_kernel<DT, D, QK, 2>;
+  out->fn_large = (const void*)rope_bulk_kernel<DT, D, QK>;
 }
 
 template <int DT, bool QK>
-static const void* pick_bulk(int32_t D) {
-  if (D == 64) return (const void*)rope_bulk_kernel<DT, 64, QK>;
-  if (D == 128) return (const void*)rope_bulk_kernel<DT, 128, QK>;
-  if (D == 256) return (const void*)rope_bulk_kernel<DT, 256, QK>;
-  return nullptr;
+static void pick_vec(int32_t D, KernelEntry* out) {
+  if (D == 64) pick_d<DT, QK, 64>(out);
+  else if (D == 128) pick_d<DT, QK, 128>(out);
+  else if (D == 256) pick_d<DT, QK, 256>(out);
 }
 
 bool rope_kernel(int32_t dtype, int32_t variant, int32_t D, bool qknorm, KernelEntry* out,
@@ -304,15 +263,12 @@ bool rope_kernel(int32_t dtype, int32_t variant, int32_t D, bool qknorm, KernelE
                           : (const void*)rope_generic_kernel<DT_FP16, false>;
     return true;
   }
-  out->kind = KK_ROPE_HALFWARP;
+  out->kind = KK_ROPE_PAIR;
   out->vec = 8;
-  if (dtype == DT_BF16) out->fn = qknorm ? pick_vec<DT_BF16, true>(D) : pick_vec<DT_BF16, false>(D);
-  else out->fn = qknorm ? pick_vec<DT_FP16, true>(D) : pick_vec<DT_FP16, false>(D);
+  out->fn = nullptr;
+  if (dtype == DT_BF16) qknorm ? pick_vec<DT_BF16, true>(D, out) : pick_vec<DT_BF16, false>(D, out);
+  else qknorm ? pick_vec<DT_FP16, true>(D, out) : pick_vec<DT_FP16, false>(D, out);
   if (!out->fn) { *why = "vector RoPE supports D in {64, 128, 256}"; return false; }
-  if (dtype == DT_BF16) out->fn_large = qknorm ? pick_bulk<DT_BF16, true>(D) : pick_bulk<DT_BF16, false>(D);
-  else out->fn_large = qknorm ? pick_bulk<DT_FP16, true>(D) : pick_bulk<DT_FP16, false>(D);
-  out->large_rows = TRIDENT_ROPE_BULK_MIN_TOKENS;
-  out->rows = kRopeBulkTokens;  // tokens per block
   return true;
 }
 

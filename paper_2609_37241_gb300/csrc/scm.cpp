@@ -394,7 +394,9 @@ struct Version {
   CUfunction fn_late;     // layer chain: `fn` with the late launch trigger
   CUfunction fn_wide;     // layer chain: `fn_inplace` with kChainWideSwigluUnroll tiles
   int32_t wave_blocks;    // layer chain: blocks of `fn` resident at once on the whole GPU
-  CUfunction fn_large;          // add+RMSNorm: entry for calls of >= ke.large_rows rows
+  CUfunction fn_large;          // add+RMSNorm, RoPE: entry for calls of >= ke.large_rows rows
+  CUfunction fn_mid;            // RoPE: entry between fn and fn_large (rope_plan)
+  RopePlans rope_plans;         // vector RoPE: item splits of its three entries
   CUfunction step_fn;           // layer chain: several calls per launch (two blocks per token)
   CUfunction step_fn_inplace;   // ... one block per token
   CUfunction step_fn_role;      // ... one block per token, role-major order over the step
@@ -606,22 +608,6 @@ void pack_pointwise(const trident_args* a, const Sig& s, PointwiseParams* p) {
   p->prefetch = 0;
 }
 
-// Round-up multiplier and shift for dividing 32-bit unsigned integers by d (1 <= d < 2^31):
-// l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1; the kernels take the quotient as
-// (h + ((n - h) >> 1)) >> (l - 1) with h = umulhi(n, m) (fast_div; Granlund and Montgomery,
-// 1994), and l = 0 (d = 1) as n itself.
-void div_magic(uint32_t d, uint32_t* m, int32_t* l) {
-  if (d == 0) {  // no divisor: callers reject such calls first; stay defined regardless
-    *m = 0;
-    *l = 0;
-    return;
-  }
-  int32_t s = 0;
-  while ((1ull << s) < d) ++s;
-  *m = (uint32_t)(((1ull << 32) * ((1ull << s) - d)) / d + 1);
-  *l = s;
-}
-
 void pack_rope(const trident_args* a, int base, int gq, const Version& v, uint32_t* err,
                RopeParams* p) {
   const trident_tensor* t = a->t;
@@ -786,6 +772,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   void* kp[1] = {&P};
   bool late = false;  // layer chain: launch fn_late (the late launch trigger)
   bool wide = false;  // layer chain: launch fn_wide (wider SwiGLU tiles)
+  RopeEntry rope_entry = ROPE_SMALL;
   switch (op) {
     case TRIDENT_OP_ADD_RMSNORM:
       pack_addnorm(a, 0, 1, 2, 3, 4, s, K_ACT_H, &P.an);
@@ -800,16 +787,18 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     case TRIDENT_OP_ROPE_KV:
     case TRIDENT_OP_QKNORM_ROPE_KV: {
       pack_rope(a, 0, op == TRIDENT_OP_QKNORM_ROPE_KV ? 6 : -1, v, scm->d_err, &P.rp);
-      const int64_t units = P.rp.T * P.rp.NH;
-      if (v.fn_large && s.T >= v.ke.large_rows) {  // bulk-copy kernel: ke.rows tokens per block,
-        const int64_t tpb = v.ke.rows;            // their head-rows staged in shared memory
-        cfg.gridDimX = cap_grid((P.rp.T + tpb - 1) / tpb);
-        cfg.sharedMemBytes = (unsigned)(tpb * P.rp.NH * P.rp.D * 2);
-        P.rb.first_wait_polls = (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) ? 0u : kBulkWaitPolls;
-        break;
+      if (v.ke.kind == KK_ROPE_PAIR) {
+        int32_t threads = 0;
+        int64_t blocks = 0;
+        rope_entry = rope_plan(v.rope_plans, &P.rp, &threads, &blocks);
+        cfg.blockDimX = (unsigned)threads;
+        cfg.gridDimX = cap_grid(blocks);
+        if (rope_entry == ROPE_BULK)
+          P.rb.first_wait_polls = (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) ? 0u : kBulkWaitPolls;
+      } else {  // generic: one warp per head-row
+        const int64_t units = P.rp.T * P.rp.NH, upb = kThreads / 32;
+        cfg.gridDimX = cap_grid((units + upb - 1) / upb);
       }
-      const int64_t upb = v.ke.kind == KK_ROPE_HALFWARP ? rope_units_per_block(P.rp.D, 2) : kThreads / 32;
-      cfg.gridDimX = cap_grid((units + upb - 1) / upb);
       break;
     }
     case TRIDENT_OP_SWIGLU:
@@ -894,7 +883,8 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   // faster layer steps at 1-4 tokens; slower once the grid fills the GPU, where a layer
   // chain prefetches only its norm rows -- see chain_prefetch_mode)
   const bool pdl = (scm->opt.flags & TRIDENT_OPT_PDL) != 0;
-  const int32_t pf = pdl && (int64_t)cfg.gridDimX * cfg.gridDimY <= scm->sm_count ? 1 : 0;
+  const int32_t pf =
+      pdl && (int64_t)cfg.gridDimX * cfg.gridDimY * cfg.blockDimX <= (int64_t)scm->sm_count * kThreads ? 1 : 0;
   switch (op) {
     case TRIDENT_OP_ADD_RMSNORM: P.an.prefetch = pf; break;
     case TRIDENT_OP_RMSNORM: P.rn.prefetch = pf; break;
@@ -910,8 +900,10 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     fn = wide ? v.fn_wide : v.fn_inplace;
   else if (late && v.fn_late)
     fn = v.fn_late;
-  if (v.fn_large && s.T >= v.ke.large_rows) fn = v.fn_large;  // many rows: add+RMSNorm's bulk-copy
-                                                              // kernel, RoPE's several rows per lane
+  if (v.ke.kind == KK_ROPE_PAIR)
+    fn = rope_entry == ROPE_BULK ? v.fn_large : (rope_entry == ROPE_MID ? v.fn_mid : v.fn);
+  else if (v.fn_large && s.T >= v.ke.large_rows)
+    fn = v.fn_large;  // many rows: add+RMSNorm's bulk-copy kernel
   return launch_on(scm, &cfg, fn, kp);
 }
 
@@ -1296,6 +1288,8 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
   v.rope = g_ops[desc->op].rope;
   st = resolve_kernel(v.d, &v.ke);
   if (st != TRIDENT_OK) return st;
+  if (v.ke.kind == KK_ROPE_PAIR)
+    rope_plans(desc->fixed[0] + 2 * desc->fixed[1], (int32_t)desc->fixed[2], &v.rope_plans);
   std::lock_guard<std::mutex> lk(scm->reg_mu);
   const int32_t n = scm->count.load(std::memory_order_relaxed);
   if (n >= scm->opt.max_specs) return fail(TRIDENT_ERR_CAPACITY, "version table full (%d)", n);
@@ -1310,27 +1304,12 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
         if (cudaGetFuncBySymbol(&h, v.ke.fn_large) != cudaSuccess || !h)
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the large-call kernel entry");
         v.fn_large = reinterpret_cast<CUfunction>(h);
-        if (v.ke.kind == KK_ROPE_HALFWARP) {
-          // the bulk-copy RoPE kernel stages ke.rows tokens' head-rows in dynamic shared memory:
-          // allow up to what the device gives a block (one setting for every version), or
-          // leave such calls to the vector kernel when a version's rows do not fit
-          const int64_t need = (int64_t)v.ke.rows * (v.d.fixed[0] + 2 * v.d.fixed[1]) * v.d.fixed[2] * 2;
-          int dev = 0, optin = 0;
-          cudaFuncAttributes fa;
-          if (cudaGetDevice(&dev) != cudaSuccess ||
-              cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-              cudaFuncGetAttributes(&fa, v.ke.fn_large) != cudaSuccess)
-            return fail(TRIDENT_ERR_CUDA, "cannot read the shared-memory limits");
-          const int64_t room = (int64_t)optin - (int64_t)fa.sharedSizeBytes;
-          if (need > room) {
-            v.fn_large = nullptr;
-          } else if (cudaFuncSetAttribute(v.ke.fn_large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) !=
-                         cudaSuccess ||
-                     cudaFuncSetAttribute(v.ke.fn_large, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                          (int)cudaSharedmemCarveoutMaxShared) != cudaSuccess) {
-            return fail(TRIDENT_ERR_CUDA, "cannot set the RoPE kernel's shared-memory size");
-          }
-        }
+      }
+      if (v.ke.fn_mid) {
+        cudaFunction_t m = nullptr;
+        if (cudaGetFuncBySymbol(&m, v.ke.fn_mid) != cudaSuccess || !m)
+          return fail(TRIDENT_ERR_CUDA, "cannot resolve the mid-size RoPE kernel entry");
+        v.fn_mid = reinterpret_cast<CUfunction>(m);
       }
       if (v.ke.fn_inplace) {
         cudaFunction_t g = nullptr;

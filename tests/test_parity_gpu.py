@@ -400,6 +400,19 @@ def test_rope_kv_many_tokens(S, T, Hq, Hkv, D, S_, qk, dtype, layout):
     check_rope(ref, got, inp, dtype)
 
 
+@pytest.mark.parametrize("T,Hq,Hkv,D,qk,dtype", [
+    (38, 32, 8, 128, True, BF16), (39, 32, 8, 128, False, FP16),   # both sides of the one-row limit
+    (511, 5, 1, 128, True, BF16), (300, 3, 2, 256, True, FP16),    # head-rows that fill no whole item
+    (511, 1, 1, 64, False, BF16), (512, 1, 1, 64, True, FP16),     # both sides of the bulk-copy limit
+    (777, 13, 1, 256, True, BF16)])
+def test_rope_kv_item_edges(S, T, Hq, Hkv, D, qk, dtype):
+    """Warp items of one, two and three head-rows per lane group at the limits of their ranges,
+    with q, k and v rows meeting inside an item and a last item only partly filled."""
+    ref, got, inp = run_rope(S, T, Hq, Hkv, D, 1024, 5e5, qk, dtype=dtype, layout="fused", seed=T + Hq)
+    assert got["status"] == 0 and ref["bad"] == 0
+    check_rope(ref, got, inp, dtype)
+
+
 def test_rope_kv_many_tokens_bad_positions(S):
     T = 603
     pos = synth.positions(np.random.default_rng(5), T, 8192)
