@@ -150,7 +150,8 @@ typedef enum trident_layout {
 /* Kernel family of a version. AUTO picks VECTOR when the version allows it. */
 typedef enum trident_variant {
   TRIDENT_VARIANT_AUTO = 0,
-  TRIDENT_VARIANT_GENERIC = 1,  /* scalar element access: any alignment, any row width  */
+  TRIDENT_VARIANT_GENERIC = 1,  /* any alignment, any row width (16-byte accesses only
+                                   where a call's own alignment allows them)            */
   TRIDENT_VARIANT_VECTOR = 2    /* 128/256-bit accesses: align_bytes 16, supported sizes */
 } trident_variant;
 

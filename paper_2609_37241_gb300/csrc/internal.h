@@ -45,9 +45,15 @@ struct RmsNormParams {
   int32_t prefetch;
 };
 
-// Pointwise operators over T rows of W elements (a: x or the first addend; b: the second
-// addend; mask: u8 for MASKED_FILL). Row strides in elements.
-enum PointwiseOp : int32_t { PW_SILU = 8, PW_ADD = 9, PW_NEG = 10, PW_MASKED_FILL = 11 };
+// Elementwise operators over T rows of W elements (a: x, the first addend or the gate; b: the
+// second addend or up; mask: u8 for MASKED_FILL). Row strides in elements. The vector kernels
+// run over `units` 16-byte vectors of y:
+//   flat  dense tensors that all start at the same offset from a 16-byte boundary, taken as
+//         one row of T * W elements: `peel` elements before the first boundary, units vectors,
+//         `tail` elements after them
+//   rows  16-byte aligned rows of `row_vecs` vectors (units = T * row_vecs); the row of a
+//         vector by fast_div where units < 2^31
+enum PointwiseOp : int32_t { PW_SWIGLU = 4, PW_SILU = 8, PW_ADD = 9, PW_NEG = 10, PW_MASKED_FILL = 11 };
 struct PointwiseParams {
   const void* a;
   const void* b;
@@ -57,6 +63,11 @@ struct PointwiseParams {
   int64_t a_rs, b_rs, m_rs, y_rs;
   float scalar;
   int32_t prefetch;
+  int64_t units, row_vecs;
+  int32_t peel, tail;
+  int32_t mask_vec;   // masks can be read a vector's elements at a time (aligned)
+  uint32_t magic;     // division by row_vecs (rows kernel) or by W (generic kernel)
+  int32_t shift;
 };
 
 // RoPE on q/k (optionally after per-head RMSNorm) plus KV-cache append.
@@ -92,7 +103,7 @@ struct RopeBulkParams {
                               // TRIDENT_OPT_TEST_WAIT_TIMEOUT)
 };
 
-// out = silu(g) * u over T rows of I elements.
+// out = silu(g) * u over T rows of I elements (the layer chain's role).
 struct SwigluParams {
   const void* g;
   const void* u;
@@ -144,6 +155,13 @@ struct ChainStepParams {
   ChainParams c[kStepMax];
 };
 
+// Elementwise entries (pointwise_plan): flat and rows kernels with one or two vectors per
+// thread, and the generic kernel.
+enum PointwiseEntry : int32_t { PW_FLAT, PW_FLAT2, PW_ROWS, PW_ROWS2, PW_GENERIC, kPwEntries };
+// Picks the entry of a call (index into pw_fn) from its packed params, fills their vector
+// fields and sets the grid. eb: element size.
+int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks);
+
 // Kernel entry (host stub address) plus its launch shape rule.
 struct KernelEntry {
   const void* fn = nullptr;
@@ -156,6 +174,7 @@ struct KernelEntry {
   const void* fn_large = nullptr;  // add+RMSNorm: the entry for calls of >= large_rows rows;
                                    // RoPE: the bulk-copy entry
   const void* fn_mid = nullptr;    // RoPE: the entry between fn and fn_large (rope_plan chooses)
+  const void* pw_fn[kPwEntries] = {};  // elementwise, by PointwiseEntry
   int32_t large_rows = 0;
   int32_t kind = 0;      // which grid rule the host applies (KernelKind)
   int32_t vec = 0;       // elements per vector (VE), or tile width for SwiGLU
@@ -167,8 +186,7 @@ enum KernelKind : int32_t {
   KK_ADDNORM_ROW = 1,   // grid = T rows, one block per row
   KK_ROPE_PAIR = 2,     // vector: grid by rope_plan
   KK_ROPE_WARP = 3,     // generic: one warp per head-row
-  KK_SWIGLU_TILE = 4,   // grid = (tiles per row, rows)
-  KK_SWIGLU_FLAT = 5,   // generic: flat grid-stride
+  KK_POINTWISE = 4,     // flat, rows or generic entry by the call's layout (pw_fn)
   KK_CHAIN = 6,
   KK_NORM_ROWS = 7      // grid = ceil(T / rows): several rows per block
 };
@@ -180,7 +198,6 @@ bool pointwise_kernel(int32_t op, int32_t dtype, int32_t variant, int64_t W, Ker
                       const char** why);
 bool rope_kernel(int32_t dtype, int32_t variant, int32_t D, bool qknorm, KernelEntry* out,
                  const char** why);
-bool swiglu_kernel(int32_t dtype, int32_t variant, int64_t I, KernelEntry* out, const char** why);
 bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry* out,
                   const char** why);
 const void* empty_kernel_entry();  // the latency-floor probe's kernel (does nothing)

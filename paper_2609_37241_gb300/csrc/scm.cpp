@@ -397,6 +397,7 @@ struct Version {
   CUfunction fn_large;          // add+RMSNorm, RoPE: entry for calls of >= ke.large_rows rows
   CUfunction fn_mid;            // RoPE: entry between fn and fn_large (rope_plan)
   RopePlans rope_plans;         // vector RoPE: item splits of its three entries
+  CUfunction pw_fn[kPwEntries];  // elementwise: entries by layout and size (pointwise_plan)
   CUfunction step_fn;           // layer chain: several calls per launch (two blocks per token)
   CUfunction step_fn_inplace;   // ... one block per token
   CUfunction step_fn_role;      // ... one block per token, role-major order over the step
@@ -593,16 +594,17 @@ void pack_rmsnorm(const trident_args* a, const Sig& s, RmsNormParams* p) {
 void pack_pointwise(const trident_args* a, const Sig& s, PointwiseParams* p) {
   const trident_tensor* t = a->t;
   const int op = a->op;
-  const int yi = (op == TRIDENT_OP_SILU || op == TRIDENT_OP_NEG) ? 1 : 2;
+  const bool binary = op == TRIDENT_OP_ADD || op == TRIDENT_OP_SWIGLU, masked = op == TRIDENT_OP_MASKED_FILL;
+  const int yi = binary || masked ? 2 : 1;
   p->a = t[0].data;
-  p->b = op == TRIDENT_OP_ADD ? t[1].data : nullptr;
-  p->mask = op == TRIDENT_OP_MASKED_FILL ? (const uint8_t*)t[1].data : nullptr;
+  p->b = binary ? t[1].data : nullptr;
+  p->mask = masked ? (const uint8_t*)t[1].data : nullptr;
   p->y = t[yi].data;
   p->T = s.T;
   p->W = s.fixed[0];
   p->a_rs = row_stride(t[0], K_ACT_H);
-  p->b_rs = op == TRIDENT_OP_ADD ? row_stride(t[1], K_ACT_H) : 0;
-  p->m_rs = op == TRIDENT_OP_MASKED_FILL ? row_stride(t[1], K_MASK_H) : 0;
+  p->b_rs = binary ? row_stride(t[1], K_ACT_H) : 0;
+  p->m_rs = masked ? row_stride(t[1], K_MASK_H) : 0;
   p->y_rs = row_stride(t[yi], K_ACT_H);
   p->scalar = (float)a->scalar;
   p->prefetch = 0;
@@ -766,13 +768,13 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     PointwiseParams pw;
     RopeParams rp;
     RopeBulkParams rb;  // rb.rp is rp
-    SwigluParams sw;
     ChainParams ch;
   } P;
   void* kp[1] = {&P};
   bool late = false;  // layer chain: launch fn_late (the late launch trigger)
   bool wide = false;  // layer chain: launch fn_wide (wider SwiGLU tiles)
   RopeEntry rope_entry = ROPE_SMALL;
+  int pw_entry = PW_GENERIC;
   switch (op) {
     case TRIDENT_OP_ADD_RMSNORM:
       pack_addnorm(a, 0, 1, 2, 3, 4, s, K_ACT_H, &P.an);
@@ -806,22 +808,10 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     case TRIDENT_OP_ADD:
     case TRIDENT_OP_NEG:
     case TRIDENT_OP_MASKED_FILL: {
-      int64_t W;
-      if (op == TRIDENT_OP_SWIGLU) {
-        pack_swiglu(a, 0, 1, 2, s.T, &P.sw);
-        W = P.sw.I;
-      } else {
-        pack_pointwise(a, s, &P.pw);
-        W = P.pw.W;
-      }
-      if (v.ke.kind == KK_SWIGLU_TILE) {  // (column tiles, rows)
-        const int64_t per = (int64_t)v.ke.unroll * kThreads * v.ke.vec;
-        cfg.gridDimX = cap_grid((W + per - 1) / per);
-        cfg.gridDimY = (unsigned)(s.T < 65535 ? (s.T < 1 ? 1 : s.T) : 65535);
-      } else {  // flat grid-stride
-        const int64_t blocks = (s.T * W + kThreads - 1) / kThreads;
-        cfg.gridDimX = cap_grid(blocks < 152 * 64 ? blocks : 152 * 64);
-      }
+      pack_pointwise(a, s, &P.pw);
+      int64_t blocks = 0;
+      pw_entry = pointwise_plan(&P.pw, op, elem_size(v.d.dtype), &blocks);
+      cfg.gridDimX = cap_grid(blocks);
       break;
     }
     case TRIDENT_OP_LAYER_CHAIN:
@@ -890,7 +880,6 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     case TRIDENT_OP_RMSNORM: P.rn.prefetch = pf; break;
     case TRIDENT_OP_ROPE_KV:
     case TRIDENT_OP_QKNORM_ROPE_KV: P.rp.prefetch = pf; break;
-    case TRIDENT_OP_SWIGLU: P.sw.prefetch = pf; break;
     case TRIDENT_OP_LAYER_CHAIN:
     case TRIDENT_OP_LAYER_CHAIN_QKNORM: P.ch.prefetch = chain_prefetch_mode(pdl, pf != 0 && !late, true); break;
     default: P.pw.prefetch = pf; break;
@@ -900,7 +889,9 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     fn = wide ? v.fn_wide : v.fn_inplace;
   else if (late && v.fn_late)
     fn = v.fn_late;
-  if (v.ke.kind == KK_ROPE_PAIR)
+  if (v.ke.kind == KK_POINTWISE)
+    fn = v.pw_fn[pw_entry];
+  else if (v.ke.kind == KK_ROPE_PAIR)
     fn = rope_entry == ROPE_BULK ? v.fn_large : (rope_entry == ROPE_MID ? v.fn_mid : v.fn);
   else if (v.fn_large && s.T >= v.ke.large_rows)
     fn = v.fn_large;  // many rows: add+RMSNorm's bulk-copy kernel
@@ -1145,8 +1136,8 @@ int32_t resolve_kernel(const trident_spec_desc& d, KernelEntry* ke) {
       case TRIDENT_OP_SILU:
       case TRIDENT_OP_ADD:
       case TRIDENT_OP_NEG:
-      case TRIDENT_OP_MASKED_FILL: return pointwise_kernel(d.op, d.dtype, var, d.fixed[0], ke, &why);
-      case TRIDENT_OP_SWIGLU: return swiglu_kernel(d.dtype, var, d.fixed[0], ke, &why);
+      case TRIDENT_OP_MASKED_FILL:
+      case TRIDENT_OP_SWIGLU: return pointwise_kernel(d.op, d.dtype, var, d.fixed[0], ke, &why);
       case TRIDENT_OP_ROPE_KV:
       case TRIDENT_OP_QKNORM_ROPE_KV:
         return rope_kernel(d.dtype, var, (int32_t)d.fixed[2], d.op == TRIDENT_OP_QKNORM_ROPE_KV, ke, &why);
@@ -1304,6 +1295,14 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
         if (cudaGetFuncBySymbol(&h, v.ke.fn_large) != cudaSuccess || !h)
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the large-call kernel entry");
         v.fn_large = reinterpret_cast<CUfunction>(h);
+      }
+      if (v.ke.kind == KK_POINTWISE) {
+        for (int k = 0; k < kPwEntries; ++k) {
+          cudaFunction_t e = nullptr;
+          if (cudaGetFuncBySymbol(&e, v.ke.pw_fn[k]) != cudaSuccess || !e)
+            return fail(TRIDENT_ERR_CUDA, "cannot resolve the elementwise kernel entries");
+          v.pw_fn[k] = reinterpret_cast<CUfunction>(e);
+        }
       }
       if (v.ke.fn_mid) {
         cudaFunction_t m = nullptr;

@@ -295,6 +295,49 @@ def test_pointwise_parity(S, name, dtype, W, T, layout, variant):
         P.check_act(got, ref, ref_bits, dtype, name, exact_frac=0.99)
 
 
+@pytest.mark.parametrize("name", ["silu", "add", "neg", "masked_fill", "swiglu"])
+@pytest.mark.parametrize("dtype,T,W,form", [
+    (BF16, 1, 3, "offset"), (BF16, 1, 9, "offset"),        # shorter than a head; a head and a tail
+    (BF16, 37, 1001, "dense"), (FP16, 5, 2047, "offset"),  # odd widths as one long row
+    (FP32, 3, 4099, "offset"), (BF16, 255, 8, "padded"),   # vectors of many short rows
+    (FP16, 130, 264, "padded"), (FP32, 70, 516, "padded"),
+    (BF16, 9, 520, "mask"),                                # a mask row no vector of it can read
+    (BF16, 11, 96, "apart"), (FP32, 6, 77, "rows"),        # offsets that differ; odd row strides
+    (BF16, 1200, 4096, "dense"), (FP16, 1200, 4096, "padded")])  # two vectors per thread
+def test_elementwise_layouts(S, name, dtype, T, W, form):
+    """Every path of the elementwise operators' layout rule, against the oracle: dense tensors
+    with a common offset, aligned row views, and tensors neither covers."""
+    g = np.random.default_rng(W + T)
+    tdt = synth._TORCH_DT[dtype]
+    pad = {"padded": 64, "rows": 3}.get(form, 0)
+    off = {"offset": 1, "rows": 1}.get(form, 0)
+
+    def place(t, extra=0):
+        o = off + extra
+        buf = torch.zeros(T * (W + pad) + o + 16, dtype=t.dtype, device="cuda")
+        view = buf[o:o + T * (W + pad)].view(T, W + pad)[:, :W]
+        return view.copy_(t)
+
+    a, b = synth.act(g, (T, W), dtype, std=3.0), synth.act(g, (T, W), dtype)
+    mask = (g.random((T, W)) < 0.4).astype(np.uint8)
+    ad, bd = place(P.dev(a, dtype)), place(P.dev(b, dtype))
+    yd = place(torch.zeros((T, W), dtype=tdt, device="cuda"), extra=2 if form == "apart" else 0)
+    md = place(torch.from_numpy(mask).cuda(), extra=1 if form == "mask" else 0)
+    op, ts = {"silu": (S.OP_SILU, [ad, yd]), "neg": (S.OP_NEG, [ad, yd]), "add": (S.OP_ADD, [ad, bd, yd]),
+              "masked_fill": (S.OP_MASKED_FILL, [ad, md, yd]), "swiglu": (S.OP_SWIGLU, [ad, bd, yd])}[name]
+    desc = S.make_spec(op, dtype, [W], 1, 1 << 20, layout=S.LAYOUT_ANY,
+                       align_bytes=4 if dtype == FP32 else 2)
+    invoke_ok(one_version_scm(S, desc), S, S.make_args(op, ts, scalar=-2.5))
+    got = P.host_bits(yd, dtype)
+    if name in ("silu", "swiglu"):
+        ref, ref_bits = L.silu(a, dtype) if name == "silu" else L.swiglu(a, b, dtype)
+        P.check_act(got, ref, ref_bits, dtype, f"{name} {dtype} {T}x{W} {form}")
+    else:
+        ref_bits = {"add": lambda: L.add(a, b, dtype), "neg": lambda: L.neg(a, dtype),
+                    "masked_fill": lambda: L.masked_fill(a, mask, -2.5, dtype)}[name]()[1]
+        assert np.array_equal(got, ref_bits), (name, dtype, T, W, form)
+
+
 def test_pointwise_in_place(S):
     g = np.random.default_rng(21)
     a = synth.act(g, (8, 4096), BF16)
