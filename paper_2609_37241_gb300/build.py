@@ -15,7 +15,7 @@ INC = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libtrident_scm.so")
-SOURCES = ["scm.cpp", "tree.cpp", "addnorm.cu", "rmsnorm.cu", "rope.cu", "pointwise.cu", "chain.cu",
+SOURCES = ["scm.cpp", "tree.cpp", "norm.cu", "rope.cu", "pointwise.cu", "chain.cu",
            "noalloc.cu"]
 HEADERS = ["internal.h", "device_common.cuh", "tree.h", "measure.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -41,8 +41,8 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
     __shared__ float2 red[kThreads / 32];
     constexpr int PP = VPT / SPLIT;  // vectors per thread this CTA writes
     static_assert(VPT % SPLIT == 0, "split");
-    const AddNormParams& n1 = c.n1;
-    const AddNormParams& n2 = c.n2;
+    const NormParams& n1 = c.n1;
+    const NormParams& n2 = c.n2;
     uint4 hv[VPT], rv[VPT], av[VPT];
     float ga[PP][VE], gm[PP][VE];
     const uint4* hp = reinterpret_cast<const uint4*>(row_ptr(n1.x, row, n1.x_rs, EB));

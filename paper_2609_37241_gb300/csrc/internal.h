@@ -14,8 +14,9 @@ enum : int32_t { DT_BF16 = 1, DT_FP16 = 2, DT_FP32 = 3 };
 
 constexpr int kThreads = 256;  // block size of every kernel in this library
 
-// add + RMSNorm over T rows of H elements. Row strides in elements.
-struct AddNormParams {
+// RMSNorm over T rows of H elements, with a residual add or without (r, r_out unused). Row
+// strides in elements.
+struct NormParams {
   const void* x;
   const void* r;
   const float* gamma;
@@ -25,6 +26,7 @@ struct AddNormParams {
   int64_t x_rs, r_rs, y_rs, ro_rs;
   float eps, inv_H;
   int32_t prefetch;  // 1: prefetch this block's first lines into L2 before the PDL wait
+  int32_t nvec;      // whole 16-byte vectors per row (H / VE)
   uint32_t first_wait_polls;  // bulk-copy kernel: polls of its first wait for the copies
                               // (kBulkWaitPolls; 0 under TRIDENT_OPT_TEST_WAIT_TIMEOUT)
   uint32_t* err;     // device status word (the bulk-copy kernel reports a timed-out wait)
@@ -33,17 +35,6 @@ struct AddNormParams {
 // Bound of every mbarrier wait of the bulk-copy kernel (try_wait polls, each itself bounded
 // by the hardware's suspend time).
 constexpr uint32_t kBulkWaitPolls = 1u << 20;
-
-// RMSNorm over T rows of H elements (no residual). Row strides in elements.
-struct RmsNormParams {
-  const void* x;
-  const float* gamma;
-  void* y;
-  int64_t T, H;
-  int64_t x_rs, y_rs;
-  float eps, inv_H;
-  int32_t prefetch;
-};
 
 // Elementwise operators over T rows of W elements (a: x, the first addend or the gate; b: the
 // second addend or up; mask: u8 for MASKED_FILL). Row strides in elements. The vector kernels
@@ -116,8 +107,8 @@ struct SwigluParams {
 // One decoder layer's chain in one launch. Blocks [0, nA) run the two add+RMSNorm steps
 // of one token each, [nA, nA+nB) the RoPE/KV head-rows, the rest SwiGLU tiles.
 struct ChainParams {
-  AddNormParams n1;   // h, r0 -> x1, r1
-  AddNormParams n2;   // attn_out, (r1 from registers) -> x2, r2; n2.r is unused
+  NormParams n1;   // h, r0 -> x1, r1
+  NormParams n2;   // attn_out, (r1 from registers) -> x2, r2; n2.r is unused
   RopeParams rope;
   SwigluParams sw;
   int32_t nA, nB, nC, sw_tiles_per_row;
@@ -162,6 +153,11 @@ enum PointwiseEntry : int32_t { PW_FLAT, PW_FLAT2, PW_ROWS, PW_ROWS2, PW_GENERIC
 // fields and sets the grid. eb: element size.
 int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks);
 
+// Norm entries (norm_plan): 16-byte aligned rows, rows at any common offset, scalar accesses,
+// and the entry of long calls (bulk copies, or two rows at a time for short rows).
+constexpr int kNormBlockVecs = 2048;  // norm_block_kernel, norm_bulk_kernel: vectors of a row at most
+enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_GENERIC, NM_LARGE, kNormEntries };
+
 // Kernel entry (host stub address) plus its launch shape rule.
 struct KernelEntry {
   const void* fn = nullptr;
@@ -171,35 +167,39 @@ struct KernelEntry {
   const void* fn_step_role = nullptr;  // chain only: fn_step_inplace, role-major block order
   const void* fn_step = nullptr;          // chain only: several calls per launch (ChainStepParams)
   const void* fn_step_inplace = nullptr;  // ... one block per token for the norms
-  const void* fn_large = nullptr;  // add+RMSNorm: the entry for calls of >= large_rows rows;
-                                   // RoPE: the bulk-copy entry
+  const void* fn_large = nullptr;  // RoPE: the bulk-copy entry (rope_plan chooses)
   const void* fn_mid = nullptr;    // RoPE: the entry between fn and fn_large (rope_plan chooses)
   const void* pw_fn[kPwEntries] = {};  // elementwise, by PointwiseEntry
-  int32_t large_rows = 0;
+  int64_t large_rows = 0;  // norms: rows from which a call takes the NM_LARGE entry
+  int32_t large_per = 1;   // ... that entry's rows per block
+  int32_t large_smem = 0;  // ... and its dynamic shared memory (rows staged by bulk copies)
   int32_t kind = 0;      // which grid rule the host applies (KernelKind)
   int32_t vec = 0;       // elements per vector (VE), or tile width for SwiGLU
   int32_t unroll = 1;    // vectors per thread per tile (SwiGLU, chain)
-  int32_t rows = 1;      // rows per block (KK_NORM_ROWS)
+  const void* nm_fn[kNormEntries] = {};  // norms, by NormEntry (NULL: none for this H)
+  int32_t nm_threads[kNormEntries] = {};
+  int32_t rows = 1;      // norms: rows per block of the NM_VEC entry
 };
 
 enum KernelKind : int32_t {
-  KK_ADDNORM_ROW = 1,   // grid = T rows, one block per row
+  KK_NORM = 1,          // entry, block size and grid by norm_plan
   KK_ROPE_PAIR = 2,     // vector: grid by rope_plan
   KK_ROPE_WARP = 3,     // generic: one warp per head-row
   KK_POINTWISE = 4,     // flat, rows or generic entry by the call's layout (pw_fn)
-  KK_CHAIN = 6,
-  KK_NORM_ROWS = 7      // grid = ceil(T / rows): several rows per block
+  KK_CHAIN = 6
 };
 
 // Lookup of compiled kernels. Return false (with a reason) if no kernel fits.
-bool addnorm_kernel(int32_t dtype, int32_t variant, int64_t H, KernelEntry* out, const char** why);
-bool rmsnorm_kernel(int32_t dtype, int32_t variant, int64_t H, KernelEntry* out, const char** why);
+bool norm_kernel(bool res, int32_t dtype, int32_t variant, int64_t H, KernelEntry* out, const char** why);
 bool pointwise_kernel(int32_t op, int32_t dtype, int32_t variant, int64_t W, KernelEntry* out,
                       const char** why);
 bool rope_kernel(int32_t dtype, int32_t variant, int32_t D, bool qknorm, KernelEntry* out,
                  const char** why);
 bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry* out,
                   const char** why);
+// The entry a call takes from its packed params (sets p->nvec), its block size and grid.
+NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, int32_t* threads, int64_t* blocks,
+                    int32_t* smem);
 const void* empty_kernel_entry();  // the latency-floor probe's kernel (does nothing)
 
 // Validation, guard-equivalent checks (sizes, layouts, 16-byte alignment, overlap) and

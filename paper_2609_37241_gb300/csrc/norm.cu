@@ -1,0 +1,558 @@
+// norm.cu -- RMSNorm, with or without a fused residual add (sm_103a).
+//
+//   RMSNORM      y = round(x * rsqrt(mean(x^2) + eps) * gamma)
+//   ADD_RMSNORM  s = x + r (fp32);  r_out = round(s);  y = round(s * rsqrt(mean(s^2) + eps) * gamma)
+//
+// rms_norm is the paper's running example (Fig. 1, §2.3; its motivation experiment uses
+// x (1024, 128)); the residual add fused in front of it is how decoder layers call it. All
+// kernels but the last two read a row once and write it once:
+//   norm_rows_kernel   rows of at most 128 vectors: LPR lanes per row, reduced by shuffles alone
+//   norm_block_kernel  longer rows, one block per row, one or two vectors per thread, one barrier.
+//                      EDGE: rows at any element offset that all tensors share (odd widths,
+//                      shifted bases), the vectors between a scalar head and tail
+//   norm_bulk_kernel   long calls of such rows: the row staged by bulk copies
+//   addnorm_row_kernel long ADD_RMSNORM calls of H = 4096 in 16 bits
+//   norm_loop_kernel   16-byte rows of more than 2048 vectors (two passes)
+//   norm_generic_kernel  anything else (scalar accesses)
+//
+// Bound: HBM for long calls; below about a thousand rows the launch and one row's dependent
+// phases (load, reduce, scale, store). Before, only power-of-two widths kept their row in
+// registers, in blocks of 256 threads; other widths read it twice, in a loop, and odd widths went
+// element by element. Device time per call, before -> now:
+//   add 1 x 4096 bf16      1.48 -> 1.03 us     rms 131072 x 128 bf16    15.6 -> 12.1 us
+//   add 24 x 5120 bf16     2.72 -> 1.35        rms 30000 x 192 bf16     32.0 -> 5.1
+//   add 64 x 8192 bf16     3.11 -> 1.83        rms 2050 x 3000 fp32     10.9 -> 8.7
+//   add 256 x 4096 bf16    3.17 -> 1.95        rms 4096 x 4096 bf16     12.9 -> 11.7
+//   add 3001 x 5120 bf16   23.7 -> 19.6        rms 16384 x 5120 bf16    59.5 -> 50.7
+//   add 4096 x 8192 bf16   40.4 -> 40.1        rms 2000 x 16384 fp16    36.1 -> 23.7
+//   add 4096 x 12288 bf16  65.1 -> 59.4        add 3000 x 2585 bf16     21.3 -> 14.3
+//   add 20000 x 576 bf16   34.9 -> 19.4        rms 1 x 4096 bf16        1.39 -> 1.11
+// The long residual rows run at the 6.8 TB/s copy rate (4096 x 8192: 6.7, 4096 x 12288: 6.8).
+#include "device_common.cuh"
+
+namespace trident {
+// Long calls take norm_bulk_kernel (or addnorm_row_kernel) from this many bytes of x, with a
+// residual add / without; norm_block_kernel against norm_bulk_kernel, bf16: with it 600 x 8192
+// 7.7 / 8.1, 1000 x 8192 14.0 / 11.9 us; 600 x 5120 5.7 / 5.8, 1000 x 5120 9.0 / 8.4; without
+// 1000 x 4096 4.2 / 4.9, 1600 x 4096 6.2 / 5.8; 600 x 8192 4.9 / 5.2, 1000 x 8192 8.7 / 7.8. fp32
+// residual rows of up to 1024 vectors stay with one vector per thread (2995 x 4096 28.6 / 30.2).
+constexpr int64_t kNormBulkResBytes = 8 << 20;
+constexpr int64_t kNormBulkBytes = 10 << 20;
+// Two rows per lane group of norm_rows_kernel (no residual, one vector per lane) from this many
+// vectors of x: half the threads have twice the loads in flight (16384 x 128 3.26 -> 2.90 us,
+// 131072 x 128 15.3 -> 12.1; 8192 x 64, below the line, 1.98 / 2.16).
+constexpr int64_t kNormRows2Vecs = 152 * 1024;
+
+template <int DT>
+__device__ __forceinline__ void load_gamma(const float* g, float* out) {
+#pragma unroll
+  for (int q = 0; q < Act<DT>::VE / 4; ++q) {
+    const float4 v = ldg_f4(g + 4 * q);
+    out[4 * q] = v.x; out[4 * q + 1] = v.y; out[4 * q + 2] = v.z; out[4 * q + 3] = v.w;
+  }
+}
+
+// LPR lanes per row, VPT vectors per lane (VPT > 1 only with 32 lanes); lane l owns the
+// vectors l + LPR * v. FULL: the lanes' vectors are exactly the row's. R rows per lane group at
+// a time, their loads issued together.
+template <int DT, bool RES, int LPR, int VPT, bool FULL, int R>
+__global__ void __launch_bounds__(kThreads) norm_rows_kernel(const NormParams p) {
+  pdl_trigger();
+  constexpr int VE = Act<DT>::VE;
+  constexpr int EB = Act<DT>::BYTES;
+  constexpr int RPB = kThreads / LPR;
+  const int lane = threadIdx.x % LPR;
+  const unsigned mask =
+      (LPR == 32) ? 0xffffffffu : (((1u << LPR) - 1u) << ((threadIdx.x & 31) & ~(LPR - 1)));
+  const int64_t row0 = (int64_t)blockIdx.x * (RPB * R) + threadIdx.x / LPR;
+  if (p.prefetch && (lane & 7) == 0) {  // the first row's lines (prefetch_l2)
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      const int vi = lane + LPR * v;
+      if (row0 < p.T && vi < p.nvec) {
+        prefetch_l2(row_ptr(p.x, row0, p.x_rs, EB) + vi * 16);
+        if (RES) prefetch_l2(row_ptr(p.r, row0, p.r_rs, EB) + vi * 16);
+      }
+    }
+  }
+  pdl_wait();
+  for (int64_t base = row0; base < p.T; base += (int64_t)gridDim.x * (RPB * R)) {
+    uint4 xv[R][VPT], rv[R][VPT];
+    float g[VPT][VE];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const int64_t row = R == 1 ? base : min(base + k * RPB, p.T - 1);
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        const int vi = lane + LPR * v;
+        if (FULL || vi < p.nvec) {
+          xv[k][v] = ldg16(row_ptr(p.x, row, p.x_rs, EB) + vi * 16);
+          if (RES) rv[k][v] = ldg16(row_ptr(p.r, row, p.r_rs, EB) + vi * 16);
+          if (k == 0) load_gamma<DT>(p.gamma + vi * VE, g[v]);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const int64_t row = base + k * RPB;
+      const bool on = R == 1 || row < p.T;
+      float s[VPT][VE], ss = 0.f;
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        const int vi = lane + LPR * v;
+        if (FULL || vi < p.nvec) {
+          unpack<DT>(xv[k][v], s[v]);
+          if (RES) {
+            float rf[VE];
+            unpack<DT>(rv[k][v], rf);
+#pragma unroll
+            for (int e = 0; e < VE; ++e) s[v][e] += rf[e];
+            if (on) st16(row_ptr(p.r_out, row, p.ro_rs, EB) + vi * 16, pack<DT>(s[v]));
+          }
+#pragma unroll
+          for (int e = 0; e < VE; ++e) ss = fmaf(s[v][e], s[v][e], ss);
+        }
+      }
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(mask, ss, o, LPR);
+      const float inv = rsqrtf(ss * p.inv_H + p.eps);
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        const int vi = lane + LPR * v;
+        if (FULL || vi < p.nvec) {
+#pragma unroll
+          for (int e = 0; e < VE; ++e) s[v][e] = s[v][e] * inv * g[v][e];
+          if (on) st16(row_ptr(p.y, row, p.y_rs, EB) + vi * 16, pack<DT>(s[v]));
+        }
+      }
+    }
+  }
+}
+
+// Sum over a block of any number of whole warps; every thread gets the same total. Up to 16
+// warps by reading every warp's sum, beyond by a second round of shuffles.
+__device__ __forceinline__ float norm_block_sum(float v, float* red) {
+  const int nw = blockDim.x >> 5;
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  if (threadIdx.x < 32 && (int)threadIdx.x >= nw) red[threadIdx.x] = 0.f;
+  __syncthreads();
+  if (nw <= 16) {
+    const float4* r4 = reinterpret_cast<const float4*>(red);
+    const float4 a = r4[0], b = r4[1], c = r4[2], d = r4[3];
+    return ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w)) +
+           (((c.x + c.y) + (c.z + c.w)) + ((d.x + d.y) + (d.z + d.w)));
+  }
+  return warp_sum(red[threadIdx.x & 31]);
+}
+
+// Thread `tid` owns the row's vectors tid + blockDim.x * v, v < VPT. One vector per thread where
+// the row allows it: at call sizes where latency counts, more threads with less each are faster
+// (24 x 5120 1.35 us against 1.8 with two and 2.1 with four). Threads past the row's end load its
+// last vector and drop it: with the loads behind a branch the compiler finished them before
+// leaving it (256 x 4096 3.3 us). FULL: no such threads. EDGE: the row's tensors
+// start at one common offset from a 16-byte boundary; the first peel and last tail elements
+// (fewer than a vector each) go to threads of their own, and gamma is read by element.
+template <int DT, bool RES, int VPT, bool EDGE, bool FULL>
+__global__ void __launch_bounds__(1024) norm_block_kernel(const NormParams p) {
+  pdl_trigger();
+  __shared__ __align__(16) float red[32];
+  constexpr int VE = Act<DT>::VE;
+  constexpr int EB = Act<DT>::BYTES;
+  const int tid = threadIdx.x;
+  const int64_t row = blockIdx.x;
+  const char* xr = row_ptr(p.x, row, p.x_rs, EB);
+  const char* rr = RES ? row_ptr(p.r, row, p.r_rs, EB) : nullptr;
+  int nvec = p.nvec, peel = 0, edge = -1;  // edge: this thread's scalar element
+  if (EDGE) {
+    peel = (int)((16 - (reinterpret_cast<uintptr_t>(xr) & 15)) & 15) / EB;
+    if (peel > p.H) peel = (int)p.H;
+    nvec = (int)(p.H - peel) / VE;
+    const int tail = (int)p.H - peel - nvec * VE;
+    if (tid < peel) edge = tid;
+    else if (tid < peel + tail) edge = nvec * VE + tid;
+    xr += peel * EB;
+    if (RES) rr += peel * EB;
+  }
+  if (p.prefetch && (tid & 7) == 0) {  // the row's lines (prefetch_l2)
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      const int vi = tid + (int)blockDim.x * v;
+      if (vi < nvec) {
+        prefetch_l2(xr + (int64_t)vi * 16);
+        if (RES) prefetch_l2(rr + (int64_t)vi * 16);
+      }
+    }
+  }
+  pdl_wait();
+  uint4 xv[VPT], rv[VPT];
+  float g[VPT][VE], s[VPT][VE], es = 0.f, eg = 0.f;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = FULL ? tid + (int)blockDim.x * v : min(tid + (int)blockDim.x * v, nvec - 1);
+    xv[v] = ldg16(xr + (int64_t)vi * 16);
+    if (RES) rv[v] = ldg16(rr + (int64_t)vi * 16);
+    if (EDGE) {
+#pragma unroll
+      for (int e = 0; e < VE; ++e) g[v][e] = __ldg(p.gamma + peel + vi * VE + e);
+    } else {
+      load_gamma<DT>(p.gamma + (int64_t)vi * VE, g[v]);
+    }
+  }
+  if (EDGE && edge >= 0) {
+    es = load_elem<DT>(p.x, row * p.x_rs + edge);
+    if (RES) es += load_elem<DT>(p.r, row * p.r_rs + edge);
+    eg = __ldg(p.gamma + edge);
+  }
+  char* ro = RES ? row_ptr(p.r_out, row, p.ro_rs, EB) + peel * EB : nullptr;
+  float ss = EDGE ? es * es : 0.f;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = tid + (int)blockDim.x * v;
+    float sv[VE], sq = 0.f;
+    unpack<DT>(xv[v], sv);
+    if (RES) {
+      float rf[VE];
+      unpack<DT>(rv[v], rf);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) s[v][e] = sv[e] = sv[e] + rf[e];
+      if (FULL || vi < nvec) st16(ro + (int64_t)vi * 16, pack<DT>(sv));
+    }
+#pragma unroll
+    for (int e = 0; e < VE; ++e) sq = fmaf(sv[e], sv[e], sq);
+    ss += FULL || vi < nvec ? sq : 0.f;
+  }
+  if (EDGE && RES && edge >= 0) store_elem<DT>(p.r_out, row * p.ro_rs + edge, es);
+  const float inv = rsqrtf(norm_block_sum(ss, red) * p.inv_H + p.eps);
+  char* yr = row_ptr(p.y, row, p.y_rs, EB) + peel * EB;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = tid + (int)blockDim.x * v;
+    if (!RES) unpack<DT>(xv[v], s[v]);
+#pragma unroll
+    for (int e = 0; e < VE; ++e) s[v][e] = s[v][e] * inv * g[v][e];
+    if (FULL || vi < nvec) st16(yr + (int64_t)vi * 16, pack<DT>(s[v]));
+  }
+  if (EDGE && edge >= 0) store_elem<DT>(p.y, row * p.y_rs + edge, es * inv * eg);
+}
+
+// Long calls: the row's x (and r) are staged in shared memory by bulk copies (cp.async.bulk,
+// completion counted on an mbarrier) issued by one thread, while every thread loads its gamma
+// vectors; s = x + r is formed from shared memory twice (the same fp32 addition both times). With
+// the rows out of the registers more of them are in flight per SM. Two vectors per thread with a
+// residual (40 registers), four without, where the fewer threads leave room for more blocks
+// (16384 x 5120 50.7 us against 52-61 with two). gamma loaded after the reduction instead cost
+// 2-3 us per call. The wait is bounded: if it runs out, the block sets TRIDENT_DEVERR_TIMEOUT,
+// waits again (bounded) for its copies and returns without writing.
+template <int DT, bool RES, int VPT, bool FULL>
+__global__ void __launch_bounds__(512, RES ? (VPT == 2 ? 3 : 2) : 1) norm_bulk_kernel(const NormParams p) {
+  constexpr int VE = Act<DT>::VE;
+  constexpr int EB = Act<DT>::BYTES;
+  extern __shared__ __align__(128) uint4 s_rows[];
+  __shared__ __align__(8) unsigned long long bar;
+  __shared__ __align__(16) float red[32];
+  const int tid = threadIdx.x, nt = blockDim.x, nvec = p.nvec;
+  const int64_t row = blockIdx.x;
+  const uint32_t bar_a = (uint32_t)__cvta_generic_to_shared(&bar);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar_a) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  pdl_trigger();
+  pdl_wait();
+  if (tid == 0) {
+    const uint32_t rb = (uint32_t)nvec * 16;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                 :: "r"(bar_a), "r"((RES ? 2 : 1) * rb) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(s_rows)), "l"(row_ptr(p.x, row, p.x_rs, EB)),
+                    "r"(rb), "r"(bar_a) : "memory");
+    if (RES)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   :: "r"((uint32_t)__cvta_generic_to_shared(s_rows + nvec)), "l"(row_ptr(p.r, row, p.r_rs, EB)),
+                      "r"(rb), "r"(bar_a) : "memory");
+  }
+  float g[VPT][VE];
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) load_gamma<DT>(p.gamma + (int64_t)(FULL ? tid + nt * v : min(tid + nt * v, nvec - 1)) * VE, g[v]);
+  __syncthreads();  // the barrier is initialised before anyone waits on it
+  auto landed = [&](uint32_t polls) -> bool {
+    uint32_t done = 0;
+    for (uint32_t it = 0; it < polls && !done; ++it)
+      asm volatile("{ .reg .pred q; mbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0; selp.u32 %0, 1, 0, q; }"
+                   : "=r"(done) : "r"(bar_a) : "memory");
+    return done != 0;
+  };
+  const bool ok = landed(p.first_wait_polls);
+  if (__syncthreads_or(!ok)) {  // one decision for the whole block
+    if (tid == 0 && p.err) atomicOr(p.err, kErrTimeout);
+    if (!ok) landed(kBulkWaitPolls);  // a second bounded wait for the copies before the block exits
+    return;
+  }
+  char* ro = RES ? row_ptr(p.r_out, row, p.ro_rs, EB) : nullptr;
+  float ss = 0.f;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = tid + nt * v, vc = FULL ? vi : min(vi, nvec - 1);
+    float sv[VE], sq = 0.f;
+    unpack<DT>(s_rows[vc], sv);
+    if (RES) {
+      float rf[VE];
+      unpack<DT>(s_rows[nvec + vc], rf);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) sv[e] += rf[e];
+      if (FULL || vi < nvec) st16(ro + (int64_t)vi * 16, pack<DT>(sv));
+    }
+#pragma unroll
+    for (int e = 0; e < VE; ++e) sq = fmaf(sv[e], sv[e], sq);
+    ss += FULL || vi < nvec ? sq : 0.f;
+  }
+  const float inv = rsqrtf(norm_block_sum(ss, red) * p.inv_H + p.eps);
+  char* yr = row_ptr(p.y, row, p.y_rs, EB);
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = tid + nt * v, vc = FULL ? vi : min(vi, nvec - 1);
+    float sv[VE];
+    unpack<DT>(s_rows[vc], sv);
+    if (RES) {
+      float rf[VE];
+      unpack<DT>(s_rows[nvec + vc], rf);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) sv[e] += rf[e];
+    }
+#pragma unroll
+    for (int e = 0; e < VE; ++e) sv[e] = sv[e] * inv * g[v][e];
+    if (FULL || vi < nvec) st16(yr + (int64_t)vi * 16, pack<DT>(sv));
+  }
+}
+
+// ADD_RMSNORM, H = 4096 in bf16 / fp16, long calls: exactly two vectors per thread of 256. The
+// one width where this order of loads and stores beat the bulk copies (1600 / 3001 / 6000 rows
+// 9.25 / 15.6 / 29.1 us against 9.49 / 15.8 / 29.6; at 5120 the two-pass kernel it replaced took
+// 23.7, the bulk copies 19.6).
+template <int DT>
+__global__ void __launch_bounds__(kThreads) addnorm_row_kernel(const NormParams p) {
+  pdl_trigger();
+  __shared__ float red[kThreads / 32];
+  constexpr int VPT = 2;
+  constexpr int EB = Act<DT>::BYTES;
+  constexpr int VE = Act<DT>::VE;
+  const int tid = threadIdx.x;
+  pdl_wait();
+  for (int64_t row = blockIdx.x; row < p.T; row += gridDim.x) {
+    const uint4* xp = reinterpret_cast<const uint4*>(row_ptr(p.x, row, p.x_rs, EB));
+    const uint4* rp = reinterpret_cast<const uint4*>(row_ptr(p.r, row, p.r_rs, EB));
+    uint4 xv[VPT], rv[VPT];
+    float g[VPT][VE], s[VPT][VE];
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      const int64_t vi = (int64_t)v * kThreads + tid;
+      xv[v] = ldg16(xp + vi);
+      rv[v] = ldg16(rp + vi);
+      load_gamma<DT>(p.gamma + vi * VE, g[v]);
+    }
+    uint4* rop = reinterpret_cast<uint4*>(row_ptr(p.r_out, row, p.ro_rs, EB));
+    float ss = 0.f;
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      float xf[VE], rf[VE];
+      unpack<DT>(xv[v], xf);
+      unpack<DT>(rv[v], rf);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) {
+        s[v][e] = xf[e] + rf[e];
+        ss = fmaf(s[v][e], s[v][e], ss);
+      }
+      st16(rop + (int64_t)v * kThreads + tid, pack<DT>(s[v]));
+    }
+    const float inv = rsqrtf(block_sum(ss, red) * p.inv_H + p.eps);
+    uint4* yp = reinterpret_cast<uint4*>(row_ptr(p.y, row, p.y_rs, EB));
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      float y[VE];
+#pragma unroll
+      for (int e = 0; e < VE; ++e) y[e] = s[v][e] * inv * g[v][e];
+      st16(yp + (int64_t)v * kThreads + tid, pack<DT>(y));
+    }
+    __syncthreads();  // `red` is reused by the next row
+  }
+}
+
+// Two passes: the first only reduces, the second recomputes s and writes, so that in-place
+// calls (r_out = r, y = x) never read a value they already overwrote.
+template <int DT, bool RES>
+__global__ void __launch_bounds__(kThreads) norm_loop_kernel(const NormParams p) {
+  pdl_prologue();
+  __shared__ __align__(16) float red[32];
+  constexpr int EB = Act<DT>::BYTES;
+  constexpr int VE = Act<DT>::VE;
+  const int tid = threadIdx.x;
+  const int64_t row = blockIdx.x, nvec = p.H / VE;
+  const uint4* x = reinterpret_cast<const uint4*>(row_ptr(p.x, row, p.x_rs, EB));
+  const uint4* r = RES ? reinterpret_cast<const uint4*>(row_ptr(p.r, row, p.r_rs, EB)) : nullptr;
+  float ss = 0.f;
+  for (int64_t vi = tid; vi < nvec; vi += kThreads) {
+    float xf[VE], rf[VE];
+    unpack<DT>(ld16(x + vi), xf);
+    if (RES) unpack<DT>(ld16(r + vi), rf);
+#pragma unroll
+    for (int e = 0; e < VE; ++e) {
+      const float s = RES ? xf[e] + rf[e] : xf[e];
+      ss = fmaf(s, s, ss);
+    }
+  }
+  const float inv = rsqrtf(norm_block_sum(ss, red) * p.inv_H + p.eps);
+  uint4* y = reinterpret_cast<uint4*>(row_ptr(p.y, row, p.y_rs, EB));
+  uint4* ro = RES ? reinterpret_cast<uint4*>(row_ptr(p.r_out, row, p.ro_rs, EB)) : nullptr;
+  for (int64_t vi = tid; vi < nvec; vi += kThreads) {
+    float xf[VE], rf[VE], g[VE];
+    unpack<DT>(ld16(x + vi), xf);
+    if (RES) {
+      unpack<DT>(ld16(r + vi), rf);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) xf[e] += rf[e];
+      st16(ro + vi, pack<DT>(xf));
+    }
+    load_gamma<DT>(p.gamma + vi * VE, g);
+#pragma unroll
+    for (int e = 0; e < VE; ++e) xf[e] = xf[e] * inv * g[e];
+    st16(y + vi, pack<DT>(xf));
+  }
+}
+
+template <int DT, bool RES>
+__global__ void __launch_bounds__(kThreads) norm_generic_kernel(const NormParams p) {
+  pdl_prologue();
+  __shared__ __align__(16) float red[32];
+  const int tid = threadIdx.x;
+  for (int64_t row = blockIdx.x; row < p.T; row += gridDim.x) {
+    const int64_t xo = row * p.x_rs, ro = row * p.r_rs;
+    float ss = 0.f;
+    for (int64_t j = tid; j < p.H; j += kThreads) {
+      const float s = RES ? load_elem<DT>(p.x, xo + j) + load_elem<DT>(p.r, ro + j) : load_elem<DT>(p.x, xo + j);
+      ss = fmaf(s, s, ss);
+    }
+    const float inv = rsqrtf(norm_block_sum(ss, red) * p.inv_H + p.eps);
+    for (int64_t j = tid; j < p.H; j += kThreads) {
+      const float s = RES ? load_elem<DT>(p.x, xo + j) + load_elem<DT>(p.r, ro + j) : load_elem<DT>(p.x, xo + j);
+      if (RES) store_elem<DT>(p.r_out, row * p.ro_rs + j, s);
+      store_elem<DT>(p.y, row * p.y_rs + j, s * inv * p.gamma[j]);
+    }
+    __syncthreads();  // `red` is reused by the next row
+  }
+}
+
+constexpr int kNormRowsVecs = 128;    // rows of at most this many vectors: norm_rows_kernel
+
+// Threads of a block for a row of nvec vectors at vpt per thread.
+static int norm_threads(int64_t nvec, int vpt) { return (int)(((nvec + vpt - 1) / vpt + 31) / 32 * 32); }
+
+template <int DT, bool RES, int LPR, int VPT>
+static void pick_rows(int64_t nvec, KernelEntry* out) {
+  const bool full = nvec == LPR * VPT;
+  out->rows = kThreads / LPR;
+  out->nm_fn[NM_VEC] = full ? (const void*)norm_rows_kernel<DT, RES, LPR, VPT, true, 1>
+                            : (const void*)norm_rows_kernel<DT, RES, LPR, VPT, false, 1>;
+  if constexpr (!RES && VPT == 1) {
+    out->nm_fn[NM_LARGE] = full ? (const void*)norm_rows_kernel<DT, RES, LPR, VPT, true, 2>
+                                : (const void*)norm_rows_kernel<DT, RES, LPR, VPT, false, 2>;
+    out->large_per = kThreads / LPR * 2;
+    out->large_rows = kNormRows2Vecs / nvec;
+  }
+}
+
+template <int DT, bool RES>
+static void pick(int64_t H, KernelEntry* out) {
+  constexpr int VE = Act<DT>::VE;
+  const int64_t nvec = H / VE;
+  for (int k = 0; k < kNormEntries; ++k) {
+    out->nm_fn[k] = nullptr;
+    out->nm_threads[k] = kThreads;
+  }
+  out->nm_fn[NM_GENERIC] = (const void*)norm_generic_kernel<DT, RES>;
+  out->rows = out->large_per = 1;
+  out->large_rows = 0;
+  out->large_smem = 0;
+  const int vpt = nvec <= 1024 ? 1 : 2;
+  const int threads = norm_threads(nvec, vpt);
+  // rows that begin anywhere hold nvec or nvec - 1 whole vectors, and at least one
+  if (nvec >= 2 && nvec <= kNormBlockVecs) {
+    out->nm_threads[NM_EDGE] = threads;
+    out->nm_fn[NM_EDGE] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, true, false>
+                                   : (const void*)norm_block_kernel<DT, RES, 2, true, false>;
+  }
+  if (H % VE != 0) return;
+  if (nvec <= kNormRowsVecs) {
+    if (nvec > 64) pick_rows<DT, RES, 32, 4>(nvec, out);
+    else if (nvec > 32) pick_rows<DT, RES, 32, 2>(nvec, out);
+    else if (nvec > 16) pick_rows<DT, RES, 32, 1>(nvec, out);
+    else if (nvec > 8) pick_rows<DT, RES, 16, 1>(nvec, out);
+    else if (nvec > 4) pick_rows<DT, RES, 8, 1>(nvec, out);
+    else if (nvec > 2) pick_rows<DT, RES, 4, 1>(nvec, out);
+    else if (nvec > 1) pick_rows<DT, RES, 2, 1>(nvec, out);
+    else pick_rows<DT, RES, 1, 1>(nvec, out);
+  } else if (nvec <= kNormBlockVecs) {
+    const bool full = threads * vpt == nvec;
+    out->nm_threads[NM_VEC] = threads;
+    out->nm_fn[NM_VEC] = vpt == 1 ? (full ? (const void*)norm_block_kernel<DT, RES, 1, false, true>
+                                          : (const void*)norm_block_kernel<DT, RES, 1, false, false>)
+                                  : (full ? (const void*)norm_block_kernel<DT, RES, 2, false, true>
+                                          : (const void*)norm_block_kernel<DT, RES, 2, false, false>);
+    if (!(RES && DT == DT_FP32 && vpt == 1)) {
+      const int bv = RES && nvec <= 1024 ? 2 : 4;
+      const int bt = norm_threads(nvec, bv);
+      const bool bfull = bt * bv == nvec;
+      out->nm_threads[NM_LARGE] = bt;
+      out->nm_fn[NM_LARGE] = bv == 2 ? (bfull ? (const void*)norm_bulk_kernel<DT, RES, 2, true>
+                                              : (const void*)norm_bulk_kernel<DT, RES, 2, false>)
+                                     : (bfull ? (const void*)norm_bulk_kernel<DT, RES, 4, true>
+                                              : (const void*)norm_bulk_kernel<DT, RES, 4, false>);
+      out->large_smem = (int32_t)(nvec * 16 * (RES ? 2 : 1));
+      if constexpr (RES && VE == 8) {
+        if (nvec == 2 * kThreads) {
+          out->nm_fn[NM_LARGE] = (const void*)addnorm_row_kernel<DT>;
+          out->large_smem = 0;
+        }
+      }
+      out->large_rows = ((RES ? kNormBulkResBytes : kNormBulkBytes) + nvec * 16 - 1) / (nvec * 16);
+    }
+  } else {
+    out->nm_fn[NM_VEC] = (const void*)norm_loop_kernel<DT, RES>;
+  }
+}
+
+bool norm_kernel(bool res, int32_t dtype, int32_t variant, int64_t H, KernelEntry* out, const char** why) {
+  if (dtype != DT_BF16 && dtype != DT_FP16 && dtype != DT_FP32) { *why = "dtype"; return false; }
+  if (H < 1) { *why = "H must be >= 1"; return false; }
+  const int eb = dtype == DT_FP32 ? 4 : 2;
+  if (variant != 1 && (H * eb) % 16 != 0) { *why = "the vector norms need H * elem_size % 16 == 0"; return false; }
+  out->kind = KK_NORM;
+  out->vec = 16 / eb;
+  if (dtype == DT_BF16) res ? pick<DT_BF16, true>(H, out) : pick<DT_BF16, false>(H, out);
+  else if (dtype == DT_FP16) res ? pick<DT_FP16, true>(H, out) : pick<DT_FP16, false>(H, out);
+  else res ? pick<DT_FP32, true>(H, out) : pick<DT_FP32, false>(H, out);
+  out->fn = out->nm_fn[NM_GENERIC];
+  return true;
+}
+
+NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, int32_t* threads, int64_t* blocks,
+                    int32_t* smem) {
+  const uintptr_t off = (uintptr_t)p->x & 15;
+  const int64_t ve = 16 / eb, rs = p->x_rs % ve;
+  // all rows of all tensors share their offsets from 16-byte boundaries
+  const bool together = ((uintptr_t)p->y & 15) == off &&
+                        (!res || (((uintptr_t)p->r & 15) == off && ((uintptr_t)p->r_out & 15) == off)) &&
+                        (p->T <= 1 || (p->y_rs % ve == rs && (!res || (p->r_rs % ve == rs && p->ro_rs % ve == rs))));
+  const bool aligned = together && off == 0 && (p->T <= 1 || rs == 0) && ((uintptr_t)p->gamma & 15) == 0;
+  p->nvec = (int32_t)(p->H / ve < INT32_MAX ? p->H / ve : INT32_MAX);  // the loop kernel counts its own
+  NormEntry e = NM_GENERIC;
+  if (aligned && ke.nm_fn[NM_VEC]) e = ke.nm_fn[NM_LARGE] && p->T >= ke.large_rows ? NM_LARGE : NM_VEC;
+  else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX) e = NM_EDGE;  // one block per row
+  *threads = ke.nm_threads[e];
+  *smem = e == NM_LARGE ? ke.large_smem : 0;
+  const int64_t per = e == NM_VEC ? ke.rows : (e == NM_LARGE ? ke.large_per : 1);
+  *blocks = (p->T + per - 1) / per;
+  return e;
+}
+
+}  // namespace trident

@@ -394,10 +394,11 @@ struct Version {
   CUfunction fn_late;     // layer chain: `fn` with the late launch trigger
   CUfunction fn_wide;     // layer chain: `fn_inplace` with kChainWideSwigluUnroll tiles
   int32_t wave_blocks;    // layer chain: blocks of `fn` resident at once on the whole GPU
-  CUfunction fn_large;          // add+RMSNorm, RoPE: entry for calls of >= ke.large_rows rows
+  CUfunction fn_large;          // RoPE: the bulk-copy entry
   CUfunction fn_mid;            // RoPE: entry between fn and fn_large (rope_plan)
   RopePlans rope_plans;         // vector RoPE: item splits of its three entries
   CUfunction pw_fn[kPwEntries];  // elementwise: entries by layout and size (pointwise_plan)
+  CUfunction nm_fn[kNormEntries];  // norms: entries by layout and size (norm_plan)
   CUfunction step_fn;           // layer chain: several calls per launch (two blocks per token)
   CUfunction step_fn_inplace;   // ... one block per token
   CUfunction step_fn_role;      // ... one block per token, role-major order over the step
@@ -565,7 +566,7 @@ int32_t check_overlap(const trident_args* a, const OpInfo& oi) {
 inline int64_t row_stride(const trident_tensor& t, Kind k) { return rows_of(t, k).stride; }
 
 void pack_addnorm(const trident_args* a, int x, int r, int g, int y, int ro, const Sig& s,
-                  Kind kind, AddNormParams* p) {
+                  Kind kind, NormParams* p) {
   const trident_tensor* t = a->t;
   p->x = t[x].data; p->r = t[r].data; p->gamma = (const float*)t[g].data;
   p->y = t[y].data; p->r_out = t[ro].data;
@@ -576,19 +577,24 @@ void pack_addnorm(const trident_args* a, int x, int r, int g, int y, int ro, con
   p->eps = (float)a->eps;
   p->inv_H = (float)(1.0 / (double)p->H);
   p->prefetch = 0;
+  p->nvec = 0;
   p->first_wait_polls = kBulkWaitPolls;
   p->err = nullptr;
 }
 
-void pack_rmsnorm(const trident_args* a, const Sig& s, RmsNormParams* p) {
+void pack_rmsnorm(const trident_args* a, const Sig& s, NormParams* p) {
   const trident_tensor* t = a->t;
   p->x = t[0].data; p->gamma = (const float*)t[1].data; p->y = t[2].data;
+  p->r = nullptr; p->r_out = nullptr;
   p->T = s.T;
   p->H = t[1].shape[0];
   p->x_rs = row_stride(t[0], K_ACT_H); p->y_rs = row_stride(t[2], K_ACT_H);
+  p->r_rs = p->ro_rs = 0;
   p->eps = (float)a->eps;
   p->inv_H = (float)(1.0 / (double)p->H);
   p->prefetch = 0;
+  p->first_wait_polls = kBulkWaitPolls;
+  p->err = nullptr;
 }
 
 void pack_pointwise(const trident_args* a, const Sig& s, PointwiseParams* p) {
@@ -763,8 +769,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   CUlaunchAttribute attr;
   base_config(scm, stream, &cfg, &attr);
   union {
-    AddNormParams an;
-    RmsNormParams rn;
+    NormParams nm;
     PointwiseParams pw;
     RopeParams rp;
     RopeBulkParams rb;  // rb.rp is rp
@@ -775,17 +780,26 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   bool wide = false;  // layer chain: launch fn_wide (wider SwiGLU tiles)
   RopeEntry rope_entry = ROPE_SMALL;
   int pw_entry = PW_GENERIC;
+  NormEntry nm_entry = NM_GENERIC;
   switch (op) {
     case TRIDENT_OP_ADD_RMSNORM:
-      pack_addnorm(a, 0, 1, 2, 3, 4, s, K_ACT_H, &P.an);
-      P.an.err = scm->d_err;
-      if (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) P.an.first_wait_polls = 0;
-      cfg.gridDimX = cap_grid(s.T);
+    case TRIDENT_OP_RMSNORM: {
+      const bool res = op == TRIDENT_OP_ADD_RMSNORM;
+      if (res) {
+        pack_addnorm(a, 0, 1, 2, 3, 4, s, K_ACT_H, &P.nm);
+      } else {
+        pack_rmsnorm(a, s, &P.nm);
+      }
+      P.nm.err = scm->d_err;
+      P.nm.first_wait_polls = (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) ? 0u : kBulkWaitPolls;
+      int32_t threads = 0, smem = 0;
+      int64_t blocks = 0;
+      nm_entry = norm_plan(v.ke, &P.nm, res, elem_size(v.d.dtype), &threads, &blocks, &smem);
+      cfg.sharedMemBytes = (unsigned)smem;
+      cfg.blockDimX = (unsigned)threads;
+      cfg.gridDimX = cap_grid(blocks);
       break;
-    case TRIDENT_OP_RMSNORM:
-      pack_rmsnorm(a, s, &P.rn);
-      cfg.gridDimX = v.ke.kind == KK_NORM_ROWS ? cap_grid((s.T + v.ke.rows - 1) / v.ke.rows) : cap_grid(s.T);
-      break;
+    }
     case TRIDENT_OP_ROPE_KV:
     case TRIDENT_OP_QKNORM_ROPE_KV: {
       pack_rope(a, 0, op == TRIDENT_OP_QKNORM_ROPE_KV ? 6 : -1, v, scm->d_err, &P.rp);
@@ -876,8 +890,8 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   const int32_t pf =
       pdl && (int64_t)cfg.gridDimX * cfg.gridDimY * cfg.blockDimX <= (int64_t)scm->sm_count * kThreads ? 1 : 0;
   switch (op) {
-    case TRIDENT_OP_ADD_RMSNORM: P.an.prefetch = pf; break;
-    case TRIDENT_OP_RMSNORM: P.rn.prefetch = pf; break;
+    case TRIDENT_OP_ADD_RMSNORM:
+    case TRIDENT_OP_RMSNORM: P.nm.prefetch = pf; break;
     case TRIDENT_OP_ROPE_KV:
     case TRIDENT_OP_QKNORM_ROPE_KV: P.rp.prefetch = pf; break;
     case TRIDENT_OP_LAYER_CHAIN:
@@ -893,8 +907,8 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     fn = v.pw_fn[pw_entry];
   else if (v.ke.kind == KK_ROPE_PAIR)
     fn = rope_entry == ROPE_BULK ? v.fn_large : (rope_entry == ROPE_MID ? v.fn_mid : v.fn);
-  else if (v.fn_large && s.T >= v.ke.large_rows)
-    fn = v.fn_large;  // many rows: add+RMSNorm's bulk-copy kernel
+  else if (v.ke.kind == KK_NORM)
+    fn = v.nm_fn[nm_entry];
   return launch_on(scm, &cfg, fn, kp);
 }
 
@@ -1131,8 +1145,9 @@ int32_t resolve_kernel(const trident_spec_desc& d, KernelEntry* ke) {
   const bool chain = d.op == TRIDENT_OP_LAYER_CHAIN || d.op == TRIDENT_OP_LAYER_CHAIN_QKNORM;
   auto try_variant = [&](int32_t var) -> bool {
     switch (d.op) {
-      case TRIDENT_OP_ADD_RMSNORM: return addnorm_kernel(d.dtype, var, d.fixed[0], ke, &why);
-      case TRIDENT_OP_RMSNORM: return rmsnorm_kernel(d.dtype, var, d.fixed[0], ke, &why);
+      case TRIDENT_OP_ADD_RMSNORM:
+      case TRIDENT_OP_RMSNORM:
+        return norm_kernel(d.op == TRIDENT_OP_ADD_RMSNORM, d.dtype, var, d.fixed[0], ke, &why);
       case TRIDENT_OP_SILU:
       case TRIDENT_OP_ADD:
       case TRIDENT_OP_NEG:
@@ -1290,20 +1305,29 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
       if (cudaGetFuncBySymbol(&f, v.ke.fn) != cudaSuccess || !f)
         return fail(TRIDENT_ERR_CUDA, "cannot resolve the kernel entry");
       v.fn = reinterpret_cast<CUfunction>(f);
+      // one limit for every version of a kernel: rows of up to kNormBlockVecs vectors, x and r
+      if (v.ke.large_smem > 0 &&
+          cudaFuncSetAttribute(v.ke.nm_fn[NM_LARGE], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               2 * kNormBlockVecs * 16) != cudaSuccess)
+        return fail(TRIDENT_ERR_CUDA, "cannot set the norm kernel's shared-memory size");
       if (v.ke.fn_large) {
         cudaFunction_t h = nullptr;
         if (cudaGetFuncBySymbol(&h, v.ke.fn_large) != cudaSuccess || !h)
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the large-call kernel entry");
         v.fn_large = reinterpret_cast<CUfunction>(h);
       }
-      if (v.ke.kind == KK_POINTWISE) {
-        for (int k = 0; k < kPwEntries; ++k) {
-          cudaFunction_t e = nullptr;
-          if (cudaGetFuncBySymbol(&e, v.ke.pw_fn[k]) != cudaSuccess || !e)
-            return fail(TRIDENT_ERR_CUDA, "cannot resolve the elementwise kernel entries");
-          v.pw_fn[k] = reinterpret_cast<CUfunction>(e);
-        }
-      }
+      auto resolve = [&](const void* entry, CUfunction* out_fn) {
+        cudaFunction_t e = nullptr;
+        if (entry && (cudaGetFuncBySymbol(&e, entry) != cudaSuccess || !e)) return false;
+        *out_fn = reinterpret_cast<CUfunction>(e);
+        return true;
+      };
+      for (int k = 0; k < kPwEntries; ++k)
+        if (!resolve(v.ke.pw_fn[k], &v.pw_fn[k]))
+          return fail(TRIDENT_ERR_CUDA, "cannot resolve the elementwise kernel entries");
+      for (int k = 0; k < kNormEntries; ++k)
+        if (!resolve(v.ke.nm_fn[k], &v.nm_fn[k]))
+          return fail(TRIDENT_ERR_CUDA, "cannot resolve the norm kernel entries");
       if (v.ke.fn_mid) {
         cudaFunction_t m = nullptr;
         if (cudaGetFuncBySymbol(&m, v.ke.fn_mid) != cudaSuccess || !m)

@@ -295,6 +295,51 @@ def test_pointwise_parity(S, name, dtype, W, T, layout, variant):
         P.check_act(got, ref, ref_bits, dtype, name, exact_frac=0.99)
 
 
+@pytest.mark.parametrize("dtype,T,H,form", [
+    (BF16, 5, 24, "dense"), (FP32, 67, 20, "dense"),       # fewer vectors than the row's lanes
+    (BF16, 33, 264, "padded"), (FP32, 9, 516, "dense"),    # two and more vectors per lane
+    (BF16, 7, 1032, "dense"), (FP16, 5, 8200, "padded"),   # blocks with idle threads in the last round
+    (FP16, 3, 16384, "dense"), (FP32, 2, 8192, "dense"),   # two vectors per thread, exactly full
+    (BF16, 3, 16392, "dense"),                             # longer than a block holds: two passes
+    (BF16, 19, 1001, "dense"), (FP16, 6, 4099, "offset"),  # rows at every offset
+    (FP32, 8, 9, "offset"), (BF16, 9, 15, "offset"),       # one whole vector between the edges; none
+    (FP16, 5, 2048, "gamma"), (BF16, 6, 520, "apart"),     # weights, or one tensor, at another offset
+    (BF16, 1025, 4096, "dense"), (FP16, 1100, 5120, "padded"), (FP16, 420, 16000, "dense"),  # bulk copies
+    (FP32, 500, 8192, "dense"), (BF16, 20001, 64, "dense"), (FP16, 12001, 128, "padded")])   # two rows a time
+def test_norm_layouts(S, dtype, T, H, form):
+    """Every path of the norms' rule over sizes and layouts, with and without the residual, out
+    of place and in place, against the oracle."""
+    g = np.random.default_rng(H + T)
+    tdt = synth._TORCH_DT[dtype]
+    es = 4 if dtype == FP32 else 2
+    pad, off = (64, 0) if form == "padded" else (0, 1 if form == "offset" else 0)
+
+    def place(t, extra=0):
+        o = off + extra
+        buf = torch.zeros(T * (H + pad) + o + 16, dtype=tdt, device="cuda")
+        return buf[o:o + T * (H + pad)].view(T, H + pad)[:, :H].copy_(t)
+
+    x, r = synth.act(g, (T, H), dtype), synth.act(g, (T, H), dtype)
+    gam = synth.gamma(g, H)
+    gbuf = torch.zeros(H + 4, device="cuda")
+    gd = gbuf[1 if form == "gamma" else 0:][:H].copy_(torch.from_numpy(gam).cuda())
+    zero = torch.zeros((T, H), dtype=tdt, device="cuda")
+    for res in (True, False):
+        op = S.OP_ADD_RMSNORM if res else S.OP_RMSNORM
+        ref = L.add_rmsnorm(x, r, gam, 1e-6, dtype) if res else L.rmsnorm(x, gam, 1e-6, dtype)
+        s = one_version_scm(S, S.make_spec(op, dtype, [H], 1, 1 << 20, layout=S.LAYOUT_ANY, align_bytes=es))
+        for inplace in (False, True):
+            xd, rd = place(P.dev(x, dtype)), place(P.dev(r, dtype))
+            yd = xd if inplace else place(zero, extra=2 if form == "apart" else 0)
+            rod = rd if inplace else place(zero)
+            invoke_ok(s, S, S.make_args(op, [xd, rd, gd, yd, rod] if res else [xd, gd, yd], eps=1e-6))
+            assert S.trident_scm_device_status(s.h, stream()) == (S.OK, 0)
+            if res:
+                assert np.array_equal(P.host_bits(rod, dtype), ref[2])
+            P.check_act(P.host_bits(yd, dtype), ref[0], ref[1], dtype, f"norm {res} {inplace} {T}x{H} {form}")
+        s.close()
+
+
 @pytest.mark.parametrize("name", ["silu", "add", "neg", "masked_fill", "swiglu"])
 @pytest.mark.parametrize("dtype,T,W,form", [
     (BF16, 1, 3, "offset"), (BF16, 1, 9, "offset"),        # shorter than a head; a head and a tail
