@@ -9,8 +9,8 @@
 // horizontal fusion where blocks take different roles:
 //   norm     two add+RMSNorm steps, one or two blocks per token (the longest per-block
 //            work)
-//   RoPE     RoPE/KV head-rows, (256 / (D/8)) per block, or three times that (three rows
-//            of one token per lane group) on grids several waves long
+//   RoPE     RoPE/KV head-rows, eight warp items per block (RopeGeom): one head-row per lane
+//            group, or up to three of one token on grids several waves long
 //   SwiGLU   tiles of one row each, twice as wide on grids of many waves
 // Grids are role-major ([norms | RoPE | SwiGLU], so the longest blocks start first), the
 // smallest ones token-major (chain_block_tok), so that consecutive blocks mix roles. Under
@@ -135,26 +135,34 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
   }
 }
 
-// RoPE role: RoPE block rb (< nB), i.e. head-rows [rb * UPB, (rb + 1) * UPB) with UPB =
-// rope_k * 256 / LPH (rope_rows with rope_k = 3 on grids several waves long); fq holds the
-// lane's frequencies (rope_lane_freqs).
-// Only the one-CTA-per-token entries (SPLIT 1: in-place calls, and grids too large for one
-// wave) carry the rope_rows path, so the others keep their registers.
-template <int DT, int D, bool QKNORM, bool ROWS3>
-__device__ __forceinline__ void chain_rope(const ChainParams& c, const int64_t rb, const float* fq) {
-  constexpr int LPH = D / Act<DT>::VE;
-  if (ROWS3 && c.rope_k == 3) {
-    rope_rows<DT, D, QKNORM, 3>(c.rope, rb, threadIdx.x % LPH, threadIdx.x / LPH, fq);
-    return;
-  }
-  const int64_t unit = rb * (kThreads / LPH) + threadIdx.x / LPH;
-  if (unit < c.rope.T * c.rope.NH) rope_head_row<DT, D, QKNORM>(c.rope, unit, threadIdx.x % LPH, fq);
+// RoPE role: RoPE block rb (< nB), i.e. the warp items [8 rb, 8 rb + 8) of the call (RopeGeom);
+// fq holds the lane's frequencies. Items of at most one head-row per lane group, or of
+// kChainRopeRows on grids several waves long (rope_k), which only the one-CTA-per-token entries
+// (ROWS) carry, so the others keep their registers.
+template <int DT, int D, bool QKNORM, bool ROWS>
+__device__ __forceinline__ void chain_rope_rows(const ChainParams& c, int64_t t, int first, int end, const float4* fq) {
+  if (ROWS && c.rope_k > 1) rope_pair_rows<DT, D, QKNORM, kChainRopeRows, false>(c.rope, t, first, end, fq);
+  else rope_pair_rows<DT, D, QKNORM, 1, false>(c.rope, t, first, end, fq);
+}
+template <int DT, int D, bool QKNORM, bool ROWS>
+__device__ __forceinline__ void chain_rope(const ChainParams& c, const int64_t rb, const float4* fq) {
+  int64_t t;
+  int first, end;
+  if (rope_item(c.rope, rb * (kThreads / 32) + threadIdx.x / 32, &t, &first, &end))
+    chain_rope_rows<DT, D, QKNORM, ROWS>(c, t, first, end, fq);
+}
+// The item of this warp in RoPE block `part` of token t (token-major grids).
+__device__ __forceinline__ bool chain_tok_item(const ChainParams& c, int part, int* first, int* end) {
+  const int item = part * (kThreads / 32) + (int)threadIdx.x / 32;
+  *first = item * c.rope.rpi;
+  *end = min(c.rope.NH, *first + c.rope.rpi);
+  return item < c.rope.ipt;
 }
 
 // Before the PDL wait: the RoPE lane frequencies of a RoPE block (other roles load none).
 template <int DT, int D>
-__device__ __forceinline__ void chain_rope_freqs(const ChainParams& c, const bool is_rope, float* fq) {
-  if (is_rope) rope_lane_freqs<DT, D>(c.rope.inv_freq, threadIdx.x % (D / Act<DT>::VE), fq);
+__device__ __forceinline__ void chain_rope_freqs(const ChainParams& c, const bool is_rope, float4* fq) {
+  if (is_rope) rope_pair_freqs(c.rope.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
 }
 
 // SwiGLU role: column tile `col_tile` of row `row`, SWU x 256 16-byte vectors of g and of u
@@ -176,7 +184,7 @@ __device__ __forceinline__ int64_t swiglu_tile_row(const ChainParams& c, const i
 
 // Block b of one call's role-major grid (b < nA + nB + nC): [norms | RoPE | SwiGLU].
 template <int DT, int VPT, int SPLIT, int D, bool QKNORM, int SWU, bool STEP>
-__device__ __forceinline__ void chain_block(const ChainParams& c, const int b, const float* fq) {
+__device__ __forceinline__ void chain_block(const ChainParams& c, const int b, const float4* fq) {
   if (b < c.nA) {
     const int64_t row = b / SPLIT;
     chain_norm<DT, VPT, SPLIT>(c, row, b - (int)row * SPLIT);
@@ -198,12 +206,14 @@ __device__ __forceinline__ void chain_block(const ChainParams& c, const int b, c
 // give one SM four norm blocks (160 KB) while another gets 24 KB. Both indices come from
 // special registers, so no remapped index stays live in a register through the body.
 template <int DT, int VPT, int SPLIT, int D, bool QKNORM>
-__device__ __forceinline__ void chain_block_tok(const ChainParams& c, const float* fq) {
+__device__ __forceinline__ void chain_block_tok(const ChainParams& c, const float4* fq) {
   const int q = blockIdx.x;
   if (q < SPLIT) {
     chain_norm<DT, VPT, SPLIT>(c, blockIdx.y, q);
   } else if (q < SPLIT + c.rope_per_tok) {
-    chain_rope<DT, D, QKNORM, false>(c, (int64_t)blockIdx.y * c.rope_per_tok + (q - SPLIT), fq);
+    int first, end;
+    if (chain_tok_item(c, q - SPLIT, &first, &end))
+      chain_rope_rows<DT, D, QKNORM, false>(c, blockIdx.y, first, end, fq);
   } else {
     chain_swiglu<DT, kChainSwigluUnroll>(c, blockIdx.y, q - SPLIT - c.rope_per_tok);
   }
@@ -240,14 +250,12 @@ __device__ __forceinline__ void norm_prefetch(const ChainParams& c, const int64_
 // SPLIT takes head-rows [p * ceil(NH / SPLIT), ...), one thread per 128-byte line.
 template <int DT, int SPLIT, int D>
 __device__ __forceinline__ void norm_rope_prefetch(const ChainParams& c, const int64_t row, const int part) {
-  constexpr int VE = Act<DT>::VE;
-  constexpr int EB = Act<DT>::BYTES;
-  constexpr int LINES = (D * EB + 127) / 128;      // 128-byte lines per head-row
-  constexpr int LANES_PER_LINE = 128 / (VE * EB);  // lanes of a head-row per line
+  constexpr int LINES = (D * Act<DT>::BYTES + 127) / 128;  // 128-byte lines per head-row
   const int per = (c.rope.NH + SPLIT - 1) / SPLIT;
   const int k = threadIdx.x / LINES;
   if (k >= per || part * per + k >= c.rope.NH) return;
-  rope_prefetch<DT, D>(c.rope, row * c.rope.NH + part * per + k, (threadIdx.x % LINES) * LANES_PER_LINE);
+  prefetch_l2(rope_row_src<D>(c.rope, row, part * per + k) + (threadIdx.x % LINES) * 128);
+  if (threadIdx.x == 0) prefetch_l2(c.rope.pos + row);
 }
 
 // prefetch == 1: every block its own first lines; prefetch == 2: only the norm blocks, which
@@ -255,7 +263,6 @@ __device__ __forceinline__ void norm_rope_prefetch(const ChainParams& c, const i
 // hundreds of blocks while the previous kernel finishes, measured slower).
 template <int DT, int VPT, int SPLIT, int D, int SWU, bool STEP>
 __device__ __forceinline__ void chain_prefetch(const ChainParams& c, const int b) {
-  constexpr int LPH = D / Act<DT>::VE;
   const int tid = threadIdx.x;
   if (b < c.nA) {
     norm_prefetch<DT, VPT, SPLIT>(c, b / SPLIT, b % SPLIT);
@@ -264,7 +271,10 @@ __device__ __forceinline__ void chain_prefetch(const ChainParams& c, const int b
     return;
   } else if (b < c.nA + c.nB) {
     if (c.rope_k != 1) return;  // several head-rows per lane group: grids too long to prefetch
-    rope_prefetch<DT, D>(c.rope, (int64_t)(b - c.nA) * (kThreads / LPH) + tid / LPH, tid % LPH);
+    int64_t t;
+    int first, end;
+    if (rope_item(c.rope, (int64_t)(b - c.nA) * (kThreads / 32) + tid / 32, &t, &first, &end))
+      rope_item_prefetch<D, 1>(c.rope, t, first, end);
   } else {
     const int64_t tile = b - c.nA - c.nB;
     if (tile >= c.sw_tiles) return;
@@ -275,13 +285,12 @@ __device__ __forceinline__ void chain_prefetch(const ChainParams& c, const int b
 
 template <int DT, int VPT, int SPLIT, int D>
 __device__ __forceinline__ void chain_prefetch_tok(const ChainParams& c) {
-  constexpr int LPH = D / Act<DT>::VE;
   const int tid = threadIdx.x, q = blockIdx.x;
   if (q < SPLIT) {
     norm_prefetch<DT, VPT, SPLIT>(c, blockIdx.y, q);
   } else if (q < SPLIT + c.rope_per_tok) {
-    const int64_t rb = (int64_t)blockIdx.y * c.rope_per_tok + (q - SPLIT);
-    rope_prefetch<DT, D>(c.rope, rb * (kThreads / LPH) + tid / LPH, tid % LPH);
+    int first, end;
+    if (chain_tok_item(c, q - SPLIT, &first, &end)) rope_item_prefetch<D, 1>(c.rope, blockIdx.y, first, end);
   } else {
     swiglu_prefetch<DT, kChainSwigluUnroll>(
         c.sw, blockIdx.y, (int64_t)(q - SPLIT - c.rope_per_tok) * kChainSwigluUnroll * kThreads, tid);
@@ -300,7 +309,7 @@ template <int DT, int VPT, int SPLIT, int D, bool QKNORM, bool LATE, int SWU>
 __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
     chain_kernel(const __grid_constant__ ChainParams c) {
   if (!LATE || (int)blockIdx.x < c.nA) pdl_trigger();
-  float fq[2 * Act<DT>::VE];
+  float4 fq[4];
   if (!LATE && SWU == kChainSwigluUnroll && c.tok_grid) {
     if (c.prefetch) chain_prefetch_tok<DT, VPT, SPLIT, D>(c);
     chain_rope_freqs<DT, D>(c, (int)blockIdx.x >= SPLIT && (int)blockIdx.x < SPLIT + c.rope_per_tok, fq);
@@ -339,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
     }
     const ChainParams& c = p.c[lo];
     const int bl = b - f[lo] + (r == 0 ? 0 : (r == 1 ? c.nA : c.nA + c.nB));
-    float fq[2 * Act<DT>::VE];
+    float4 fq[4];
     chain_rope_freqs<DT, D>(c, r == 1, fq);
     pdl_wait();
     chain_block<DT, VPT, SPLIT, D, QKNORM, kChainStepSwigluUnroll, true>(c, bl, fq);
@@ -352,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
     const ChainParams& c = p.c[lo];
     const int bl = b - p.first[lo];
     if (c.prefetch) chain_prefetch<DT, VPT, SPLIT, D, kChainStepSwigluUnroll, true>(c, bl);
-    float fq[2 * Act<DT>::VE];
+    float4 fq[4];
     chain_rope_freqs<DT, D>(c, bl >= c.nA && bl < c.nA + c.nB, fq);
     pdl_wait();
     chain_block<DT, VPT, SPLIT, D, QKNORM, kChainStepSwigluUnroll, true>(c, bl, fq);

@@ -178,7 +178,7 @@ __device__ __forceinline__ void rope_sincos(float pos, float fhi, float flo, flo
   __sincosf(r + al, s, c);
 }
 
-// ---------------------------------------------------------------- RoPE head-row
+// ---------------------------------------------------------------- division
 // n / d for a 32-bit n and a divisor d known per launch, from the host's round-up multiplier
 // m and shift l for d (div_magic; Granlund and Montgomery, "Division by invariant integers
 // using multiplication", 1994): (h + ((n - h) >> 1)) >> (l - 1) with h = umulhi(n, m), exact
@@ -188,282 +188,6 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, uint32_t m, int32_t l) 
   if (l == 0) return n;
   const uint32_t h = __umulhi(n, m);
   return (h + ((n - h) >> 1)) >> (l - 1);
-}
-
-// Token and head-row of a unit: unit = t * NH + hh (units below 2^32, every grid in practice,
-// by fast_div).
-__device__ __forceinline__ void rope_unit_split(const RopeParams& p, int64_t unit, int64_t* t, int* hh) {
-  if (unit <= 0xffffffffll) {
-    const uint32_t u = (uint32_t)unit;
-    const uint32_t q = fast_div(u, p.nh_magic, p.nh_shift);
-    *t = q;
-    *hh = (int)(u - q * (uint32_t)p.NH);
-  } else {
-    *t = unit / p.NH;
-    *hh = (int)(unit - *t * p.NH);
-  }
-}
-
-// q, k or v head of head-row hh of a token.
-__device__ __forceinline__ void rope_head_of(const RopeParams& p, int hh, int* h, bool* is_q, bool* is_v) {
-  *is_v = hh >= p.Hq + p.Hkv;
-  *is_q = hh < p.Hq;
-  *h = *is_q ? hh : (*is_v ? hh - p.Hq - p.Hkv : hh - p.Hq);
-}
-
-// L2 prefetch of head-row `unit`'s source line(s) and position (lanes on a line boundary).
-template <int DT, int D>
-__device__ __forceinline__ void rope_prefetch(const RopeParams& p, int64_t unit, int lane) {
-  constexpr int VE = Act<DT>::VE;
-  constexpr int EB = Act<DT>::BYTES;
-  if (unit >= p.T * p.NH || (lane * VE * EB) % 128 != 0) return;
-  int64_t t;
-  int hh, h;
-  bool is_q, is_v;
-  rope_unit_split(p, unit, &t, &hh);
-  rope_head_of(p, hh, &h, &is_q, &is_v);
-  const char* src = is_q ? row_ptr(p.q, t, p.q_rs, EB) : is_v ? row_ptr(p.v, t, p.v_rs, EB)
-                                                             : row_ptr(p.k, t, p.k_rs, EB);
-  prefetch_l2(src + ((int64_t)h * D + lane * VE) * EB);
-  if (lane == 0) prefetch_l2(p.pos + t);
-}
-
-// The (hi, lo) frequencies of lane `lane` of a head-row, for its VE elements
-// i = (lane % (LPH/2)) * VE + e. The frequency table belongs to the version: it is written
-// once, when the version is registered (and the registration waits for that copy), and is
-// never written again, so kernels read it before griddepcontrol.wait, while the previous
-// kernel of the stream still runs. Every RoPE lane of a grid reads the same few lines of
-// the table; read after the wait, those reads queue behind each other at the L2 slices
-// that hold the lines, on the critical path of every RoPE block. The same lane position
-// has the same frequencies in every head-row, so a lane loads them once.
-template <int DT, int D>
-__device__ __forceinline__ void rope_lane_freqs(const float2* inv_freq, int lane, float* fq) {
-  constexpr int VE = Act<DT>::VE;
-  constexpr int HALF = D / VE / 2;
-  const float* fr = reinterpret_cast<const float*>(inv_freq) + 2 * (lane % HALF) * VE;
-#pragma unroll
-  for (int q = 0; q < VE / 2; ++q) {
-    const float4 f4 = ldg_f4(fr + 4 * q);
-    fq[4 * q] = f4.x; fq[4 * q + 1] = f4.y; fq[4 * q + 2] = f4.z; fq[4 * q + 3] = f4.w;
-  }
-}
-
-// One head-row (token t, head hh) handled by LPH = D / VE consecutive lanes, each lane
-// owning VE consecutive elements. Rotate-half pairs element i with i + D/2, i.e. lane
-// l with lane l ^ (LPH/2). hh < Hq: q head (rotated in place); hh < Hq + Hkv: k head
-// (rotated into k_cache); else v head (copied into v_cache). fq holds the lane's
-// frequencies (rope_lane_freqs). A head-row is processed in two steps: rope_row_load issues
-// every load it needs -- the row slice, the position and the norm weights -- and
-// rope_row_finish uses them, so a lane group that owns several head-rows issues all of
-// their loads before it waits for any (one memory round trip in all).
-template <int DT, int D>
-__device__ __forceinline__ void rope_row_where(const RopeParams& p, int64_t unit, int64_t* t, int* h,
-                                               bool* is_q, bool* is_v) {
-  int hh;
-  rope_unit_split(p, unit, t, &hh);
-  rope_head_of(p, hh, h, is_q, is_v);
-}
-
-template <int DT, int D, bool QKNORM>
-__device__ __forceinline__ void rope_row_load(const RopeParams& p, int64_t unit, int lane, uint4* raw,
-                                              int32_t* pos, float* gg) {
-  constexpr int VE = Act<DT>::VE;
-  constexpr int EB = Act<DT>::BYTES;
-  int64_t t;
-  int h;
-  bool is_q, is_v;
-  rope_row_where<DT, D>(p, unit, &t, &h, &is_q, &is_v);
-  const char* src = is_q ? row_ptr(p.q, t, p.q_rs, EB) : is_v ? row_ptr(p.v, t, p.v_rs, EB)
-                                                             : row_ptr(p.k, t, p.k_rs, EB);
-  src += ((int64_t)h * D + lane * VE) * EB;
-  *raw = is_q ? ld16(src) : ldg16(src);
-  *pos = __ldg(p.pos + t);
-  if (QKNORM && !is_v) {
-    const float* gam = (is_q ? p.gamma_q : p.gamma_k) + lane * VE;
-#pragma unroll
-    for (int q = 0; q < VE / 4; ++q) {
-      const float4 g4 = ldg_f4(gam + 4 * q);
-      gg[4 * q] = g4.x; gg[4 * q + 1] = g4.y; gg[4 * q + 2] = g4.z; gg[4 * q + 3] = g4.w;
-    }
-  }
-}
-
-template <int DT, int D, bool QKNORM>
-__device__ __forceinline__ void rope_row_finish(const RopeParams& p, int64_t unit, int lane, const uint4 raw,
-                                                const int32_t pos, const float* gg, const float* fq) {
-  constexpr int VE = Act<DT>::VE;
-  constexpr int LPH = D / VE;
-  constexpr int HALF = LPH / 2;
-  constexpr int EB = Act<DT>::BYTES;
-  static_assert(LPH >= 2 && LPH <= 32 && (LPH & (LPH - 1)) == 0, "head size");
-  const unsigned group_mask =
-      (LPH == 32) ? 0xffffffffu : (((1u << LPH) - 1u) << ((threadIdx.x & 31) & ~(LPH - 1)));
-  int64_t t;
-  int h;
-  bool is_q, is_v;
-  rope_row_where<DT, D>(p, unit, &t, &h, &is_q, &is_v);
-  if (pos < 0 || (int64_t)pos >= p.S) {
-    if (lane == 0) atomicOr(p.err, kErrPos);
-    return;
-  }
-  if (is_v) {  // bit copy into the cache
-    st16(reinterpret_cast<char*>(p.v_cache) + (((int64_t)h * p.S + pos) * D + lane * VE) * EB, raw);
-    return;
-  }
-  float x[VE];
-  unpack<DT>(raw, x);
-  if (QKNORM) {
-    float ss = 0.f;
-#pragma unroll
-    for (int e = 0; e < VE; ++e) ss = fmaf(x[e], x[e], ss);
-#pragma unroll
-    for (int o = LPH / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(group_mask, ss, o, LPH);
-    const float inv = rsqrtf(ss * p.inv_D + p.eps);
-#pragma unroll
-    for (int e = 0; e < VE; ++e) x[e] = x[e] * inv * gg[e];
-  }
-  float other[VE];
-#pragma unroll
-  for (int e = 0; e < VE; ++e) other[e] = __shfl_xor_sync(group_mask, x[e], HALF, LPH);
-  const bool low = lane < HALF;
-  const float fpos = (float)pos;
-  float y[VE];
-#pragma unroll
-  for (int e = 0; e < VE; ++e) {
-    float sn, cs;
-    rope_sincos(fpos, fq[2 * e], fq[2 * e + 1], &sn, &cs);
-    // low half: x_i c - x_{i+D/2} s;  high half: x_{i+D/2} c + x_i s
-    y[e] = low ? fmaf(x[e], cs, -other[e] * sn) : fmaf(x[e], cs, other[e] * sn);
-  }
-  if (is_q) {
-    st16(row_ptr(p.q, t, p.q_rs, EB) + ((int64_t)h * D + lane * VE) * EB, pack<DT>(y));
-  } else {
-    char* dst = reinterpret_cast<char*>(p.k_cache) + (((int64_t)h * p.S + pos) * D + lane * VE) * EB;
-    st16(dst, pack<DT>(y));
-  }
-}
-
-template <int DT, int D, bool QKNORM>
-__device__ __forceinline__ void rope_head_row(const RopeParams& p, int64_t unit, int lane, const float* fq) {
-  uint4 raw;
-  int32_t pos;
-  float gg[Act<DT>::VE];
-  rope_row_load<DT, D, QKNORM>(p, unit, lane, &raw, &pos, gg);
-  rope_row_finish<DT, D, QKNORM>(p, unit, lane, raw, pos, gg, fq);
-}
-
-// K head-rows per lane group, for grids several waves long: lane group g (of G = 256 / LPH)
-// of RoPE block rb owns the units rb * G * K + g + G * j, j < K -- with NH = 48 and K = 3 one
-// token's q, k and v rows. A block then moves K times the bytes for the same fixed costs,
-// which pays where blocks queue for slots (a 1024-token layer 39.7 -> 34.8 us) and not where
-// a block's own latency is the step (one wave: slower per block). Rows of one token share
-// the position and so every angle: the lane computes its sines and cosines once, for the
-// token of the first row, and again only for a row of another token (NH not a multiple of
-// G), reloading its frequencies then. All K rows' loads are issued before any is used.
-template <int DT, int D, bool QKNORM, int K>
-__device__ __forceinline__ void rope_rows(const RopeParams& p, const int64_t rb, const int lane, const int g,
-                                          const float* fq) {
-  constexpr int VE = Act<DT>::VE;
-  constexpr int LPH = D / VE;
-  constexpr int HALF = LPH / 2;
-  constexpr int EB = Act<DT>::BYTES;
-  constexpr int G = kThreads / LPH;
-  const unsigned group_mask =
-      (LPH == 32) ? 0xffffffffu : (((1u << LPH) - 1u) << ((threadIdx.x & 31) & ~(LPH - 1)));
-  const int64_t nunits = p.T * p.NH;
-  const int64_t u0 = rb * (int64_t)(G * K) + g;
-  if (u0 >= nunits) return;
-  // rows u0 + G * j: token and head-row of the first by one division, the rest by stepping
-  int64_t t0;
-  int hh0;
-  rope_unit_split(p, u0, &t0, &hh0);
-  uint4 raw[K];
-  {
-    int64_t t = t0;
-    int hh = hh0;
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      if (j > 0) {
-        hh += G;
-        while (hh >= p.NH) { hh -= p.NH; ++t; }
-      }
-      if (u0 + (int64_t)G * j < nunits) {
-        int h;
-        bool is_q, is_v;
-        rope_head_of(p, hh, &h, &is_q, &is_v);
-        const char* src = is_q ? row_ptr(p.q, t, p.q_rs, EB) : is_v ? row_ptr(p.v, t, p.v_rs, EB)
-                                                                   : row_ptr(p.k, t, p.k_rs, EB);
-        src += ((int64_t)h * D + lane * VE) * EB;
-        raw[j] = is_q ? ld16(src) : ldg16(src);
-      }
-    }
-  }
-  const int32_t pos0 = __ldg(p.pos + t0);
-  float sn[VE], cs[VE];
-#pragma unroll
-  for (int e = 0; e < VE; ++e) rope_sincos((float)pos0, fq[2 * e], fq[2 * e + 1], &sn[e], &cs[e]);
-  const bool low = lane < HALF;
-  int64_t t = t0;
-  int hh = hh0;
-#pragma unroll
-  for (int j = 0; j < K; ++j) {
-    if (j > 0) {
-      hh += G;
-      while (hh >= p.NH) { hh -= p.NH; ++t; }
-    }
-    if (u0 + (int64_t)G * j >= nunits) break;
-    int h;
-    bool is_q, is_v;
-    rope_head_of(p, hh, &h, &is_q, &is_v);
-    // units ascend, so once a row belongs to a later token every following row does too
-    const bool same = t == t0;
-    const int32_t pos = same ? pos0 : __ldg(p.pos + t);
-    if (pos < 0 || (int64_t)pos >= p.S) {
-      if (lane == 0) atomicOr(p.err, kErrPos);
-      continue;
-    }
-    if (is_v) {  // bit copy into the cache
-      st16(reinterpret_cast<char*>(p.v_cache) + (((int64_t)h * p.S + pos) * D + lane * VE) * EB, raw[j]);
-      continue;
-    }
-    float x[VE];
-    unpack<DT>(raw[j], x);
-    if (QKNORM) {
-      const float* gam = (is_q ? p.gamma_q : p.gamma_k) + lane * VE;
-      float gg[VE];
-#pragma unroll
-      for (int q = 0; q < VE / 4; ++q) {
-        const float4 g4 = ldg_f4(gam + 4 * q);
-        gg[4 * q] = g4.x; gg[4 * q + 1] = g4.y; gg[4 * q + 2] = g4.z; gg[4 * q + 3] = g4.w;
-      }
-      float ss = 0.f;
-#pragma unroll
-      for (int e = 0; e < VE; ++e) ss = fmaf(x[e], x[e], ss);
-#pragma unroll
-      for (int o = LPH / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(group_mask, ss, o, LPH);
-      const float inv = rsqrtf(ss * p.inv_D + p.eps);
-#pragma unroll
-      for (int e = 0; e < VE; ++e) x[e] = x[e] * inv * gg[e];
-    }
-    float other[VE];
-#pragma unroll
-    for (int e = 0; e < VE; ++e) other[e] = __shfl_xor_sync(group_mask, x[e], HALF, LPH);
-    if (!same) {
-      float f2[2 * VE];
-      rope_lane_freqs<DT, D>(p.inv_freq, lane, f2);
-#pragma unroll
-      for (int e = 0; e < VE; ++e) rope_sincos((float)pos, f2[2 * e], f2[2 * e + 1], &sn[e], &cs[e]);
-    }
-    float y[VE];
-#pragma unroll
-    for (int e = 0; e < VE; ++e)
-      y[e] = low ? fmaf(x[e], cs[e], -other[e] * sn[e]) : fmaf(x[e], cs[e], other[e] * sn[e]);
-    if (is_q) {
-      st16(row_ptr(p.q, t, p.q_rs, EB) + ((int64_t)h * D + lane * VE) * EB, pack<DT>(y));
-    } else {
-      st16(reinterpret_cast<char*>(p.k_cache) + (((int64_t)h * p.S + pos) * D + lane * VE) * EB, pack<DT>(y));
-    }
-  }
 }
 
 // ---------------------------------------------------------------- packed fp32 pairs
@@ -555,58 +279,59 @@ __device__ __forceinline__ void rope_pair_gamma(const float* gamma, int lane, Ro
   }
 }
 
-// Finishes head-row hh of token t from its two vectors: [q/k norm,] rotation, store (v: copy).
-// *kind says whose weights *g holds (0: none yet); rows of an item mostly share them.
-template <int DT, int D, bool QKNORM>
-__device__ __forceinline__ void rope_pair_finish(const RopeParams& p, int64_t t, int hh, int lane, int32_t pos,
-                                                 const uint4& lo, const uint4& hi, const RopeAngles& an,
-                                                 RopeGamma* g, int* kind) {
-  constexpr int LPG = RopeGeom<D>::LPG;
-  const bool is_q = hh < p.Hq, is_v = hh >= p.Hq + p.Hkv;
-  char* dst = is_q ? row_ptr(p.q, t, p.q_rs, 2) + (int64_t)hh * (D * 2)
-                   : reinterpret_cast<char*>(is_v ? p.v_cache : p.k_cache) +
-                         ((int64_t)(hh - p.Hq - (is_v ? p.Hkv : 0)) * p.S + pos) * (D * 2);
-  dst += lane * 16;
-  if (is_v) {  // bit copy into the cache
-    st16(dst, lo);
-    st16(dst + D, hi);
-    return;
-  }
+template <int DT>
+__device__ __forceinline__ void rope_unpack(const uint4& lo, const uint4& hi, F2* A, F2* B) {
   float a[8], b[8];
   unpack<DT>(lo, a);
   unpack<DT>(hi, b);
-  F2 A[4], B[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     A[q] = f2_pack(a[2 * q], a[2 * q + 1]);
     B[q] = f2_pack(b[2 * q], b[2 * q + 1]);
   }
-  if (QKNORM) {
-    F2 s2 = f2_mul(A[0], A[0]);
+}
+
+// 1 / rms of a head-row held by the lane group (LPG lanes), in both halves of a pair.
+template <int D>
+__device__ __forceinline__ F2 rope_inv_rms(const RopeParams& p, const F2* A, const F2* B) {
+  constexpr int LPG = RopeGeom<D>::LPG;
+  F2 s2 = f2_mul(A[0], A[0]);
 #pragma unroll
-    for (int q = 1; q < 4; ++q) s2 = f2_fma(A[q], A[q], s2);
+  for (int q = 1; q < 4; ++q) s2 = f2_fma(A[q], A[q], s2);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) s2 = f2_fma(B[q], B[q], s2);
-    float s0, s1;
-    f2_unpack(s2, &s0, &s1);
-    float ss = s0 + s1;
-    const unsigned mask =
-        LPG == 32 ? 0xffffffffu : (((1u << LPG) - 1u) << ((threadIdx.x & 31) & ~(LPG - 1)));
+  for (int q = 0; q < 4; ++q) s2 = f2_fma(B[q], B[q], s2);
+  float s0, s1;
+  f2_unpack(s2, &s0, &s1);
+  float ss = s0 + s1;
+  const unsigned mask =
+      LPG == 32 ? 0xffffffffu : (((1u << LPG) - 1u) << ((threadIdx.x & 31) & ~(LPG - 1)));
 #pragma unroll
-    for (int o = LPG / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(mask, ss, o, LPG);
-    const float inv = rsqrtf(ss * p.inv_D + p.eps);
-    const int want = is_q ? 1 : 2;
-    if (*kind != want) {
-      rope_pair_gamma<D>(is_q ? p.gamma_q : p.gamma_k, lane, g);
-      *kind = want;
-    }
-    const F2 iv = f2_pack(inv, inv);
+  for (int o = LPG / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(mask, ss, o, LPG);
+  const float inv = rsqrtf(ss * p.inv_D + p.eps);
+  return f2_pack(inv, inv);
+}
+__device__ __forceinline__ void rope_scale(F2 inv, const RopeGamma& g, F2* A, F2* B) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      A[q] = f2_mul(f2_mul(A[q], iv), g->lo[q]);
-      B[q] = f2_mul(f2_mul(B[q], iv), g->hi[q]);
-    }
+  for (int q = 0; q < 4; ++q) {
+    A[q] = f2_mul(f2_mul(A[q], inv), g.lo[q]);
+    B[q] = f2_mul(f2_mul(B[q], inv), g.hi[q]);
   }
+}
+
+// Where head-row hh of token t goes (its lane-0 vector).
+template <int D>
+__device__ __forceinline__ char* rope_row_dst(const RopeParams& p, int64_t t, int hh, int32_t pos) {
+  constexpr int RB = D * 2;
+  if (hh < p.Hq) return row_ptr(p.q, t, p.q_rs, 2) + (int64_t)hh * RB;
+  const bool is_v = hh >= p.Hq + p.Hkv;
+  return reinterpret_cast<char*>(is_v ? p.v_cache : p.k_cache) +
+         ((int64_t)(hh - p.Hq - (is_v ? p.Hkv : 0)) * p.S + pos) * RB;
+}
+
+// Rotates a lane's pairs and stores them at dst (the lane's low vector).
+template <int DT, int D>
+__device__ __forceinline__ void rope_rotate(char* dst, const RopeAngles& an, const F2* A, const F2* B) {
+  float a[8], b[8];
   // low half: x_i c - x_{i+D/2} s;  high half: x_{i+D/2} c + x_i s
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -617,26 +342,76 @@ __device__ __forceinline__ void rope_pair_finish(const RopeParams& p, int64_t t,
   st16(dst + D, pack<DT>(b));
 }
 
+// Finishes head-row hh of token t from its two vectors: [q/k norm,] rotation, store (v: copy).
+// KEEP: *g holds a kind's weights (*kind; 0: none yet) from row to row, as rows of an item
+// mostly share them; otherwise each row loads its own (fewer registers).
+template <int DT, int D, bool QKNORM, bool KEEP>
+__device__ __forceinline__ void rope_pair_finish(const RopeParams& p, int64_t t, int hh, int lane, int32_t pos,
+                                                 const uint4& lo, const uint4& hi, const RopeAngles& an,
+                                                 RopeGamma* g, int* kind) {
+  char* dst = rope_row_dst<D>(p, t, hh, pos) + lane * 16;
+  if (hh >= p.Hq + p.Hkv) {  // bit copy into the cache
+    st16(dst, lo);
+    st16(dst + D, hi);
+    return;
+  }
+  F2 A[4], B[4];
+  rope_unpack<DT>(lo, hi, A, B);
+  if (QKNORM) {
+    const bool is_q = hh < p.Hq;
+    const F2 inv = rope_inv_rms<D>(p, A, B);
+    if (KEEP) {
+      const int want = is_q ? 1 : 2;
+      if (*kind != want) {
+        rope_pair_gamma<D>(is_q ? p.gamma_q : p.gamma_k, lane, g);
+        *kind = want;
+      }
+      rope_scale(inv, *g, A, B);
+    } else {
+      RopeGamma own;
+      rope_pair_gamma<D>(is_q ? p.gamma_q : p.gamma_k, lane, &own);
+      rope_scale(inv, own, A, B);
+    }
+  }
+  rope_rotate<DT, D>(dst, an, A, B);
+}
+
+// L2 prefetch of an item's row lines (at most R rows per lane group) and position.
+template <int D, int R>
+__device__ __forceinline__ void rope_item_prefetch(const RopeParams& p, int64_t t, int first, int end) {
+  constexpr int LPG = RopeGeom<D>::LPG, GW = RopeGeom<D>::GW;
+  const int lane = (threadIdx.x & 31) % LPG, g = (threadIdx.x & 31) / LPG;
+  if (lane % 8 != 0) return;
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    if (first + g + j * GW < end) {
+      const char* src = rope_row_src<D>(p, t, first + g + j * GW) + lane * 16;
+      prefetch_l2(src);
+      prefetch_l2(src + D);
+    }
+  }
+  if ((threadIdx.x & 31) == 0) prefetch_l2(p.pos + t);
+}
+
 // One item's rows [first, end) of token t, at most R per lane group: every load the rows need
-// is issued first. fq: the lane's frequencies.
-template <int DT, int D, bool QKNORM, int R>
+// is issued first, without a branch (with one per row the loads followed one another). fq: the
+// lane's frequencies.
+template <int DT, int D, bool QKNORM, int R, bool KEEP>
 __device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, int first, int end, const float4* fq) {
   constexpr int LPG = RopeGeom<D>::LPG, GW = RopeGeom<D>::GW;
   const int lane = (threadIdx.x & 31) % LPG;
   const int hh0 = first + (threadIdx.x & 31) / LPG;
   uint4 lo[R], hi[R];
 #pragma unroll
-  for (int j = 0; j < R; ++j) {
-    if (hh0 + j * GW < end) {
-      const char* src = rope_row_src<D>(p, t, hh0 + j * GW) + lane * 16;
-      lo[j] = ld16(src);
-      hi[j] = ld16(src + D);
-    }
+  for (int j = 0; j < R; ++j) {  // groups past the item's end load its last row and drop it
+    const char* src = rope_row_src<D>(p, t, min(hh0 + j * GW, end - 1)) + lane * 16;
+    lo[j] = ld16(src);
+    hi[j] = ld16(src + D);
   }
   const int32_t pos = __ldg(p.pos + t);
   RopeGamma g;
   int kind = 0;
-  if (QKNORM && hh0 < end && hh0 < p.Hq + p.Hkv) {
+  if (QKNORM && (KEEP || R == 1)) {
     kind = hh0 < p.Hq ? 1 : 2;
     rope_pair_gamma<D>(kind == 1 ? p.gamma_q : p.gamma_k, lane, &g);
   }
@@ -645,11 +420,26 @@ __device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, i
     return;
   }
   RopeAngles an;
+  if (QKNORM && R == 1) {  // the norm first: its weights' registers are free before the angles'
+    if (hh0 >= end) return;
+    F2 A[4], B[4];
+    rope_unpack<DT>(lo[0], hi[0], A, B);
+    rope_scale(rope_inv_rms<D>(p, A, B), g, A, B);
+    rope_angles(pos, fq, &an);
+    char* dst = rope_row_dst<D>(p, t, hh0, pos) + lane * 16;
+    if (hh0 >= p.Hq + p.Hkv) {  // bit copy into the cache
+      st16(dst, lo[0]);
+      st16(dst + D, hi[0]);
+    } else {
+      rope_rotate<DT, D>(dst, an, A, B);
+    }
+    return;
+  }
   rope_angles(pos, fq, &an);
 #pragma unroll
   for (int j = 0; j < R; ++j)
     if (hh0 + j * GW < end)
-      rope_pair_finish<DT, D, QKNORM>(p, t, hh0 + j * GW, lane, pos, lo[j], hi[j], an, &g, &kind);
+      rope_pair_finish<DT, D, QKNORM, KEEP>(p, t, hh0 + j * GW, lane, pos, lo[j], hi[j], an, &g, &kind);
 }
 
 // ---------------------------------------------------------------- SwiGLU tile
@@ -697,14 +487,13 @@ __device__ __forceinline__ void swiglu_tile(const SwigluParams& p, int64_t row, 
   const uint4* g = reinterpret_cast<const uint4*>(row_ptr(p.g, row, p.g_rs, EB));
   const uint4* u = reinterpret_cast<const uint4*>(row_ptr(p.u, row, p.u_rs, EB));
   uint4* o = reinterpret_cast<uint4*>(row_ptr(p.out, row, p.o_rs, EB));
+  if (v0 >= nvec) return;  // the same for the whole block
   uint4 gv[UNROLL], uv[UNROLL];
 #pragma unroll
-  for (int k = 0; k < UNROLL; ++k) {
-    const int64_t vi = v0 + (int64_t)k * kThreads + tid;
-    if (vi < nvec) {
-      gv[k] = ldg16(g + vi);
-      uv[k] = ldg16(u + vi);
-    }
+  for (int k = 0; k < UNROLL; ++k) {  // threads past the row's end load its last vector and drop it
+    const int64_t vi = min(v0 + (int64_t)k * kThreads + tid, nvec - 1);
+    gv[k] = ldg16(g + vi);
+    uv[k] = ldg16(u + vi);
   }
 #pragma unroll
   for (int k = 0; k < UNROLL; ++k) {

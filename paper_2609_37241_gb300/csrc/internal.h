@@ -80,8 +80,6 @@ struct RopeParams {
   int32_t Hq, Hkv, D, NH;  // NH = Hq + 2 Hkv head-rows per token
   float eps, inv_D;
   int32_t prefetch;
-  uint32_t nh_magic;  // unit / NH for units below 2^32 by fast_div
-  int32_t nh_shift;
   int32_t ipt, rpi;    // warp items per token, head-rows per item (RopeSplit)
   uint32_t ipt_magic;  // item / ipt by fast_div
   int32_t ipt_shift;
@@ -117,7 +115,8 @@ struct ChainParams {
                      // 2 only the norm blocks' rows, 0 none
   int32_t tok_grid;  // 1: grid (a_split + rope_per_tok + sw_tiles_per_row, T), token-major
   int32_t rope_per_tok;  // RoPE blocks per token (token-major grid: nB = T * rope_per_tok)
-  int32_t rope_k;    // head-rows per RoPE lane group: 1, or 3 on grids several waves long
+  int32_t rope_k;    // head-rows per RoPE lane group at most: 1, or kChainRopeRows on grids several
+                     // waves long
   uint32_t sw_magic;  // tile / sw_tiles_per_row by fast_div
   int32_t sw_shift;
   int64_t sw_tiles;  // T * sw_tiles_per_row (valid SwiGLU tiles)
@@ -133,6 +132,7 @@ constexpr int kStepMax = 48;
 // step's grid, several waves long, does better with fewer, larger tiles (measured on 36 Qwen3
 // layers: 8 tokens 11.7 -> 11.4 us, 32 tokens 39.1 -> 37.2 us, 128 tokens 155 -> 150 us;
 // the same change on single calls made them slower, 64 tokens 3.56 -> 4.09 us).
+constexpr int kChainRopeRows = 3;
 constexpr int kChainSwigluUnroll = 2;
 constexpr int kChainStepSwigluUnroll = 4;
 // A single call's grid of many waves (one CTA per token) takes the wider tiles too: blocks
@@ -252,11 +252,5 @@ struct RopePlans {
 };
 void rope_plans(int64_t NH, int32_t D, RopePlans* out);
 RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks);
-
-// Units (head-rows) handled by one RoPE block of the layer chain for head size D.
-inline int32_t rope_units_per_block(int32_t D, int32_t elem_bytes) {
-  int32_t lanes_per_head = D * elem_bytes / 16;
-  return kThreads / lanes_per_head;
-}
 
 }  // namespace trident

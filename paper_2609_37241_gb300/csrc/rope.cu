@@ -45,26 +45,14 @@ constexpr int32_t kRopeBulkTokens = 512;
 template <int DT, int D, bool QKNORM, int R>
 __global__ void __launch_bounds__(kRopeThreads) rope_pair_kernel(const RopeParams p) {
   pdl_trigger();
-  constexpr int LPG = RopeGeom<D>::LPG, GW = RopeGeom<D>::GW;
-  const int lane = (threadIdx.x & 31) % LPG, g = (threadIdx.x & 31) / LPG;
   int64_t t;
   int first, end;
   const bool live = rope_item(p, (int64_t)blockIdx.x * (kRopeThreads / 32) + threadIdx.x / 32, &t, &first, &end);
   float4 fq[4];
-  rope_pair_freqs(p.inv_freq, lane, fq);
-  if (p.prefetch && live && lane % 8 == 0) {
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      if (first + g + j * GW < end) {
-        const char* src = rope_row_src<D>(p, t, first + g + j * GW) + lane * 16;
-        prefetch_l2(src);
-        prefetch_l2(src + D);
-      }
-    }
-    if ((threadIdx.x & 31) == 0) prefetch_l2(p.pos + t);
-  }
+  rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
+  if (p.prefetch && live) rope_item_prefetch<D, R>(p, t, first, end);
   pdl_wait();
-  if (live) rope_pair_rows<DT, D, QKNORM, R>(p, t, first, end, fq);
+  if (live) rope_pair_rows<DT, D, QKNORM, R, true>(p, t, first, end, fq);
 }
 
 // Calls of many tokens: a warp's item is three head-rows per lane group (3 KB), staged in the
@@ -150,7 +138,7 @@ __global__ void __launch_bounds__(kRopeBulkThreads, 6) rope_bulk_kernel(const Ro
     const int hh = hh0 + j * GW;
     if (hh >= end) break;
     const char* row = s_rows[w] + (hh - first) * RB + lane * 16;
-    rope_pair_finish<DT, D, QKNORM>(p, t, hh, lane, pos, ld16(row), ld16(row + D), an, &g, &kind);
+    rope_pair_finish<DT, D, QKNORM, true>(p, t, hh, lane, pos, ld16(row), ld16(row + D), an, &g, &kind);
   }
 }
 

@@ -397,6 +397,7 @@ struct Version {
   CUfunction fn_large;          // RoPE: the bulk-copy entry
   CUfunction fn_mid;            // RoPE: entry between fn and fn_large (rope_plan)
   RopePlans rope_plans;         // vector RoPE: item splits of its three entries
+  RopeSplit rope_split[2];      // layer chain: item splits with one and kChainRopeRows rows
   CUfunction pw_fn[kPwEntries];  // elementwise: entries by layout and size (pointwise_plan)
   CUfunction nm_fn[kNormEntries];  // norms: entries by layout and size (norm_plan)
   CUfunction step_fn;           // layer chain: several calls per launch (two blocks per token)
@@ -633,7 +634,6 @@ void pack_rope(const trident_args* a, int base, int gq, const Version& v, uint32
   p->Hkv = (int32_t)t[base + 1].shape[1];
   p->D = (int32_t)t[base].shape[2];
   p->NH = p->Hq + 2 * p->Hkv;
-  div_magic((uint32_t)p->NH, &p->nh_magic, &p->nh_shift);
   p->eps = (float)a->eps;
   p->inv_D = (float)(1.0 / (double)p->D);
   p->prefetch = 0;
@@ -696,6 +696,15 @@ void set_chain_tiles(ChainParams* c, int64_t T, int32_t unroll, int32_t vec) {
   c->sw_tiles = T * tiles;
 }
 
+// Sets the RoPE items of a chain call and returns its RoPE blocks (eight warp items each).
+int64_t chain_rope_blocks(RopeParams* p, int64_t T, const RopeSplit& r) {
+  p->ipt = r.ipt;
+  p->rpi = r.rpi;
+  p->ipt_magic = r.magic;
+  p->ipt_shift = r.shift;
+  return (T * r.ipt + kThreads / 32 - 1) / (kThreads / 32);
+}
+
 int32_t pack_chain(trident_scm* scm, const Version& v, const trident_args* a, const Sig& s,
                    int32_t unroll, ChainParams* c) {
   pack_addnorm(a, C_H, C_R0, C_GA, C_X1, C_R1, s, K_ACT_H, &c->n1);
@@ -704,8 +713,7 @@ int32_t pack_chain(trident_scm* scm, const Version& v, const trident_args* a, co
   pack_swiglu(a, C_G, C_U, C_O, s.T, &c->sw);
   const int64_t per = (int64_t)unroll * kThreads * v.ke.vec;
   const int64_t tiles = (c->sw.I + per - 1) / per;
-  const int64_t upb = rope_units_per_block(c->rope.D, 2);
-  const int64_t nB = (s.T * c->rope.NH + upb - 1) / upb, nC = s.T * tiles;
+  const int64_t nB = chain_rope_blocks(&c->rope, s.T, v.rope_split[0]), nC = s.T * tiles;
   if (2 * s.T + nB + nC > 0x7fffffff) return fail(TRIDENT_ERR_INVALID, "layer chain too large for one launch");
   c->nB = (int32_t)nB;
   set_chain_tiles(c, s.T, unroll, v.ke.vec);
@@ -726,25 +734,28 @@ bool chain_inplace(const trident_args* a) {
 
 // Sets the norm CTAs per token (split) and the RoPE head-rows per lane group (rope_k), and
 // with them nA, nB and the grid's block count.
-int32_t set_chain_split(ChainParams* c, int64_t T, int32_t split, int32_t rope_k, int64_t* blocks) {
+int32_t set_chain_split(const Version& v, ChainParams* c, int64_t T, int32_t split, int32_t rope_k,
+                        int64_t* blocks) {
   c->a_split = split;
   c->nA = (int32_t)(T * split);
   c->rope_k = rope_k;
-  const int64_t upb = (int64_t)rope_units_per_block(c->rope.D, 2) * rope_k;
-  c->nB = (int32_t)((T * c->rope.NH + upb - 1) / upb);
+  c->nB = (int32_t)chain_rope_blocks(&c->rope, T, v.rope_split[rope_k > 1]);
   *blocks = (int64_t)c->nA + c->nB + c->nC;
   return TRIDENT_OK;
 }
 
-// Three head-rows per RoPE lane group (rope_rows) on grids several waves long: a grid whose
+// Up to three head-rows per RoPE lane group on grids several waves long: a grid whose
 // one-CTA-per-token form with one head-row per lane group (`one` blocks) exceeds the resident
-// slots. There blocks queue for slots and a RoPE block that moves three rows for the same
-// fixed costs pays; within one wave a block's own latency is the step (a single-wave grid of
-// such blocks measured slower: 64 tokens 3.52 -> 4.46 us). Same-box A/B: Llama layer steps
-// at 128 tokens 5.61 -> 5.12 us, 256 tokens 9.37 -> 8.39 us; 36 Qwen3-style layers in one
-// launch at 32 / 64 / 128 / 256 tokens 36.7 / 70.5 / 142.9 / 281.0 -> 35.2 / 65.6 / 128.6 /
-// 252.7 us.
-inline int32_t chain_rope_k(int64_t one, int64_t wave_blocks) { return one > wave_blocks ? 3 : 1; }
+// slots. There blocks queue for slots and a RoPE block that moves three rows for the same fixed
+// costs pays; within one wave a block's own latency is the step. Same-box device times of the
+// role as it was (a lane per 16-byte vector, partners exchanged by shuffles, loads behind a
+// branch per row), as it is with two rows and with three: Llama layers of 128 / 256 / 1024 / 8192
+// tokens 5.16 / 8.88 / 29.4 / 221.8, 5.02 / 8.45 / 27.7 / 210.9, 4.99 / 8.30 / 27.1 / 205.4 us
+// (8192 tokens: 6.7 TB/s, 0.99 of the 6.8 TB/s copy rate); 36 layers with q/k norm in one launch
+// at 8 / 32 / 128 tokens 10.7 / 33.7 / 124.8, 10.0 / 31.0 / 116.7, 9.4 / 30.3 / 110.7 us. Within
+// one wave the two forms are level (16 tokens 2.27 / 2.25 us, 64 tokens 3.32 / 3.32, with q/k
+// norm 2.29 / 2.30 and 62 tokens 3.32 / 3.19); 80 tokens 5.11 / 3.65, which now fit one wave.
+inline int32_t chain_rope_k(int64_t one, int64_t wave_blocks) { return one > wave_blocks ? kChainRopeRows : 1; }
 
 // Layer-chain prefetch before the PDL wait: every block's first lines for grids of at most
 // one block per SM (small_grid); otherwise, when norm_rows, only the norm blocks prefetch:
@@ -845,7 +856,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       wide = split == 1 && v.fn_wide && one > 4 * (int64_t)v.wave_blocks;
       if (wide) set_chain_tiles(&c, s.T, kChainWideSwigluUnroll, v.ke.vec);
       int64_t blocks = 0;
-      st = set_chain_split(&c, s.T, split, rope_k, &blocks);
+      st = set_chain_split(v, &c, s.T, split, rope_k, &blocks);
       if (st != TRIDENT_OK) return st;
       cfg.gridDimX = (unsigned)blocks;
       // Under PDL, a role-major grid of more than a quarter block per SM whose blocks, with
@@ -867,13 +878,12 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       // layer step, 1 token 2.20 -> 2.04 us). Larger grids are role-major, which starts the
       // longest (norm) blocks first (64 tokens: 3.98 us role-major, 4.05 us token-major; 48
       // and 64 tokens in other interleaved orders were slower as well).
-      const int64_t upb = rope_units_per_block(c.rope.D, 2);
       if ((scm->opt.flags & TRIDENT_OPT_PDL) && split == 2 && v.fn_late && 4 * blocks > scm->sm_count &&
           blocks + c.nA <= v.wave_blocks + v.wave_blocks / 8) {
         late = true;
-      } else if (c.rope.NH % upb == 0 && s.T >= 1 && s.T <= 65535 && blocks <= 2 * scm->sm_count) {
+      } else if (rope_k == 1 && s.T >= 1 && s.T <= 65535 && blocks <= 2 * scm->sm_count) {
         c.tok_grid = 1;
-        c.rope_per_tok = (int32_t)(c.rope.NH / upb);
+        c.rope_per_tok = (c.rope.ipt + kThreads / 32 - 1) / (kThreads / 32);
         cfg.gridDimX = (unsigned)(split + c.rope_per_tok + c.sw_tiles_per_row);
         cfg.gridDimY = (unsigned)s.T;
       }
@@ -1296,6 +1306,10 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
   if (st != TRIDENT_OK) return st;
   if (v.ke.kind == KK_ROPE_PAIR)
     rope_plans(desc->fixed[0] + 2 * desc->fixed[1], (int32_t)desc->fixed[2], &v.rope_plans);
+  if (v.ke.kind == KK_CHAIN)
+    for (int k = 0; k < 2; ++k)
+      v.rope_split[k] = rope_split(desc->fixed[1] + 2 * desc->fixed[2], (int32_t)desc->fixed[3],
+                                   k ? kChainRopeRows : 1);
   std::lock_guard<std::mutex> lk(scm->reg_mu);
   const int32_t n = scm->count.load(std::memory_order_relaxed);
   if (n >= scm->opt.max_specs) return fail(TRIDENT_ERR_CAPACITY, "version table full (%d)", n);
@@ -1711,7 +1725,7 @@ int32_t step_chunk(trident_scm* scm, const trident_args* a, int32_t m, void* str
     int64_t first = 0;
     for (int32_t i = 0; i < m; ++i) {
       int64_t blocks = 0;
-      set_chain_split(&P.c[i], sig[i].T, split, rope_k, &blocks);
+      set_chain_split(scm->versions[sel[i]], &P.c[i], sig[i].T, split, rope_k, &blocks);
       P.first[i] = (int32_t)first;
       first += blocks;
       if (first > 0x7fffffff)
