@@ -132,12 +132,31 @@ def fastcall():
     `invoke_seq(scm, args_address, n, stream)` and `invoke_step(...)`, same arguments, on raw
     integer addresses; the default stream is 0), or None if it was not built. Same C calls
     as trident_scm_invoke / _seq / _step, without ctypes' per-call cost."""
-    try:
-        lib()
-        from . import _fastcall
-        return _fastcall
-    except ImportError:
+    global _shim
+    if _shim is False:
+        try:
+            lib()
+            from . import _fastcall
+            _shim = _fastcall
+        except ImportError:
+            _shim = None
+    return _shim
+
+
+_shim = False  # not looked for yet
+
+
+def _run(kind, scm, args, n, stream):
+    """(status, selected) through the shim, or None where the call has to go through ctypes:
+    no shim, a closed handle, or arguments that are not what ctypes' own checks accept."""
+    fc = _shim if _shim is not False else fastcall()
+    if fc is None or type(scm) is not c_vp or not scm.value:
         return None
+    if stream is None:
+        stream = 0
+    elif type(stream) is not int:
+        return None
+    return fc.run(kind, scm.value, ctypes.addressof(args), n, stream)
 
 
 class ScmError(RuntimeError):
@@ -168,6 +187,9 @@ def trident_scm_register_spec(scm, desc):
 
 
 def trident_scm_invoke(scm, args, stream=None):
+    r = _run(0, scm, args, 1, stream) if type(args) is trident_args else None
+    if r is not None:
+        return r
     sel = c_i32(-1)
     st = lib().trident_scm_invoke(scm, ctypes.byref(args), stream, ctypes.byref(sel))
     return st, sel.value
@@ -175,6 +197,9 @@ def trident_scm_invoke(scm, args, stream=None):
 
 def trident_scm_invoke_seq(scm, args_array, stream=None):
     n = len(args_array)
+    r = _run(1, scm, args_array, n, stream) if getattr(args_array, "_type_", None) is trident_args else None
+    if r is not None:
+        return r
     sel = (c_i32 * max(n, 1))()
     st = lib().trident_scm_invoke_seq(scm, args_array, n, stream, sel)
     return st, list(sel)[:n]
@@ -183,6 +208,9 @@ def trident_scm_invoke_seq(scm, args_array, stream=None):
 def trident_scm_invoke_step(scm, args_array, stream=None):
     """Like trident_scm_invoke_seq; independent layer-chain calls share one launch."""
     n = len(args_array)
+    r = _run(2, scm, args_array, n, stream) if getattr(args_array, "_type_", None) is trident_args else None
+    if r is not None:
+        return r
     sel = (c_i32 * max(n, 1))()
     st = lib().trident_scm_invoke_step(scm, args_array, n, stream, sel)
     return st, list(sel)[:n]

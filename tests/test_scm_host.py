@@ -458,6 +458,52 @@ def test_fastcall_shim_matches_ctypes(S):
     s.close()
 
 
+@pytest.mark.parametrize("n", [0, 1, 3, 64, 65, 130])
+def test_binding_calls_through_shim_equal_ctypes(S, n):
+    """invoke, invoke_seq and invoke_step of the binding go through the shim where it is built;
+    statuses, selections and statistics equal the ctypes calls', hits and misses, few and many."""
+    import ctypes
+    for miss_at in (None, 0, n // 2):
+        args = [cases.lib_args(cases.make_args({"op": 1, "T": 4 if i % 3 else 2, "H": 64})) for i in range(n)]
+        if miss_at is not None and n:
+            args[miss_at] = cases.lib_args(cases.make_args({"op": 1, "T": 40, "H": 64}))
+        arr = (S.trident_args * n)(*args)
+        got = []
+        for ctypes_path in (False, True):
+            s = dry(S)
+            s.register(S.make_spec(1, 1, [64], 1, 3))
+            s.register(S.make_spec(1, 1, [64], 1, 8))
+            out = []
+            for name in ("trident_scm_invoke_seq", "trident_scm_invoke_step"):
+                if ctypes_path:
+                    sel = (ctypes.c_int32 * max(n, 1))()
+                    out.append((getattr(S.lib(), name)(s.h, arr, n, None, sel), list(sel)[:n]))
+                else:
+                    out.append(getattr(S, name)(s.h, arr, None))
+            for a in args[:3]:
+                if ctypes_path:
+                    sel = ctypes.c_int32(-1)
+                    out.append((S.lib().trident_scm_invoke(s.h, ctypes.byref(a), None, ctypes.byref(sel)), sel.value))
+                else:
+                    out.append(s.invoke(a, 0))
+            st = s.stats()
+            got.append((out, st.invokes, st.hits, st.misses))
+            s.close()
+        assert got[0] == got[1]
+
+
+def test_binding_refuses_what_ctypes_refuses(S):
+    import ctypes
+    s = dry(S)
+    a = cases.lib_args(cases.make_args({"op": 1, "T": 4, "H": 64}))
+    with pytest.raises((ctypes.ArgumentError, TypeError)):
+        s.invoke((ctypes.c_int32 * 4)(), 0)
+    with pytest.raises((ctypes.ArgumentError, TypeError)):
+        s.invoke_seq((ctypes.c_int32 * 4)(), 0)
+    s.close()
+    assert S.trident_scm_invoke(s.h, a)[0] == S.ERR_INVALID  # a closed handle
+
+
 def test_execution_error_is_raised_not_retried(S):
     """Algorithm 1 (§3.2): when the selected P_i fails, the error propagates at once -- no
     later version is tried, the compile hook is not called, nothing is registered (§3.5).
