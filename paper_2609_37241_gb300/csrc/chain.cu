@@ -368,24 +368,23 @@ __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
   }
 }
 
-template <int DT, int SPLIT, bool QK>
-static void pick(int64_t H, const void** one, const void** step, const void** extra, const void** role) {
-  // extra: for SPLIT 2 the LATE entry, for SPLIT 1 the wide-tile entry; role: for SPLIT 1
-  // the role-major whole-step entry
-  constexpr int per = kThreads * Act<DT>::VE;
-  if (H == per * 2) {
-    *one = (const void*)chain_kernel<DT, 2, SPLIT, 128, QK, false, kChainSwigluUnroll>;
-    *step = (const void*)chain_step_kernel<DT, 2, SPLIT, 128, QK, false>;
-    if constexpr (SPLIT == 2) *extra = (const void*)chain_kernel<DT, 2, SPLIT, 128, QK, true, kChainSwigluUnroll>;
-    else *extra = (const void*)chain_kernel<DT, 2, SPLIT, 128, QK, false, kChainWideSwigluUnroll>;
-    if constexpr (SPLIT == 1) *role = (const void*)chain_step_kernel<DT, 2, SPLIT, 128, QK, true>;
-  } else if (H == per * 4) {
-    *one = (const void*)chain_kernel<DT, 4, SPLIT, 128, QK, false, kChainSwigluUnroll>;
-    *step = (const void*)chain_step_kernel<DT, 4, SPLIT, 128, QK, false>;
-    if constexpr (SPLIT == 2) *extra = (const void*)chain_kernel<DT, 4, SPLIT, 128, QK, true, kChainSwigluUnroll>;
-    else *extra = (const void*)chain_kernel<DT, 4, SPLIT, 128, QK, false, kChainWideSwigluUnroll>;
-    if constexpr (SPLIT == 1) *role = (const void*)chain_step_kernel<DT, 4, SPLIT, 128, QK, true>;
-  }
+template <int DT, bool QK, int VPT>
+static void pick(KernelEntry* out) {
+  constexpr int U = kChainSwigluUnroll;
+  out->fn = (const void*)chain_kernel<DT, VPT, 2, 128, QK, false, U>;
+  out->fn_late = (const void*)chain_kernel<DT, VPT, 2, 128, QK, true, U>;
+  out->fn_inplace = (const void*)chain_kernel<DT, VPT, 1, 128, QK, false, U>;
+  out->fn_inplace_late = (const void*)chain_kernel<DT, VPT, 1, 128, QK, true, U>;
+  out->fn_wide = (const void*)chain_kernel<DT, VPT, 1, 128, QK, false, kChainWideSwigluUnroll>;
+  out->fn_step = (const void*)chain_step_kernel<DT, VPT, 2, 128, QK, false>;
+  out->fn_step_inplace = (const void*)chain_step_kernel<DT, VPT, 1, 128, QK, false>;
+  out->fn_step_role = (const void*)chain_step_kernel<DT, VPT, 1, 128, QK, true>;
+}
+
+template <int DT, bool QK>
+static void pick(int64_t H, KernelEntry* out) {
+  if (H == kThreads * Act<DT>::VE * 2) pick<DT, QK, 2>(out);
+  else if (H == kThreads * Act<DT>::VE * 4) pick<DT, QK, 4>(out);
 }
 
 bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry* out,
@@ -395,29 +394,13 @@ bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry*
   out->kind = KK_CHAIN;
   out->vec = 8;
   out->unroll = kChainSwigluUnroll;
-  // fn: two blocks per token for the norms; fn_late: the same with the late launch trigger;
-  // fn_inplace: one block per token (calls whose outputs overwrite inputs, and grids too
-  // large for one wave); fn_wide: fn_inplace with wider SwiGLU tiles (grids of many waves);
+  // fn: two blocks per token for the norms; fn_inplace: one block per token (calls whose outputs
+  // overwrite inputs, and grids too large for one wave); fn_late, fn_inplace_late: the same with
+  // the late launch trigger; fn_wide: fn_inplace with wider SwiGLU tiles (grids of many waves);
   // fn_step*: the same for several calls per launch (fn_step_role: role-major order)
-  out->fn = out->fn_inplace = out->fn_step = out->fn_step_inplace = out->fn_late = out->fn_wide =
-      out->fn_step_role = nullptr;
-  if (dtype == DT_BF16) {
-    if (qknorm) {
-      pick<DT_BF16, 2, true>(H, &out->fn, &out->fn_step, &out->fn_late, nullptr);
-      pick<DT_BF16, 1, true>(H, &out->fn_inplace, &out->fn_step_inplace, &out->fn_wide, &out->fn_step_role);
-    } else {
-      pick<DT_BF16, 2, false>(H, &out->fn, &out->fn_step, &out->fn_late, nullptr);
-      pick<DT_BF16, 1, false>(H, &out->fn_inplace, &out->fn_step_inplace, &out->fn_wide, &out->fn_step_role);
-    }
-  } else {
-    if (qknorm) {
-      pick<DT_FP16, 2, true>(H, &out->fn, &out->fn_step, &out->fn_late, nullptr);
-      pick<DT_FP16, 1, true>(H, &out->fn_inplace, &out->fn_step_inplace, &out->fn_wide, &out->fn_step_role);
-    } else {
-      pick<DT_FP16, 2, false>(H, &out->fn, &out->fn_step, &out->fn_late, nullptr);
-      pick<DT_FP16, 1, false>(H, &out->fn_inplace, &out->fn_step_inplace, &out->fn_wide, &out->fn_step_role);
-    }
-  }
+  out->fn = nullptr;
+  if (dtype == DT_BF16) qknorm ? pick<DT_BF16, true>(H, out) : pick<DT_BF16, false>(H, out);
+  else qknorm ? pick<DT_FP16, true>(H, out) : pick<DT_FP16, false>(H, out);
   if (!out->fn) { *why = "layer chain supports H in {4096, 8192}"; return false; }
   return true;
 }

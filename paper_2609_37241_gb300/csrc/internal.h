@@ -163,6 +163,7 @@ struct KernelEntry {
   const void* fn = nullptr;
   const void* fn_inplace = nullptr;  // chain only: the entry for calls that write in place
   const void* fn_late = nullptr;     // chain only: fn with the late launch trigger (LATE)
+  const void* fn_inplace_late = nullptr;  // chain only: fn_inplace with the late launch trigger
   const void* fn_wide = nullptr;     // chain only: fn_inplace with kChainWideSwigluUnroll tiles
   const void* fn_step_role = nullptr;  // chain only: fn_step_inplace, role-major block order
   const void* fn_step = nullptr;          // chain only: several calls per launch (ChainStepParams)

@@ -392,6 +392,7 @@ struct Version {
   CUfunction fn;
   CUfunction fn_inplace;  // layer chain: one block per token when outputs alias inputs
   CUfunction fn_late;     // layer chain: `fn` with the late launch trigger
+  CUfunction fn_inplace_late;  // layer chain: `fn_inplace` with the late launch trigger
   CUfunction fn_wide;     // layer chain: `fn_inplace` with kChainWideSwigluUnroll tiles
   int32_t wave_blocks;    // layer chain: blocks of `fn` resident at once on the whole GPU
   CUfunction fn_large;          // RoPE: the bulk-copy entry
@@ -860,25 +861,22 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       if (st != TRIDENT_OK) return st;
       cfg.gridDimX = (unsigned)blocks;
       // Under PDL, a role-major grid of more than a quarter block per SM whose blocks, with
-      // its own norm blocks, fit the resident slots give or take an eighth of them launches
-      // fn_late: its RoPE and SwiGLU blocks trigger the next launch at their exit, so the
-      // next grid is placed whole while this one's norm blocks finish, one norm block per SM
-      // instead of up to four. Same-box A/B of Llama layer steps against the grids below: 6
-      // tokens 2.22 -> 2.12 us, 8 tokens 2.33 -> 2.14, 16 tokens 2.58 -> 2.29, 24 tokens
-      // 3.19 -> 2.44, 32 tokens 2.98 -> 2.57, 48 tokens 3.21 -> 2.99, 56 tokens 3.31 ->
-      // 3.19; equal at 2 and 4 tokens and at 1 token 1.5-2 % slower (nothing to place, and
-      // the next launch starts later), hence the lower bound; a few dozen blocks placed late
-      // cost less than stacked norm blocks (36 Qwen3-style launches at 64 tokens 125.9 ->
-      // 122.3 us, 62 Llama tokens equal), but at 64 Llama tokens, with 96 blocks placed late,
-      // the probe measured 3.51 -> 3.69 us, hence the upper bound.
-      // Otherwise a token-major grid (chain_block_tok) for grids of at most two blocks per SM,
-      // when every token has the same number of RoPE blocks: consecutive blocks then mix
-      // roles, so the blocks that land together on one SM are not all norm blocks (measured
-      // against role-major grids without the late trigger: 16 tokens 3.55 -> 2.85 us per
-      // layer step, 1 token 2.20 -> 2.04 us). Larger grids are role-major, which starts the
-      // longest (norm) blocks first (64 tokens: 3.98 us role-major, 4.05 us token-major; 48
-      // and 64 tokens in other interleaved orders were slower as well).
-      if ((scm->opt.flags & TRIDENT_OPT_PDL) && split == 2 && v.fn_late && 4 * blocks > scm->sm_count &&
+      // its own norm blocks, fit the resident slots give or take an eighth of them launches a
+      // late entry (fn_late, fn_inplace_late): its RoPE and SwiGLU blocks trigger the next launch
+      // at their exit, so the next grid is placed whole while this one's norm blocks finish, one
+      // norm block per SM instead of up to four. Same-box A/B of Llama layer steps against the
+      // grids below: 6 tokens 2.22 -> 2.12 us, 16 tokens 2.58 -> 2.29, 32 tokens 2.98 -> 2.57, 56
+      // tokens 3.31 -> 3.19; with one norm CTA per token 90 tokens 5.10 -> 3.80, 100 tokens 5.24 ->
+      // 4.08, H 8192 at 37 tokens 4.86 -> 3.70. Equal at 2 and 4 tokens and at 1 token 1.5-2 %
+      // slower (nothing to place, and the next launch starts later), hence the lower bound; a few
+      // dozen blocks placed late cost less than stacked norm blocks, but with 96 blocks placed
+      // late the probe measured 3.51 -> 3.69 us, hence the upper bound.
+      // Otherwise a token-major grid (chain_block_tok) for grids of at most two blocks per SM
+      // with one head-row per RoPE lane group: consecutive blocks then mix roles, so the blocks
+      // that land together on one SM are not all norm blocks (measured against role-major grids
+      // without the late trigger: 16 tokens 3.55 -> 2.85 us per layer step, 1 token 2.20 -> 2.04
+      // us). Larger grids are role-major, which starts the longest (norm) blocks first.
+      if ((scm->opt.flags & TRIDENT_OPT_PDL) && !wide && 4 * blocks > scm->sm_count &&
           blocks + c.nA <= v.wave_blocks + v.wave_blocks / 8) {
         late = true;
       } else if (rope_k == 1 && s.T >= 1 && s.T <= 65535 && blocks <= 2 * scm->sm_count) {
@@ -910,8 +908,8 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   }
   CUfunction fn = v.fn;
   if ((op == TRIDENT_OP_LAYER_CHAIN || op == TRIDENT_OP_LAYER_CHAIN_QKNORM) && P.ch.a_split == 1)
-    fn = wide ? v.fn_wide : v.fn_inplace;
-  else if (late && v.fn_late)
+    fn = wide ? v.fn_wide : (late ? v.fn_inplace_late : v.fn_inplace);
+  else if (late)
     fn = v.fn_late;
   if (v.ke.kind == KK_POINTWISE)
     fn = v.pw_fn[pw_entry];
@@ -1358,6 +1356,12 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
           if (cudaGetFuncBySymbol(&l, v.ke.fn_late) != cudaSuccess || !l)
             return fail(TRIDENT_ERR_CUDA, "cannot resolve the late-trigger kernel entry");
           v.fn_late = reinterpret_cast<CUfunction>(l);
+        }
+        if (v.ke.fn_inplace_late) {
+          cudaFunction_t l = nullptr;
+          if (cudaGetFuncBySymbol(&l, v.ke.fn_inplace_late) != cudaSuccess || !l)
+            return fail(TRIDENT_ERR_CUDA, "cannot resolve the in-place late-trigger kernel entry");
+          v.fn_inplace_late = reinterpret_cast<CUfunction>(l);
         }
         if (v.ke.fn_wide) {
           cudaFunction_t w = nullptr;
