@@ -80,6 +80,7 @@ struct RopeParams {
   int32_t Hq, Hkv, D, NH;  // NH = Hq + 2 Hkv head-rows per token
   float eps, inv_D;
   int32_t prefetch;
+  int32_t freq_late;   // 1: inv_freq may still be written by the previous kernel of the stream
   int32_t ipt, rpi;    // warp items per token, head-rows per item (RopeSplit)
   uint32_t ipt_magic;  // item / ipt by fast_div
   int32_t ipt_shift;

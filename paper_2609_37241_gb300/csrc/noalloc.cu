@@ -16,9 +16,10 @@
 // that clears the status word and rewrites the table for its own (theta, D), then the
 // RoPE kernel. The host keeps no record of what the array holds, so nothing on the host
 // can disagree with the device: whatever ran on the stream before, and whether or not an
-// earlier launch failed, the RoPE kernel reads the table its own call wrote. The RoPE
-// kernel reads its frequencies before griddepcontrol.wait; it is launched here without
-// programmatic serialisation, so it starts only after the preparing kernel has finished.
+// earlier launch failed, the RoPE kernel reads the table its own call wrote. It is launched
+// with programmatic serialisation, so that its launch overlaps the preparing kernel, and reads
+// its frequencies only after griddepcontrol.wait (RopeParams.freq_late), when that kernel has
+// finished; the preparing kernel itself starts after everything before it on the stream.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -44,13 +45,23 @@ struct DeviceScratch {
 };
 DeviceScratch g_dev[kMaxDevices];
 
+// theta^(-2 * 2^b / D) for b < 7, in fp64: the factors of every f_i = theta^(-2i/D), i < 128.
+struct FreqPowers { double p[7]; };
+
 // Prepares the scratch for one call: clears the status word and writes the frequency
-// table f_i = theta^(-2i/D) in fp64, stored as (fp32(f), fp32(f - hi)), for i < D/2.
-__global__ void prepare_scratch(uint32_t* status, float2* tab, int32_t D, double theta) {
+// table f_i = theta^(-2i/D) in fp64, stored as (fp32(f), fp32(f - hi)), for i < D/2: the product of
+// the powers at the bits of i, at most six roundings of 2^-53 where the pair keeps 2^-48. (One
+// pow per thread instead, in the kernel, was 7 us of every call: fp64 runs at a small fraction of
+// fp32's rate.)
+__global__ void prepare_scratch(uint32_t* status, float2* tab, int32_t D, const FreqPowers pw) {
+  pdl_trigger();
   const int i = threadIdx.x;
   if (i == 0) *status = 0u;
   if (i < D / 2) {
-    const double f = pow(theta, -2.0 * (double)i / (double)D);
+    double f = 1.0;
+#pragma unroll
+    for (int b = 0; b < 7; ++b)
+      if (i >> b & 1) f *= pw.p[b];
     const float hi = (float)f;
     tab[i] = make_float2(hi, (float)(f - (double)hi));
   }
@@ -94,10 +105,13 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint32_t* status = reinterpret_cast<uint32_t*>(ds.addr);
   float2* table = reinterpret_cast<float2*>(ds.addr + kTableOffset);
-  prepare_scratch<<<1, (unsigned)kMaxPairs, 0, s>>>(status, table, p.D, args->rope_theta);
+  FreqPowers pw;
+  for (int b = 0; b < 7; ++b) pw.p[b] = std::pow(args->rope_theta, -2.0 * (double)(1 << b) / (double)p.D);
+  prepare_scratch<<<1, (unsigned)kMaxPairs, 0, s>>>(status, table, p.D, pw);
   if (cudaGetLastError() != cudaSuccess)
     return internal_fail(TRIDENT_ERR_CUDA, "scratch preparation launch failed");
   p.inv_freq = table;
+  p.freq_late = 1;
   p.err = status;
   RopeBulkParams bp;
   RopePlans plans;
@@ -105,12 +119,20 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   int64_t blocks = 0;
   rope_plans(p.NH, p.D, &plans);
   const RopeEntry entry = rope_plan(plans, &p, &threads, &blocks);
-  bp.rp = p;
+  bp.rp = p;  // (its kernel reads the frequencies after the wait anyway)
   bp.first_wait_polls = kBulkWaitPolls;
   const void* fn = entry == ROPE_BULK ? ke.fn_large : (entry == ROPE_MID ? ke.fn_mid : ke.fn);
   void* kargs[1] = {entry == ROPE_BULK ? (void*)&bp : (void*)&p};
-  if (cudaLaunchKernel(fn, dim3((unsigned)(blocks < 0x7fffffff ? blocks : 0x7fffffff)),
-                       dim3((unsigned)threads), kargs, 0, s) != cudaSuccess)
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(blocks < 0x7fffffff ? blocks : 0x7fffffff));
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelExC(&cfg, fn, kargs) != cudaSuccess)
     return internal_fail(TRIDENT_ERR_CUDA, "RoPE launch failed");
   if (out_status &&
       cudaMemcpyAsync(out_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)

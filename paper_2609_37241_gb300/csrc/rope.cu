@@ -49,9 +49,10 @@ __global__ void __launch_bounds__(kRopeThreads) rope_pair_kernel(const RopeParam
   int first, end;
   const bool live = rope_item(p, (int64_t)blockIdx.x * (kRopeThreads / 32) + threadIdx.x / 32, &t, &first, &end);
   float4 fq[4];
-  rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
+  if (!p.freq_late) rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
   if (p.prefetch && live) rope_item_prefetch<D, R>(p, t, first, end);
   pdl_wait();
+  if (p.freq_late) rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
   if (live) rope_pair_rows<DT, D, QKNORM, R, true>(p, t, first, end, fq);
 }
 

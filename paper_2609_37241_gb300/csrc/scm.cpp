@@ -638,6 +638,7 @@ void pack_rope(const trident_args* a, int base, int gq, const Version& v, uint32
   p->eps = (float)a->eps;
   p->inv_D = (float)(1.0 / (double)p->D);
   p->prefetch = 0;
+  p->freq_late = 0;
 }
 
 void pack_swiglu(const trident_args* a, int g, int u, int o, int64_t T, SwigluParams* p) {
