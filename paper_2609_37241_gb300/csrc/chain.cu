@@ -26,7 +26,7 @@ namespace trident {
 
 
 // Norm role: part `part` (< SPLIT) of token `row`'s two add+RMSNorm steps.
-template <int DT, int VPT, int SPLIT>
+template <int DT, int NT, int VPT, int SPLIT>
 __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t row, const int part) {
   constexpr int EB = Act<DT>::BYTES;
   constexpr int VE = Act<DT>::VE;
@@ -38,7 +38,7 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
     // row (the sums need it) but loads only its half of both gamma vectors and writes only
     // its half of the four outputs, so no SM carries the token's full 56 KB. s1 and s2 are
     // recomputed from the packed inputs after the reduction rather than kept in registers.
-    __shared__ float2 red[kThreads / 32];
+    __shared__ float2 red[NT / 32];
     constexpr int PP = VPT / SPLIT;  // vectors per thread this CTA writes
     static_assert(VPT % SPLIT == 0, "split");
     const NormParams& n1 = c.n1;
@@ -50,7 +50,7 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
     const uint4* ap = reinterpret_cast<const uint4*>(row_ptr(n2.x, row, n2.x_rs, EB));
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
-      const int64_t vi = (int64_t)v * kThreads + tid;
+      const int64_t vi = (int64_t)v * NT + tid;
       hv[v] = ldg16(hp + vi);
       rv[v] = ldg16(rp + vi);
       av[v] = ldg16(ap + vi);
@@ -71,7 +71,7 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
     float ss1 = 0.f, ss2 = 0.f;
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
-      const int64_t vi = (int64_t)v * kThreads + tid;
+      const int64_t vi = (int64_t)v * NT + tid;
       float hf[VE], rf[VE], af[VE], s1[VE], s2[VE];
       unpack<DT>(hv[v], hf);
       unpack<DT>(rv[v], rf);
@@ -104,7 +104,7 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
     __syncthreads();
     float2 tot = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) {
+    for (int i = 0; i < NT / 32; ++i) {
       tot.x += red[i].x;
       tot.y += red[i].y;
     }
@@ -115,7 +115,7 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
       if (v / PP != part) continue;
-      const int64_t vi = (int64_t)v * kThreads + tid;
+      const int64_t vi = (int64_t)v * NT + tid;
       float hf[VE], rf[VE], af[VE], s1[VE], y1[VE], y2[VE];
       unpack<DT>(hv[v], hf);
       unpack<DT>(rv[v], rf);
@@ -144,19 +144,21 @@ __device__ __forceinline__ void chain_rope_rows(const ChainParams& c, int64_t t,
   if (ROWS && c.rope_k > 1) rope_pair_rows<DT, D, QKNORM, kChainRopeRows, false>(c.rope, t, first, end, fq);
   else rope_pair_rows<DT, D, QKNORM, 1, false>(c.rope, t, first, end, fq);
 }
-template <int DT, int D, bool QKNORM, bool ROWS>
+template <int DT, int NT, int D, bool QKNORM, bool ROWS>
 __device__ __forceinline__ void chain_rope(const ChainParams& c, const int64_t rb, const float4* fq) {
   int64_t t;
   int first, end;
-  if (rope_item(c.rope, rb * (kThreads / 32) + threadIdx.x / 32, &t, &first, &end))
+  const int w = threadIdx.x / 32;
+  if (w < c.rope_ipb && rope_item(c.rope, rb * c.rope_ipb + w, &t, &first, &end))
     chain_rope_rows<DT, D, QKNORM, ROWS>(c, t, first, end, fq);
 }
 // The item of this warp in RoPE block `part` of token t (token-major grids).
+template <int NT>
 __device__ __forceinline__ bool chain_tok_item(const ChainParams& c, int part, int* first, int* end) {
-  const int item = part * (kThreads / 32) + (int)threadIdx.x / 32;
+  const int w = (int)threadIdx.x / 32, item = part * c.rope_ipb + w;
   *first = item * c.rope.rpi;
   *end = min(c.rope.NH, *first + c.rope.rpi);
-  return item < c.rope.ipt;
+  return w < c.rope_ipb && item < c.rope.ipt;
 }
 
 // Before the PDL wait: the RoPE lane frequencies of a RoPE block (other roles load none).
@@ -166,10 +168,10 @@ __device__ __forceinline__ void chain_rope_freqs(const ChainParams& c, const boo
 }
 
 // SwiGLU role: column tile `col_tile` of row `row`, SWU x 256 16-byte vectors of g and of u
-// (kChainSwigluUnroll for one call's grid, kChainStepSwigluUnroll for a whole step's).
-template <int DT, int SWU>
+// (kChainSwigluUnroll for one call's grid, kChainStepTileVecs / NT for a whole step's).
+template <int DT, int NT, int SWU>
 __device__ __forceinline__ void chain_swiglu(const ChainParams& c, const int64_t row, const int64_t col_tile) {
-  swiglu_tile<DT, SWU>(c.sw, row, col_tile * SWU * kThreads, threadIdx.x);
+  swiglu_tile<DT, SWU, NT>(c.sw, row, col_tile * SWU * NT, threadIdx.x);
 }
 
 // Row of SwiGLU tile `tile`. A single call's kernel divides by the host's multiplier
@@ -183,18 +185,18 @@ __device__ __forceinline__ int64_t swiglu_tile_row(const ChainParams& c, const i
 }
 
 // Block b of one call's role-major grid (b < nA + nB + nC): [norms | RoPE | SwiGLU].
-template <int DT, int VPT, int SPLIT, int D, bool QKNORM, int SWU, bool STEP>
+template <int DT, int NT, int VPT, int SPLIT, int D, bool QKNORM, int SWU, bool STEP>
 __device__ __forceinline__ void chain_block(const ChainParams& c, const int b, const float4* fq) {
   if (b < c.nA) {
     const int64_t row = b / SPLIT;
-    chain_norm<DT, VPT, SPLIT>(c, row, b - (int)row * SPLIT);
+    chain_norm<DT, NT, VPT, SPLIT>(c, row, b - (int)row * SPLIT);
   } else if (b < c.nA + c.nB) {
-    chain_rope<DT, D, QKNORM, SPLIT == 1>(c, b - c.nA, fq);
+    chain_rope<DT, NT, D, QKNORM, SPLIT == 1>(c, b - c.nA, fq);
   } else {
     const int64_t tile = b - c.nA - c.nB;
     if (tile >= c.sw_tiles) return;
     const int64_t row = swiglu_tile_row<STEP>(c, tile);
-    chain_swiglu<DT, SWU>(c, row, tile - row * c.sw_tiles_per_row);
+    chain_swiglu<DT, NT, SWU>(c, row, tile - row * c.sw_tiles_per_row);
   }
 }
 
@@ -205,17 +207,17 @@ __device__ __forceinline__ void chain_block(const ChainParams& c, const int b, c
 // kernel's blocks retire, several consecutive blocks on one SM, and a role-major order can
 // give one SM four norm blocks (160 KB) while another gets 24 KB. Both indices come from
 // special registers, so no remapped index stays live in a register through the body.
-template <int DT, int VPT, int SPLIT, int D, bool QKNORM>
+template <int DT, int NT, int VPT, int SPLIT, int D, bool QKNORM>
 __device__ __forceinline__ void chain_block_tok(const ChainParams& c, const float4* fq) {
   const int q = blockIdx.x;
   if (q < SPLIT) {
-    chain_norm<DT, VPT, SPLIT>(c, blockIdx.y, q);
+    chain_norm<DT, NT, VPT, SPLIT>(c, blockIdx.y, q);
   } else if (q < SPLIT + c.rope_per_tok) {
     int first, end;
-    if (chain_tok_item(c, q - SPLIT, &first, &end))
+    if (chain_tok_item<NT>(c, q - SPLIT, &first, &end))
       chain_rope_rows<DT, D, QKNORM, false>(c, blockIdx.y, first, end, fq);
   } else {
-    chain_swiglu<DT, kChainSwigluUnroll>(c, blockIdx.y, q - SPLIT - c.rope_per_tok);
+    chain_swiglu<DT, NT, kChainTileVecs / NT>(c, blockIdx.y, q - SPLIT - c.rope_per_tok);
   }
 }
 
@@ -223,7 +225,7 @@ __device__ __forceinline__ void chain_block_tok(const ChainParams& c, const floa
 // positions, the SwiGLU tile -- one prefetch per 128-byte line, between the launch trigger
 // and the PDL wait (see prefetch_l2).
 // A token's SPLIT norm blocks share its rows' lines: part p prefetches vectors v = p mod SPLIT.
-template <int DT, int VPT, int SPLIT>
+template <int DT, int NT, int VPT, int SPLIT>
 __device__ __forceinline__ void norm_prefetch(const ChainParams& c, const int64_t row, const int part) {
   constexpr int EB = Act<DT>::BYTES;
   constexpr int VE = Act<DT>::VE;
@@ -235,7 +237,7 @@ __device__ __forceinline__ void norm_prefetch(const ChainParams& c, const int64_
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
     if (v % SPLIT != part) continue;
-    const int64_t vi = (int64_t)v * kThreads + tid;
+    const int64_t vi = (int64_t)v * NT + tid;
     if ((tid & 7) == 0) {
       prefetch_l2(hp + vi);
       prefetch_l2(rp + vi);
@@ -261,11 +263,11 @@ __device__ __forceinline__ void norm_rope_prefetch(const ChainParams& c, const i
 // prefetch == 1: every block its own first lines; prefetch == 2: only the norm blocks, which
 // take their token's rows and its RoPE head-rows (the other roles' own prefetches, issued by
 // hundreds of blocks while the previous kernel finishes, measured slower).
-template <int DT, int VPT, int SPLIT, int D, int SWU, bool STEP>
+template <int DT, int NT, int VPT, int SPLIT, int D, int SWU, bool STEP>
 __device__ __forceinline__ void chain_prefetch(const ChainParams& c, const int b) {
   const int tid = threadIdx.x;
   if (b < c.nA) {
-    norm_prefetch<DT, VPT, SPLIT>(c, b / SPLIT, b % SPLIT);
+    norm_prefetch<DT, NT, VPT, SPLIT>(c, b / SPLIT, b % SPLIT);
     if (c.prefetch == 2) norm_rope_prefetch<DT, SPLIT, D>(c, b / SPLIT, b % SPLIT);
   } else if (c.prefetch == 2) {
     return;
@@ -273,56 +275,57 @@ __device__ __forceinline__ void chain_prefetch(const ChainParams& c, const int b
     if (c.rope_k != 1) return;  // several head-rows per lane group: grids too long to prefetch
     int64_t t;
     int first, end;
-    if (rope_item(c.rope, (int64_t)(b - c.nA) * (kThreads / 32) + tid / 32, &t, &first, &end))
+    if (tid / 32 < c.rope_ipb &&
+        rope_item(c.rope, (int64_t)(b - c.nA) * c.rope_ipb + tid / 32, &t, &first, &end))
       rope_item_prefetch<D, 1>(c.rope, t, first, end);
   } else {
     const int64_t tile = b - c.nA - c.nB;
     if (tile >= c.sw_tiles) return;
     const int64_t row = swiglu_tile_row<STEP>(c, tile);
-    swiglu_prefetch<DT, SWU>(c.sw, row, (tile - row * c.sw_tiles_per_row) * SWU * kThreads, tid);
+    swiglu_prefetch<DT, SWU, NT>(c.sw, row, (tile - row * c.sw_tiles_per_row) * SWU * NT, tid);
   }
 }
 
-template <int DT, int VPT, int SPLIT, int D>
+template <int DT, int NT, int VPT, int SPLIT, int D>
 __device__ __forceinline__ void chain_prefetch_tok(const ChainParams& c) {
   const int tid = threadIdx.x, q = blockIdx.x;
   if (q < SPLIT) {
-    norm_prefetch<DT, VPT, SPLIT>(c, blockIdx.y, q);
+    norm_prefetch<DT, NT, VPT, SPLIT>(c, blockIdx.y, q);
   } else if (q < SPLIT + c.rope_per_tok) {
     int first, end;
-    if (chain_tok_item(c, q - SPLIT, &first, &end)) rope_item_prefetch<D, 1>(c.rope, blockIdx.y, first, end);
+    if (chain_tok_item<NT>(c, q - SPLIT, &first, &end)) rope_item_prefetch<D, 1>(c.rope, blockIdx.y, first, end);
   } else {
-    swiglu_prefetch<DT, kChainSwigluUnroll>(
-        c.sw, blockIdx.y, (int64_t)(q - SPLIT - c.rope_per_tok) * kChainSwigluUnroll * kThreads, tid);
+    swiglu_prefetch<DT, kChainTileVecs / NT, NT>(
+        c.sw, blockIdx.y, (int64_t)(q - SPLIT - c.rope_per_tok) * kChainTileVecs, tid);
   }
 }
 
-// Four resident blocks per SM for H 4096 (64 registers): the 64-token grid (576 blocks)
-// then fits one wave on 152 SMs; a fifth register would drop it to three blocks per SM.
+// 1024 resident threads per SM (64 registers): the 64-token grid at H 4096 (480 blocks of 256
+// threads) then fits one wave on 152 SMs; one register more would cost a quarter of them.
 // LATE (role-major grids only): only the norm blocks trigger the next launch at their start,
 // the RoPE and SwiGLU blocks at their exit. The next launch then starts once this grid's
 // short blocks are gone, and its blocks are placed while several slots per SM are free, one
 // norm block per SM, instead of filling each slot the moment it frees (up to four norm
 // blocks on one SM). The trigger is otherwise the kernel's first instruction: even one
 // parameter read ahead of it measured 0.05 us slower per launch.
-template <int DT, int VPT, int SPLIT, int D, bool QKNORM, bool LATE, int SWU>
-__global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
+template <int DT, int NT, int VPT, int SPLIT, int D, bool QKNORM, bool LATE, int SWU>
+__global__ void __launch_bounds__(NT, 1024 / NT)
     chain_kernel(const __grid_constant__ ChainParams c) {
   if (!LATE || (int)blockIdx.x < c.nA) pdl_trigger();
   float4 fq[4];
-  if (!LATE && SWU == kChainSwigluUnroll && c.tok_grid) {
-    if (c.prefetch) chain_prefetch_tok<DT, VPT, SPLIT, D>(c);
+  if (!LATE && SWU == kChainTileVecs / NT && c.tok_grid) {
+    if (c.prefetch) chain_prefetch_tok<DT, NT, VPT, SPLIT, D>(c);
     chain_rope_freqs<DT, D>(c, (int)blockIdx.x >= SPLIT && (int)blockIdx.x < SPLIT + c.rope_per_tok, fq);
     pdl_wait();
-    chain_block_tok<DT, VPT, SPLIT, D, QKNORM>(c, fq);
+    chain_block_tok<DT, NT, VPT, SPLIT, D, QKNORM>(c, fq);
   } else {
     // A role-major grid fills the GPU: its RoPE blocks become resident only as the previous
     // kernel's blocks retire, and their frequency loads measured faster after the wait.
     const int b = blockIdx.x;
-    if (c.prefetch) chain_prefetch<DT, VPT, SPLIT, D, SWU, false>(c, b);
+    if (c.prefetch) chain_prefetch<DT, NT, VPT, SPLIT, D, SWU, false>(c, b);
     pdl_wait();
     chain_rope_freqs<DT, D>(c, b >= c.nA && b < c.nA + c.nB, fq);
-    chain_block<DT, VPT, SPLIT, D, QKNORM, SWU, false>(c, b, fq);
+    chain_block<DT, NT, VPT, SPLIT, D, QKNORM, SWU, false>(c, b, fq);
   }
 }
 
@@ -332,8 +335,8 @@ __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
 // step -- every call's norm blocks, then every call's RoPE blocks, then every call's SwiGLU
 // tiles -- so that the longer blocks fill the first wave (a separate entry: the call-major
 // kernel measured about 1 % slower with this branch in it).
-template <int DT, int VPT, int SPLIT, int D, bool QKNORM, bool ROLE>
-__global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
+template <int DT, int NT, int VPT, int SPLIT, int D, bool QKNORM, bool ROLE>
+__global__ void __launch_bounds__(NT, 1024 / NT)
     chain_step_kernel(const __grid_constant__ ChainStepParams p) {
   pdl_trigger();
   const int b = blockIdx.x;
@@ -351,7 +354,7 @@ __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
     float4 fq[4];
     chain_rope_freqs<DT, D>(c, r == 1, fq);
     pdl_wait();
-    chain_block<DT, VPT, SPLIT, D, QKNORM, kChainStepSwigluUnroll, true>(c, bl, fq);
+    chain_block<DT, NT, VPT, SPLIT, D, QKNORM, kChainStepTileVecs / NT, true>(c, bl, fq);
   } else {
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
@@ -360,31 +363,38 @@ __global__ void __launch_bounds__(kThreads, VPT == 2 ? 4 : 2)
     }
     const ChainParams& c = p.c[lo];
     const int bl = b - p.first[lo];
-    if (c.prefetch) chain_prefetch<DT, VPT, SPLIT, D, kChainStepSwigluUnroll, true>(c, bl);
+    if (c.prefetch) chain_prefetch<DT, NT, VPT, SPLIT, D, kChainStepTileVecs / NT, true>(c, bl);
     float4 fq[4];
     chain_rope_freqs<DT, D>(c, bl >= c.nA && bl < c.nA + c.nB, fq);
     pdl_wait();
-    chain_block<DT, VPT, SPLIT, D, QKNORM, kChainStepSwigluUnroll, true>(c, bl, fq);
+    chain_block<DT, NT, VPT, SPLIT, D, QKNORM, kChainStepTileVecs / NT, true>(c, bl, fq);
   }
 }
 
-template <int DT, bool QK, int VPT>
+template <int DT, bool QK, int NT, int VPT>
 static void pick(KernelEntry* out) {
-  constexpr int U = kChainSwigluUnroll;
-  out->fn = (const void*)chain_kernel<DT, VPT, 2, 128, QK, false, U>;
-  out->fn_late = (const void*)chain_kernel<DT, VPT, 2, 128, QK, true, U>;
-  out->fn_inplace = (const void*)chain_kernel<DT, VPT, 1, 128, QK, false, U>;
-  out->fn_inplace_late = (const void*)chain_kernel<DT, VPT, 1, 128, QK, true, U>;
-  out->fn_wide = (const void*)chain_kernel<DT, VPT, 1, 128, QK, false, kChainWideSwigluUnroll>;
-  out->fn_step = (const void*)chain_step_kernel<DT, VPT, 2, 128, QK, false>;
-  out->fn_step_inplace = (const void*)chain_step_kernel<DT, VPT, 1, 128, QK, false>;
-  out->fn_step_role = (const void*)chain_step_kernel<DT, VPT, 1, 128, QK, true>;
+  constexpr int U = kChainTileVecs / NT;
+  out->threads = NT;
+  out->fn = (const void*)chain_kernel<DT, NT, VPT, 2, 128, QK, false, U>;
+  out->fn_late = (const void*)chain_kernel<DT, NT, VPT, 2, 128, QK, true, U>;
+  out->fn_inplace = (const void*)chain_kernel<DT, NT, VPT, 1, 128, QK, false, U>;
+  out->fn_inplace_late = (const void*)chain_kernel<DT, NT, VPT, 1, 128, QK, true, U>;
+  out->fn_wide = (const void*)chain_kernel<DT, NT, VPT, 1, 128, QK, false, kChainWideTileVecs / NT>;
+  out->fn_wide_late = (const void*)chain_kernel<DT, NT, VPT, 1, 128, QK, true, kChainWideTileVecs / NT>;
+  out->fn_step = (const void*)chain_step_kernel<DT, NT, VPT, 2, 128, QK, false>;
+  out->fn_step_inplace = (const void*)chain_step_kernel<DT, NT, VPT, 1, 128, QK, false>;
+  out->fn_step_role = (const void*)chain_step_kernel<DT, NT, VPT, 1, 128, QK, true>;
 }
 
+// H 4096: 256 threads, two vectors each. H 8192: 512 threads, two vectors each, instead of four
+// for 256 threads: at 64 registers 1024 threads fit an SM instead of 512 (28 tokens 4.70 -> 2.90
+// us, 200 tokens 12.5 -> 10.7, 3000 tokens of I 22016 167 -> 137 us; with four vectors and the
+// other changes of these kernels 3.43 us and 152). H 4096 with 512 threads of one vector lost
+// (64 tokens 3.21 / 3.76 us, 8192 tokens 205.7 / 222): twice the slots per SwiGLU tile.
 template <int DT, bool QK>
 static void pick(int64_t H, KernelEntry* out) {
-  if (H == kThreads * Act<DT>::VE * 2) pick<DT, QK, 2>(out);
-  else if (H == kThreads * Act<DT>::VE * 4) pick<DT, QK, 4>(out);
+  if (H == 4096) pick<DT, QK, 256, 2>(out);
+  else if (H == 8192) pick<DT, QK, 512, 2>(out);
 }
 
 bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry* out,
@@ -393,7 +403,6 @@ bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry*
   if (D != 128) { *why = "layer chain supports D = 128"; return false; }
   out->kind = KK_CHAIN;
   out->vec = 8;
-  out->unroll = kChainSwigluUnroll;
   // fn: two blocks per token for the norms; fn_inplace: one block per token (calls whose outputs
   // overwrite inputs, and grids too large for one wave); fn_late, fn_inplace_late: the same with
   // the late launch trigger; fn_wide: fn_inplace with wider SwiGLU tiles (grids of many waves);

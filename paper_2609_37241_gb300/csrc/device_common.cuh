@@ -411,7 +411,7 @@ __device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, i
   const int32_t pos = __ldg(p.pos + t);
   RopeGamma g;
   int kind = 0;
-  if (QKNORM && (KEEP || R == 1)) {
+  if (QKNORM && (KEEP || R == 1) && hh0 < end && hh0 < p.Hq + p.Hkv) {  // v rows need none
     kind = hh0 < p.Hq ? 1 : 2;
     rope_pair_gamma<D>(kind == 1 ? p.gamma_q : p.gamma_k, lane, &g);
   }
@@ -458,7 +458,7 @@ template <> __device__ __forceinline__ float silu_mul<DT_FP32>(float g, float u)
 }
 
 // L2 prefetch of the gate and up lines of one SwiGLU tile (threads on a line boundary).
-template <int DT, int UNROLL>
+template <int DT, int UNROLL, int NT>
 __device__ __forceinline__ void swiglu_prefetch(const SwigluParams& p, int64_t row, int64_t v0,
                                                 int tid) {
   constexpr int VE = Act<DT>::VE;
@@ -469,7 +469,7 @@ __device__ __forceinline__ void swiglu_prefetch(const SwigluParams& p, int64_t r
   const uint4* u = reinterpret_cast<const uint4*>(row_ptr(p.u, row, p.u_rs, EB));
 #pragma unroll
   for (int k = 0; k < UNROLL; ++k) {
-    const int64_t vi = v0 + (int64_t)k * kThreads + tid;
+    const int64_t vi = v0 + (int64_t)k * NT + tid;
     if (vi < nvec) {
       prefetch_l2(g + vi);
       prefetch_l2(u + vi);
@@ -477,10 +477,10 @@ __device__ __forceinline__ void swiglu_prefetch(const SwigluParams& p, int64_t r
   }
 }
 
-// One tile of UNROLL * kThreads vectors of one row, starting at vector index v0. Its loads stand
+// One tile of UNROLL * NT vectors of one row, starting at vector index v0. Its loads stand
 // in no branch (each behind its own, the compiler finishes one pair before it issues the next):
 // threads past the row's end (not FULL) load its last vector and drop it.
-template <int DT, int UNROLL, bool FULL>
+template <int DT, int UNROLL, int NT, bool FULL>
 __device__ __forceinline__ void swiglu_tile_body(const SwigluParams& p, int64_t row, int64_t v0, int tid) {
   constexpr int VE = Act<DT>::VE;
   constexpr int EB = Act<DT>::BYTES;
@@ -491,13 +491,13 @@ __device__ __forceinline__ void swiglu_tile_body(const SwigluParams& p, int64_t 
   uint4 gv[UNROLL], uv[UNROLL];
 #pragma unroll
   for (int k = 0; k < UNROLL; ++k) {
-    const int64_t vk = v0 + (int64_t)k * kThreads + tid, vi = FULL ? vk : min(vk, nvec - 1);
+    const int64_t vk = v0 + (int64_t)k * NT + tid, vi = FULL ? vk : min(vk, nvec - 1);
     gv[k] = ldg16(g + vi);
     uv[k] = ldg16(u + vi);
   }
 #pragma unroll
   for (int k = 0; k < UNROLL; ++k) {
-    const int64_t vi = v0 + (int64_t)k * kThreads + tid;
+    const int64_t vi = v0 + (int64_t)k * NT + tid;
     if (FULL || vi < nvec) {
       float gf[VE], uf[VE], of[VE];
       unpack<DT>(gv[k], gf);
@@ -513,20 +513,20 @@ __device__ __forceinline__ void swiglu_tile_body(const SwigluParams& p, int64_t 
 // I of 22016 leaves 192 of 512 vectors: 128 tokens at H 8192 10.4 us at the full width,
 // 8.5 us so; taking it in two parts instead cost a second round trip, 206 -> 209 us at 8192
 // tokens of I 14336). The width depends on the block alone.
-template <int DT, int UNROLL>
+template <int DT, int UNROLL, int NT>
 __device__ __forceinline__ void swiglu_tile(const SwigluParams& p, int64_t row, int64_t v0, int tid) {
   const int64_t left = p.I / Act<DT>::VE - v0;
-  if (left >= UNROLL * kThreads) {
-    swiglu_tile_body<DT, UNROLL, true>(p, row, v0, tid);
+  if (left >= UNROLL * NT) {
+    swiglu_tile_body<DT, UNROLL, NT, true>(p, row, v0, tid);
     return;
   }
   if constexpr (UNROLL > 1) {
-    if (left <= UNROLL / 2 * kThreads) {
-      swiglu_tile<DT, UNROLL / 2>(p, row, v0, tid);
+    if (left <= UNROLL / 2 * NT) {
+      swiglu_tile<DT, UNROLL / 2, NT>(p, row, v0, tid);
       return;
     }
   }
-  if (left > 0) swiglu_tile_body<DT, UNROLL, false>(p, row, v0, tid);
+  if (left > 0) swiglu_tile_body<DT, UNROLL, NT, false>(p, row, v0, tid);
 }
 
 }  // namespace trident

@@ -118,6 +118,7 @@ struct ChainParams {
   int32_t rope_per_tok;  // RoPE blocks per token (token-major grid: nB = T * rope_per_tok)
   int32_t rope_k;    // head-rows per RoPE lane group at most: 1, or kChainRopeRows on grids several
                      // waves long
+  int32_t rope_ipb;  // RoPE warp items per block: a warp each, fewer on grids that leave SMs idle
   uint32_t sw_magic;  // tile / sw_tiles_per_row by fast_div
   int32_t sw_shift;
   int64_t sw_tiles;  // T * sw_tiles_per_row (valid SwiGLU tiles)
@@ -128,17 +129,17 @@ struct ChainParams {
 // the single-call kernel. The struct is passed as the kernel parameter (about 25 KB, under
 // the 32 KB parameter limit), so no device buffer is written before the launch.
 constexpr int kStepMax = 48;
-// SwiGLU tile width of the layer chain's blocks, in 256-thread rounds of 16-byte vectors of
-// g and of u: one call's grid keeps tiles small (more blocks for small token counts); a whole
-// step's grid, several waves long, does better with fewer, larger tiles (measured on 36 Qwen3
-// layers: 8 tokens 11.7 -> 11.4 us, 32 tokens 39.1 -> 37.2 us, 128 tokens 155 -> 150 us;
-// the same change on single calls made them slower, 64 tokens 3.56 -> 4.09 us).
+// SwiGLU tile width of the layer chain's blocks, in 16-byte vectors of g and of u: one call's
+// grid keeps tiles small (more blocks for small token counts); a whole step's grid, several waves
+// long, does better with fewer, larger tiles (measured on 36 Qwen3 layers: 8 tokens 11.7 -> 11.4
+// us, 32 tokens 39.1 -> 37.2 us, 128 tokens 155 -> 150 us; the same change on single calls made
+// them slower, 64 tokens 3.56 -> 4.09 us). A single call's grid of many waves (one CTA per token)
+// takes the wider tiles too: blocks queue for slots there, and a tile that moves twice the bytes
+// for the same fixed costs pays.
 constexpr int kChainRopeRows = 3;
-constexpr int kChainSwigluUnroll = 2;
-constexpr int kChainStepSwigluUnroll = 4;
-// A single call's grid of many waves (one CTA per token) takes the wider tiles too: blocks
-// queue for slots there, and a tile that moves twice the bytes for the same fixed costs pays.
-constexpr int kChainWideSwigluUnroll = 4;
+constexpr int kChainTileVecs = 512;
+constexpr int kChainStepTileVecs = 1024;
+constexpr int kChainWideTileVecs = 1024;
 struct ChainStepParams {
   int32_t n;
   int32_t first[kStepMax + 1];  // call-major: call i owns blocks [first[i], first[i+1])
@@ -165,7 +166,8 @@ struct KernelEntry {
   const void* fn_inplace = nullptr;  // chain only: the entry for calls that write in place
   const void* fn_late = nullptr;     // chain only: fn with the late launch trigger (LATE)
   const void* fn_inplace_late = nullptr;  // chain only: fn_inplace with the late launch trigger
-  const void* fn_wide = nullptr;     // chain only: fn_inplace with kChainWideSwigluUnroll tiles
+  const void* fn_wide = nullptr;     // chain only: fn_inplace with kChainWideTileVecs tiles
+  const void* fn_wide_late = nullptr;  // chain only: fn_wide with the late launch trigger
   const void* fn_step_role = nullptr;  // chain only: fn_step_inplace, role-major block order
   const void* fn_step = nullptr;          // chain only: several calls per launch (ChainStepParams)
   const void* fn_step_inplace = nullptr;  // ... one block per token for the norms
@@ -176,8 +178,8 @@ struct KernelEntry {
   int32_t large_per = 1;   // ... that entry's rows per block
   int32_t large_smem = 0;  // ... and its dynamic shared memory (rows staged by bulk copies)
   int32_t kind = 0;      // which grid rule the host applies (KernelKind)
-  int32_t vec = 0;       // elements per vector (VE), or tile width for SwiGLU
-  int32_t unroll = 1;    // vectors per thread per tile (SwiGLU, chain)
+  int32_t vec = 0;       // elements per vector (VE)
+  int32_t threads = 0;   // chain: block size
   const void* nm_fn[kNormEntries] = {};  // norms, by NormEntry (NULL: none for this H)
   int32_t nm_threads[kNormEntries] = {};
   int32_t rows = 1;      // norms: rows per block of the NM_VEC entry

@@ -242,7 +242,6 @@ bool rope_kernel(int32_t dtype, int32_t variant, int32_t D, bool qknorm, KernelE
                  const char** why) {
   if (dtype != DT_BF16 && dtype != DT_FP16) { *why = "RoPE supports bf16 and fp16"; return false; }
   if (D < 2 || D % 2 != 0) { *why = "head size D must be even"; return false; }
-  out->unroll = 1;
   if (variant == 1) {  // GENERIC
     out->kind = KK_ROPE_WARP;
     out->vec = 1;

@@ -392,8 +392,9 @@ struct Version {
   CUfunction fn;
   CUfunction fn_inplace;  // layer chain: one block per token when outputs alias inputs
   CUfunction fn_late;     // layer chain: `fn` with the late launch trigger
+  CUfunction fn_wide_late;     // layer chain: `fn_wide` with the late launch trigger
   CUfunction fn_inplace_late;  // layer chain: `fn_inplace` with the late launch trigger
-  CUfunction fn_wide;     // layer chain: `fn_inplace` with kChainWideSwigluUnroll tiles
+  CUfunction fn_wide;     // layer chain: `fn_inplace` with kChainWideTileVecs tiles
   int32_t wave_blocks;    // layer chain: blocks of `fn` resident at once on the whole GPU
   CUfunction fn_large;          // RoPE: the bulk-copy entry
   CUfunction fn_mid;            // RoPE: entry between fn and fn_large (rope_plan)
@@ -424,7 +425,7 @@ struct StepMemo {
   uint64_t used;   // clock of the last store or replay (least recently used is replaced)
   int32_t m;       // calls
   int32_t ndist;   // distinct selected versions
-  unsigned grid;
+  unsigned grid, threads;
   CUfunction fn;
   int32_t sel[kStepMax];
   int32_t dist_idx[kStepMax], dist_cnt[kStepMax];
@@ -685,12 +686,12 @@ void base_config(const trident_scm* scm, void* stream, CUlaunchConfig* cfg, CUla
 }
 
 // Packs one layer-chain call: both norms, RoPE/KV, SwiGLU and the RoPE and SwiGLU block
-// counts, for SwiGLU tiles of `unroll` x 256 vectors (kChainSwigluUnroll in a call's own
-// launch, kChainStepSwigluUnroll in a whole-step launch). The norm split (set_chain_split)
+// counts, for SwiGLU tiles of `tile` vectors (kChainTileVecs in a call's own launch,
+// kChainStepTileVecs in a whole-step launch). The norm split (set_chain_split)
 // is decided by the caller.
-// SwiGLU tiles of `unroll` x 256 vectors per row: their count, nC, and the row multiplier.
-void set_chain_tiles(ChainParams* c, int64_t T, int32_t unroll, int32_t vec) {
-  const int64_t per = (int64_t)unroll * kThreads * vec;
+// SwiGLU tiles of `tile` vectors per row: their count, nC, and the row multiplier.
+void set_chain_tiles(ChainParams* c, int64_t T, int32_t tile, int32_t vec) {
+  const int64_t per = (int64_t)tile * vec;
   const int64_t tiles = (c->sw.I + per - 1) / per;
   c->nC = (int32_t)(T * tiles);
   c->sw_tiles_per_row = (int32_t)tiles;
@@ -698,27 +699,29 @@ void set_chain_tiles(ChainParams* c, int64_t T, int32_t unroll, int32_t vec) {
   c->sw_tiles = T * tiles;
 }
 
-// Sets the RoPE items of a chain call and returns its RoPE blocks (eight warp items each).
-int64_t chain_rope_blocks(RopeParams* p, int64_t T, const RopeSplit& r) {
+// Sets the RoPE items of a chain call and returns its RoPE blocks (ipb warp items each).
+int64_t chain_rope_blocks(ChainParams* c, int64_t T, const RopeSplit& r, int32_t ipb) {
+  RopeParams* p = &c->rope;
+  c->rope_ipb = ipb;
   p->ipt = r.ipt;
   p->rpi = r.rpi;
   p->ipt_magic = r.magic;
   p->ipt_shift = r.shift;
-  return (T * r.ipt + kThreads / 32 - 1) / (kThreads / 32);
+  return (T * r.ipt + ipb - 1) / ipb;
 }
 
 int32_t pack_chain(trident_scm* scm, const Version& v, const trident_args* a, const Sig& s,
-                   int32_t unroll, ChainParams* c) {
+                   int32_t tile, ChainParams* c) {
   pack_addnorm(a, C_H, C_R0, C_GA, C_X1, C_R1, s, K_ACT_H, &c->n1);
   pack_addnorm(a, C_AO, C_R1, C_GM, C_X2, C_R2, s, K_ACT_H, &c->n2);
   pack_rope(a, C_Q, a->op == TRIDENT_OP_LAYER_CHAIN_QKNORM ? C_GQ : -1, v, scm->d_err, &c->rope);
   pack_swiglu(a, C_G, C_U, C_O, s.T, &c->sw);
-  const int64_t per = (int64_t)unroll * kThreads * v.ke.vec;
+  const int64_t per = (int64_t)tile * v.ke.vec;
   const int64_t tiles = (c->sw.I + per - 1) / per;
-  const int64_t nB = chain_rope_blocks(&c->rope, s.T, v.rope_split[0]), nC = s.T * tiles;
+  const int64_t nB = chain_rope_blocks(c, s.T, v.rope_split[0], v.ke.threads / 32), nC = s.T * tiles;
   if (2 * s.T + nB + nC > 0x7fffffff) return fail(TRIDENT_ERR_INVALID, "layer chain too large for one launch");
   c->nB = (int32_t)nB;
-  set_chain_tiles(c, s.T, unroll, v.ke.vec);
+  set_chain_tiles(c, s.T, tile, v.ke.vec);
   c->prefetch = 0;
   c->tok_grid = 0;
   c->rope_per_tok = 0;
@@ -741,7 +744,7 @@ int32_t set_chain_split(const Version& v, ChainParams* c, int64_t T, int32_t spl
   c->a_split = split;
   c->nA = (int32_t)(T * split);
   c->rope_k = rope_k;
-  c->nB = (int32_t)chain_rope_blocks(&c->rope, T, v.rope_split[rope_k > 1]);
+  c->nB = (int32_t)chain_rope_blocks(c, T, v.rope_split[rope_k > 1], v.ke.threads / 32);
   *blocks = (int64_t)c->nA + c->nB + c->nC;
   return TRIDENT_OK;
 }
@@ -757,7 +760,11 @@ int32_t set_chain_split(const Version& v, ChainParams* c, int64_t T, int32_t spl
 // at 8 / 32 / 128 tokens 10.7 / 33.7 / 124.8, 10.0 / 31.0 / 116.7, 9.4 / 30.3 / 110.7 us. Within
 // one wave the two forms are level (16 tokens 2.27 / 2.25 us, 64 tokens 3.32 / 3.32, with q/k
 // norm 2.29 / 2.30 and 62 tokens 3.32 / 3.19); 80 tokens 5.11 / 3.65, which now fit one wave.
-inline int32_t chain_rope_k(int64_t one, int64_t wave_blocks) { return one > wave_blocks ? kChainRopeRows : 1; }
+// With q/k norm, whose rows are the longer, only from one and a quarter waves: 110 / 116 / 122
+// tokens 4.57 / 5.15 / 5.24 us with three rows, 4.28 / 4.88 / 4.82 with one; 128 tokens 5.36 / 4.95.
+inline int32_t chain_rope_k(int64_t one, int64_t wave_blocks, bool qknorm) {
+  return one > (qknorm ? wave_blocks + wave_blocks / 4 : wave_blocks) ? kChainRopeRows : 1;
+}
 
 // Layer-chain prefetch before the PDL wait: every block's first lines for grids of at most
 // one block per SM (small_grid); otherwise, when norm_rows, only the norm blocks prefetch:
@@ -844,22 +851,51 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     case TRIDENT_OP_LAYER_CHAIN:
     case TRIDENT_OP_LAYER_CHAIN_QKNORM: {
       ChainParams& c = P.ch;
-      int32_t st = pack_chain(scm, v, a, s, v.ke.unroll, &c);
+      cfg.blockDimX = (unsigned)v.ke.threads;
+      int32_t st = pack_chain(scm, v, a, s, kChainTileVecs, &c);
       if (st != TRIDENT_OK) return st;
       // Two CTAs per token for the norms -- so no SM carries a whole token's norm traffic --
       // while the grid still fits in one wave, and unless an output is written over an
       // input the partner CTA still reads (in-place calls keep one CTA per token).
       const int32_t split = (!chain_inplace(a) && 2 * s.T + c.nB + c.nC <= v.wave_blocks) ? 2 : 1;
       const int64_t one = s.T + c.nB + c.nC;  // one CTA per token, one head-row per lane group
-      const int32_t rope_k = split == 1 ? chain_rope_k(one, v.wave_blocks) : 1;
+      const bool qk = op == TRIDENT_OP_LAYER_CHAIN_QKNORM;
+      int32_t rope_k = split == 1 ? chain_rope_k(one, v.wave_blocks, qk) : 1;
       // Wider SwiGLU tiles (fn_wide) on grids of more than four waves: same-box probe, one
       // Llama layer at 1024 / 4096 tokens 34.2 / 122.8 -> 31.3 / 112.6 us; at 256 tokens
-      // (3.4 waves) 9.81 -> 9.75 us, at 128 tokens (1.7 waves) 4.72 -> 5.11 us.
-      wide = split == 1 && v.fn_wide && one > 4 * (int64_t)v.wave_blocks;
-      if (wide) set_chain_tiles(&c, s.T, kChainWideSwigluUnroll, v.ke.vec);
+      // (3.4 waves) 9.81 -> 9.75 us, at 128 tokens (1.7 waves) 4.72 -> 5.11 us. With blocks of
+      // 512 threads (H 8192), where a tile is one or two vectors per thread, also where the
+      // wider tiles let the grid fit one wave: 44 tokens of I 28672 5.26 -> 4.40 us, 50 of I 22016
+      // 4.65 -> 4.04 (with 256 threads, 100 and 110 tokens at H 4096, 4.14 / 4.35 -> 4.46 / 4.74).
+      wide = split == 1 && one > 4 * (int64_t)v.wave_blocks;
+      if (split == 1 && !wide && one > v.wave_blocks && v.ke.threads > kThreads) {
+        const int64_t per = (int64_t)kChainWideTileVecs * v.ke.vec, tw = (c.sw.I + per - 1) / per;
+        const int64_t rest = s.T + s.T * tw, warps = v.ke.threads / 32;
+        for (int k = 0; k < 2 && !wide; ++k) {  // with one head-row per lane group if that fits
+          if (rest + (s.T * v.rope_split[k].ipt + warps - 1) / warps <= v.wave_blocks) {
+            wide = true;
+            rope_k = k ? kChainRopeRows : 1;
+          }
+        }
+      }
+      if (wide) set_chain_tiles(&c, s.T, kChainWideTileVecs, v.ke.vec);
       int64_t blocks = 0;
       st = set_chain_split(v, &c, s.T, split, rope_k, &blocks);
       if (st != TRIDENT_OK) return st;
+      // Few blocks: a RoPE block takes four or eight items (a quarter or half of its warps) while
+      // the grid still leaves an SM to every block, or with blocks of 256 threads a quarter of
+      // the SMs idle; a warp's angles are issue-bound, and the warps of fewer items per SM finish
+      // sooner. H 8192 at 2 / 4 / 10 tokens with q/k norm 2.42 / 2.44 / 2.78 -> 2.22 / 2.24 / 2.56
+      // us, H 4096 at 10 tokens 1.85 -> 1.82 (with 144 blocks, 16 tokens, 2.23 -> 2.44).
+      const int64_t spread = v.ke.threads > kThreads ? scm->sm_count : scm->sm_count * 3 / 4;
+      for (int32_t ipb = 4; ipb < v.ke.threads / 32; ipb *= 2) {
+        const int64_t nb = (s.T * c.rope.ipt + ipb - 1) / ipb;
+        if (c.nA + nb + c.nC <= spread) {
+          c.nB = (int32_t)chain_rope_blocks(&c, s.T, v.rope_split[rope_k > 1], ipb);
+          blocks = (int64_t)c.nA + c.nB + c.nC;
+          break;
+        }
+      }
       cfg.gridDimX = (unsigned)blocks;
       // Under PDL, a role-major grid of more than a quarter block per SM whose blocks, with
       // its own norm blocks, fit the resident slots give or take an eighth of them launches a
@@ -871,18 +907,21 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       // 4.08, H 8192 at 37 tokens 4.86 -> 3.70. Equal at 2 and 4 tokens and at 1 token 1.5-2 %
       // slower (nothing to place, and the next launch starts later), hence the lower bound; a few
       // dozen blocks placed late cost less than stacked norm blocks, but with 96 blocks placed
-      // late the probe measured 3.51 -> 3.69 us, hence the upper bound.
+      // late the probe measured 3.51 -> 3.69 us, hence the upper bound; with one norm CTA per
+      // token, whose grids hold half the norm blocks, a quarter of the slots (H 8192 56 tokens 4.92 ->
+      // 4.18 us, 110 tokens with q/k norm 4.57 -> 4.32).
       // Otherwise a token-major grid (chain_block_tok) for grids of at most two blocks per SM
       // with one head-row per RoPE lane group: consecutive blocks then mix roles, so the blocks
       // that land together on one SM are not all norm blocks (measured against role-major grids
       // without the late trigger: 16 tokens 3.55 -> 2.85 us per layer step, 1 token 2.20 -> 2.04
       // us). Larger grids are role-major, which starts the longest (norm) blocks first.
-      if ((scm->opt.flags & TRIDENT_OPT_PDL) && !wide && 4 * blocks > scm->sm_count &&
-          blocks + c.nA <= v.wave_blocks + v.wave_blocks / 8) {
+      const int64_t q = v.ke.threads / kThreads;  // the bounds below count blocks of 256 threads
+      if ((scm->opt.flags & TRIDENT_OPT_PDL) && 4 * q * blocks > scm->sm_count &&
+          blocks + c.nA <= v.wave_blocks + (split == 1 ? 2 : 1) * v.wave_blocks / 8) {
         late = true;
-      } else if (rope_k == 1 && s.T >= 1 && s.T <= 65535 && blocks <= 2 * scm->sm_count) {
+      } else if (rope_k == 1 && s.T >= 1 && s.T <= 65535 && !wide && q * blocks <= 2 * scm->sm_count) {
         c.tok_grid = 1;
-        c.rope_per_tok = (c.rope.ipt + kThreads / 32 - 1) / (kThreads / 32);
+        c.rope_per_tok = (c.rope.ipt + c.rope_ipb - 1) / c.rope_ipb;
         cfg.gridDimX = (unsigned)(split + c.rope_per_tok + c.sw_tiles_per_row);
         cfg.gridDimY = (unsigned)s.T;
       }
@@ -896,8 +935,9 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   // faster layer steps at 1-4 tokens; slower once the grid fills the GPU, where a layer
   // chain prefetches only its norm rows -- see chain_prefetch_mode)
   const bool pdl = (scm->opt.flags & TRIDENT_OPT_PDL) != 0;
+  const int64_t sm_threads = v.ke.kind == KK_CHAIN ? v.ke.threads : kThreads;
   const int32_t pf =
-      pdl && (int64_t)cfg.gridDimX * cfg.gridDimY * cfg.blockDimX <= (int64_t)scm->sm_count * kThreads ? 1 : 0;
+      pdl && (int64_t)cfg.gridDimX * cfg.gridDimY * cfg.blockDimX <= scm->sm_count * sm_threads ? 1 : 0;
   switch (op) {
     case TRIDENT_OP_ADD_RMSNORM:
     case TRIDENT_OP_RMSNORM: P.nm.prefetch = pf; break;
@@ -909,7 +949,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   }
   CUfunction fn = v.fn;
   if ((op == TRIDENT_OP_LAYER_CHAIN || op == TRIDENT_OP_LAYER_CHAIN_QKNORM) && P.ch.a_split == 1)
-    fn = wide ? v.fn_wide : (late ? v.fn_inplace_late : v.fn_inplace);
+    fn = wide ? (late ? v.fn_wide_late : v.fn_wide) : (late ? v.fn_inplace_late : v.fn_inplace);
   else if (late)
     fn = v.fn_late;
   if (v.ke.kind == KK_POINTWISE)
@@ -1352,24 +1392,9 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
         if (cudaGetFuncBySymbol(&g, v.ke.fn_inplace) != cudaSuccess || !g)
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the in-place kernel entry");
         v.fn_inplace = reinterpret_cast<CUfunction>(g);
-        if (v.ke.fn_late) {
-          cudaFunction_t l = nullptr;
-          if (cudaGetFuncBySymbol(&l, v.ke.fn_late) != cudaSuccess || !l)
-            return fail(TRIDENT_ERR_CUDA, "cannot resolve the late-trigger kernel entry");
-          v.fn_late = reinterpret_cast<CUfunction>(l);
-        }
-        if (v.ke.fn_inplace_late) {
-          cudaFunction_t l = nullptr;
-          if (cudaGetFuncBySymbol(&l, v.ke.fn_inplace_late) != cudaSuccess || !l)
-            return fail(TRIDENT_ERR_CUDA, "cannot resolve the in-place late-trigger kernel entry");
-          v.fn_inplace_late = reinterpret_cast<CUfunction>(l);
-        }
-        if (v.ke.fn_wide) {
-          cudaFunction_t w = nullptr;
-          if (cudaGetFuncBySymbol(&w, v.ke.fn_wide) != cudaSuccess || !w)
-            return fail(TRIDENT_ERR_CUDA, "cannot resolve the wide-tile kernel entry");
-          v.fn_wide = reinterpret_cast<CUfunction>(w);
-        }
+        if (!resolve(v.ke.fn_late, &v.fn_late) || !resolve(v.ke.fn_inplace_late, &v.fn_inplace_late) ||
+            !resolve(v.ke.fn_wide, &v.fn_wide) || !resolve(v.ke.fn_wide_late, &v.fn_wide_late))
+          return fail(TRIDENT_ERR_CUDA, "cannot resolve the layer chain's late and wide entries");
         cudaFunction_t h = nullptr, k = nullptr;
         if (cudaGetFuncBySymbol(&h, v.ke.fn_step) != cudaSuccess || !h ||
             cudaGetFuncBySymbol(&k, v.ke.fn_step_inplace) != cudaSuccess || !k)
@@ -1383,8 +1408,8 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
           v.step_fn_role = reinterpret_cast<CUfunction>(q);
         }
         int per_sm = 0, step_per_sm = 0, sms = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.ke.fn, kThreads, 0) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&step_per_sm, v.ke.fn_step, kThreads, 0) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, v.ke.fn, v.ke.threads, 0) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&step_per_sm, v.ke.fn_step, v.ke.threads, 0) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, scm->device) != cudaSuccess)
           return fail(TRIDENT_ERR_CUDA, "occupancy query failed");
         v.wave_blocks = per_sm * sms;
@@ -1633,6 +1658,7 @@ int32_t replay_chunk(trident_scm* scm, const trident_args* a, int32_t m, uint64_
     CUlaunchAttribute attr;
     base_config(scm, stream, &cfg, &attr);
     cfg.gridDimX = e->grid;
+    cfg.blockDimX = e->threads;
     void* kp[1] = {&e->P};
     const int32_t st = launch_on(scm, &cfg, e->fn, kp);
     if (st != TRIDENT_OK) return count_error(scm, st);
@@ -1648,7 +1674,7 @@ int32_t replay_chunk(trident_scm* scm, const trident_args* a, int32_t m, uint64_
 
 // Under memo_lock: stores a fused chunk over the least recently used entry.
 void store_chunk(trident_scm* scm, const trident_args* a, int32_t m, uint64_t fp, const int32_t* sel,
-                 const ChainStepParams* P, unsigned grid, CUfunction fn) {
+                 const ChainStepParams* P, unsigned grid, unsigned threads, CUfunction fn) {
   if (!scm->memo) {
     scm->memo = static_cast<StepMemo*>(std::calloc(kMemoEntries, sizeof(StepMemo)));
     if (!scm->memo) return;  // no cache: every chunk takes the full path
@@ -1660,6 +1686,7 @@ void store_chunk(trident_scm* scm, const trident_args* a, int32_t m, uint64_t fp
   e->used = ++scm->memo_clock;
   e->m = m;
   e->grid = grid;
+  e->threads = threads;
   e->fn = fn;
   e->ndist = 0;
   for (int32_t i = 0; i < m; ++i) {
@@ -1719,14 +1746,14 @@ int32_t step_chunk(trident_scm* scm, const trident_args* a, int32_t m, void* str
     int64_t two = 0, one = 0;  // blocks with two / one CTAs per token (one head-row per lane group)
     for (int32_t i = 0; i < m; ++i) {
       ChainParams& c = P.c[i];
-      const int32_t st = pack_chain(scm, scm->versions[sel[i]], a + i, sig[i], kChainStepSwigluUnroll, &c);
+      const int32_t st = pack_chain(scm, scm->versions[sel[i]], a + i, sig[i], kChainStepTileVecs, &c);
       if (st != TRIDENT_OK) return count_error(scm, st);
       inplace = inplace || chain_inplace(a + i);
       two += 2 * sig[i].T + c.nB + c.nC;
       one += sig[i].T + c.nB + c.nC;
     }
     const int32_t split = (!inplace && two <= v0->step_wave_blocks) ? 2 : 1;
-    const int32_t rope_k = split == 1 ? chain_rope_k(one, v0->step_wave_blocks) : 1;
+    const int32_t rope_k = split == 1 ? chain_rope_k(one, v0->step_wave_blocks, a[0].op == TRIDENT_OP_LAYER_CHAIN_QKNORM) : 1;
     int64_t first = 0;
     for (int32_t i = 0; i < m; ++i) {
       int64_t blocks = 0;
@@ -1765,6 +1792,7 @@ int32_t step_chunk(trident_scm* scm, const trident_args* a, int32_t m, void* str
     grid = (unsigned)first;
     fn = split == 2 ? v0->step_fn : (role_major ? v0->step_fn_role : v0->step_fn_inplace);
     cfg.gridDimX = grid;
+    cfg.blockDimX = (unsigned)v0->ke.threads;
     void* kp[1] = {&P};
     const int32_t st = launch_on(scm, &cfg, fn, kp);
     if (st != TRIDENT_OK) return count_error(scm, st);
@@ -1779,7 +1807,7 @@ int32_t step_chunk(trident_scm* scm, const trident_args* a, int32_t m, void* str
   scm->fused_launches.fetch_add(1, std::memory_order_relaxed);
   scm->fused_calls.fetch_add((uint64_t)m, std::memory_order_relaxed);
   if (repeat && !scm->memo_lock.test_and_set(std::memory_order_acquire)) {
-    store_chunk(scm, a, m, fp, sel, scm->dry ? nullptr : &P, grid, fn);
+    store_chunk(scm, a, m, fp, sel, scm->dry ? nullptr : &P, grid, (unsigned)v0->ke.threads, fn);
     scm->memo_lock.clear(std::memory_order_release);
   }
   return TRIDENT_OK;
