@@ -183,6 +183,7 @@ struct KernelEntry {
   const void* nm_fn[kNormEntries] = {};  // norms, by NormEntry (NULL: none for this H)
   int32_t nm_threads[kNormEntries] = {};
   int32_t rows = 1;      // norms: rows per block of the NM_VEC entry
+  int32_t edge_rows = 1;  // ... and of the NM_EDGE entry
 };
 
 enum KernelKind : int32_t {

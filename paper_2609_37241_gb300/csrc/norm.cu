@@ -7,9 +7,10 @@
 // x (1024, 128)); the residual add fused in front of it is how decoder layers call it. All
 // kernels but the last two read a row once and write it once:
 //   norm_rows_kernel   rows of at most 128 vectors: LPR lanes per row, reduced by shuffles alone
+//   norm_rows_edge_kernel  such rows at any element offset that all tensors share (odd widths,
+//                      shifted bases): a warp per row, the vectors between a scalar head and tail
 //   norm_block_kernel  longer rows, one block per row, one or two vectors per thread, one barrier.
-//                      EDGE: rows at any element offset that all tensors share (odd widths,
-//                      shifted bases), the vectors between a scalar head and tail
+//                      EDGE: at any common element offset
 //   norm_bulk_kernel   long calls of such rows: the row staged by bulk copies
 //   addnorm_row_kernel long ADD_RMSNORM calls of H = 4096 in 16 bits
 //   norm_loop_kernel   16-byte rows of more than 2048 vectors (two passes)
@@ -25,7 +26,7 @@
 //   add 256 x 4096 bf16    3.17 -> 1.95        rms 4096 x 4096 bf16     12.9 -> 11.7
 //   add 3001 x 5120 bf16   23.7 -> 19.6        rms 16384 x 5120 bf16    59.5 -> 50.7
 //   add 4096 x 8192 bf16   40.4 -> 40.1        rms 2000 x 16384 fp16    36.1 -> 23.7
-//   add 4096 x 12288 bf16  65.1 -> 59.4        add 3000 x 2585 bf16     21.3 -> 14.3
+//   add 4096 x 12288 bf16  65.1 -> 59.4        add 3000 x 2585 bf16     21.3 -> 12.5
 //   add 20000 x 576 bf16   34.9 -> 19.4        rms 1 x 4096 bf16        1.39 -> 1.11
 // The long residual rows run at the 6.8 TB/s copy rate (4096 x 8192: 6.7, 4096 x 12288: 6.8).
 #include "device_common.cuh"
@@ -49,6 +50,29 @@ __device__ __forceinline__ void load_gamma(const float* g, float* out) {
   for (int q = 0; q < Act<DT>::VE / 4; ++q) {
     const float4 v = ldg_f4(g + 4 * q);
     out[4 * q] = v.x; out[4 * q + 1] = v.y; out[4 * q + 2] = v.z; out[4 * q + 3] = v.w;
+  }
+}
+
+// The weights of a vector whose first element is i, not a multiple of 4 (its offset from one, the
+// same for the whole block): the aligned float4s around them, shifted, where those lie within
+// the H weights and gamma itself is aligned; by element otherwise. By element everywhere, every
+// weight load of a warp touched 32 sectors for 128 bytes.
+template <int DT>
+__device__ __forceinline__ void load_gamma_at(const float* gamma, int i, int H, float* out) {
+  constexpr int VE = Act<DT>::VE;
+  const int sh = i & 3, b = i - sh;
+  if ((reinterpret_cast<uintptr_t>(gamma) & 15) == 0 && b + VE + 4 <= H) {
+    float t[VE + 4];
+#pragma unroll
+    for (int q = 0; q < VE / 4 + 1; ++q) {
+      const float4 v = ldg_f4(gamma + b + 4 * q);
+      t[4 * q] = v.x; t[4 * q + 1] = v.y; t[4 * q + 2] = v.z; t[4 * q + 3] = v.w;
+    }
+#pragma unroll
+    for (int e = 0; e < VE; ++e) out[e] = sh < 2 ? (sh == 0 ? t[e] : t[e + 1]) : (sh == 2 ? t[e + 2] : t[e + 3]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < VE; ++e) out[e] = __ldg(gamma + i + e);
   }
 }
 
@@ -193,8 +217,7 @@ __global__ void __launch_bounds__(1024) norm_block_kernel(const NormParams p) {
     xv[v] = ldg16(xr + (int64_t)vi * 16);
     if (RES) rv[v] = ldg16(rr + (int64_t)vi * 16);
     if (EDGE) {
-#pragma unroll
-      for (int e = 0; e < VE; ++e) g[v][e] = __ldg(p.gamma + peel + vi * VE + e);
+      load_gamma_at<DT>(p.gamma, peel + vi * VE, (int)p.H, g[v]);
     } else {
       load_gamma<DT>(p.gamma + (int64_t)vi * VE, g[v]);
     }
@@ -234,6 +257,67 @@ __global__ void __launch_bounds__(1024) norm_block_kernel(const NormParams p) {
     if (FULL || vi < nvec) st16(yr + (int64_t)vi * 16, pack<DT>(s[v]));
   }
   if (EDGE && edge >= 0) store_elem<DT>(p.y, row * p.y_rs + edge, es * inv * eg);
+}
+
+// EDGE rows of at most 128 vectors: a warp per row, eight rows per block, VPT vectors per lane;
+// a block per row (of one warp) was bound by the rate at which blocks start (20000 x 101 20.4 us).
+template <int DT, bool RES, int VPT>
+__global__ void __launch_bounds__(kThreads) norm_rows_edge_kernel(const NormParams p) {
+  pdl_prologue();
+  constexpr int VE = Act<DT>::VE;
+  constexpr int EB = Act<DT>::BYTES;
+  const int lane = threadIdx.x & 31, H = (int)p.H;
+  const int64_t row = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
+  if (row >= p.T) return;
+  const char* xr = row_ptr(p.x, row, p.x_rs, EB);
+  const int peel = (int)((16 - (reinterpret_cast<uintptr_t>(xr) & 15)) & 15) / EB;
+  const int nvec = (H - peel) / VE, tail = H - peel - nvec * VE;
+  const int edge = lane < peel ? lane : (lane < peel + tail ? nvec * VE + lane : -1);
+  xr += peel * EB;
+  const char* rr = RES ? row_ptr(p.r, row, p.r_rs, EB) + peel * EB : nullptr;
+  uint4 xv[VPT], rv[VPT];
+  float g[VPT][VE], s[VPT][VE], es = 0.f, eg = 0.f, ss = 0.f;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {  // lanes past the row's end load its last vector and drop it
+    const int vi = min(lane + 32 * v, nvec - 1);
+    xv[v] = ldg16(xr + vi * 16);
+    if (RES) rv[v] = ldg16(rr + vi * 16);
+    load_gamma_at<DT>(p.gamma, peel + vi * VE, H, g[v]);
+  }
+  if (edge >= 0) {
+    es = load_elem<DT>(p.x, row * p.x_rs + edge);
+    if (RES) es += load_elem<DT>(p.r, row * p.r_rs + edge);
+    eg = __ldg(p.gamma + edge);
+    ss = es * es;
+    if (RES) store_elem<DT>(p.r_out, row * p.ro_rs + edge, es);
+  }
+  char* ro = RES ? row_ptr(p.r_out, row, p.ro_rs, EB) + peel * EB : nullptr;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = lane + 32 * v;
+    float sq = 0.f;
+    unpack<DT>(xv[v], s[v]);
+    if (RES) {
+      float rf[VE];
+      unpack<DT>(rv[v], rf);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) s[v][e] += rf[e];
+      if (vi < nvec) st16(ro + vi * 16, pack<DT>(s[v]));
+    }
+#pragma unroll
+    for (int e = 0; e < VE; ++e) sq = fmaf(s[v][e], s[v][e], sq);
+    ss += vi < nvec ? sq : 0.f;
+  }
+  const float inv = rsqrtf(warp_sum(ss) * p.inv_H + p.eps);
+  char* yr = row_ptr(p.y, row, p.y_rs, EB) + peel * EB;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) {
+    const int vi = lane + 32 * v;
+#pragma unroll
+    for (int e = 0; e < VE; ++e) s[v][e] = s[v][e] * inv * g[v][e];
+    if (vi < nvec) st16(yr + vi * 16, pack<DT>(s[v]));
+  }
+  if (edge >= 0) store_elem<DT>(p.y, row * p.y_rs + edge, es * inv * eg);
 }
 
 // Long calls: the row's x (and r) are staged in shared memory by bulk copies (cp.async.bulk,
@@ -476,7 +560,13 @@ static void pick(int64_t H, KernelEntry* out) {
   const int vpt = nvec <= 1024 ? 1 : 2;
   const int threads = norm_threads(nvec, vpt);
   // rows that begin anywhere hold nvec or nvec - 1 whole vectors, and at least one
-  if (nvec >= 2 && nvec <= kNormBlockVecs) {
+  out->edge_rows = 1;
+  if (nvec >= 2 && nvec <= kNormRowsVecs) {
+    out->edge_rows = kThreads / 32;
+    out->nm_fn[NM_EDGE] = nvec <= 32 ? (const void*)norm_rows_edge_kernel<DT, RES, 1>
+                        : nvec <= 64 ? (const void*)norm_rows_edge_kernel<DT, RES, 2>
+                                     : (const void*)norm_rows_edge_kernel<DT, RES, 4>;
+  } else if (nvec >= 2 && nvec <= kNormBlockVecs) {
     out->nm_threads[NM_EDGE] = threads;
     out->nm_fn[NM_EDGE] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, true, false>
                                    : (const void*)norm_block_kernel<DT, RES, 2, true, false>;
@@ -550,7 +640,7 @@ NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, 
   else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX) e = NM_EDGE;  // one block per row
   *threads = ke.nm_threads[e];
   *smem = e == NM_LARGE ? ke.large_smem : 0;
-  const int64_t per = e == NM_VEC ? ke.rows : (e == NM_LARGE ? ke.large_per : 1);
+  const int64_t per = e == NM_VEC ? ke.rows : e == NM_LARGE ? ke.large_per : e == NM_EDGE ? ke.edge_rows : 1;
   *blocks = (p->T + per - 1) / per;
   return e;
 }

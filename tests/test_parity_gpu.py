@@ -302,6 +302,7 @@ def test_pointwise_parity(S, name, dtype, W, T, layout, variant):
     (FP16, 3, 16384, "dense"), (FP32, 2, 8192, "dense"),   # two vectors per thread, exactly full
     (BF16, 3, 16392, "dense"),                             # longer than a block holds: two passes
     (BF16, 19, 1001, "dense"), (FP16, 6, 4099, "offset"),  # rows at every offset
+    (BF16, 1003, 101, "dense"), (FP16, 37, 333, "offset"), (FP32, 65, 511, "dense"), (BF16, 41, 1023, "dense"),
     (FP32, 8, 9, "offset"), (BF16, 9, 15, "offset"),       # one whole vector between the edges; none
     (FP16, 5, 2048, "gamma"), (BF16, 6, 520, "apart"),     # weights, or one tensor, at another offset
     (BF16, 1025, 4096, "dense"), (FP16, 1100, 5120, "padded"), (FP16, 420, 16000, "dense"),  # bulk copies
