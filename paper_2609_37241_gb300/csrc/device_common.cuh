@@ -239,12 +239,15 @@ __device__ __forceinline__ bool rope_item(const RopeParams& p, int64_t item, int
 }
 
 // Source of head-row hh of token t (its lane-0 vector).
-template <int D>
-__device__ __forceinline__ const char* rope_row_src(const RopeParams& p, int64_t t, int hh) {
-  constexpr int RB = D * 2;
+__device__ __forceinline__ const char* rope_row_src(const RopeParams& p, int64_t t, int hh, int D) {
+  const int RB = D * 2;
   return hh < p.Hq ? row_ptr(p.q, t, p.q_rs, 2) + (int64_t)hh * RB
        : hh < p.Hq + p.Hkv ? row_ptr(p.k, t, p.k_rs, 2) + (int64_t)(hh - p.Hq) * RB
                            : row_ptr(p.v, t, p.v_rs, 2) + (int64_t)(hh - p.Hq - p.Hkv) * RB;
+}
+template <int D>
+__device__ __forceinline__ const char* rope_row_src(const RopeParams& p, int64_t t, int hh) {
+  return rope_row_src(p, t, hh, D);
 }
 
 // Sines and cosines of a lane's eight pairs for position pos; fq holds the lane's frequencies.
@@ -267,8 +270,7 @@ __device__ __forceinline__ void rope_pair_freqs(const float2* inv_freq, int lane
 
 // A lane's q- or k-norm weights (kind 1: q, 2: k), for its low and high halves.
 struct RopeGamma { F2 lo[4], hi[4]; };
-template <int D>
-__device__ __forceinline__ void rope_pair_gamma(const float* gamma, int lane, RopeGamma* g) {
+__device__ __forceinline__ void rope_pair_gamma(const float* gamma, int lane, int D, RopeGamma* g) {
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     const float4 a = ldg_f4(gamma + lane * 8 + 4 * q), b = ldg_f4(gamma + D / 2 + lane * 8 + 4 * q);
@@ -291,10 +293,10 @@ __device__ __forceinline__ void rope_unpack(const uint4& lo, const uint4& hi, F2
   }
 }
 
-// 1 / rms of a head-row held by the lane group (LPG lanes), in both halves of a pair.
-template <int D>
-__device__ __forceinline__ F2 rope_inv_rms(const RopeParams& p, const F2* A, const F2* B) {
-  constexpr int LPG = RopeGeom<D>::LPG;
+// 1 / rms of a head-row held by the lane group (LPG lanes; on: the lane holds part of it), in
+// both halves of a pair.
+template <int LPG>
+__device__ __forceinline__ F2 rope_inv_rms(const RopeParams& p, const F2* A, const F2* B, bool on = true) {
   F2 s2 = f2_mul(A[0], A[0]);
 #pragma unroll
   for (int q = 1; q < 4; ++q) s2 = f2_fma(A[q], A[q], s2);
@@ -302,7 +304,7 @@ __device__ __forceinline__ F2 rope_inv_rms(const RopeParams& p, const F2* A, con
   for (int q = 0; q < 4; ++q) s2 = f2_fma(B[q], B[q], s2);
   float s0, s1;
   f2_unpack(s2, &s0, &s1);
-  float ss = s0 + s1;
+  float ss = on ? s0 + s1 : 0.f;
   const unsigned mask =
       LPG == 32 ? 0xffffffffu : (((1u << LPG) - 1u) << ((threadIdx.x & 31) & ~(LPG - 1)));
 #pragma unroll
@@ -319,18 +321,17 @@ __device__ __forceinline__ void rope_scale(F2 inv, const RopeGamma& g, F2* A, F2
 }
 
 // Where head-row hh of token t goes (its lane-0 vector).
-template <int D>
-__device__ __forceinline__ char* rope_row_dst(const RopeParams& p, int64_t t, int hh, int32_t pos) {
-  constexpr int RB = D * 2;
+__device__ __forceinline__ char* rope_row_dst(const RopeParams& p, int64_t t, int hh, int32_t pos, int D) {
+  const int RB = D * 2;
   if (hh < p.Hq) return row_ptr(p.q, t, p.q_rs, 2) + (int64_t)hh * RB;
   const bool is_v = hh >= p.Hq + p.Hkv;
   return reinterpret_cast<char*>(is_v ? p.v_cache : p.k_cache) +
          ((int64_t)(hh - p.Hq - (is_v ? p.Hkv : 0)) * p.S + pos) * RB;
 }
 
-// Rotates a lane's pairs and stores them at dst (the lane's low vector).
-template <int DT, int D>
-__device__ __forceinline__ void rope_rotate(char* dst, const RopeAngles& an, const F2* A, const F2* B) {
+// Rotates a lane's pairs and stores them at dst (the lane's low vector; D bytes on, the high one).
+template <int DT>
+__device__ __forceinline__ void rope_rotate(char* dst, int D, const RopeAngles& an, const F2* A, const F2* B) {
   float a[8], b[8];
   // low half: x_i c - x_{i+D/2} s;  high half: x_{i+D/2} c + x_i s
 #pragma unroll
@@ -349,7 +350,7 @@ template <int DT, int D, bool QKNORM, bool KEEP>
 __device__ __forceinline__ void rope_pair_finish(const RopeParams& p, int64_t t, int hh, int lane, int32_t pos,
                                                  const uint4& lo, const uint4& hi, const RopeAngles& an,
                                                  RopeGamma* g, int* kind) {
-  char* dst = rope_row_dst<D>(p, t, hh, pos) + lane * 16;
+  char* dst = rope_row_dst(p, t, hh, pos, D) + lane * 16;
   if (hh >= p.Hq + p.Hkv) {  // bit copy into the cache
     st16(dst, lo);
     st16(dst + D, hi);
@@ -357,23 +358,24 @@ __device__ __forceinline__ void rope_pair_finish(const RopeParams& p, int64_t t,
   }
   F2 A[4], B[4];
   rope_unpack<DT>(lo, hi, A, B);
+  constexpr int LPG = RopeGeom<D>::LPG;
   if (QKNORM) {
     const bool is_q = hh < p.Hq;
-    const F2 inv = rope_inv_rms<D>(p, A, B);
+    const F2 inv = rope_inv_rms<LPG>(p, A, B);
     if (KEEP) {
       const int want = is_q ? 1 : 2;
       if (*kind != want) {
-        rope_pair_gamma<D>(is_q ? p.gamma_q : p.gamma_k, lane, g);
+        rope_pair_gamma(is_q ? p.gamma_q : p.gamma_k, lane, D, g);
         *kind = want;
       }
       rope_scale(inv, *g, A, B);
     } else {
       RopeGamma own;
-      rope_pair_gamma<D>(is_q ? p.gamma_q : p.gamma_k, lane, &own);
+      rope_pair_gamma(is_q ? p.gamma_q : p.gamma_k, lane, D, &own);
       rope_scale(inv, own, A, B);
     }
   }
-  rope_rotate<DT, D>(dst, an, A, B);
+  rope_rotate<DT>(dst, D, an, A, B);
 }
 
 // L2 prefetch of an item's row lines (at most R rows per lane group) and position.
@@ -413,7 +415,7 @@ __device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, i
   int kind = 0;
   if (QKNORM && (KEEP || R == 1) && hh0 < end && hh0 < p.Hq + p.Hkv) {  // v rows need none
     kind = hh0 < p.Hq ? 1 : 2;
-    rope_pair_gamma<D>(kind == 1 ? p.gamma_q : p.gamma_k, lane, &g);
+    rope_pair_gamma(kind == 1 ? p.gamma_q : p.gamma_k, lane, D, &g);
   }
   if (pos < 0 || (int64_t)pos >= p.S) {  // uniform over the warp: one token per item
     if ((threadIdx.x & 31) == 0) atomicOr(p.err, kErrPos);
@@ -424,14 +426,14 @@ __device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, i
     if (hh0 >= end) return;
     F2 A[4], B[4];
     rope_unpack<DT>(lo[0], hi[0], A, B);
-    rope_scale(rope_inv_rms<D>(p, A, B), g, A, B);
+    rope_scale(rope_inv_rms<LPG>(p, A, B), g, A, B);
     rope_angles(pos, fq, &an);
-    char* dst = rope_row_dst<D>(p, t, hh0, pos) + lane * 16;
+    char* dst = rope_row_dst(p, t, hh0, pos, D) + lane * 16;
     if (hh0 >= p.Hq + p.Hkv) {  // bit copy into the cache
       st16(dst, lo[0]);
       st16(dst + D, hi[0]);
     } else {
-      rope_rotate<DT, D>(dst, an, A, B);
+      rope_rotate<DT>(dst, D, an, A, B);
     }
     return;
   }

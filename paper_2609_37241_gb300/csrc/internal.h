@@ -172,6 +172,7 @@ struct KernelEntry {
   const void* fn_step = nullptr;          // chain only: several calls per launch (ChainStepParams)
   const void* fn_step_inplace = nullptr;  // ... one block per token for the norms
   const void* fn_large = nullptr;  // RoPE: the bulk-copy entry (rope_plan chooses)
+  const void* any_fn[2] = {};      // RoPE versions of the generic kind: rope_any_kernel (or NULL)
   const void* fn_mid = nullptr;    // RoPE: the entry between fn and fn_large (rope_plan chooses)
   const void* pw_fn[kPwEntries] = {};  // elementwise, by PointwiseEntry
   int64_t large_rows = 0;  // norms: rows from which a call takes the NM_LARGE entry
@@ -232,15 +233,15 @@ inline void div_magic(uint32_t d, uint32_t* m, int32_t* l) {
 }
 
 // How a token's NH head-rows are split into warp items of at most `max_rows` rows per lane
-// group (a warp has 512 / D groups), as evenly as the groups allow.
+// group (gw groups per warp), as evenly as the groups allow.
 struct RopeSplit {
   int32_t ipt, rpi;  // items per token, head-rows per item
   uint32_t magic;    // item / ipt by fast_div
   int32_t shift;
 };
-inline RopeSplit rope_split(int64_t NH, int32_t D, int32_t max_rows) {
+inline RopeSplit rope_split(int64_t NH, int64_t gw, int32_t max_rows) {
   RopeSplit r{};
-  const int64_t gw = 512 / D, quads = (NH + gw - 1) / gw, ipt = (quads + max_rows - 1) / max_rows;
+  const int64_t quads = (NH + gw - 1) / gw, ipt = (quads + max_rows - 1) / max_rows;
   if (ipt < 1) return r;
   const int64_t rpi = (quads + ipt - 1) / ipt * gw;
   r.rpi = (int32_t)rpi;
@@ -254,8 +255,10 @@ inline RopeSplit rope_split(int64_t NH, int32_t D, int32_t max_rows) {
 enum RopeEntry : int32_t { ROPE_SMALL = 0, ROPE_MID = 1, ROPE_BULK = 2 };
 struct RopePlans {
   RopeSplit split[3];  // by RopeEntry
+  RopeSplit any[2];    // rope_any_kernel with one and with three rows per lane group (ipt 0: none)
 };
 void rope_plans(int64_t NH, int32_t D, RopePlans* out);
 RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks);
+int rope_any_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks);
 
 }  // namespace trident

@@ -7,8 +7,9 @@
 // needs no exchange between lanes and a token's angles are computed once per lane and item.
 // Three entries, by the call's size (rope_plan): one head-row per lane group where latency
 // counts, two in between, and for calls of many tokens three, staged in shared memory by
-// cp.async.bulk (rope_bulk_kernel). The generic kernel gives each head-row one warp and scalar
-// accesses (any alignment, any even D). All compute (cos, sin) of pos * theta^(-2i/D) in the
+// cp.async.bulk (rope_bulk_kernel). Other head sizes that
+// are multiples of 16 take rope_any_kernel, the same with lanes left over; the generic kernel gives
+// each head-row one warp and scalar accesses (any alignment, any even D). All compute (cos, sin) of pos * theta^(-2i/D) in the
 // kernel from the version's double-float frequency table [D/2], which the host splits from
 // fp64 at registration.
 //
@@ -143,6 +144,58 @@ __global__ void __launch_bounds__(kRopeBulkThreads, 6) rope_bulk_kernel(const Ro
   }
 }
 
+// Head sizes without a kernel of their own, and versions that promise no alignment, when a call's
+// tensors are 16-byte aligned and D is a multiple of 16 of at most 256: the pair layout with LPG
+// lanes per head-row, D / 16 of them holding part of it.
+template <int DT, int LPG, bool QKNORM, int R>
+__global__ void __launch_bounds__(kRopeThreads) rope_any_kernel(const RopeParams p) {
+  pdl_prologue();
+  constexpr int GW = 32 / LPG;
+  const int D = p.D, l = (threadIdx.x & 31) % LPG, lane = min(l, D / 16 - 1);
+  const bool on = l == lane;
+  int64_t t;
+  int first, end;
+  if (!rope_item(p, (int64_t)blockIdx.x * (kRopeThreads / 32) + threadIdx.x / 32, &t, &first, &end)) return;
+  const int hh0 = first + (threadIdx.x & 31) / LPG;
+  uint4 lo[R], hi[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) {  // groups past the item's end load its last row and drop it
+    const char* src = rope_row_src(p, t, min(hh0 + j * GW, end - 1), D) + lane * 16;
+    lo[j] = ld16(src);
+    hi[j] = ld16(src + D);
+  }
+  const int32_t pos = __ldg(p.pos + t);
+  if (pos < 0 || (int64_t)pos >= p.S) {
+    if ((threadIdx.x & 31) == 0) atomicOr(p.err, kErrPos);
+    return;
+  }
+  float4 fq[4];
+  rope_pair_freqs(p.inv_freq, lane, fq);
+  RopeAngles an;
+  rope_angles(pos, fq, &an);
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int hh = hh0 + j * GW;
+    if (hh >= end) break;
+    char* dst = rope_row_dst(p, t, hh, pos, D) + lane * 16;
+    if (hh >= p.Hq + p.Hkv) {  // bit copy into the cache
+      if (on) {
+        st16(dst, lo[j]);
+        st16(dst + D, hi[j]);
+      }
+      continue;
+    }
+    F2 A[4], B[4];
+    rope_unpack<DT>(lo[j], hi[j], A, B);
+    if (QKNORM) {
+      RopeGamma g;
+      rope_pair_gamma(hh < p.Hq ? p.gamma_q : p.gamma_k, lane, D, &g);
+      rope_scale(rope_inv_rms<LPG>(p, A, B, on), g, A, B);
+    }
+    if (on) rope_rotate<DT>(dst, D, an, A, B);
+  }
+}
+
 template <int DT, bool QKNORM>
 __global__ void __launch_bounds__(kThreads) rope_generic_kernel(const RopeParams p) {
   pdl_prologue();
@@ -205,10 +258,20 @@ __global__ void __launch_bounds__(kThreads) rope_generic_kernel(const RopeParams
   }
 }
 
+static int rope_any_lanes(int32_t D) {  // 0: no such kernel
+  if (D < 32 || D > 256 || D % 16 != 0) return 0;
+  return D <= 64 ? 4 : D <= 128 ? 8 : 16;
+}
+
 void rope_plans(int64_t NH, int32_t D, RopePlans* out) {
-  out->split[ROPE_SMALL] = rope_split(NH, D, 1);
-  out->split[ROPE_MID] = rope_split(NH, D, 2);
-  out->split[ROPE_BULK] = rope_split(NH, D, kRopeBulkRows);
+  if (const int lanes = rope_any_lanes(D)) {
+    out->any[0] = rope_split(NH, 32 / lanes, 1);
+    out->any[1] = rope_split(NH, 32 / lanes, 3);
+  }
+  if (D != 64 && D != 128 && D != 256) return;
+  out->split[ROPE_SMALL] = rope_split(NH, 512 / D, 1);
+  out->split[ROPE_MID] = rope_split(NH, 512 / D, 2);
+  out->split[ROPE_BULK] = rope_split(NH, 512 / D, kRopeBulkRows);
 }
 
 RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks) {
@@ -222,6 +285,41 @@ RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int
   *threads = e == ROPE_BULK ? kRopeBulkThreads : kRopeThreads;
   *blocks = (p->T * r.ipt + *threads / 32 - 1) / (*threads / 32);
   return e;
+}
+
+// The rope_any_kernel entry of a call of a version without an aligned kernel, or -1: one row per
+// lane group below about three items per SM, three from there. D 96, 32 + 8 + 8 heads, against
+// the generic kernel, with q/k norm / without: 20 tokens 3.50 -> 2.31 / 2.44 -> 2.01 us, 3000
+// tokens 55.7 -> 14.6 / 41.4 -> 10.9; D 160, 16 + 8 + 8 heads with the norm 40.5 -> 18.5.
+int rope_any_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks) {
+  if (plans.any[0].ipt == 0) return -1;
+  const uintptr_t ptrs = (uintptr_t)p->q | (uintptr_t)p->k | (uintptr_t)p->v | (uintptr_t)p->k_cache |
+                         (uintptr_t)p->v_cache | (uintptr_t)p->gamma_q | (uintptr_t)p->gamma_k;
+  if (ptrs % 16 != 0 || (p->T > 1 && (p->q_rs % 8 != 0 || p->k_rs % 8 != 0 || p->v_rs % 8 != 0))) return -1;
+  const int e = p->T * plans.any[0].ipt > kRopeSmallItems ? 1 : 0;
+  const RopeSplit& r = plans.any[e];
+  p->ipt = r.ipt;
+  p->rpi = r.rpi;
+  p->ipt_magic = r.magic;
+  p->ipt_shift = r.shift;
+  *threads = kRopeThreads;
+  *blocks = (p->T * r.ipt + kRopeThreads / 32 - 1) / (kRopeThreads / 32);
+  return e;
+}
+
+template <int DT, bool QK>
+static void pick_any(int32_t D, KernelEntry* out) {
+  const int lanes = rope_any_lanes(D);
+  if (lanes == 4) {
+    out->any_fn[0] = (const void*)rope_any_kernel<DT, 4, QK, 1>;
+    out->any_fn[1] = (const void*)rope_any_kernel<DT, 4, QK, 3>;
+  } else if (lanes == 8) {
+    out->any_fn[0] = (const void*)rope_any_kernel<DT, 8, QK, 1>;
+    out->any_fn[1] = (const void*)rope_any_kernel<DT, 8, QK, 3>;
+  } else if (lanes == 16) {
+    out->any_fn[0] = (const void*)rope_any_kernel<DT, 16, QK, 1>;
+    out->any_fn[1] = (const void*)rope_any_kernel<DT, 16, QK, 3>;
+  }
 }
 
 template <int DT, bool QK, int D>
@@ -244,6 +342,8 @@ bool rope_kernel(int32_t dtype, int32_t variant, int32_t D, bool qknorm, KernelE
   if (D < 2 || D % 2 != 0) { *why = "head size D must be even"; return false; }
   if (variant == 1) {  // GENERIC
     out->kind = KK_ROPE_WARP;
+    if (dtype == DT_BF16) qknorm ? pick_any<DT_BF16, true>(D, out) : pick_any<DT_BF16, false>(D, out);
+    else qknorm ? pick_any<DT_FP16, true>(D, out) : pick_any<DT_FP16, false>(D, out);
     out->vec = 1;
     if (dtype == DT_BF16) out->fn = qknorm ? (const void*)rope_generic_kernel<DT_BF16, true>
                                            : (const void*)rope_generic_kernel<DT_BF16, false>;

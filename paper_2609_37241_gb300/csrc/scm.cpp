@@ -401,6 +401,7 @@ struct Version {
   RopePlans rope_plans;         // vector RoPE: item splits of its three entries
   RopeSplit rope_split[2];      // layer chain: item splits with one and kChainRopeRows rows
   CUfunction pw_fn[kPwEntries];  // elementwise: entries by layout and size (pointwise_plan)
+  CUfunction any_fn[2];            // RoPE versions of the generic kind: rope_any_kernel
   CUfunction nm_fn[kNormEntries];  // norms: entries by layout and size (norm_plan)
   CUfunction step_fn;           // layer chain: several calls per launch (two blocks per token)
   CUfunction step_fn_inplace;   // ... one block per token
@@ -799,6 +800,8 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   bool late = false;  // layer chain: launch fn_late (the late launch trigger)
   bool wide = false;  // layer chain: launch fn_wide (wider SwiGLU tiles)
   RopeEntry rope_entry = ROPE_SMALL;
+  int rope_any = -1;
+  int64_t rope_blocks = 0;
   int pw_entry = PW_GENERIC;
   NormEntry nm_entry = NM_GENERIC;
   switch (op) {
@@ -831,6 +834,10 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
         cfg.gridDimX = cap_grid(blocks);
         if (rope_entry == ROPE_BULK)
           P.rb.first_wait_polls = (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) ? 0u : kBulkWaitPolls;
+      } else if (int32_t threads = 0; v.any_fn[0] &&
+                 (rope_any = rope_any_plan(v.rope_plans, &P.rp, &threads, &rope_blocks)) >= 0) {
+        cfg.blockDimX = (unsigned)threads;
+        cfg.gridDimX = cap_grid(rope_blocks);
       } else {  // generic: one warp per head-row
         const int64_t units = P.rp.T * P.rp.NH, upb = kThreads / 32;
         cfg.gridDimX = cap_grid((units + upb - 1) / upb);
@@ -958,6 +965,8 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     fn = rope_entry == ROPE_BULK ? v.fn_large : (rope_entry == ROPE_MID ? v.fn_mid : v.fn);
   else if (v.ke.kind == KK_NORM)
     fn = v.nm_fn[nm_entry];
+  else if (rope_any >= 0)
+    fn = v.any_fn[rope_any];
   return launch_on(scm, &cfg, fn, kp);
 }
 
@@ -1343,11 +1352,11 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
   v.rope = g_ops[desc->op].rope;
   st = resolve_kernel(v.d, &v.ke);
   if (st != TRIDENT_OK) return st;
-  if (v.ke.kind == KK_ROPE_PAIR)
+  if (v.ke.kind == KK_ROPE_PAIR || v.ke.any_fn[0])
     rope_plans(desc->fixed[0] + 2 * desc->fixed[1], (int32_t)desc->fixed[2], &v.rope_plans);
   if (v.ke.kind == KK_CHAIN)
     for (int k = 0; k < 2; ++k)
-      v.rope_split[k] = rope_split(desc->fixed[1] + 2 * desc->fixed[2], (int32_t)desc->fixed[3],
+      v.rope_split[k] = rope_split(desc->fixed[1] + 2 * desc->fixed[2], 512 / desc->fixed[3],
                                    k ? kChainRopeRows : 1);
   std::lock_guard<std::mutex> lk(scm->reg_mu);
   const int32_t n = scm->count.load(std::memory_order_relaxed);
@@ -1378,6 +1387,9 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
       for (int k = 0; k < kPwEntries; ++k)
         if (!resolve(v.ke.pw_fn[k], &v.pw_fn[k]))
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the elementwise kernel entries");
+      for (int k = 0; k < 2; ++k)
+        if (!resolve(v.ke.any_fn[k], &v.any_fn[k]))
+          return fail(TRIDENT_ERR_CUDA, "cannot resolve the RoPE kernel entries");
       for (int k = 0; k < kNormEntries; ++k)
         if (!resolve(v.ke.nm_fn[k], &v.nm_fn[k]))
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the norm kernel entries");

@@ -502,6 +502,21 @@ def test_rope_kv_item_edges(S, T, Hq, Hkv, D, qk, dtype):
     check_rope(ref, got, inp, dtype)
 
 
+@pytest.mark.parametrize("D,T,Hq,Hkv,variant,dtype,layout", [
+    (96, 7, 4, 2, 0, BF16, "fused"), (96, 300, 5, 1, 0, FP16, "separate"), (80, 33, 3, 1, 0, BF16, "separate"),
+    (112, 150, 7, 2, 0, FP16, "fused"), (160, 40, 3, 2, 0, BF16, "fused"), (240, 90, 2, 1, 0, BF16, "separate"),
+    (32, 200, 9, 3, 0, BF16, "fused"), (48, 1, 1, 1, 0, FP16, "separate"),  # few lanes per head-row
+    (128, 60, 4, 2, 1, BF16, "separate"), (256, 3, 2, 1, 1, FP16, "separate"),  # aligned calls, any-alignment version
+    (40, 9, 2, 1, 0, BF16, "separate"), (272, 5, 2, 1, 0, BF16, "separate")])  # neither: scalar accesses
+def test_rope_kv_other_head_sizes(S, D, T, Hq, Hkv, variant, dtype, layout):
+    """Head sizes without a kernel of their own, and versions of any alignment on aligned calls."""
+    for qk in (False, True):
+        ref, got, inp = run_rope(S, T, Hq, Hkv, D, 512, 1e4, qk, dtype=dtype, layout=layout, variant=variant,
+                                 seed=D + T)
+        assert got["status"] == 0
+        check_rope(ref, got, inp, dtype)
+
+
 def test_rope_kv_many_tokens_bad_positions(S):
     T = 603
     pos = synth.positions(np.random.default_rng(5), T, 8192)
