@@ -425,16 +425,16 @@ __device__ __forceinline__ void rope_pair_rows(const RopeParams& p, int64_t t, i
   if (QKNORM && R == 1) {  // the norm first: its weights' registers are free before the angles'
     if (hh0 >= end) return;
     F2 A[4], B[4];
+    if (hh0 >= p.Hq + p.Hkv) {  // bit copy into the cache
+      char* dst = rope_row_dst(p, t, hh0, pos, D) + lane * 16;
+      st16(dst, lo[0]);
+      st16(dst + D, hi[0]);
+      return;
+    }
     rope_unpack<DT>(lo[0], hi[0], A, B);
     rope_scale(rope_inv_rms<LPG>(p, A, B), g, A, B);
     rope_angles(pos, fq, &an);
-    char* dst = rope_row_dst(p, t, hh0, pos, D) + lane * 16;
-    if (hh0 >= p.Hq + p.Hkv) {  // bit copy into the cache
-      st16(dst, lo[0]);
-      st16(dst + D, hi[0]);
-    } else {
-      rope_rotate<DT>(dst, D, an, A, B);
-    }
+    rope_rotate<DT>(rope_row_dst(p, t, hh0, pos, D) + lane * 16, D, an, A, B);
     return;
   }
   rope_angles(pos, fq, &an);
