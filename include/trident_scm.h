@@ -170,9 +170,9 @@ typedef enum trident_variant {
                                           step of a hit reports ERR_CUDA without launching */
 #define TRIDENT_OPT_NO_STEP_REPLAY 0x20 /* invoke_step never replays a stored chunk */
 #define TRIDENT_OPT_TEST_WAIT_TIMEOUT 0x40 /* for tests of the device-side timeout path: the
-                                          bulk-copy add+RMSNorm kernel gives up its first
-                                          wait for its copies at once (0 polls), so every
-                                          block takes the timeout path -- sets
+                                          bulk-copy norm and RoPE kernels give up their first
+                                          wait for their copies at once (0 polls), so every
+                                          block (warp) takes the timeout path -- sets
                                           TRIDENT_DEVERR_TIMEOUT, drains its copies with the
                                           full bounded wait and returns without writing */
 

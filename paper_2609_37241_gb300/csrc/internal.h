@@ -12,7 +12,7 @@ namespace trident {
 // Activation element types (values equal trident_dtype).
 enum : int32_t { DT_BF16 = 1, DT_FP16 = 2, DT_FP32 = 3 };
 
-constexpr int kThreads = 256;  // block size of every kernel in this library
+constexpr int kThreads = 256;  // block size of the kernels that do not say otherwise
 
 // RMSNorm over T rows of H elements, with a residual add or without (r, r_out unused). Row
 // strides in elements.
