@@ -6,7 +6,7 @@
 // lanes per head-row, each lane holding both halves of its rotated pairs, so that a rotation
 // needs no exchange between lanes and a token's angles are computed once per lane and item.
 // Three entries, by the call's size (rope_plan): one head-row per lane group where latency
-// counts, two in between, and for calls of many tokens three, staged in shared memory by
+// counts, two where it pays, and for calls of many tokens three, staged in shared memory by
 // cp.async.bulk (rope_bulk_kernel). Other head sizes that
 // are multiples of 16 take rope_any_kernel, the same with lanes left over; the generic kernel gives
 // each head-row one warp and scalar accesses (any alignment, any even D). All compute (cos, sin) of pos * theta^(-2i/D) in the
@@ -22,23 +22,38 @@
 //   120 tokens   3.58 -> 3.01 / 3.18 -> 2.77 us     3333 tokens   26.5 -> 15.1 / 20.8 -> 13.7 us
 //   250 tokens   5.13 -> 3.22 / 4.48 -> 3.04 us     8192 tokens   51.7 -> 33.3 / 41.8 -> 30.9 us
 // (8192 tokens without the norm: 0.96 of the copy rate.) D 64 at 250 tokens without the norm
-// is the one size of that sweep that lost (2.63 -> 3.01 us).
+// is the one size of the sweeps that lost (2.63 -> 2.88 us).
 #include "device_common.cuh"
 
 namespace trident {
 
 // Small and mid entries: 64 threads, two items per block (128 threads: the same within 3 %).
 constexpr int kRopeThreads = 64;
-// Calls of at most this many one-row items (three per SM) take one head-row per lane group:
-// the call is one memory round trip, and a second row per group only lengthens it. Above, two
-// rows per group halve the warps that fetch the same frequency and weight lines: 60 tokens with
-// q/k norm 2.33 us against 2.62 with one row, 500 tokens 4.67 against 5.51.
-constexpr int64_t kRopeSmallItems = 456;
-// Calls of at least this many tokens take the bulk-copy entry: at 512 tokens it is level with two
-// register-held rows per group (with q/k norm 5.0 against 4.9 us, without 4.6 against 3.9), from
-// about 1024 ahead (2048 tokens 10.5 / 8.9 against 12.3 / 10.5 us; 8192 33.3 / 30.9 against
-// 38.0 / 32.8).
+// One head-row per lane group (small entry) or two (mid), by the call's one-row items per SM. Up
+// to three the call is one memory round trip, and a second row only lengthens it; on long calls
+// two rows halve the warps that fetch the same frequency and weight lines (60 tokens of 32 + 8 + 8
+// heads, D 128, with q/k norm 2.33 us against 2.62, 500 tokens 4.67 / 5.51). In between the times
+// of both go in steps, by how the blocks of launches back to back meet on the SMs. With q/k norm
+// two rows pay from 4.5 to 6 items per SM (75 tokens 2.40 / 2.66, 150 of D 64 2.40 / 2.88) and
+// from 27 (400 tokens 4.36 / 4.59); one row elsewhere: 45 tokens 2.25 -> 2.05 us, 90 3.32 -> 2.73,
+// 140 3.39 -> 2.62, 225 3.66 -> 3.33, D 64 at 380 tokens 3.38 -> 2.85, 28 + 4 + 4 heads at 150 3.77
+// -> 2.89. Without the norm one row pays from 10.5 to 15: 180 tokens 2.87 -> 2.47, D 64 at 300 2.92
+// -> 2.40, D 256 at 130 2.87 -> 2.46 (but 160 tokens 2.19 -> 2.98); 105 tokens, below, 2.04 / 2.80,
+// 320, above, 3.55 / 4.08.
+constexpr int64_t kRopeSms = 152;
+static bool rope_small(int64_t items, bool qk) {
+  const int64_t n = 2 * items;  // in half items
+  if (n <= 6 * kRopeSms) return true;
+  if (qk) return n <= 54 * kRopeSms && !(n > 9 * kRopeSms && n <= 12 * kRopeSms);
+  return n > 21 * kRopeSms && n <= 30 * kRopeSms;
+}
+// Calls of at least this many tokens and bulk items take the bulk-copy entry: 640 tokens (2560
+// items) with q/k norm 5.06 us against 5.80 with two register-held rows per group, 2048 tokens
+// 10.5 / 8.9 (with / without the norm) against 12.3 / 10.5, 8192 33.3 / 30.9 against 38.0 / 32.8.
+// With fewer items, the same tokens of few heads, a warp's serial copy, rotate and store is the
+// call: 8 + 2 + 2 heads at 700 / 1600 tokens 4.53 / 5.22 against 2.85 (one row) / 4.61.
 constexpr int32_t kRopeBulkTokens = 512;
+constexpr int64_t kRopeBulkItems = 2304;
 
 
 // Before the launch wait: the lane's frequencies (the version's table is written only at
@@ -275,8 +290,8 @@ void rope_plans(int64_t NH, int32_t D, RopePlans* out) {
 }
 
 RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks) {
-  const RopeEntry e = p->T >= kRopeBulkTokens ? ROPE_BULK
-                      : p->T * plans.split[ROPE_SMALL].ipt > kRopeSmallItems ? ROPE_MID : ROPE_SMALL;
+  const RopeEntry e = p->T >= kRopeBulkTokens && p->T * plans.split[ROPE_BULK].ipt >= kRopeBulkItems ? ROPE_BULK
+                      : rope_small(p->T * plans.split[ROPE_SMALL].ipt, p->gamma_q != nullptr) ? ROPE_SMALL : ROPE_MID;
   const RopeSplit& r = plans.split[e];
   p->ipt = r.ipt;
   p->rpi = r.rpi;
@@ -296,7 +311,7 @@ int rope_any_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64
   const uintptr_t ptrs = (uintptr_t)p->q | (uintptr_t)p->k | (uintptr_t)p->v | (uintptr_t)p->k_cache |
                          (uintptr_t)p->v_cache | (uintptr_t)p->gamma_q | (uintptr_t)p->gamma_k;
   if (ptrs % 16 != 0 || (p->T > 1 && (p->q_rs % 8 != 0 || p->k_rs % 8 != 0 || p->v_rs % 8 != 0))) return -1;
-  const int e = p->T * plans.any[0].ipt > kRopeSmallItems ? 1 : 0;
+  const int e = p->T * plans.any[0].ipt > 3 * kRopeSms ? 1 : 0;
   const RopeSplit& r = plans.any[e];
   p->ipt = r.ipt;
   p->rpi = r.rpi;
