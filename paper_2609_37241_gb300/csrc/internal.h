@@ -155,10 +155,11 @@ enum PointwiseEntry : int32_t { PW_FLAT, PW_FLAT2, PW_ROWS, PW_ROWS2, PW_GENERIC
 // fields and sets the grid. eb: element size.
 int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks);
 
-// Norm entries (norm_plan): 16-byte aligned rows, rows at any common offset, scalar accesses,
-// and the entry of long calls (bulk copies, or two rows at a time for short rows).
+// Norm entries (norm_plan): 16-byte aligned rows, rows at any common offset (few or many rows),
+// scalar accesses, and the entry of long aligned calls (bulk copies, or two rows at a time for
+// short rows).
 constexpr int kNormBlockVecs = 2048;  // norm_block_kernel, norm_bulk_kernel: vectors of a row at most
-enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_GENERIC, NM_LARGE, kNormEntries };
+enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_EDGE_MANY, NM_GENERIC, NM_LARGE, kNormEntries };
 
 // Kernel entry (host stub address) plus its launch shape rule.
 struct KernelEntry {
@@ -184,7 +185,8 @@ struct KernelEntry {
   const void* nm_fn[kNormEntries] = {};  // norms, by NormEntry (NULL: none for this H)
   int32_t nm_threads[kNormEntries] = {};
   int32_t rows = 1;      // norms: rows per block of the NM_VEC entry
-  int32_t edge_rows = 1;  // ... and of the NM_EDGE entry
+  int32_t edge_rows = 1;  // ... and of the NM_EDGE_MANY entry,
+  int64_t edge_many = 0;  // which calls of at least this many rows take
 };
 
 enum KernelKind : int32_t {

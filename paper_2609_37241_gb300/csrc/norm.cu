@@ -7,8 +7,9 @@
 // x (1024, 128)); the residual add fused in front of it is how decoder layers call it. All
 // kernels but the last two read a row once and write it once:
 //   norm_rows_kernel   rows of at most 128 vectors: LPR lanes per row, reduced by shuffles alone
-//   norm_rows_edge_kernel  such rows at any element offset that all tensors share (odd widths,
-//                      shifted bases): a warp per row, the vectors between a scalar head and tail
+//   norm_rows_edge_kernel  long calls of such rows at any element offset that all tensors share
+//                      (odd widths, shifted bases): a warp per row, the vectors between a scalar
+//                      head and tail
 //   norm_block_kernel  longer rows, one block per row, one or two vectors per thread, one barrier.
 //                      EDGE: at any common element offset
 //   norm_bulk_kernel   long calls of such rows: the row staged by bulk copies
@@ -43,6 +44,18 @@ constexpr int64_t kNormBulkBytes = 10 << 20;
 // vectors of x: half the threads have twice the loads in flight (16384 x 128 3.26 -> 2.90 us,
 // 131072 x 128 15.3 -> 12.1; 8192 x 64, below the line, 1.98 / 2.16).
 constexpr int64_t kNormRows2Vecs = 152 * 1024;
+// EDGE rows of 33 to 128 vectors take a block per row below this many rows, a warp per row (two or
+// four vectors per lane, one after the other) from there, where the rate at which blocks start
+// bounds the block per row; with the residual and more than 64 vectors always a block. Warp / block
+// per row: 832 bf16 at 24 / 600 / 2400 / 5000 rows 2.59 / 1.65, 4.34 / 3.20, 5.02 / 4.51, 6.13 /
+// 6.98 us; 333 at 2400 / 5000 4.11 / 4.08, 3.30 / 5.29; the residual on 1000 fp16 at 3 / 5000 /
+// 30000 2.74 / 1.59, 12.4 / 8.1, 51.8 / 38.0. Up to 32 vectors a warp is enough: 101 at 24 / 2400
+// rows 1.50 / 1.59, 2.88 / 3.45.
+constexpr int64_t kNormEdgeRows = 3072;
+// fp32 EDGE rows of more than 512 vectors take two vectors per thread from this many rows (more
+// rows resident): 4000 x 3001 25.4 -> 20.6 us, with the residual 34.8 -> 30.7; 8559 x 2222 35.7 ->
+// 29.6; at 300 rows 2.31 / 2.76. (16 bits: 3000 x 3999 12.5 / 13.7.)
+constexpr int64_t kNormEdgeWideRows = 2048;
 
 template <int DT>
 __device__ __forceinline__ void load_gamma(const float* g, float* out) {
@@ -259,7 +272,7 @@ __global__ void __launch_bounds__(1024) norm_block_kernel(const NormParams p) {
   if (EDGE && edge >= 0) store_elem<DT>(p.y, row * p.y_rs + edge, es * inv * eg);
 }
 
-// EDGE rows of at most 128 vectors: a warp per row, eight rows per block, VPT vectors per lane;
+// Long calls of EDGE rows of at most 128 vectors: a warp per row, eight rows per block, VPT vectors per lane;
 // a block per row (of one warp) was bound by the rate at which blocks start (20000 x 101 20.4 us).
 template <int DT, bool RES, int VPT>
 __global__ void __launch_bounds__(kThreads) norm_rows_edge_kernel(const NormParams p) {
@@ -561,15 +574,22 @@ static void pick(int64_t H, KernelEntry* out) {
   const int threads = norm_threads(nvec, vpt);
   // rows that begin anywhere hold nvec or nvec - 1 whole vectors, and at least one
   out->edge_rows = 1;
-  if (nvec >= 2 && nvec <= kNormRowsVecs) {
-    out->edge_rows = kThreads / 32;
-    out->nm_fn[NM_EDGE] = nvec <= 32 ? (const void*)norm_rows_edge_kernel<DT, RES, 1>
-                        : nvec <= 64 ? (const void*)norm_rows_edge_kernel<DT, RES, 2>
-                                     : (const void*)norm_rows_edge_kernel<DT, RES, 4>;
-  } else if (nvec >= 2 && nvec <= kNormBlockVecs) {
+  out->edge_many = INT64_MAX;
+  if (nvec >= 2 && nvec <= kNormBlockVecs) {
     out->nm_threads[NM_EDGE] = threads;
     out->nm_fn[NM_EDGE] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, true, false>
                                    : (const void*)norm_block_kernel<DT, RES, 2, true, false>;
+    if (nvec <= 64 || (!RES && nvec <= kNormRowsVecs)) {
+      out->edge_rows = kThreads / 32;
+      out->edge_many = nvec <= 32 ? 0 : kNormEdgeRows;
+      if (nvec <= 32) out->nm_fn[NM_EDGE_MANY] = (const void*)norm_rows_edge_kernel<DT, RES, 1>;
+      else if (nvec <= 64) out->nm_fn[NM_EDGE_MANY] = (const void*)norm_rows_edge_kernel<DT, RES, 2>;
+      else if constexpr (!RES) out->nm_fn[NM_EDGE_MANY] = (const void*)norm_rows_edge_kernel<DT, RES, 4>;
+    } else if (VE == 4 && vpt == 1 && nvec > 512) {
+      out->edge_many = kNormEdgeWideRows;
+      out->nm_threads[NM_EDGE_MANY] = norm_threads(nvec, 2);
+      out->nm_fn[NM_EDGE_MANY] = (const void*)norm_block_kernel<DT, RES, 2, true, false>;
+    }
   }
   if (H % VE != 0) return;
   if (nvec <= kNormRowsVecs) {
@@ -637,10 +657,10 @@ NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, 
   p->nvec = (int32_t)(p->H / ve < INT32_MAX ? p->H / ve : INT32_MAX);  // the loop kernel counts its own
   NormEntry e = NM_GENERIC;
   if (aligned && ke.nm_fn[NM_VEC]) e = ke.nm_fn[NM_LARGE] && p->T >= ke.large_rows ? NM_LARGE : NM_VEC;
-  else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX) e = NM_EDGE;  // one block per row
+  else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX) e = p->T >= ke.edge_many ? NM_EDGE_MANY : NM_EDGE;
   *threads = ke.nm_threads[e];
   *smem = e == NM_LARGE ? ke.large_smem : 0;
-  const int64_t per = e == NM_VEC ? ke.rows : e == NM_LARGE ? ke.large_per : e == NM_EDGE ? ke.edge_rows : 1;
+  const int64_t per = e == NM_VEC ? ke.rows : e == NM_LARGE ? ke.large_per : e == NM_EDGE_MANY ? ke.edge_rows : 1;
   *blocks = (p->T + per - 1) / per;
   return e;
 }

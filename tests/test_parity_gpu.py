@@ -304,6 +304,8 @@ def test_pointwise_parity(S, name, dtype, W, T, layout, variant):
     (BF16, 19, 1001, "dense"), (FP16, 6, 4099, "offset"),  # rows at every offset
     (BF16, 1003, 101, "dense"), (FP16, 37, 333, "offset"), (FP32, 65, 511, "dense"), (BF16, 41, 1023, "dense"),
     (FP32, 8, 9, "offset"), (BF16, 9, 15, "offset"),       # one whole vector between the edges; none
+    (BF16, 3071, 333, "offset"), (FP16, 3075, 333, "dense"), (BF16, 3073, 1021, "offset"),  # a warp per such row
+    (FP32, 2047, 2222, "dense"), (FP32, 2050, 2055, "offset"),  # ... and two vectors per thread
     (FP16, 5, 2048, "gamma"), (BF16, 6, 520, "apart"),     # weights, or one tensor, at another offset
     (BF16, 1025, 4096, "dense"), (FP16, 1100, 5120, "padded"), (FP16, 420, 16000, "dense"),  # bulk copies
     (FP32, 500, 8192, "dense"), (BF16, 20001, 64, "dense"), (FP16, 12001, 128, "padded")])   # two rows a time
