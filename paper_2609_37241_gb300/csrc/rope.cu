@@ -21,8 +21,8 @@
 //   30 tokens    3.36 -> 2.06 / 2.95 -> 1.91 us      500 tokens    7.66 -> 4.67 / 6.86 -> 4.20 us
 //   120 tokens   3.58 -> 3.01 / 3.18 -> 2.77 us     3333 tokens   26.5 -> 15.1 / 20.8 -> 13.7 us
 //   250 tokens   5.13 -> 3.22 / 4.48 -> 3.04 us     8192 tokens   51.7 -> 33.3 / 41.8 -> 30.9 us
-// (8192 tokens without the norm: 0.96 of the copy rate.) D 64 at 250 tokens without the norm
-// is the one size of the sweeps that lost (2.63 -> 2.88 us).
+// (8192 tokens without the norm: 0.96 of the copy rate.) D 64 without the norm lost at sizes
+// between 240 and 350 tokens (2.63 -> 2.7-3.05 us).
 #include "device_common.cuh"
 
 namespace trident {
@@ -37,15 +37,17 @@ constexpr int kRopeThreads = 64;
 // two rows pay from 4.5 to 6 items per SM (75 tokens 2.40 / 2.66, 150 of D 64 2.40 / 2.88) and
 // from 27 (400 tokens 4.36 / 4.59); one row elsewhere: 45 tokens 2.25 -> 2.05 us, 90 3.32 -> 2.73,
 // 140 3.39 -> 2.62, 225 3.66 -> 3.33, D 64 at 380 tokens 3.38 -> 2.85, 28 + 4 + 4 heads at 150 3.77
-// -> 2.89. Without the norm one row pays from 10.5 to 15: 180 tokens 2.87 -> 2.47, D 64 at 300 2.92
-// -> 2.40, D 256 at 130 2.87 -> 2.46 (but 160 tokens 2.19 -> 2.98); 105 tokens, below, 2.04 / 2.80,
-// 320, above, 3.55 / 4.08.
+// -> 2.89. Without the norm one row pays where its two-item blocks just fit a whole number per SM
+// or leave half a one, from 10.5 to 12 and from 13 to 15 items: 28 head-rows (20 + 4 + 4) at 240 /
+// 257 tokens 2.87 / 2.87 -> 2.33 / 2.35, 180 tokens of 48 2.87 -> 2.47, D 64 at 300 2.91 -> 2.40, D
+// 256 at 130 2.87 -> 2.46; between those, 28 head-rows at 264 tokens (12.2) 2.84 / 3.31, and outside,
+// 105 tokens of 48 (8.3) 2.04 / 2.80, 320 (25) 3.55 / 4.08.
 constexpr int64_t kRopeSms = 152;
 static bool rope_small(int64_t items, bool qk) {
   const int64_t n = 2 * items;  // in half items
   if (n <= 6 * kRopeSms) return true;
   if (qk) return n <= 54 * kRopeSms && !(n > 9 * kRopeSms && n <= 12 * kRopeSms);
-  return n > 21 * kRopeSms && n <= 30 * kRopeSms;
+  return (n > 21 * kRopeSms && n <= 24 * kRopeSms) || (n > 26 * kRopeSms && n <= 30 * kRopeSms);
 }
 // Calls of at least this many tokens and bulk items take the bulk-copy entry: 640 tokens (2560
 // items) with q/k norm 5.06 us against 5.80 with two register-held rows per group, 2048 tokens

@@ -498,7 +498,8 @@ def test_rope_kv_many_tokens(S, T, Hq, Hkv, D, S_, qk, dtype, layout):
     (767, 45, 2, 64, True, BF16), (768, 45, 2, 64, False, FP16),   # both sides of the bulk-copy limit
     (777, 13, 1, 256, True, BF16), (1024, 22, 2, 128, True, FP16),
     (57, 32, 8, 128, True, BF16), (58, 32, 8, 128, True, FP16), (77, 32, 8, 128, True, FP16),  # one row or two
-    (343, 32, 8, 128, True, BF16), (134, 32, 8, 128, False, BF16), (191, 32, 8, 128, False, FP16)])
+    (343, 32, 8, 128, True, BF16), (134, 32, 8, 128, False, BF16), (191, 32, 8, 128, False, FP16),
+    (152, 32, 8, 128, False, FP16), (153, 32, 8, 128, False, BF16)])
 def test_rope_kv_item_edges(S, T, Hq, Hkv, D, qk, dtype):
     """Warp items of one, two and three head-rows per lane group at the limits of their ranges,
     with q, k and v rows meeting inside an item and a last item only partly filled."""
