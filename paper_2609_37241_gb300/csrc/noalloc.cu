@@ -19,7 +19,8 @@
 // earlier launch failed, the RoPE kernel reads the table its own call wrote. It is launched
 // with programmatic serialisation, so that its launch overlaps the preparing kernel, and reads
 // its frequencies only after griddepcontrol.wait (RopeParams.freq_late), when that kernel has
-// finished; the preparing kernel itself starts after everything before it on the stream.
+// finished, by coherent loads (rope_pair_freqs_late); the preparing kernel itself starts after
+// everything before it on the stream.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -50,9 +51,9 @@ struct FreqPowers { double p[7]; };
 
 // Prepares the scratch for one call: clears the status word and writes the frequency
 // table f_i = theta^(-2i/D) in fp64, stored as (fp32(f), fp32(f - hi)), for i < D/2: the product of
-// the powers at the bits of i, at most six roundings of 2^-53 where the pair keeps 2^-48. (One
-// pow per thread instead, in the kernel, was 7 us of every call: fp64 runs at a small fraction of
-// fp32's rate.)
+// the powers at the bits of i. At most seven factors, each off by at most 2^-52 (pow), and six
+// roundings of 2^-53: 20 * 2^-53 in all, below the 2^-48 that the pair keeps. (One pow per thread
+// instead, in the kernel, was 7 us of every call: fp64 runs at a small fraction of fp32's rate.)
 __global__ void prepare_scratch(uint32_t* status, float2* tab, int32_t D, const FreqPowers pw) {
   pdl_trigger();
   const int i = threadIdx.x;
@@ -119,7 +120,7 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   int64_t blocks = 0;
   rope_plans(p.NH, p.D, &plans);
   const RopeEntry entry = rope_plan(plans, &p, &threads, &blocks);
-  bp.rp = p;  // (its kernel reads the frequencies after the wait anyway)
+  bp.rp = p;
   bp.first_wait_polls = kBulkWaitPolls;
   const void* fn = entry == ROPE_BULK ? ke.fn_large : (entry == ROPE_MID ? ke.fn_mid : ke.fn);
   void* kargs[1] = {entry == ROPE_BULK ? (void*)&bp : (void*)&p};

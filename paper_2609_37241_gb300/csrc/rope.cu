@@ -59,7 +59,7 @@ constexpr int64_t kRopeBulkItems = 2304;
 
 
 // Before the launch wait: the lane's frequencies (the version's table is written only at
-// registration), and with p.prefetch the L2 prefetch of the item's row lines and position.
+// registration; with p.freq_late the previous kernel writes it, and they are read after), and with p.prefetch the L2 prefetch of the item's row lines and position.
 template <int DT, int D, bool QKNORM, int R>
 __global__ void __launch_bounds__(kRopeThreads) rope_pair_kernel(const RopeParams p) {
   pdl_trigger();
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kRopeThreads) rope_pair_kernel(const RopeParam
   if (!p.freq_late) rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
   if (p.prefetch && live) rope_item_prefetch<D, R>(p, t, first, end);
   pdl_wait();
-  if (p.freq_late) rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
+  if (p.freq_late) rope_pair_freqs_late(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
   if (live) rope_pair_rows<DT, D, QKNORM, R, true>(p, t, first, end, fq);
 }
 
@@ -129,7 +129,8 @@ __global__ void __launch_bounds__(kRopeBulkThreads, 6) rope_bulk_kernel(const Ro
   RopeAngles an;
   {
     float4 fq[4];
-    rope_pair_freqs(p.inv_freq, lane, fq);
+    if (p.freq_late) rope_pair_freqs_late(p.inv_freq, lane, fq);
+    else rope_pair_freqs(p.inv_freq, lane, fq);
     rope_angles(pos_ok ? pos : 0, fq, &an);
   }
   auto landed = [&](uint32_t polls) -> bool {

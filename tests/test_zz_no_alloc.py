@@ -108,6 +108,31 @@ def test_noalloc_calls_in_a_row_match_the_oracle_and_the_scm(S):
         assert np.array_equal(got_h["v_cache"], via_h["v_cache"])
 
 
+@pytest.mark.parametrize("D,Hq,Hkv,T,qknorm", [
+    (256, 4, 2, 9, True), (256, 4, 2, 150, False),  # frequency pairs above 64: all seven factors
+    (256, 8, 4, 1030, True), (128, 32, 8, 770, True), (64, 45, 2, 773, False)])  # bulk copies
+def test_noalloc_tables_alternate_back_to_back(S, D, Hq, Hkv, T, qknorm):
+    """Calls queued one behind the other, each with another theta: every RoPE kernel, resident
+    while the kernel before it rewrites the table, must read its own call's frequencies."""
+    stream = torch.cuda.current_stream().cuda_stream
+    Sl, thetas = 4096, [1e4, 1e6, 5e5, 1e4]
+    op = S.OP_QKNORM_ROPE_KV if qknorm else S.OP_ROPE_KV
+    sets, cs = [], []
+    for i, theta in enumerate(thetas):
+        case = make_case(D + T + i, T, Hq, Hkv, D, Sl)
+        sets.append(device_tensors(case, qknorm))
+        cs.append(case)
+    args = [S.make_args(op, ts, eps=1e-6, rope_theta=theta) for ts, theta in zip(sets, thetas)]
+    torch.cuda.synchronize()
+    for a in args:
+        assert S.trident_rope_kv_noalloc(a, stream) == S.OK, S.trident_scm_last_error()
+    torch.cuda.synchronize()
+    for case, ts, theta in zip(cs, sets, thetas):
+        ref = L.rope_kv(case["q"], case["k"], case["v"], case["pos"], case["kc"], case["vc"], theta, BF16,
+                        qknorm=qknorm, gamma_q=case["gq"], gamma_k=case["gk"], eps=1e-6)
+        P.check_rope(ref, host_outputs(ts), (case["q"], case["k"], case["v"], case["pos"]))
+
+
 def test_noalloc_without_status_word(S):
     """out_status may be NULL: the call still runs and matches the oracle."""
     Sl, D, Hq, Hkv = 512, 64, 4, 2
