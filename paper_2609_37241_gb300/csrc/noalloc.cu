@@ -108,8 +108,18 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   float2* table = reinterpret_cast<float2*>(ds.addr + kTableOffset);
   FreqPowers pw;
   for (int b = 0; b < 7; ++b) pw.p[b] = std::pow(args->rope_theta, -2.0 * (double)(1 << b) / (double)p.D);
-  prepare_scratch<<<1, (unsigned)kMaxPairs, 0, s>>>(status, table, p.D, pw);
-  if (cudaGetLastError() != cudaSuccess)
+  // Every failure is read from the failing call itself and taken out of the thread's last error:
+  // an error that some earlier call left there is not this call's.
+  auto failed = [](cudaError_t e) {
+    if (e == cudaSuccess) return false;
+    (void)cudaGetLastError();
+    return true;
+  };
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3((unsigned)kMaxPairs);
+  cfg.stream = s;
+  if (failed(cudaLaunchKernelEx(&cfg, prepare_scratch, status, table, p.D, pw)))
     return internal_fail(TRIDENT_ERR_CUDA, "scratch preparation launch failed");
   p.inv_freq = table;
   p.freq_late = 1;
@@ -127,17 +137,12 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(blocks < 0x7fffffff ? blocks : 0x7fffffff));
   cfg.blockDim = dim3((unsigned)threads);
-  cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelExC(&cfg, fn, kargs) != cudaSuccess)
-    return internal_fail(TRIDENT_ERR_CUDA, "RoPE launch failed");
-  if (out_status &&
-      cudaMemcpyAsync(out_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+  if (failed(cudaLaunchKernelExC(&cfg, fn, kargs))) return internal_fail(TRIDENT_ERR_CUDA, "RoPE launch failed");
+  if (out_status && failed(cudaMemcpyAsync(out_status, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)))
     return internal_fail(TRIDENT_ERR_CUDA, "status copy failed");
-  if (cudaGetLastError() != cudaSuccess) return internal_fail(TRIDENT_ERR_CUDA, "launch error");
   return TRIDENT_OK;
 }

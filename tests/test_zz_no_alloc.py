@@ -146,6 +146,25 @@ def test_noalloc_without_status_word(S):
     P.check_rope(ref, host_outputs(ts), (case["q"], case["k"], case["v"], case["pos"]))
 
 
+def test_noalloc_does_not_report_an_earlier_calls_error(S):
+    """A CUDA error that an earlier, unrelated call left behind (here the creation of an SCM on a
+    device that does not exist) is not taken for a failure of this call."""
+    Sl, D, Hq, Hkv = 512, 128, 4, 2
+    case = make_case(8, 6, Hq, Hkv, D, Sl)
+    ref = L.rope_kv(case["q"], case["k"], case["v"], case["pos"], case["kc"], case["vc"], 1e4, BF16)
+    ts = device_tensors(case, False)
+    torch.cuda.synchronize()
+    with pytest.raises(S.ScmError):
+        S.Scm(device=torch.cuda.device_count())
+    word = torch.full((1,), -1, dtype=torch.int32).pin_memory()
+    st = S.trident_rope_kv_noalloc(S.make_args(S.OP_ROPE_KV, ts, rope_theta=1e4),
+                                   torch.cuda.current_stream().cuda_stream, status_word=word.data_ptr())
+    assert st == S.OK, S.trident_scm_last_error()
+    torch.cuda.synchronize()
+    assert int(word.item()) == 0
+    P.check_rope(ref, host_outputs(ts), (case["q"], case["k"], case["v"], case["pos"]))
+
+
 def test_noalloc_rejects_sizes_beyond_its_scratch(S):
     """A head size above 256 needs more than the static array's 128 frequency pairs: a clear
     error, nothing launched."""
