@@ -6,12 +6,14 @@ one trident_scm_invoke per step from Python -- guards, argument packing and one 
 launch -- timed with CUDA events over K back-to-back steps, inputs rotated over enough
 buffer sets that the working set exceeds twice the L2.
 
-Also reported on the same line: every token count of that workload fused and unfused,
-the 36-layer Qwen3-style step, host nanoseconds per cache hit (single add+RMSNorm call,
-1 token), the 100k-call dynamic-shape guard stress (hit/miss counts checked against the
-oracle replay), the HBM bandwidth sweep (add+RMSNorm and SwiGLU, 1..32768 tokens), the
-roofline of the dominant kernel, the end-to-end step with host copies, and the CPU
-oracle as a reported baseline.
+The line also carries the end-to-end step with host copies, the roofline of the dominant
+kernel, the clocks and the CPU oracle as a baseline. It stays short (LINE_MAX), so that a
+reader who keeps only the end of the output still has all of it; the whole record goes to
+stderr, one JSON object behind "[bench record] ": besides those, every token count of that
+workload fused and unfused, the 36-layer Qwen3-style step, host nanoseconds per cache hit
+(single add+RMSNorm call, 1 token), the 100k-call dynamic-shape guard stress (hit/miss
+counts checked against the oracle replay) and the HBM bandwidth sweep (add+RMSNorm and
+SwiGLU, 1..32768 tokens).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference] [--quick]
                  [--sections LIST] [--tokens LIST]
@@ -42,6 +44,25 @@ NOMINAL_HBM_GBS = 8000.0
 CHAIN_SOURCES = ["paper_2609_37241_gb300/csrc/chain.cu", "paper_2609_37241_gb300/csrc/device_common.cuh",
                  "paper_2609_37241_gb300/csrc/internal.h"]
 CHAIN_COUNTERS = "profiles/chain_kernel_llama_t64.json"
+
+
+LINE_MAX = 1500  # characters of the line on stdout
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline",
+             "python_binding")
+LINE_SUBKEYS = {"e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+                "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic"),
+                "cpu_baseline": ("value", "unit", "cores", "kind")}
+
+
+def headline_line(record):
+    """The line on stdout: the record's headline keys, its nested sections left out."""
+    line = {}
+    for k in LINE_KEYS:
+        if k in record:
+            v = record[k]
+            line[k] = {s: v[s] for s in LINE_SUBKEYS[k] if s in v} if k in LINE_SUBKEYS else v
+    return json.dumps(line)
 
 
 def chain_sources_sha256():
@@ -1399,7 +1420,8 @@ def run_ours(a):
             line["cpu_baseline_all_cores"] = cpu_all
         if ck:
             line["clocks"] = ck
-        print(json.dumps(line), flush=True)
+        print("[bench record] " + json.dumps(line), file=sys.stderr, flush=True)
+        print(headline_line(line), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()

@@ -72,6 +72,33 @@ def test_committed_dram_counters_match_the_algorithmic_bytes():
     assert abs(rd - r_alg) <= 0.1 * r_alg and abs(wr - w_alg) <= 0.1 * w_alg
 
 
+def test_headline_line_is_short_and_whole():
+    """The line on stdout carries every contract key with the record's values and stays within
+    LINE_MAX however long the record's sections are."""
+    sections = {str(i): dict(us=1.0 / 3, notes="x" * 40) for i in range(300)}
+    record = dict(metric=bench.METRIC, value=12345.678, unit=bench.UNIT, n_gpus=8, steps=100000, warmup=1000,
+                  ms_per_step=12.345678, higher_is_better=False, scaling="weak", vs_baseline=None, dtype="bf16",
+                  data="d" * 130, config=dict(workload="w" * 140, tokens=64, path="p" * 45, l2="l" * 60,
+                                              parallelism="single GPU"),
+                  timing=dict(lead="t" * 400), gpu_launches=100000, gpu_launches_whole_run=1 << 30,
+                  python_binding="fastcall", llama_per_tokens=sections, hbm_sweep=sections,
+                  roofline=dict(bound="hbm", achieved=3327.6, peak=6784.2, unit="GB/s", frac=0.49,
+                                traffic=10676117, kernel="k" * 40, copy_floor=sections),
+                  e2e=dict(value=12345.67, unit=bench.UNIT, h2d_bytes_per_step=10 ** 7, d2h_bytes_per_step=10 ** 7,
+                           serial=sections),
+                  cpu_baseline=dict(value=40000.0, unit=bench.UNIT, cores=1, kind="oracle", sample="s" * 90),
+                  clocks=dict(sm_mhz=2070.0, sm_max_mhz=2070.0, reasons=["sw_power_cap"], samples=999))
+    text = bench.headline_line(record)
+    assert len(text) <= bench.LINE_MAX and "\n" not in text
+    line = json.loads(text)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks"):
+        assert line[k] == record[k]
+    for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"):
+        assert line["e2e"][k] == record["e2e"][k]
+    assert line["roofline"]["frac"] == 0.49 and line["cpu_baseline"]["kind"] == "oracle"
+
+
 def _run_reference(env_extra):
     import subprocess
     import sys
