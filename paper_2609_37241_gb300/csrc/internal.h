@@ -156,10 +156,10 @@ enum PointwiseEntry : int32_t { PW_FLAT, PW_FLAT2, PW_ROWS, PW_ROWS2, PW_GENERIC
 int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks);
 
 // Norm entries (norm_plan): 16-byte aligned rows, rows at any common offset (few or many rows),
-// scalar accesses, and the entry of long aligned calls (bulk copies, or two rows at a time for
-// short rows).
+// scalar accesses, the entry of long aligned calls (bulk copies, more vectors per thread, or two
+// rows at a time for short rows), and one for some calls in between (norm_row_kernel).
 constexpr int kNormBlockVecs = 2048;  // norm_block_kernel, norm_bulk_kernel: vectors of a row at most
-enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_EDGE_MANY, NM_GENERIC, NM_LARGE, kNormEntries };
+enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_EDGE_MANY, NM_GENERIC, NM_LARGE, NM_MID, kNormEntries };
 
 // Kernel entry (host stub address) plus its launch shape rule.
 struct KernelEntry {
@@ -176,7 +176,8 @@ struct KernelEntry {
   const void* any_fn[2] = {};      // RoPE versions of the generic kind: rope_any_kernel (or NULL)
   const void* fn_mid = nullptr;    // RoPE: the entry between fn and fn_large (rope_plan chooses)
   const void* pw_fn[kPwEntries] = {};  // elementwise, by PointwiseEntry
-  int64_t large_rows = 0;  // norms: rows from which a call takes the NM_LARGE entry
+  float large_sm = 0;      // norms: calls of more rows per SM take the NM_LARGE entry
+  float mid_lo = 0, mid_hi = 0;  // ... and of rows per SM in (mid_lo, mid_hi] the NM_MID entry
   int32_t large_per = 1;   // ... that entry's rows per block
   int32_t large_smem = 0;  // ... and its dynamic shared memory (rows staged by bulk copies)
   int32_t kind = 0;      // which grid rule the host applies (KernelKind)
@@ -207,7 +208,7 @@ bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry*
                   const char** why);
 // The entry a call takes from its packed params (sets p->nvec), its block size and grid.
 NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, int32_t* threads, int64_t* blocks,
-                    int32_t* smem);
+                    int32_t* smem, int32_t sms);
 const void* empty_kernel_entry();  // the latency-floor probe's kernel (does nothing)
 
 // Validation, guard-equivalent checks (sizes, layouts, 16-byte alignment, overlap) and

@@ -10,10 +10,10 @@
 //   norm_rows_edge_kernel  long calls of such rows at any element offset that all tensors share
 //                      (odd widths, shifted bases): a warp per row, the vectors between a scalar
 //                      head and tail
-//   norm_block_kernel  longer rows, one block per row, one or two vectors per thread, one barrier.
-//                      EDGE: at any common element offset
-//   norm_bulk_kernel   long calls of such rows: the row staged by bulk copies
-//   addnorm_row_kernel long ADD_RMSNORM calls of H = 4096 in 16 bits
+//   norm_block_kernel  longer rows, one block per row, one barrier; one or two vectors per thread,
+//                      four or eight in long fp32 calls. EDGE: at any common element offset
+//   norm_bulk_kernel   long calls of such rows in 16 bits: the row staged by bulk copies
+//   norm_row_kernel    some calls of 256, 512 and 1024 vectors in 16 bits: blocks of 256 threads
 //   norm_loop_kernel   16-byte rows of more than 2048 vectors (two passes)
 //   norm_generic_kernel  anything else (scalar accesses)
 //
@@ -33,17 +33,36 @@
 #include "device_common.cuh"
 
 namespace trident {
-// Long calls take norm_bulk_kernel (or addnorm_row_kernel) from this many bytes of x, with a
-// residual add / without; norm_block_kernel against norm_bulk_kernel, bf16: with it 600 x 8192
-// 7.7 / 8.1, 1000 x 8192 14.0 / 11.9 us; 600 x 5120 5.7 / 5.8, 1000 x 5120 9.0 / 8.4; without
-// 1000 x 4096 4.2 / 4.9, 1600 x 4096 6.2 / 5.8; 600 x 8192 4.9 / 5.2, 1000 x 8192 8.7 / 7.8. fp32
-// residual rows of up to 1024 vectors stay with one vector per thread (2995 x 4096 28.6 / 30.2).
-constexpr int64_t kNormBulkResBytes = 8 << 20;
-constexpr int64_t kNormBulkBytes = 10 << 20;
+// Calls of more rows than a number of waves of norm_block_kernel's blocks (norm_block_sm rows per SM
+// and wave) take the entry of long calls: two waves with one vector per thread, one with two. Within
+// them the short-lived blocks win, beyond them rows kept in fewer registers per SM do. In 16 bits that
+// entry is norm_bulk_kernel, block / bulk either side of the line: residual 560 x 6144 6.0 / 6.4, 620
+// 7.8 / 6.6; 850 x 5120 6.7 / 7.7, 1000 9.1 / 8.6; 600 x 8192 7.7 / 8.6, 680 10.0 / 9.3; 152 x 12288
+// 4.1 / 4.6, 228 6.8 / 6.1; without it 600 x 6144 4.0 / 4.4, 680 5.4 / 4.7; 1200 x 4096 4.6 / 4.7, 1400
+// 5.7 / 5.4. In fp32 without the residual it is norm_block_kernel with four vectors per thread, eight
+// from more than 1280 vectors (us, block / this / bulk copies): 600 x 4096 4.5 / 4.8 / 5.2, 1000 8.0 /
+// 6.5 / 6.9; 1400 x 2048 5.3 / 4.8 / 5.2; 500 x 8192 7.8 / 6.7 / 8.3, 1200 15.2 / 12.9 / 15.8; with it
+// nothing beats the block (500 x 8192 11.5 against 13.4 with bulk copies, 1000 x 6144 16.0 / 17.0).
+// Rows of up to 256 vectors without the residual hold out four waves (3000 x 2048 bf16 5.5 / 6.0, 7000
+// 10.9 / 10.5); shorter ones in 16 bits any number (7000 x 1536 8.7 / 10.2).
+static float norm_block_sm(int threads, int vpt, int ve) {
+  return vpt == 2 && ve == 8 ? 1.f : (float)(2048 / threads);  // two 16-bit vectors per thread: 64 registers
+}
+// norm_row_kernel's ranges, in rows per SM: where its blocks still fit one wave (or two fit better
+// than norm_block_kernel's). Block or bulk / this: residual 1400 x 2048 5.36 / 5.20; 640 x 4096 5.16 /
+// 4.88, 760 5.66 / 5.52, 850 5.94 / 5.96; 620 x 8192 8.79 / 8.24, 850 10.75 / 10.50, 1000 11.9 / 12.0;
+// without it 700 x 4096 3.10 / 2.96, 760 3.40 / 3.22, 680 2.94 / 2.94. Residual calls of 512 vectors
+// beyond two waves take it too: 1600 / 3001 / 6000 rows 9.25 / 15.6 / 29.1 us against 9.49 / 15.8 /
+// 29.6 with bulk copies.
+struct NormRange { float lo, hi; };
+static NormRange norm_row_range(bool res, int vpt) {
+  if (!res) return vpt == 2 ? NormRange{4.5f, 5.25f} : NormRange{0.f, 0.f};
+  return vpt == 1 ? NormRange{8.f, 12.f} : vpt == 2 ? NormRange{4.f, 5.25f} : NormRange{4.f, 6.f};
+}
 // Two rows per lane group of norm_rows_kernel (no residual, one vector per lane) from this many
-// vectors of x: half the threads have twice the loads in flight (16384 x 128 3.26 -> 2.90 us,
+// vectors of x per SM: half the threads have twice the loads in flight (16384 x 128 3.26 -> 2.90 us,
 // 131072 x 128 15.3 -> 12.1; 8192 x 64, below the line, 1.98 / 2.16).
-constexpr int64_t kNormRows2Vecs = 152 * 1024;
+constexpr float kNormRows2Vecs = 1024.f;
 // EDGE rows of 33 to 128 vectors take a block per row below this many rows, a warp per row (two or
 // four vectors per lane, one after the other) from there, where the rate at which blocks start
 // bounds the block per row; with the residual and more than 64 vectors always a block. Warp / block
@@ -189,9 +208,9 @@ __device__ __forceinline__ float norm_block_sum(float v, float* red) {
 // last vector and drop it: with the loads behind a branch the compiler finished them before
 // leaving it (256 x 4096 3.3 us). FULL: no such threads. EDGE: the row's tensors
 // start at one common offset from a 16-byte boundary; the first peel and last tail elements
-// (fewer than a vector each) go to threads of their own, and gamma is read by element.
+// (fewer than a vector each) go to threads of their own, and gamma is read by load_gamma_at.
 template <int DT, bool RES, int VPT, bool EDGE, bool FULL>
-__global__ void __launch_bounds__(1024) norm_block_kernel(const NormParams p) {
+__global__ void __launch_bounds__(VPT >= 8 ? 256 : VPT >= 4 ? 512 : 1024) norm_block_kernel(const NormParams p) {
   pdl_trigger();
   __shared__ __align__(16) float red[32];
   constexpr int VE = Act<DT>::VE;
@@ -423,55 +442,56 @@ __global__ void __launch_bounds__(512, RES ? (VPT == 2 ? 3 : 2) : 1) norm_bulk_k
   }
 }
 
-// ADD_RMSNORM, H = 4096 in bf16 / fp16, long calls: exactly two vectors per thread of 256. The
-// one width where this order of loads and stores beat the bulk copies (1600 / 3001 / 6000 rows
-// 9.25 / 15.6 / 29.1 us against 9.49 / 15.8 / 29.6; at 5120 the two-pass kernel it replaced took
-// 23.7, the bulk copies 19.6).
-template <int DT>
-__global__ void __launch_bounds__(kThreads) addnorm_row_kernel(const NormParams p) {
+// Rows of exactly VPT vectors per thread of 256, in 16 bits: fewer and longer-lived blocks than
+// norm_block_kernel's, which fit one wave up to a third more rows (norm_row_range). A block has one
+// row, so the loop runs once; it holds the weights' loads in front of the reduction, behind which
+// ptxas otherwise moves them, a second round trip (residual 700 x 8192 9.2 us, without it 11.1).
+template <int DT, bool RES, int VPT>
+__global__ void __launch_bounds__(kThreads) norm_row_kernel(const NormParams p) {
   pdl_trigger();
   __shared__ float red[kThreads / 32];
-  constexpr int VPT = 2;
   constexpr int EB = Act<DT>::BYTES;
   constexpr int VE = Act<DT>::VE;
   const int tid = threadIdx.x;
   pdl_wait();
   for (int64_t row = blockIdx.x; row < p.T; row += gridDim.x) {
     const uint4* xp = reinterpret_cast<const uint4*>(row_ptr(p.x, row, p.x_rs, EB));
-    const uint4* rp = reinterpret_cast<const uint4*>(row_ptr(p.r, row, p.r_rs, EB));
+    const uint4* rp = RES ? reinterpret_cast<const uint4*>(row_ptr(p.r, row, p.r_rs, EB)) : nullptr;
     uint4 xv[VPT], rv[VPT];
     float g[VPT][VE], s[VPT][VE];
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
       const int64_t vi = (int64_t)v * kThreads + tid;
       xv[v] = ldg16(xp + vi);
-      rv[v] = ldg16(rp + vi);
+      if (RES) rv[v] = ldg16(rp + vi);
       load_gamma<DT>(p.gamma + vi * VE, g[v]);
     }
-    uint4* rop = reinterpret_cast<uint4*>(row_ptr(p.r_out, row, p.ro_rs, EB));
+    uint4* rop = RES ? reinterpret_cast<uint4*>(row_ptr(p.r_out, row, p.ro_rs, EB)) : nullptr;
     float ss = 0.f;
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
-      float xf[VE], rf[VE];
-      unpack<DT>(xv[v], xf);
-      unpack<DT>(rv[v], rf);
+      unpack<DT>(xv[v], s[v]);
+      if (RES) {
+        float rf[VE];
+        unpack<DT>(rv[v], rf);
 #pragma unroll
-      for (int e = 0; e < VE; ++e) {
-        s[v][e] = xf[e] + rf[e];
-        ss = fmaf(s[v][e], s[v][e], ss);
+        for (int e = 0; e < VE; ++e) s[v][e] += rf[e];
       }
-      st16(rop + (int64_t)v * kThreads + tid, pack<DT>(s[v]));
+#pragma unroll
+      for (int e = 0; e < VE; ++e) ss = fmaf(s[v][e], s[v][e], ss);
+      if (RES) st16(rop + (int64_t)v * kThreads + tid, pack<DT>(s[v]));
     }
     const float inv = rsqrtf(block_sum(ss, red) * p.inv_H + p.eps);
     uint4* yp = reinterpret_cast<uint4*>(row_ptr(p.y, row, p.y_rs, EB));
 #pragma unroll
     for (int v = 0; v < VPT; ++v) {
       float y[VE];
+      if (!RES) unpack<DT>(xv[v], s[v]);
 #pragma unroll
       for (int e = 0; e < VE; ++e) y[e] = s[v][e] * inv * g[v][e];
       st16(yp + (int64_t)v * kThreads + tid, pack<DT>(y));
     }
-    __syncthreads();  // `red` is reused by the next row
+    __syncthreads();  // before the next row's sums
   }
 }
 
@@ -554,7 +574,7 @@ static void pick_rows(int64_t nvec, KernelEntry* out) {
     out->nm_fn[NM_LARGE] = full ? (const void*)norm_rows_kernel<DT, RES, LPR, VPT, true, 2>
                                 : (const void*)norm_rows_kernel<DT, RES, LPR, VPT, false, 2>;
     out->large_per = kThreads / LPR * 2;
-    out->large_rows = kNormRows2Vecs / nvec;
+    out->large_sm = kNormRows2Vecs / (float)nvec;
   }
 }
 
@@ -568,7 +588,7 @@ static void pick(int64_t H, KernelEntry* out) {
   }
   out->nm_fn[NM_GENERIC] = (const void*)norm_generic_kernel<DT, RES>;
   out->rows = out->large_per = 1;
-  out->large_rows = 0;
+  out->large_sm = out->mid_lo = out->mid_hi = 0.f;
   out->large_smem = 0;
   const int vpt = nvec <= 1024 ? 1 : 2;
   const int threads = norm_threads(nvec, vpt);
@@ -608,23 +628,43 @@ static void pick(int64_t H, KernelEntry* out) {
                                           : (const void*)norm_block_kernel<DT, RES, 1, false, false>)
                                   : (full ? (const void*)norm_block_kernel<DT, RES, 2, false, true>
                                           : (const void*)norm_block_kernel<DT, RES, 2, false, false>);
-    if (!(RES && DT == DT_FP32 && vpt == 1)) {
-      const int bv = RES && nvec <= 1024 ? 2 : 4;
+    const float wave = norm_block_sm(threads, vpt, VE);
+    out->large_sm = vpt == 2 ? wave : (!RES && nvec <= 256 ? 4 : 2) * wave;
+    if constexpr (VE == 8) {
+      if (RES || nvec >= 256) {
+        const int bv = RES && nvec <= 1024 ? 2 : 4;
+        const int bt = norm_threads(nvec, bv);
+        const bool bfull = bt * bv == nvec;
+        out->nm_threads[NM_LARGE] = bt;
+        out->nm_fn[NM_LARGE] = bv == 2 ? (bfull ? (const void*)norm_bulk_kernel<DT, RES, 2, true>
+                                                : (const void*)norm_bulk_kernel<DT, RES, 2, false>)
+                                       : (bfull ? (const void*)norm_bulk_kernel<DT, RES, 4, true>
+                                                : (const void*)norm_bulk_kernel<DT, RES, 4, false>);
+        out->large_smem = (int32_t)(nvec * 16 * (RES ? 2 : 1));
+      }
+      const int rv = nvec % kThreads == 0 ? (int)(nvec / kThreads) : 0;
+      if (RES && rv == 1) out->nm_fn[NM_MID] = (const void*)norm_row_kernel<DT, RES, 1>;
+      if (RES && rv == 4) out->nm_fn[NM_MID] = (const void*)norm_row_kernel<DT, RES, 4>;
+      if (rv == 2) out->nm_fn[NM_MID] = (const void*)norm_row_kernel<DT, RES, 2>;
+      if (out->nm_fn[NM_MID]) {
+        const NormRange r = norm_row_range(RES, rv);
+        out->mid_lo = r.lo;
+        out->mid_hi = r.hi;
+      }
+      if (RES && rv == 2) {
+        out->nm_threads[NM_LARGE] = kThreads;
+        out->nm_fn[NM_LARGE] = out->nm_fn[NM_MID];
+        out->large_smem = 0;
+      }
+    } else if constexpr (!RES) {
+      const int bv = nvec <= 1280 ? 4 : 8;
       const int bt = norm_threads(nvec, bv);
       const bool bfull = bt * bv == nvec;
       out->nm_threads[NM_LARGE] = bt;
-      out->nm_fn[NM_LARGE] = bv == 2 ? (bfull ? (const void*)norm_bulk_kernel<DT, RES, 2, true>
-                                              : (const void*)norm_bulk_kernel<DT, RES, 2, false>)
-                                     : (bfull ? (const void*)norm_bulk_kernel<DT, RES, 4, true>
-                                              : (const void*)norm_bulk_kernel<DT, RES, 4, false>);
-      out->large_smem = (int32_t)(nvec * 16 * (RES ? 2 : 1));
-      if constexpr (RES && VE == 8) {
-        if (nvec == 2 * kThreads) {
-          out->nm_fn[NM_LARGE] = (const void*)addnorm_row_kernel<DT>;
-          out->large_smem = 0;
-        }
-      }
-      out->large_rows = ((RES ? kNormBulkResBytes : kNormBulkBytes) + nvec * 16 - 1) / (nvec * 16);
+      out->nm_fn[NM_LARGE] = bv == 4 ? (bfull ? (const void*)norm_block_kernel<DT, RES, 4, false, true>
+                                              : (const void*)norm_block_kernel<DT, RES, 4, false, false>)
+                                     : (bfull ? (const void*)norm_block_kernel<DT, RES, 8, false, true>
+                                              : (const void*)norm_block_kernel<DT, RES, 8, false, false>);
     }
   } else {
     out->nm_fn[NM_VEC] = (const void*)norm_loop_kernel<DT, RES>;
@@ -646,7 +686,7 @@ bool norm_kernel(bool res, int32_t dtype, int32_t variant, int64_t H, KernelEntr
 }
 
 NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, int32_t* threads, int64_t* blocks,
-                    int32_t* smem) {
+                    int32_t* smem, int32_t sms) {
   const uintptr_t off = (uintptr_t)p->x & 15;
   const int64_t ve = 16 / eb, rs = p->x_rs % ve;
   // all rows of all tensors share their offsets from 16-byte boundaries
@@ -656,8 +696,12 @@ NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, 
   const bool aligned = together && off == 0 && (p->T <= 1 || rs == 0) && ((uintptr_t)p->gamma & 15) == 0;
   p->nvec = (int32_t)(p->H / ve < INT32_MAX ? p->H / ve : INT32_MAX);  // the loop kernel counts its own
   NormEntry e = NM_GENERIC;
-  if (aligned && ke.nm_fn[NM_VEC]) e = ke.nm_fn[NM_LARGE] && p->T >= ke.large_rows ? NM_LARGE : NM_VEC;
-  else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX) e = p->T >= ke.edge_many ? NM_EDGE_MANY : NM_EDGE;
+  const float rows_sm = (float)p->T / (float)sms;
+  if (aligned && ke.nm_fn[NM_VEC])
+    e = ke.nm_fn[NM_MID] && rows_sm > ke.mid_lo && rows_sm <= ke.mid_hi ? NM_MID
+        : ke.nm_fn[NM_LARGE] && rows_sm > ke.large_sm ? NM_LARGE : NM_VEC;
+  else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX)
+    e = p->T >= ke.edge_many ? NM_EDGE_MANY : NM_EDGE;
   *threads = ke.nm_threads[e];
   *smem = e == NM_LARGE ? ke.large_smem : 0;
   const int64_t per = e == NM_VEC ? ke.rows : e == NM_LARGE ? ke.large_per : e == NM_EDGE_MANY ? ke.edge_rows : 1;

@@ -817,7 +817,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       P.nm.first_wait_polls = (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) ? 0u : kBulkWaitPolls;
       int32_t threads = 0, smem = 0;
       int64_t blocks = 0;
-      nm_entry = norm_plan(v.ke, &P.nm, res, elem_size(v.d.dtype), &threads, &blocks, &smem);
+      nm_entry = norm_plan(v.ke, &P.nm, res, elem_size(v.d.dtype), &threads, &blocks, &smem, scm->sm_count);
       cfg.sharedMemBytes = (unsigned)smem;
       cfg.blockDimX = (unsigned)threads;
       cfg.gridDimX = cap_grid(blocks);

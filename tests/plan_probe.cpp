@@ -1,0 +1,53 @@
+// plan_probe.cpp -- prints the kernel entry that a call's dispatch rule chooses, one line per input
+// line, without a GPU: it is linked with the library's own objects and calls the rules that the host
+// core calls. Lines (152 SMs):
+//   norm RES DTYPE H T OFF RS    RES 0/1, rows at element offset OFF of a 16-byte boundary, row stride RS
+#include <cinttypes>
+#include <cstdio>
+#include <cstring>
+
+#include <cuda_runtime.h>
+
+#include "internal.h"
+
+using namespace trident;
+
+constexpr int32_t kSms = 152;
+
+static void norm_line(const char* s) {
+  int res, dtype;
+  int64_t H, T, off, rs;
+  if (std::sscanf(s, "%d %d %" SCNd64 " %" SCNd64 " %" SCNd64 " %" SCNd64, &res, &dtype, &H, &T, &off, &rs) != 6) return;
+  const int eb = dtype == DT_FP32 ? 4 : 2;
+  KernelEntry ke;
+  const char* why = "";
+  if (!norm_kernel(res != 0, dtype, (H * eb) % 16 != 0 ? 1 : 0, H, &ke, &why)) {
+    std::printf("error %s\n", why);
+    return;
+  }
+  NormParams p;
+  std::memset(&p, 0, sizeof p);
+  const uintptr_t at = 4096 + (uintptr_t)(off * eb);
+  p.x = reinterpret_cast<const void*>(at);
+  p.r = res ? p.x : nullptr;
+  p.y = reinterpret_cast<void*>(at);
+  p.r_out = res ? p.y : nullptr;
+  p.gamma = reinterpret_cast<const float*>((uintptr_t)4096);
+  p.T = T;
+  p.H = H;
+  p.x_rs = p.r_rs = p.y_rs = p.ro_rs = rs;
+  int32_t threads = 0, smem = 0;
+  int64_t blocks = 0;
+  const NormEntry e = norm_plan(ke, &p, res != 0, eb, &threads, &blocks, &smem, kSms);
+  static const char* const names[kNormEntries] = {"vec", "edge", "edge_many", "generic", "large", "mid"};
+  std::printf("%s%s\n", names[e], e == NM_LARGE ? (smem ? "_bulk" : ke.large_per > 1 ? "_rows2" : "_regs") : "");
+}
+
+int main() {
+  char line[256];
+  while (std::fgets(line, sizeof line, stdin)) {
+    if (std::strncmp(line, "norm ", 5) == 0) norm_line(line + 5);
+    else std::printf("error unknown line\n");
+  }
+  return 0;
+}

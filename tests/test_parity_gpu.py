@@ -8,6 +8,7 @@ import torch
 from oracle import layer as L
 from paper_2609_37241_gb300 import synth
 from tests import parity as P
+from tests import plans
 
 pytestmark = pytest.mark.gpu
 BF16, FP16, FP32 = 1, 2, 3
@@ -312,6 +313,17 @@ def test_pointwise_parity(S, name, dtype, W, T, layout, variant):
 def test_norm_layouts(S, dtype, T, H, form):
     """Every path of the norms' rule over sizes and layouts, with and without the residual, out
     of place and in place, against the oracle."""
+    check_norm_layout(S, dtype, T, H, form)
+
+
+@pytest.mark.parametrize("dtype,T,H,off,res,plain", plans.NORM_LIMITS)
+def test_norm_entry_limits(S, dtype, T, H, off, res, plain):
+    """Both sides of each line of the norms' rule."""
+    assert (plans.norm(True, dtype, H, T, off), plans.norm(False, dtype, H, T, off)) == (res, plain)
+    check_norm_layout(S, dtype, T, H, "offset" if off else "dense")
+
+
+def check_norm_layout(S, dtype, T, H, form):
     g = np.random.default_rng(H + T)
     tdt = synth._TORCH_DT[dtype]
     es = 4 if dtype == FP32 else 2

@@ -1,0 +1,11 @@
+"""Which kernel entry calls at the limits of the dispatch rules take (no GPU): the GPU tests that
+run these calls then reach the entries they mean to."""
+import pytest
+
+from tests import plans
+
+
+@pytest.mark.parametrize("dtype,T,H,off,res,plain", plans.NORM_LIMITS)
+def test_norm_entries(dtype, T, H, off, res, plain):
+    assert plans.norm(True, dtype, H, T, off) == res
+    assert plans.norm(False, dtype, H, T, off) == plain
