@@ -76,6 +76,20 @@ constexpr int64_t kNormEdgeRows = 3072;
 // 29.6; at 300 rows 2.31 / 2.76. (16 bits: 3000 x 3999 12.5 / 13.7.)
 constexpr int64_t kNormEdgeWideRows = 2048;
 
+// Calls of few rows, in rows per SM. Rows of 33 to 128 vectors: norm_block_kernel, a vector per thread,
+// instead of two or four per lane one after the other (warp / block, us): 64 x 1024 bf16 1.87 / 1.19, 2200
+// 3.20 / 3.00, 3000 3.62 / 3.85; 1300 x 512 2.60 / 1.98, 2200 2.67 / 3.02; 1300 x 320 2.05 / 1.93, 1700
+// 2.06 / 2.25; residual 64 x 1024 2.06 / 1.11, 4500 7.33 / 6.91, 7000 10.2 / 10.2; 1300 x 320 2.25 / 2.10,
+// 2200 2.65 / 3.22. Rows of 2048 vectors: eight per thread of 256 instead of two per thread of 1024, whose
+// one block per SM waits longest on itself: 64 / 152 x 16384 bf16 2.63 / 3.63 -> 2.34 / 3.13, residual 3.91
+// / 4.91 -> 3.42 / 4.17; fp32 only below half a row per SM (64 x 8192 3.04 -> 2.53, 100 3.40 / 3.97), with
+// the residual only above 0.4 (40 x 8192 3.74 / 4.07, 100 4.75 -> 4.29).
+static NormRange norm_few_range(bool res, int ve, int64_t nvec) {
+  if (nvec == kNormBlockVecs) return ve == 8 ? NormRange{0.f, 1.f} : res ? NormRange{0.4f, 1.f} : NormRange{0.f, 0.5f};
+  if (nvec > 32 && nvec <= 64) return {0.f, 9.f};
+  if (nvec > 64 && nvec <= 128) return {0.f, res ? 40.f : 14.f};
+  return {0.f, 0.f};
+}
 template <int DT>
 __device__ __forceinline__ void load_gamma(const float* g, float* out) {
 #pragma unroll
@@ -559,7 +573,7 @@ __global__ void __launch_bounds__(kThreads) norm_generic_kernel(const NormParams
   }
 }
 
-constexpr int kNormRowsVecs = 128;    // rows of at most this many vectors: norm_rows_kernel
+constexpr int kNormRowsVecs = 128;    // rows of at most this many vectors: norm_rows_kernel, but in calls of few rows
 
 // Threads of a block for a row of nvec vectors at vpt per thread.
 static int norm_threads(int64_t nvec, int vpt) { return (int)(((nvec + vpt - 1) / vpt + 31) / 32 * 32); }
@@ -588,10 +602,21 @@ static void pick(int64_t H, KernelEntry* out) {
   }
   out->nm_fn[NM_GENERIC] = (const void*)norm_generic_kernel<DT, RES>;
   out->rows = out->large_per = 1;
-  out->large_sm = out->mid_lo = out->mid_hi = 0.f;
+  out->large_sm = out->mid_lo = out->mid_hi = out->few_lo = out->few_hi = 0.f;
   out->large_smem = 0;
   const int vpt = nvec <= 1024 ? 1 : 2;
   const int threads = norm_threads(nvec, vpt);
+  const NormRange few = norm_few_range(RES, VE, nvec);
+  if (H % VE == 0 && few.hi > 0.f) {
+    const int fv = nvec <= kNormRowsVecs ? 1 : 8;
+    const int ft = norm_threads(nvec, fv);
+    out->few_lo = few.lo;
+    out->few_hi = few.hi;
+    out->nm_threads[NM_FEW] = ft;
+    out->nm_fn[NM_FEW] = fv == 8 ? (const void*)norm_block_kernel<DT, RES, 8, false, true>
+                         : ft == nvec ? (const void*)norm_block_kernel<DT, RES, 1, false, true>
+                                      : (const void*)norm_block_kernel<DT, RES, 1, false, false>;
+  }
   // rows that begin anywhere hold nvec or nvec - 1 whole vectors, and at least one
   out->edge_rows = 1;
   out->edge_many = INT64_MAX;
@@ -698,7 +723,8 @@ NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, 
   NormEntry e = NM_GENERIC;
   const float rows_sm = (float)p->T / (float)sms;
   if (aligned && ke.nm_fn[NM_VEC])
-    e = ke.nm_fn[NM_MID] && rows_sm > ke.mid_lo && rows_sm <= ke.mid_hi ? NM_MID
+    e = ke.nm_fn[NM_FEW] && rows_sm > ke.few_lo && rows_sm <= ke.few_hi ? NM_FEW
+        : ke.nm_fn[NM_MID] && rows_sm > ke.mid_lo && rows_sm <= ke.mid_hi ? NM_MID
         : ke.nm_fn[NM_LARGE] && rows_sm > ke.large_sm ? NM_LARGE : NM_VEC;
   else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX)
     e = p->T >= ke.edge_many ? NM_EDGE_MANY : NM_EDGE;

@@ -45,4 +45,8 @@ NORM_LIMITS = [
     (2, 913, 8192, 0, "large_bulk", "large_bulk"),
     (3, 1217, 2048, 0, "vec", "large_regs"), (3, 457, 5000, 0, "vec", "large_regs"),    # four per thread
     (3, 305, 8192, 0, "vec", "large_regs"), (3, 305, 7000, 0, "vec", "large_regs"),     # eight
+    (1, 1368, 264, 0, "few", "few"), (1, 1369, 264, 0, "vec", "vec"),  # few rows
+    (2, 2128, 1024, 0, "few", "few"), (2, 2129, 1024, 0, "few", "vec"), (3, 6081, 512, 0, "vec", "vec"),
+    (3, 1, 148, 0, "few", "few"), (1, 152, 16384, 0, "few", "few"), (2, 153, 16384, 0, "large_bulk", "large_bulk"),
+    (3, 61, 8192, 0, "few", "few"), (3, 77, 8192, 0, "few", "vec"), (3, 60, 8192, 0, "vec", "few"),
 ]
