@@ -157,9 +157,11 @@ int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks);
 
 // Norm entries (norm_plan): 16-byte aligned rows, rows at any common offset (few or many rows),
 // scalar accesses, the entry of long aligned calls (bulk copies, more vectors per thread, or two
-// rows at a time for short rows), and those of few rows and of some in between (norm_row_kernel).
+// rows at a time for short rows), those of few rows and of some in between (norm_row_kernel), and rows
+// at other offsets with the loads out of branches.
 constexpr int kNormBlockVecs = 2048;  // norm_block_kernel, norm_bulk_kernel: vectors of a row at most
-enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_EDGE_MANY, NM_GENERIC, NM_LARGE, NM_FEW, NM_MID, kNormEntries };
+enum NormEntry : int32_t { NM_VEC, NM_EDGE, NM_EDGE_MANY, NM_GENERIC, NM_LARGE, NM_FEW, NM_MID,
+                           NM_EDGE_FLAT, kNormEntries };
 
 // Kernel entry (host stub address) plus its launch shape rule.
 struct KernelEntry {
@@ -179,6 +181,7 @@ struct KernelEntry {
   float large_sm = 0;      // norms: calls of more rows per SM take the NM_LARGE entry
   float few_lo = 0, few_hi = 0;  // ... of rows per SM in (few_lo, few_hi] the NM_FEW entry
   float mid_lo = 0, mid_hi = 0;  // ... and of rows per SM in (mid_lo, mid_hi] the NM_MID entry
+  float edge_lo = 0, edge_hi = 0;  // the same for rows at other offsets and the NM_EDGE_FLAT entry
   int32_t large_per = 1;   // ... that entry's rows per block
   int32_t large_smem = 0;  // ... and its dynamic shared memory (rows staged by bulk copies)
   int32_t kind = 0;      // which grid rule the host applies (KernelKind)

@@ -90,6 +90,13 @@ static NormRange norm_few_range(bool res, int ve, int64_t nvec) {
   if (nvec > 64 && nvec <= 128) return {0.f, res ? 40.f : 14.f};
   return {0.f, 0.f};
 }
+// EDGE rows in 16 bits, a block per row: from lo to hi threads per SM the loads stand in no branch
+// (EDGE 2). With fewer, the branches' round trips hide in the launch; with more, the loads they save
+// count. Branches / none, at an odd offset: 600 x 333 2.05 / 2.87 us, 900 3.67 / 2.93; 300 x 1001 2.42 /
+// 3.29, 450 3.94 / 3.37, 900 4.08 / 3.34, 2000 4.56 / 4.67; 300 x 1537 3.81 / 3.42, 1333 4.26 / 4.42;
+// residual 450 x 333 1.94 / 2.86, 1333 3.59 / 2.97; 600 x 1001 3.60 / 3.40, 900 3.19 / 3.82. In fp32, with half the weights per vector, the branches are faster (600 x 1001 2.06 / 2.48).
+static NormRange norm_edge_range(bool res) { return res ? NormRange{200.f, 570.f} : NormRange{300.f, 1280.f}; }
+
 template <int DT>
 __device__ __forceinline__ void load_gamma(const float* g, float* out) {
 #pragma unroll
@@ -102,17 +109,23 @@ __device__ __forceinline__ void load_gamma(const float* g, float* out) {
 // The weights of a vector whose first element is i, not a multiple of 4 (its offset from one, the
 // same for the whole block): the aligned float4s around them, shifted, where those lie within
 // the H weights and gamma itself is aligned; by element otherwise. By element everywhere, every
-// weight load of a warp touched 32 sectors for 128 bytes.
-template <int DT>
+// weight load of a warp touched 32 sectors for 128 bytes. FLAT: without the branch that only a row's
+// last vectors take: the last float4's weights one by one (past the row's end: the last weight, not
+// used).
+template <int DT, bool FLAT>
 __device__ __forceinline__ void load_gamma_at(const float* gamma, int i, int H, float* out) {
   constexpr int VE = Act<DT>::VE;
   const int sh = i & 3, b = i - sh;
-  if ((reinterpret_cast<uintptr_t>(gamma) & 15) == 0 && b + VE + 4 <= H) {
+  if ((reinterpret_cast<uintptr_t>(gamma) & 15) == 0 && (FLAT || b + VE + 4 <= H)) {
     float t[VE + 4];
 #pragma unroll
-    for (int q = 0; q < VE / 4 + 1; ++q) {
+    for (int q = 0; q < VE / 4 + (FLAT ? 0 : 1); ++q) {
       const float4 v = ldg_f4(gamma + b + 4 * q);
       t[4 * q] = v.x; t[4 * q + 1] = v.y; t[4 * q + 2] = v.z; t[4 * q + 3] = v.w;
+    }
+    if (FLAT) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) t[VE + j] = __ldg(gamma + min(b + VE + j, H - 1));
     }
 #pragma unroll
     for (int e = 0; e < VE; ++e) out[e] = sh < 2 ? (sh == 0 ? t[e] : t[e + 1]) : (sh == 2 ? t[e + 2] : t[e + 3]);
@@ -222,8 +235,9 @@ __device__ __forceinline__ float norm_block_sum(float v, float* red) {
 // last vector and drop it: with the loads behind a branch the compiler finished them before
 // leaving it (256 x 4096 3.3 us). FULL: no such threads. EDGE: the row's tensors
 // start at one common offset from a 16-byte boundary; the first peel and last tail elements
-// (fewer than a vector each) go to threads of their own, and gamma is read by load_gamma_at.
-template <int DT, bool RES, int VPT, bool EDGE, bool FULL>
+// (fewer than a vector each) go to threads of their own, and gamma is read by load_gamma_at. EDGE 2:
+// every load without a branch (norm_edge_range).
+template <int DT, bool RES, int VPT, int EDGE, bool FULL>
 __global__ void __launch_bounds__(VPT >= 8 ? 256 : VPT >= 4 ? 512 : 1024) norm_block_kernel(const NormParams p) {
   pdl_trigger();
   __shared__ __align__(16) float red[32];
@@ -263,15 +277,17 @@ __global__ void __launch_bounds__(VPT >= 8 ? 256 : VPT >= 4 ? 512 : 1024) norm_b
     xv[v] = ldg16(xr + (int64_t)vi * 16);
     if (RES) rv[v] = ldg16(rr + (int64_t)vi * 16);
     if (EDGE) {
-      load_gamma_at<DT>(p.gamma, peel + vi * VE, (int)p.H, g[v]);
+      load_gamma_at<DT, EDGE == 2>(p.gamma, peel + vi * VE, (int)p.H, g[v]);
     } else {
       load_gamma<DT>(p.gamma + (int64_t)vi * VE, g[v]);
     }
   }
-  if (EDGE && edge >= 0) {
-    es = load_elem<DT>(p.x, row * p.x_rs + edge);
-    if (RES) es += load_elem<DT>(p.r, row * p.r_rs + edge);
-    eg = __ldg(p.gamma + edge);
+  if (EDGE == 2 || (EDGE && edge >= 0)) {  // 2: threads without an edge element load the first and drop it
+    const int ec = EDGE == 2 ? max(edge, 0) : edge;
+    es = load_elem<DT>(p.x, row * p.x_rs + ec);
+    if (RES) es += load_elem<DT>(p.r, row * p.r_rs + ec);
+    eg = __ldg(p.gamma + ec);
+    if (EDGE == 2 && edge < 0) es = 0.f;
   }
   char* ro = RES ? row_ptr(p.r_out, row, p.ro_rs, EB) + peel * EB : nullptr;
   float ss = EDGE ? es * es : 0.f;
@@ -328,7 +344,7 @@ __global__ void __launch_bounds__(kThreads) norm_rows_edge_kernel(const NormPara
     const int vi = min(lane + 32 * v, nvec - 1);
     xv[v] = ldg16(xr + vi * 16);
     if (RES) rv[v] = ldg16(rr + vi * 16);
-    load_gamma_at<DT>(p.gamma, peel + vi * VE, H, g[v]);
+    load_gamma_at<DT, false>(p.gamma, peel + vi * VE, H, g[v]);
   }
   if (edge >= 0) {
     es = load_elem<DT>(p.x, row * p.x_rs + edge);
@@ -602,7 +618,7 @@ static void pick(int64_t H, KernelEntry* out) {
   }
   out->nm_fn[NM_GENERIC] = (const void*)norm_generic_kernel<DT, RES>;
   out->rows = out->large_per = 1;
-  out->large_sm = out->mid_lo = out->mid_hi = out->few_lo = out->few_hi = 0.f;
+  out->large_sm = out->mid_lo = out->mid_hi = out->few_lo = out->few_hi = out->edge_lo = out->edge_hi = 0.f;
   out->large_smem = 0;
   const int vpt = nvec <= 1024 ? 1 : 2;
   const int threads = norm_threads(nvec, vpt);
@@ -613,17 +629,25 @@ static void pick(int64_t H, KernelEntry* out) {
     out->few_lo = few.lo;
     out->few_hi = few.hi;
     out->nm_threads[NM_FEW] = ft;
-    out->nm_fn[NM_FEW] = fv == 8 ? (const void*)norm_block_kernel<DT, RES, 8, false, true>
-                         : ft == nvec ? (const void*)norm_block_kernel<DT, RES, 1, false, true>
-                                      : (const void*)norm_block_kernel<DT, RES, 1, false, false>;
+    out->nm_fn[NM_FEW] = fv == 8 ? (const void*)norm_block_kernel<DT, RES, 8, 0, true>
+                         : ft == nvec ? (const void*)norm_block_kernel<DT, RES, 1, 0, true>
+                                      : (const void*)norm_block_kernel<DT, RES, 1, 0, false>;
   }
   // rows that begin anywhere hold nvec or nvec - 1 whole vectors, and at least one
   out->edge_rows = 1;
   out->edge_many = INT64_MAX;
   if (nvec >= 2 && nvec <= kNormBlockVecs) {
     out->nm_threads[NM_EDGE] = threads;
-    out->nm_fn[NM_EDGE] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, true, false>
-                                   : (const void*)norm_block_kernel<DT, RES, 2, true, false>;
+    if constexpr (VE == 8) {
+      const NormRange r = norm_edge_range(RES);
+      out->edge_lo = r.lo / (float)threads;
+      out->edge_hi = r.hi / (float)threads;
+      out->nm_threads[NM_EDGE_FLAT] = threads;
+      out->nm_fn[NM_EDGE_FLAT] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, 2, false>
+                                          : (const void*)norm_block_kernel<DT, RES, 2, 2, false>;
+    }
+    out->nm_fn[NM_EDGE] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, 1, false>
+                                   : (const void*)norm_block_kernel<DT, RES, 2, 1, false>;
     if (nvec <= 64 || (!RES && nvec <= kNormRowsVecs)) {
       out->edge_rows = kThreads / 32;
       out->edge_many = nvec <= 32 ? 0 : kNormEdgeRows;
@@ -633,7 +657,7 @@ static void pick(int64_t H, KernelEntry* out) {
     } else if (VE == 4 && vpt == 1 && nvec > 512) {
       out->edge_many = kNormEdgeWideRows;
       out->nm_threads[NM_EDGE_MANY] = norm_threads(nvec, 2);
-      out->nm_fn[NM_EDGE_MANY] = (const void*)norm_block_kernel<DT, RES, 2, true, false>;
+      out->nm_fn[NM_EDGE_MANY] = (const void*)norm_block_kernel<DT, RES, 2, 1, false>;
     }
   }
   if (H % VE != 0) return;
@@ -649,10 +673,10 @@ static void pick(int64_t H, KernelEntry* out) {
   } else if (nvec <= kNormBlockVecs) {
     const bool full = threads * vpt == nvec;
     out->nm_threads[NM_VEC] = threads;
-    out->nm_fn[NM_VEC] = vpt == 1 ? (full ? (const void*)norm_block_kernel<DT, RES, 1, false, true>
-                                          : (const void*)norm_block_kernel<DT, RES, 1, false, false>)
-                                  : (full ? (const void*)norm_block_kernel<DT, RES, 2, false, true>
-                                          : (const void*)norm_block_kernel<DT, RES, 2, false, false>);
+    out->nm_fn[NM_VEC] = vpt == 1 ? (full ? (const void*)norm_block_kernel<DT, RES, 1, 0, true>
+                                          : (const void*)norm_block_kernel<DT, RES, 1, 0, false>)
+                                  : (full ? (const void*)norm_block_kernel<DT, RES, 2, 0, true>
+                                          : (const void*)norm_block_kernel<DT, RES, 2, 0, false>);
     const float wave = norm_block_sm(threads, vpt, VE);
     out->large_sm = vpt == 2 ? wave : (!RES && nvec <= 256 ? 4 : 2) * wave;
     if constexpr (VE == 8) {
@@ -686,10 +710,10 @@ static void pick(int64_t H, KernelEntry* out) {
       const int bt = norm_threads(nvec, bv);
       const bool bfull = bt * bv == nvec;
       out->nm_threads[NM_LARGE] = bt;
-      out->nm_fn[NM_LARGE] = bv == 4 ? (bfull ? (const void*)norm_block_kernel<DT, RES, 4, false, true>
-                                              : (const void*)norm_block_kernel<DT, RES, 4, false, false>)
-                                     : (bfull ? (const void*)norm_block_kernel<DT, RES, 8, false, true>
-                                              : (const void*)norm_block_kernel<DT, RES, 8, false, false>);
+      out->nm_fn[NM_LARGE] = bv == 4 ? (bfull ? (const void*)norm_block_kernel<DT, RES, 4, 0, true>
+                                              : (const void*)norm_block_kernel<DT, RES, 4, 0, false>)
+                                     : (bfull ? (const void*)norm_block_kernel<DT, RES, 8, 0, true>
+                                              : (const void*)norm_block_kernel<DT, RES, 8, 0, false>);
     }
   } else {
     out->nm_fn[NM_VEC] = (const void*)norm_loop_kernel<DT, RES>;
@@ -727,7 +751,8 @@ NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, 
         : ke.nm_fn[NM_MID] && rows_sm > ke.mid_lo && rows_sm <= ke.mid_hi ? NM_MID
         : ke.nm_fn[NM_LARGE] && rows_sm > ke.large_sm ? NM_LARGE : NM_VEC;
   else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX)
-    e = p->T >= ke.edge_many ? NM_EDGE_MANY : NM_EDGE;
+    e = p->T >= ke.edge_many ? NM_EDGE_MANY
+        : ke.nm_fn[NM_EDGE_FLAT] && rows_sm > ke.edge_lo && rows_sm <= ke.edge_hi ? NM_EDGE_FLAT : NM_EDGE;
   *threads = ke.nm_threads[e];
   *smem = e == NM_LARGE ? ke.large_smem : 0;
   const int64_t per = e == NM_VEC ? ke.rows : e == NM_LARGE ? ke.large_per : e == NM_EDGE_MANY ? ke.edge_rows : 1;

@@ -39,7 +39,7 @@ static void norm_line(const char* s) {
   int32_t threads = 0, smem = 0;
   int64_t blocks = 0;
   const NormEntry e = norm_plan(ke, &p, res != 0, eb, &threads, &blocks, &smem, kSms);
-  static const char* const names[kNormEntries] = {"vec", "edge", "edge_many", "generic", "large", "few", "mid"};
+  static const char* const names[kNormEntries] = {"vec", "edge", "edge_many", "generic", "large", "few", "mid", "edge_flat"};
   std::printf("%s%s\n", names[e], e == NM_LARGE ? (smem ? "_bulk" : ke.large_per > 1 ? "_rows2" : "_regs") : "");
 }
 

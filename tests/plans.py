@@ -49,4 +49,8 @@ NORM_LIMITS = [
     (2, 2128, 1024, 0, "few", "few"), (2, 2129, 1024, 0, "few", "vec"), (3, 6081, 512, 0, "vec", "vec"),
     (3, 1, 148, 0, "few", "few"), (1, 152, 16384, 0, "few", "few"), (2, 153, 16384, 0, "large_bulk", "large_bulk"),
     (3, 61, 8192, 0, "few", "few"), (3, 77, 8192, 0, "few", "vec"), (3, 60, 8192, 0, "vec", "few"),
+    (1, 475, 333, 1, "edge", "edge"), (2, 713, 333, 1, "edge_flat", "edge_flat"),       # rows at odd offsets
+    (1, 1354, 333, 1, "edge", "edge_flat"), (2, 357, 1023, 1, "edge_flat", "edge_flat"),
+    (1, 88, 4001, 1, "edge_flat", "edge"), (2, 91, 4095, 1, "edge_flat", "edge_flat"),
+    (1, 40, 9001, 1, "edge", "edge"), (2, 85, 9007, 1, "edge_flat", "edge_flat"),       # two vectors per thread
 ]
