@@ -267,15 +267,14 @@ __device__ __forceinline__ void rope_pair_freqs(const float2* inv_freq, int lane
 #pragma unroll
   for (int q = 0; q < 4; ++q) fq[q] = ldg_f4(reinterpret_cast<const float*>(inv_freq) + 16 * lane + 4 * q);
 }
-// The same from a table that the previous kernel of the stream wrote, called after pdl_wait: that
-// kernel may have written it while this grid was already resident, so the loads are coherent ones
-// (__ldg is defined only for what nothing writes during the kernel) and stay behind the wait.
+// The same from a table that the previous kernel of the stream may have written, called after
+// pdl_wait: that kernel may have written it while this grid was already resident, so the loads are
+// plain, coherent ones (__ldg is defined only for what nothing writes during the kernel), which
+// pdl_wait's memory clobber keeps behind it.
 __device__ __forceinline__ void rope_pair_freqs_late(const float2* inv_freq, int lane, float4* fq) {
 #pragma unroll
   for (int q = 0; q < 4; ++q)
-    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(fq[q].x), "=f"(fq[q].y), "=f"(fq[q].z), "=f"(fq[q].w)
-                 : "l"(reinterpret_cast<const float*>(inv_freq) + 16 * lane + 4 * q) : "memory");
+    fq[q] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(inv_freq) + 16 * lane + 4 * q);
 }
 
 // A lane's q- or k-norm weights (kind 1: q, 2: k), for its low and high halves.

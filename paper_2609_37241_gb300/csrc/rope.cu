@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(kRopeBulkThreads, 6) rope_bulk_kernel(const Ro
   RopeAngles an;
   {
     float4 fq[4];
-    if (p.freq_late) rope_pair_freqs_late(p.inv_freq, lane, fq);
-    else rope_pair_freqs(p.inv_freq, lane, fq);
+    rope_pair_freqs_late(p.inv_freq, lane, fq);
     rope_angles(pos_ok ? pos : 0, fq, &an);
   }
   auto landed = [&](uint32_t polls) -> bool {
