@@ -80,7 +80,7 @@ struct RopeParams {
   int32_t Hq, Hkv, D, NH;  // NH = Hq + 2 Hkv head-rows per token
   float eps, inv_D;
   int32_t prefetch;
-  int32_t freq_late;   // 1: inv_freq may still be written by the previous kernel of the stream
+  int32_t freq_late;   // 1: inv_freq is written by the previous kernel of the stream: read it after the wait
   int32_t ipt, rpi;    // warp items per token, head-rows per item (RopeSplit)
   uint32_t ipt_magic;  // item / ipt by fast_div
   int32_t ipt_shift;
@@ -176,7 +176,8 @@ struct KernelEntry {
   const void* fn_step_inplace = nullptr;  // ... one block per token for the norms
   const void* fn_large = nullptr;  // RoPE: the bulk-copy entry (rope_plan chooses)
   const void* any_fn[2] = {};      // RoPE versions of the generic kind: rope_any_kernel (or NULL)
-  const void* fn_mid = nullptr;    // RoPE: the entry between fn and fn_large (rope_plan chooses)
+  const void* fn_mid = nullptr;    // RoPE: two head-rows per lane group
+  const void* fn_blocks = nullptr;  // RoPE: fn for blocks of 128 or 256 threads
   const void* pw_fn[kPwEntries] = {};  // elementwise, by PointwiseEntry
   float large_sm = 0;      // norms: calls of more rows per SM take the NM_LARGE entry
   float few_lo = 0, few_hi = 0;  // ... of rows per SM in (few_lo, few_hi] the NM_FEW entry
@@ -259,13 +260,13 @@ inline RopeSplit rope_split(int64_t NH, int64_t gw, int32_t max_rows) {
 
 // Which vector RoPE entry a call of T tokens takes, and its launch shape. The splits depend
 // only on the version's head counts and head size (rope_plans, at registration).
-enum RopeEntry : int32_t { ROPE_SMALL = 0, ROPE_MID = 1, ROPE_BULK = 2 };
+enum RopeEntry : int32_t { ROPE_SMALL = 0, ROPE_MID = 1, ROPE_BULK = 2, ROPE_BLOCKS = 3, kRopeEntries };
 struct RopePlans {
-  RopeSplit split[3];  // by RopeEntry
+  RopeSplit split[kRopeEntries];  // by RopeEntry
   RopeSplit any[2];    // rope_any_kernel with one and with three rows per lane group (ipt 0: none)
 };
 void rope_plans(int64_t NH, int32_t D, RopePlans* out);
-RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks);
-int rope_any_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks);
+RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks, int32_t sms);
+int rope_any_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int64_t* blocks, int32_t sms);
 
 }  // namespace trident

@@ -43,6 +43,7 @@ struct DeviceScratch {
   std::once_flag once;
   cudaError_t setup_error = cudaSuccess;
   unsigned char* addr = nullptr;  // device address of g_scratch on this device
+  int sms = 0;                    // its multiprocessors
 };
 DeviceScratch g_dev[kMaxDevices];
 
@@ -93,15 +94,17 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   if (!rope_kernel(dtype, TRIDENT_VARIANT_VECTOR, p.D, qknorm, &ke, &why))
     return internal_fail(TRIDENT_ERR_INVALID, why);
 
-  // one-time set-up on this device: the device address of the static array
+  // one-time set-up on this device: the device address of the static array, the SM count
   DeviceScratch& ds = g_dev[dev];
   std::call_once(ds.once, [&] {
     void* a = nullptr;
     ds.setup_error = cudaGetSymbolAddress(&a, g_scratch);
     ds.addr = static_cast<unsigned char*>(a);
+    if (ds.setup_error == cudaSuccess)
+      ds.setup_error = cudaDeviceGetAttribute(&ds.sms, cudaDevAttrMultiProcessorCount, dev);
   });
   if (ds.setup_error != cudaSuccess || !ds.addr)
-    return internal_fail(TRIDENT_ERR_CUDA, "cudaGetSymbolAddress of the scratch array failed");
+    return internal_fail(TRIDENT_ERR_CUDA, "set-up of the scratch array failed");
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint32_t* status = reinterpret_cast<uint32_t*>(ds.addr);
@@ -129,10 +132,11 @@ extern "C" __attribute__((visibility("default"))) int32_t trident_rope_kv_noallo
   int32_t threads = 0;
   int64_t blocks = 0;
   rope_plans(p.NH, p.D, &plans);
-  const RopeEntry entry = rope_plan(plans, &p, &threads, &blocks);
+  const RopeEntry entry = rope_plan(plans, &p, &threads, &blocks, ds.sms);
   bp.rp = p;
   bp.first_wait_polls = kBulkWaitPolls;
-  const void* fn = entry == ROPE_BULK ? ke.fn_large : (entry == ROPE_MID ? ke.fn_mid : ke.fn);
+  const void* const fns[kRopeEntries] = {ke.fn, ke.fn_mid, ke.fn_large, ke.fn_blocks};  // by RopeEntry
+  const void* fn = fns[entry];
   void* kargs[1] = {entry == ROPE_BULK ? (void*)&bp : (void*)&p};
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -396,9 +396,8 @@ struct Version {
   CUfunction fn_inplace_late;  // layer chain: `fn_inplace` with the late launch trigger
   CUfunction fn_wide;     // layer chain: `fn_inplace` with kChainWideTileVecs tiles
   int32_t wave_blocks;    // layer chain: blocks of `fn` resident at once on the whole GPU
-  CUfunction fn_large;          // RoPE: the bulk-copy entry
-  CUfunction fn_mid;            // RoPE: entry between fn and fn_large (rope_plan)
-  RopePlans rope_plans;         // vector RoPE: item splits of its three entries
+  CUfunction rope_fn[kRopeEntries];  // vector RoPE: entries by size (rope_plan)
+  RopePlans rope_plans;         // vector RoPE: item splits of its entries
   RopeSplit rope_split[2];      // layer chain: item splits with one and kChainRopeRows rows
   CUfunction pw_fn[kPwEntries];  // elementwise: entries by layout and size (pointwise_plan)
   CUfunction any_fn[2];            // RoPE versions of the generic kind: rope_any_kernel
@@ -829,13 +828,13 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       if (v.ke.kind == KK_ROPE_PAIR) {
         int32_t threads = 0;
         int64_t blocks = 0;
-        rope_entry = rope_plan(v.rope_plans, &P.rp, &threads, &blocks);
+        rope_entry = rope_plan(v.rope_plans, &P.rp, &threads, &blocks, scm->sm_count);
         cfg.blockDimX = (unsigned)threads;
         cfg.gridDimX = cap_grid(blocks);
         if (rope_entry == ROPE_BULK)
           P.rb.first_wait_polls = (scm->opt.flags & TRIDENT_OPT_TEST_WAIT_TIMEOUT) ? 0u : kBulkWaitPolls;
       } else if (int32_t threads = 0; v.any_fn[0] &&
-                 (rope_any = rope_any_plan(v.rope_plans, &P.rp, &threads, &rope_blocks)) >= 0) {
+                 (rope_any = rope_any_plan(v.rope_plans, &P.rp, &threads, &rope_blocks, scm->sm_count)) >= 0) {
         cfg.blockDimX = (unsigned)threads;
         cfg.gridDimX = cap_grid(rope_blocks);
       } else {  // generic: one warp per head-row
@@ -962,7 +961,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
   if (v.ke.kind == KK_POINTWISE)
     fn = v.pw_fn[pw_entry];
   else if (v.ke.kind == KK_ROPE_PAIR)
-    fn = rope_entry == ROPE_BULK ? v.fn_large : (rope_entry == ROPE_MID ? v.fn_mid : v.fn);
+    fn = v.rope_fn[rope_entry];
   else if (v.ke.kind == KK_NORM)
     fn = v.nm_fn[nm_entry];
   else if (rope_any >= 0)
@@ -1372,12 +1371,6 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
           cudaFuncSetAttribute(v.ke.nm_fn[NM_LARGE], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                2 * kNormBlockVecs * 16) != cudaSuccess)
         return fail(TRIDENT_ERR_CUDA, "cannot set the norm kernel's shared-memory size");
-      if (v.ke.fn_large) {
-        cudaFunction_t h = nullptr;
-        if (cudaGetFuncBySymbol(&h, v.ke.fn_large) != cudaSuccess || !h)
-          return fail(TRIDENT_ERR_CUDA, "cannot resolve the large-call kernel entry");
-        v.fn_large = reinterpret_cast<CUfunction>(h);
-      }
       auto resolve = [&](const void* entry, CUfunction* out_fn) {
         cudaFunction_t e = nullptr;
         if (entry && (cudaGetFuncBySymbol(&e, entry) != cudaSuccess || !e)) return false;
@@ -1393,11 +1386,11 @@ int32_t append_version(trident_scm_t* scm, const trident_spec_desc* desc, int32_
       for (int k = 0; k < kNormEntries; ++k)
         if (!resolve(v.ke.nm_fn[k], &v.nm_fn[k]))
           return fail(TRIDENT_ERR_CUDA, "cannot resolve the norm kernel entries");
-      if (v.ke.fn_mid) {
-        cudaFunction_t m = nullptr;
-        if (cudaGetFuncBySymbol(&m, v.ke.fn_mid) != cudaSuccess || !m)
-          return fail(TRIDENT_ERR_CUDA, "cannot resolve the mid-size RoPE kernel entry");
-        v.fn_mid = reinterpret_cast<CUfunction>(m);
+      if (v.ke.kind == KK_ROPE_PAIR) {
+        const void* const entries[kRopeEntries] = {v.ke.fn, v.ke.fn_mid, v.ke.fn_large, v.ke.fn_blocks};  // by RopeEntry
+        for (int k = 0; k < kRopeEntries; ++k)
+          if (!resolve(entries[k], &v.rope_fn[k]))
+            return fail(TRIDENT_ERR_CUDA, "cannot resolve the RoPE kernel entries");
       }
       if (v.ke.fn_inplace) {
         cudaFunction_t g = nullptr;

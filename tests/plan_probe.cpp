@@ -2,6 +2,7 @@
 // line, without a GPU: it is linked with the library's own objects and calls the rules that the host
 // core calls. Lines (152 SMs):
 //   norm RES DTYPE H T OFF RS    RES 0/1, rows at element offset OFF of a 16-byte boundary, row stride RS
+//   rope ANY QK HQ HKV D T       ANY 1: a version of any alignment; QK 1: with q/k norm
 #include <cinttypes>
 #include <cstdio>
 #include <cstring>
@@ -43,10 +44,43 @@ static void norm_line(const char* s) {
   std::printf("%s%s\n", names[e], e == NM_LARGE ? (smem ? "_bulk" : ke.large_per > 1 ? "_rows2" : "_regs") : "");
 }
 
+static void rope_line(const char* s) {
+  int qk, Hq, Hkv, D, any;
+  int64_t T;
+  if (std::sscanf(s, "%d %d %d %d %d %" SCNd64, &any, &qk, &Hq, &Hkv, &D, &T) != 6) return;
+  KernelEntry ke;
+  const char* why = "";
+  if (!rope_kernel(DT_BF16, any ? 1 : 2, D, qk != 0, &ke, &why)) {
+    std::printf("error %s\n", why);
+    return;
+  }
+  RopeParams p;
+  std::memset(&p, 0, sizeof p);
+  p.gamma_q = p.gamma_k = qk ? reinterpret_cast<const float*>((uintptr_t)4096) : nullptr;
+  p.T = T;
+  p.Hq = Hq;
+  p.Hkv = Hkv;
+  p.D = D;
+  p.NH = Hq + 2 * Hkv;
+  p.q_rs = p.k_rs = p.v_rs = (int64_t)p.NH * D;
+  RopePlans plans{};
+  rope_plans(p.NH, D, &plans);
+  int32_t threads = 0;
+  int64_t blocks = 0;
+  if (any) {
+    const int e = rope_any_plan(plans, &p, &threads, &blocks, kSms);
+    std::printf("%s\n", e < 0 ? "generic" : e == 0 ? "any1" : "any3");
+    return;
+  }
+  const RopeEntry e = rope_plan(plans, &p, &threads, &blocks, kSms);
+  std::printf("%s_%d\n", e == ROPE_MID ? "two" : e == ROPE_BULK ? "bulk" : "one", threads);
+}
+
 int main() {
   char line[256];
   while (std::fgets(line, sizeof line, stdin)) {
     if (std::strncmp(line, "norm ", 5) == 0) norm_line(line + 5);
+    else if (std::strncmp(line, "rope ", 5) == 0) rope_line(line + 5);
     else std::printf("error unknown line\n");
   }
   return 0;

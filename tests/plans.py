@@ -35,6 +35,10 @@ def norm(res, dtype, H, T, off=0, rs=None):
     return plans([f"norm {int(res)} {dtype} {H} {T} {off} {H if rs is None else rs}"])[0]
 
 
+def rope(T, Hq, Hkv, D, qk, any_align=False):
+    return plans([f"rope {int(any_align)} {int(qk)} {Hq} {Hkv} {D} {T}"])[0]
+
+
 # Norm calls at the limits of their entries: (dtype, T, H, rows' element offset from a 16-byte boundary,
 # entry with the residual, entry without); BF16 1, FP16 2, FP32 3.
 NORM_LIMITS = [
@@ -53,4 +57,16 @@ NORM_LIMITS = [
     (1, 1354, 333, 1, "edge", "edge_flat"), (2, 357, 1023, 1, "edge_flat", "edge_flat"),
     (1, 88, 4001, 1, "edge_flat", "edge"), (2, 91, 4095, 1, "edge_flat", "edge_flat"),
     (1, 40, 9001, 1, "edge", "edge"), (2, 85, 9007, 1, "edge_flat", "edge_flat"),       # two vectors per thread
+]
+
+# RoPE calls at the limits of their entries: (T, Hq, Hkv, D, q/k norm, entry and block size).
+ROPE_LIMITS = [
+    (38, 32, 8, 128, False, "one_64"), (39, 32, 8, 128, False, "two_64"), (115, 32, 8, 128, False, "two_64"),
+    (116, 32, 8, 128, False, "one_256"), (139, 32, 8, 128, False, "one_128"), (152, 32, 8, 128, False, "one_128"),
+    (153, 32, 8, 128, False, "one_256"), (304, 32, 8, 128, False, "one_256"), (305, 32, 8, 128, False, "two_64"),
+    (575, 32, 8, 128, False, "two_64"), (576, 32, 8, 128, False, "bulk_128"),
+    (57, 32, 8, 128, True, "one_64"), (58, 32, 8, 128, True, "two_64"), (87, 32, 8, 128, True, "two_64"),
+    (88, 32, 8, 128, True, "one_128"), (405, 32, 8, 128, True, "one_128"), (406, 32, 8, 128, True, "two_64"),
+    (347, 16, 4, 64, False, "one_64"), (405, 16, 4, 64, False, "one_64"), (406, 16, 4, 64, False, "one_256"),
+    (511, 5, 1, 128, True, "two_64"), (400, 3, 2, 256, False, "one_256"), (333, 3, 3, 256, True, "one_128"),
 ]

@@ -490,31 +490,44 @@ def test_rope_bad_positions_flag_and_skip(S):
 
 
 @pytest.mark.parametrize("T,Hq,Hkv,D,S_,qk,dtype,layout", [
-    (515, 32, 8, 128, 8192, False, BF16, "fused"),     # Llama heads; the last block holds 3 tokens
+    (577, 32, 8, 128, 8192, False, BF16, "fused"),     # Llama heads
     (1024, 32, 8, 128, 8192, True, FP16, "separate"),  # Qwen3-style q/k norm
-    (601, 4, 2, 64, 1024, True, BF16, "fused"),
-    (512, 8, 8, 256, 600, False, FP16, "separate"),
-    (2050, 16, 1, 128, 4096, False, BF16, "fused")])
+    (2305, 4, 2, 64, 4096, True, BF16, "fused"),       # one item per token: the last block holds one
+    (577, 8, 8, 256, 600, False, FP16, "separate"),
+    (2051, 16, 1, 128, 4096, False, BF16, "fused")])   # two items per token: the last block holds two
 def test_rope_kv_many_tokens(S, T, Hq, Hkv, D, S_, qk, dtype, layout):
-    """Calls of at least 512 tokens: the bulk-copy kernel (a few tokens per block, their rows
-    staged in shared memory, each token's angles computed once), ragged last blocks included."""
+    """Calls of many tokens: the bulk-copy kernel (a warp per item of up to three head-rows per
+    lane group, staged in shared memory, the angles computed once per item), ragged last blocks
+    included."""
+    assert plans.rope(T, Hq, Hkv, D, qk) == "bulk_128"
     ref, got, inp = run_rope(S, T, Hq, Hkv, D, S_, 5e5, qk, dtype=dtype, layout=layout, seed=T + D)
     assert got["status"] == 0 and ref["bad"] == 0
     check_rope(ref, got, inp, dtype)
 
 
 @pytest.mark.parametrize("T,Hq,Hkv,D,qk,dtype", [
-    (38, 32, 8, 128, True, BF16), (39, 32, 8, 128, False, FP16),   # both sides of the one-row limit
     (511, 5, 1, 128, True, BF16), (300, 3, 2, 256, True, FP16),    # head-rows that fill no whole item
     (511, 1, 1, 64, False, BF16), (512, 1, 1, 64, True, FP16),
     (767, 45, 2, 64, True, BF16), (768, 45, 2, 64, False, FP16),   # both sides of the bulk-copy limit
     (777, 13, 1, 256, True, BF16), (1024, 22, 2, 128, True, FP16),
-    (57, 32, 8, 128, True, BF16), (58, 32, 8, 128, True, FP16), (77, 32, 8, 128, True, FP16),  # one row or two
-    (343, 32, 8, 128, True, BF16), (134, 32, 8, 128, False, BF16), (191, 32, 8, 128, False, FP16),
-    (152, 32, 8, 128, False, FP16), (153, 32, 8, 128, False, BF16)])
+    (38, 32, 8, 128, True, BF16), (39, 32, 8, 128, False, FP16), (57, 32, 8, 128, True, BF16),
+    (58, 32, 8, 128, True, FP16), (77, 32, 8, 128, True, FP16), (343, 32, 8, 128, True, BF16),
+    (134, 32, 8, 128, False, BF16), (191, 32, 8, 128, False, FP16), (152, 32, 8, 128, False, FP16),
+    (153, 32, 8, 128, False, BF16), (515, 32, 8, 128, False, BF16), (601, 4, 2, 64, True, BF16),
+    (512, 8, 8, 256, False, FP16)])
 def test_rope_kv_item_edges(S, T, Hq, Hkv, D, qk, dtype):
     """Warp items of one, two and three head-rows per lane group at the limits of their ranges,
     with q, k and v rows meeting inside an item and a last item only partly filled."""
+    ref, got, inp = run_rope(S, T, Hq, Hkv, D, 1024, 5e5, qk, dtype=dtype, layout="fused", seed=T + Hq)
+    assert got["status"] == 0 and ref["bad"] == 0
+    check_rope(ref, got, inp, dtype)
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,D,qk,entry", plans.ROPE_LIMITS)
+def test_rope_kv_entry_limits(S, T, Hq, Hkv, D, qk, entry):
+    """Both sides of each line of the RoPE kernels' rule."""
+    assert plans.rope(T, Hq, Hkv, D, qk) == entry
+    dtype = FP16 if T % 2 else BF16
     ref, got, inp = run_rope(S, T, Hq, Hkv, D, 1024, 5e5, qk, dtype=dtype, layout="fused", seed=T + Hq)
     assert got["status"] == 0 and ref["bad"] == 0
     check_rope(ref, got, inp, dtype)

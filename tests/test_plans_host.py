@@ -9,3 +9,8 @@ from tests import plans
 def test_norm_entries(dtype, T, H, off, res, plain):
     assert plans.norm(True, dtype, H, T, off) == res
     assert plans.norm(False, dtype, H, T, off) == plain
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,D,qk,entry", plans.ROPE_LIMITS)
+def test_rope_entries(T, Hq, Hkv, D, qk, entry):
+    assert plans.rope(T, Hq, Hkv, D, qk) == entry
