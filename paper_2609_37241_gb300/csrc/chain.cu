@@ -9,8 +9,9 @@
 // horizontal fusion where blocks take different roles:
 //   norm     two add+RMSNorm steps, one or two blocks per token (the longest per-block
 //            work)
-//   RoPE     RoPE/KV head-rows, eight warp items per block (RopeGeom): one head-row per lane
-//            group, or up to three of one token on grids several waves long
+//   RoPE     RoPE/KV head-rows, a warp item per warp (RopeGeom), or per few warps of a block on
+//            small grids: one head-row per lane group, or up to three of one token on grids
+//            several waves long
 //   SwiGLU   tiles of one row each, twice as wide on grids of many waves
 // Grids are role-major ([norms | RoPE | SwiGLU], so the longest blocks start first), the
 // smallest ones token-major (chain_block_tok), so that consecutive blocks mix roles. Under
@@ -23,7 +24,6 @@
 #include "device_common.cuh"
 
 namespace trident {
-
 
 // Norm role: part `part` (< SPLIT) of token `row`'s two add+RMSNorm steps.
 template <int DT, int NT, int VPT, int SPLIT>
@@ -135,8 +135,8 @@ __device__ __forceinline__ void chain_norm(const ChainParams& c, const int64_t r
   }
 }
 
-// RoPE role: RoPE block rb (< nB), i.e. the warp items [8 rb, 8 rb + 8) of the call (RopeGeom);
-// fq holds the lane's frequencies. Items of at most one head-row per lane group, or of
+// RoPE role: RoPE block rb (< nB), i.e. the warp items [ipb rb, ipb (rb + 1)) of the call (RopeGeom),
+// ipb = rope_ipb; fq holds the lane's frequencies. Items of at most one head-row per lane group, or of
 // kChainRopeRows on grids several waves long (rope_k), which only the one-CTA-per-token entries
 // (ROWS) carry, so the others keep their registers.
 template <int DT, int D, bool QKNORM, bool ROWS>
@@ -167,8 +167,8 @@ __device__ __forceinline__ void chain_rope_freqs(const ChainParams& c, const boo
   if (is_rope) rope_pair_freqs(c.rope.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
 }
 
-// SwiGLU role: column tile `col_tile` of row `row`, SWU x 256 16-byte vectors of g and of u
-// (kChainSwigluUnroll for one call's grid, kChainStepTileVecs / NT for a whole step's).
+// SwiGLU role: column tile `col_tile` of row `row`, SWU x NT 16-byte vectors of g and of u
+// (kChainTileVecs or kChainWideTileVecs in all for one call's grid, kChainStepTileVecs for a step's).
 template <int DT, int NT, int SWU>
 __device__ __forceinline__ void chain_swiglu(const ChainParams& c, const int64_t row, const int64_t col_tile) {
   swiglu_tile<DT, SWU, NT>(c.sw, row, col_tile * SWU * NT, threadIdx.x);
@@ -369,6 +369,102 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     pdl_wait();
     chain_block<DT, NT, VPT, SPLIT, D, QKNORM, kChainStepTileVecs / NT, true>(c, bl, fq);
   }
+}
+
+// Up to three head-rows per RoPE lane group on grids several waves long: a grid whose
+// one-CTA-per-token form with one head-row per lane group (`one` blocks) exceeds the resident
+// slots. There blocks queue for slots and a RoPE block that moves three rows for the same fixed
+// costs pays; within one wave a block's own latency is the step. Same-box device times of the
+// role as it was (a lane per 16-byte vector, partners exchanged by shuffles, loads behind a
+// branch per row), as it is with two rows and with three: Llama layers of 128 / 256 / 1024 / 8192
+// tokens 5.16 / 8.88 / 29.4 / 221.8, 5.02 / 8.45 / 27.7 / 210.9, 4.99 / 8.30 / 27.1 / 205.4 us
+// (8192 tokens: 6.7 TB/s, 0.99 of the 6.8 TB/s copy rate); 36 layers with q/k norm in one launch
+// at 8 / 32 / 128 tokens 10.7 / 33.7 / 124.8, 10.0 / 31.0 / 116.7, 9.4 / 30.3 / 110.7 us. 80 tokens
+// 5.11 / 3.65, which now fit one wave.
+// With q/k norm, whose rows are the longer, only from one and a quarter waves: 110 / 116 / 122
+// tokens 4.57 / 5.15 / 5.24 us with three rows, 4.28 / 4.88 / 4.82 with one; 128 tokens 5.36 / 4.95.
+int32_t chain_rope_k(int64_t one, int64_t wave, bool qk) {
+  return one > (qk ? wave + wave / 4 : wave) ? kChainRopeRows : 1;
+}
+
+ChainPlan chain_plan(int64_t T, int64_t I, const RopeSplit* rope, int32_t threads, int32_t vec, int64_t wave, int32_t sms,
+                     bool inplace, bool qk, bool pdl) {
+  const int32_t warps = threads / 32;
+  const bool big = threads > kThreads;  // blocks of 512 threads (H 8192)
+  auto tiles = [&](int64_t width) { return T * ((I + width * vec - 1) / (width * vec)); };
+  auto items = [&](int k, int64_t ipb) { return (T * rope[k].ipt + ipb - 1) / ipb; };
+  int64_t nC = tiles(kChainTileVecs);
+  const int64_t one = T + items(0, warps) + nC;  // one norm CTA per token, one head-row per lane group
+  ChainPlan pl{};
+  // Two CTAs per token for the norms -- so no SM carries a whole token's norm traffic -- while the
+  // grid still fits in one wave, and unless an output is written over an input the partner CTA still
+  // reads (in-place calls keep one CTA per token).
+  pl.split = !inplace && T + one <= wave ? 2 : 1;
+  pl.rope_k = pl.split == 1 ? chain_rope_k(one, wave, qk) : 1;
+  bool early = false;  // no late trigger
+  // Wider SwiGLU tiles on grids of more than four waves: same-box probe, one Llama layer at 1024 /
+  // 4096 tokens 34.2 / 122.8 -> 31.3 / 112.6 us; at 256 tokens (3.4 waves) 9.81 -> 9.75 us, at 128
+  // tokens (1.7 waves) 4.72 -> 5.11 us.
+  pl.wide = pl.split == 1 && one > 4 * wave;
+  // With blocks of 512 threads, where a tile is one or two vectors per thread, beyond one wave: with one
+  // head-row per lane group where the wider tiles let the grid fit one wave (44 tokens of I 28672 5.26
+  // -> 4.40 us), with q/k norm up to 1.7 waves (50 / 62 / 80 tokens 5.27 / 5.53 / 6.25 -> 4.71 / 5.11 /
+  // 5.96 us; three rows 6.10 / 5.59 / 5.97, which at 100 tokens take 6.66, one row 7.01); three rows
+  // beyond that (without the norm 66 / 80 / 128 tokens 5.23 / 6.02 / 8.80 -> 5.03 / 5.58 / 7.78). (With
+  // 256 threads, 100 and 110 tokens at H 4096, 4.14 / 4.35 -> 4.46 / 4.74.) Past one wave the late
+  // trigger loses (50 tokens with q/k norm 4.71 / 4.59, 54 4.85 / 4.98, 62 5.11 / 5.38).
+  if (pl.split == 1 && !pl.wide && big && one > wave) {
+    const int64_t rest = T + tiles(kChainWideTileVecs);
+    const int64_t w1 = rest + items(0, warps);
+    pl.wide = true;
+    pl.rope_k = w1 <= wave || (qk && 10 * w1 <= 17 * wave) ? 1 : kChainRopeRows;
+    early = rest + items(pl.rope_k > 1, warps) > wave;
+  }
+  if (pl.wide) nC = tiles(kChainWideTileVecs);
+  const int64_t nA = T * pl.split;
+  const int k = pl.rope_k > 1;
+  pl.ipb = warps;
+  // Few blocks: a RoPE block takes four or eight items (a quarter or half of its warps) while the grid
+  // still leaves an SM to every block, or with blocks of 256 threads a quarter of the SMs idle; a warp's
+  // angles are issue-bound, and the warps of fewer items per SM finish sooner. With q/k norm, where a
+  // lane's norm is added to its angles, and two norm CTAs per token up to 1.6 blocks per SM, or in blocks of 512 threads eight items up to two if the late trigger below still applies (without
+  // the norm 18 tokens 1.86 / 1.91). H 8192 at 2 / 4 / 10 tokens with q/k norm 2.42 / 2.44 / 2.78 -> 2.22 /
+  // 2.24 / 2.56 us, 16 / 18 / 20 2.67 / 2.70 / 2.70 -> 2.52 / 2.55 / 2.58 (28 of I 22016, too many for the
+  // late trigger, 2.84 / 3.58); H 4096 at 10 tokens 1.85 -> 1.82, with q/k norm 17 / 24 / 30 2.00 / 2.04 /
+  // 2.18 -> 1.91 / 1.99 / 2.14, 32 2.18 / 2.26.
+  for (int32_t ipb = 4; ipb < warps; ipb *= 2) {
+    const int64_t blocks = nA + items(k, ipb) + nC;
+    const bool more = qk && pl.split == 2 &&
+                      (big ? ipb == 8 && blocks <= 2 * (int64_t)sms && blocks + nA <= wave + wave / 8
+                           : 5 * blocks <= 8 * (int64_t)sms);
+    if (blocks <= (big ? sms : sms * 3 / 4) || more) {
+      pl.ipb = ipb;
+      break;
+    }
+  }
+  pl.blocks = nA + items(k, pl.ipb) + nC;
+  // Under PDL, a role-major grid of more than a quarter block per SM whose blocks, with
+  // its own norm blocks, fit the resident slots give or take an eighth of them launches a
+  // late entry (fn_late, fn_inplace_late): its RoPE and SwiGLU blocks trigger the next launch
+  // at their exit, so the next grid is placed whole while this one's norm blocks finish, one
+  // norm block per SM instead of up to four. Same-box A/B of Llama layer steps against the
+  // grids below: 6 tokens 2.22 -> 2.12 us, 16 tokens 2.58 -> 2.29, 32 tokens 2.98 -> 2.57, 56
+  // tokens 3.31 -> 3.19; with one norm CTA per token 90 tokens 5.10 -> 3.80, 100 tokens 5.24 ->
+  // 4.08, H 8192 at 37 tokens 4.86 -> 3.70. Equal at 2 and 4 tokens and at 1 token 1.5-2 %
+  // slower (nothing to place, and the next launch starts later), hence the lower bound; a few
+  // dozen blocks placed late cost less than stacked norm blocks, but with 96 blocks placed
+  // late the probe measured 3.51 -> 3.69 us, hence the upper bound; with one norm CTA per
+  // token, whose grids hold half the norm blocks, a quarter of the slots (H 8192 56 tokens 4.92 ->
+  // 4.18 us, 110 tokens with q/k norm 4.57 -> 4.32).
+  // Otherwise a token-major grid (chain_block_tok) for grids of at most two blocks per SM
+  // with one head-row per RoPE lane group: consecutive blocks then mix roles, so the blocks
+  // that land together on one SM are not all norm blocks (measured against role-major grids
+  // without the late trigger: 16 tokens 3.55 -> 2.85 us per layer step, 1 token 2.20 -> 2.04
+  // us). Larger grids are role-major, which starts the longest (norm) blocks first.
+  const int64_t q = threads / kThreads;  // the bounds below count blocks of 256 threads
+  pl.late = pdl && !early && 4 * q * pl.blocks > sms && pl.blocks + nA <= wave + (pl.split == 1 ? 2 : 1) * wave / 8;
+  pl.tok = !pl.late && pl.rope_k == 1 && T >= 1 && T <= 65535 && !pl.wide && q * pl.blocks <= 2 * (int64_t)sms;
+  return pl;
 }
 
 template <int DT, bool QK, int NT, int VPT>

@@ -214,17 +214,6 @@ bool chain_kernel(int32_t dtype, int64_t H, int32_t D, bool qknorm, KernelEntry*
 // The entry a call takes from its packed params (sets p->nvec), its block size and grid.
 NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, int32_t* threads, int64_t* blocks,
                     int32_t* smem, int32_t sms);
-const void* empty_kernel_entry();  // the latency-floor probe's kernel (does nothing)
-
-// Validation, guard-equivalent checks (sizes, layouts, 16-byte alignment, overlap) and
-// parameter packing of a ROPE_KV / QKNORM_ROPE_KV argument tuple without an SCM. Leaves
-// p->cs and p->err NULL. Returns a trident_status (message in trident_scm_last_error).
-int32_t prepare_rope_args(const void* trident_args_ptr, RopeParams* p, int32_t* dtype,
-                          bool* qknorm);
-
-// Sets the thread-local last-error message and returns `status`.
-int32_t internal_fail(int32_t status, const char* msg);
-
 // Round-up multiplier and shift for dividing 32-bit unsigned integers by d (1 <= d < 2^31):
 // l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1; the kernels take the quotient as
 // (h + ((n - h) >> 1)) >> (l - 1) with h = umulhi(n, m) (fast_div; Granlund and Montgomery,
@@ -257,6 +246,28 @@ inline RopeSplit rope_split(int64_t NH, int64_t gw, int32_t max_rows) {
   div_magic((uint32_t)r.ipt, &r.magic, &r.shift);
   return r;
 }
+
+// A single chain call's launch: norm CTAs per token, RoPE head-rows per lane group at most and items
+// per block, SwiGLU tile width, launch trigger and block order. rope: the call's item splits with one
+// and with kChainRopeRows rows; wave: blocks resident at once.
+struct ChainPlan {
+  int32_t split, rope_k, ipb;
+  bool wide, late, tok;
+  int64_t blocks;  // role-major grid
+};
+ChainPlan chain_plan(int64_t T, int64_t I, const RopeSplit* rope, int32_t threads, int32_t vec, int64_t wave, int32_t sms,
+                     bool inplace, bool qk, bool pdl);
+int32_t chain_rope_k(int64_t one, int64_t wave, bool qk);
+const void* empty_kernel_entry();  // the latency-floor probe's kernel (does nothing)
+
+// Validation, guard-equivalent checks (sizes, layouts, 16-byte alignment, overlap) and
+// parameter packing of a ROPE_KV / QKNORM_ROPE_KV argument tuple without an SCM. Leaves
+// p->cs and p->err NULL. Returns a trident_status (message in trident_scm_last_error).
+int32_t prepare_rope_args(const void* trident_args_ptr, RopeParams* p, int32_t* dtype,
+                          bool* qknorm);
+
+// Sets the thread-local last-error message and returns `status`.
+int32_t internal_fail(int32_t status, const char* msg);
 
 // Which vector RoPE entry a call of T tokens takes, and its launch shape. The splits depend
 // only on the version's head counts and head size (rope_plans, at registration).

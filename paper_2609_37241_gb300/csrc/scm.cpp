@@ -737,33 +737,14 @@ bool chain_inplace(const trident_args* a) {
          t[C_R2].data == t[C_R0].data || t[C_X2].data == t[C_AO].data;
 }
 
-// Sets the norm CTAs per token (split) and the RoPE head-rows per lane group (rope_k), and
-// with them nA, nB and the grid's block count.
-int32_t set_chain_split(const Version& v, ChainParams* c, int64_t T, int32_t split, int32_t rope_k,
-                        int64_t* blocks) {
+// Sets the norm CTAs per token (split), the RoPE head-rows per lane group (rope_k) and items per
+// block (ipb), and with them nA and nB; returns the grid's block count.
+int64_t set_chain_split(const Version& v, ChainParams* c, int64_t T, int32_t split, int32_t rope_k, int32_t ipb) {
   c->a_split = split;
   c->nA = (int32_t)(T * split);
   c->rope_k = rope_k;
-  c->nB = (int32_t)chain_rope_blocks(c, T, v.rope_split[rope_k > 1], v.ke.threads / 32);
-  *blocks = (int64_t)c->nA + c->nB + c->nC;
-  return TRIDENT_OK;
-}
-
-// Up to three head-rows per RoPE lane group on grids several waves long: a grid whose
-// one-CTA-per-token form with one head-row per lane group (`one` blocks) exceeds the resident
-// slots. There blocks queue for slots and a RoPE block that moves three rows for the same fixed
-// costs pays; within one wave a block's own latency is the step. Same-box device times of the
-// role as it was (a lane per 16-byte vector, partners exchanged by shuffles, loads behind a
-// branch per row), as it is with two rows and with three: Llama layers of 128 / 256 / 1024 / 8192
-// tokens 5.16 / 8.88 / 29.4 / 221.8, 5.02 / 8.45 / 27.7 / 210.9, 4.99 / 8.30 / 27.1 / 205.4 us
-// (8192 tokens: 6.7 TB/s, 0.99 of the 6.8 TB/s copy rate); 36 layers with q/k norm in one launch
-// at 8 / 32 / 128 tokens 10.7 / 33.7 / 124.8, 10.0 / 31.0 / 116.7, 9.4 / 30.3 / 110.7 us. Within
-// one wave the two forms are level (16 tokens 2.27 / 2.25 us, 64 tokens 3.32 / 3.32, with q/k
-// norm 2.29 / 2.30 and 62 tokens 3.32 / 3.19); 80 tokens 5.11 / 3.65, which now fit one wave.
-// With q/k norm, whose rows are the longer, only from one and a quarter waves: 110 / 116 / 122
-// tokens 4.57 / 5.15 / 5.24 us with three rows, 4.28 / 4.88 / 4.82 with one; 128 tokens 5.36 / 4.95.
-inline int32_t chain_rope_k(int64_t one, int64_t wave_blocks, bool qknorm) {
-  return one > (qknorm ? wave_blocks + wave_blocks / 4 : wave_blocks) ? kChainRopeRows : 1;
+  c->nB = (int32_t)chain_rope_blocks(c, T, v.rope_split[rope_k > 1], ipb);
+  return (int64_t)c->nA + c->nB + c->nC;
 }
 
 // Layer-chain prefetch before the PDL wait: every block's first lines for grids of at most
@@ -860,75 +841,18 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
       cfg.blockDimX = (unsigned)v.ke.threads;
       int32_t st = pack_chain(scm, v, a, s, kChainTileVecs, &c);
       if (st != TRIDENT_OK) return st;
-      // Two CTAs per token for the norms -- so no SM carries a whole token's norm traffic --
-      // while the grid still fits in one wave, and unless an output is written over an
-      // input the partner CTA still reads (in-place calls keep one CTA per token).
-      const int32_t split = (!chain_inplace(a) && 2 * s.T + c.nB + c.nC <= v.wave_blocks) ? 2 : 1;
-      const int64_t one = s.T + c.nB + c.nC;  // one CTA per token, one head-row per lane group
-      const bool qk = op == TRIDENT_OP_LAYER_CHAIN_QKNORM;
-      int32_t rope_k = split == 1 ? chain_rope_k(one, v.wave_blocks, qk) : 1;
-      // Wider SwiGLU tiles (fn_wide) on grids of more than four waves: same-box probe, one
-      // Llama layer at 1024 / 4096 tokens 34.2 / 122.8 -> 31.3 / 112.6 us; at 256 tokens
-      // (3.4 waves) 9.81 -> 9.75 us, at 128 tokens (1.7 waves) 4.72 -> 5.11 us. With blocks of
-      // 512 threads (H 8192), where a tile is one or two vectors per thread, also where the
-      // wider tiles let the grid fit one wave: 44 tokens of I 28672 5.26 -> 4.40 us, 50 of I 22016
-      // 4.65 -> 4.04 (with 256 threads, 100 and 110 tokens at H 4096, 4.14 / 4.35 -> 4.46 / 4.74).
-      wide = split == 1 && one > 4 * (int64_t)v.wave_blocks;
-      if (split == 1 && !wide && one > v.wave_blocks && v.ke.threads > kThreads) {
-        const int64_t per = (int64_t)kChainWideTileVecs * v.ke.vec, tw = (c.sw.I + per - 1) / per;
-        const int64_t rest = s.T + s.T * tw, warps = v.ke.threads / 32;
-        for (int k = 0; k < 2 && !wide; ++k) {  // with one head-row per lane group if that fits
-          if (rest + (s.T * v.rope_split[k].ipt + warps - 1) / warps <= v.wave_blocks) {
-            wide = true;
-            rope_k = k ? kChainRopeRows : 1;
-          }
-        }
-      }
+      const ChainPlan pl = chain_plan(s.T, c.sw.I, v.rope_split, v.ke.threads, v.ke.vec, v.wave_blocks, scm->sm_count,
+                                      chain_inplace(a), op == TRIDENT_OP_LAYER_CHAIN_QKNORM,
+                                      (scm->opt.flags & TRIDENT_OPT_PDL) != 0);
+      wide = pl.wide;
+      late = pl.late;
       if (wide) set_chain_tiles(&c, s.T, kChainWideTileVecs, v.ke.vec);
-      int64_t blocks = 0;
-      st = set_chain_split(v, &c, s.T, split, rope_k, &blocks);
-      if (st != TRIDENT_OK) return st;
-      // Few blocks: a RoPE block takes four or eight items (a quarter or half of its warps) while
-      // the grid still leaves an SM to every block, or with blocks of 256 threads a quarter of
-      // the SMs idle; a warp's angles are issue-bound, and the warps of fewer items per SM finish
-      // sooner. H 8192 at 2 / 4 / 10 tokens with q/k norm 2.42 / 2.44 / 2.78 -> 2.22 / 2.24 / 2.56
-      // us, H 4096 at 10 tokens 1.85 -> 1.82 (with 144 blocks, 16 tokens, 2.23 -> 2.44).
-      const int64_t spread = v.ke.threads > kThreads ? scm->sm_count : scm->sm_count * 3 / 4;
-      for (int32_t ipb = 4; ipb < v.ke.threads / 32; ipb *= 2) {
-        const int64_t nb = (s.T * c.rope.ipt + ipb - 1) / ipb;
-        if (c.nA + nb + c.nC <= spread) {
-          c.nB = (int32_t)chain_rope_blocks(&c, s.T, v.rope_split[rope_k > 1], ipb);
-          blocks = (int64_t)c.nA + c.nB + c.nC;
-          break;
-        }
-      }
-      cfg.gridDimX = (unsigned)blocks;
-      // Under PDL, a role-major grid of more than a quarter block per SM whose blocks, with
-      // its own norm blocks, fit the resident slots give or take an eighth of them launches a
-      // late entry (fn_late, fn_inplace_late): its RoPE and SwiGLU blocks trigger the next launch
-      // at their exit, so the next grid is placed whole while this one's norm blocks finish, one
-      // norm block per SM instead of up to four. Same-box A/B of Llama layer steps against the
-      // grids below: 6 tokens 2.22 -> 2.12 us, 16 tokens 2.58 -> 2.29, 32 tokens 2.98 -> 2.57, 56
-      // tokens 3.31 -> 3.19; with one norm CTA per token 90 tokens 5.10 -> 3.80, 100 tokens 5.24 ->
-      // 4.08, H 8192 at 37 tokens 4.86 -> 3.70. Equal at 2 and 4 tokens and at 1 token 1.5-2 %
-      // slower (nothing to place, and the next launch starts later), hence the lower bound; a few
-      // dozen blocks placed late cost less than stacked norm blocks, but with 96 blocks placed
-      // late the probe measured 3.51 -> 3.69 us, hence the upper bound; with one norm CTA per
-      // token, whose grids hold half the norm blocks, a quarter of the slots (H 8192 56 tokens 4.92 ->
-      // 4.18 us, 110 tokens with q/k norm 4.57 -> 4.32).
-      // Otherwise a token-major grid (chain_block_tok) for grids of at most two blocks per SM
-      // with one head-row per RoPE lane group: consecutive blocks then mix roles, so the blocks
-      // that land together on one SM are not all norm blocks (measured against role-major grids
-      // without the late trigger: 16 tokens 3.55 -> 2.85 us per layer step, 1 token 2.20 -> 2.04
-      // us). Larger grids are role-major, which starts the longest (norm) blocks first.
-      const int64_t q = v.ke.threads / kThreads;  // the bounds below count blocks of 256 threads
-      if ((scm->opt.flags & TRIDENT_OPT_PDL) && 4 * q * blocks > scm->sm_count &&
-          blocks + c.nA <= v.wave_blocks + (split == 1 ? 2 : 1) * v.wave_blocks / 8) {
-        late = true;
-      } else if (rope_k == 1 && s.T >= 1 && s.T <= 65535 && !wide && q * blocks <= 2 * scm->sm_count) {
+      set_chain_split(v, &c, s.T, pl.split, pl.rope_k, pl.ipb);
+      cfg.gridDimX = (unsigned)pl.blocks;
+      if (pl.tok) {
         c.tok_grid = 1;
         c.rope_per_tok = (c.rope.ipt + c.rope_ipb - 1) / c.rope_ipb;
-        cfg.gridDimX = (unsigned)(split + c.rope_per_tok + c.sw_tiles_per_row);
+        cfg.gridDimX = (unsigned)(pl.split + c.rope_per_tok + c.sw_tiles_per_row);
         cfg.gridDimY = (unsigned)s.T;
       }
       break;
@@ -1761,8 +1685,8 @@ int32_t step_chunk(trident_scm* scm, const trident_args* a, int32_t m, void* str
     const int32_t rope_k = split == 1 ? chain_rope_k(one, v0->step_wave_blocks, a[0].op == TRIDENT_OP_LAYER_CHAIN_QKNORM) : 1;
     int64_t first = 0;
     for (int32_t i = 0; i < m; ++i) {
-      int64_t blocks = 0;
-      set_chain_split(scm->versions[sel[i]], &P.c[i], sig[i].T, split, rope_k, &blocks);
+      const int64_t blocks = set_chain_split(scm->versions[sel[i]], &P.c[i], sig[i].T, split, rope_k,
+                                             v0->ke.threads / 32);
       P.first[i] = (int32_t)first;
       first += blocks;
       if (first > 0x7fffffff)

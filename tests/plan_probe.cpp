@@ -2,6 +2,8 @@
 // line, without a GPU: it is linked with the library's own objects and calls the rules that the host
 // core calls. Lines (152 SMs):
 //   norm RES DTYPE H T OFF RS    RES 0/1, rows at element offset OFF of a 16-byte boundary, row stride RS
+//   chain QK H HQ HKV I T INPLACE PDL    norm CTAs per token, SwiGLU tiles, launch trigger, block order;
+//                                        head-rows per RoPE lane group and items per RoPE block
 //   rope ANY QK HQ HKV D T       ANY 1: a version of any alignment; QK 1: with q/k norm
 #include <cinttypes>
 #include <cstdio>
@@ -76,11 +78,30 @@ static void rope_line(const char* s) {
   std::printf("%s_%d\n", e == ROPE_MID ? "two" : e == ROPE_BULK ? "bulk" : "one", threads);
 }
 
+static void chain_line(const char* s) {
+  int qk, Hq, Hkv, inplace, pdl;
+  int64_t H, I, T;
+  if (std::sscanf(s, "%d %" SCNd64 " %d %d %" SCNd64 " %" SCNd64 " %d %d", &qk, &H, &Hq, &Hkv, &I, &T, &inplace, &pdl) != 8)
+    return;
+  KernelEntry ke;
+  const char* why = "";
+  if (!chain_kernel(DT_BF16, H, 128, qk != 0, &ke, &why)) {
+    std::printf("error %s\n", why);
+    return;
+  }
+  const RopeSplit split[2] = {rope_split(Hq + 2 * Hkv, 4, 1), rope_split(Hq + 2 * Hkv, 4, kChainRopeRows)};
+  const int64_t wave = (int64_t)kSms * (1024 / ke.threads);  // the kernels' launch bounds
+  const ChainPlan p = chain_plan(T, I, split, ke.threads, ke.vec, wave, kSms, inplace != 0, qk != 0, pdl != 0);
+  std::printf("%s%s%s rows%d ipb%d\n", p.split == 2 ? "two" : p.wide ? "wide" : "one", p.late ? "_late" : "",
+              p.tok ? "_tok" : "", p.rope_k, p.ipb);
+}
+
 int main() {
   char line[256];
   while (std::fgets(line, sizeof line, stdin)) {
     if (std::strncmp(line, "norm ", 5) == 0) norm_line(line + 5);
     else if (std::strncmp(line, "rope ", 5) == 0) rope_line(line + 5);
+    else if (std::strncmp(line, "chain ", 6) == 0) chain_line(line + 6);
     else std::printf("error unknown line\n");
   }
   return 0;

@@ -39,6 +39,10 @@ def rope(T, Hq, Hkv, D, qk, any_align=False):
     return plans([f"rope {int(any_align)} {int(qk)} {Hq} {Hkv} {D} {T}"])[0]
 
 
+def chain(qk, H, Hq, I, T, pdl=True, inplace=False, Hkv=8):
+    return plans([f"chain {int(qk)} {H} {Hq} {Hkv} {I} {T} {int(inplace)} {int(pdl)}"])[0]
+
+
 # Norm calls at the limits of their entries: (dtype, T, H, rows' element offset from a 16-byte boundary,
 # entry with the residual, entry without); BF16 1, FP16 2, FP32 3.
 NORM_LIMITS = [
@@ -69,4 +73,31 @@ ROPE_LIMITS = [
     (88, 32, 8, 128, True, "one_128"), (405, 32, 8, 128, True, "one_128"), (406, 32, 8, 128, True, "two_64"),
     (347, 16, 4, 64, False, "one_64"), (405, 16, 4, 64, False, "one_64"), (406, 16, 4, 64, False, "one_256"),
     (511, 5, 1, 128, True, "two_64"), (400, 3, 2, 256, False, "one_256"), (333, 3, 3, 256, True, "one_128"),
+]
+
+# Layer-chain calls at the limits of their entries: (H, q heads, I, q/k norm, T, PDL, in place, plan);
+# 8 k/v heads of D 128. The plan: norm CTAs per token (two, one, or one with wide SwiGLU tiles), late
+# trigger, token-major order; head-rows per RoPE lane group, items per RoPE block.
+CHAIN_LIMITS = [
+    (4096, 32, 14336, False, 4, True, False, "two_tok rows1 ipb4"), (4096, 32, 14336, False, 5, True, False, "two_late rows1 ipb4"),
+    (4096, 32, 14336, False, 13, True, False, "two_late rows1 ipb8"), (4096, 32, 14336, False, 72, True, False, "two_late rows1 ipb8"),
+    (4096, 32, 14336, False, 73, True, False, "two rows1 ipb8"), (4096, 32, 14336, False, 81, True, False, "two rows1 ipb8"),
+    (4096, 32, 14336, False, 82, True, False, "one_late rows1 ipb8"), (4096, 32, 14336, False, 94, True, False, "one_late rows3 ipb8"),
+    (4096, 32, 14336, False, 116, True, False, "one_late rows3 ipb8"), (4096, 32, 14336, False, 117, True, False, "one rows3 ipb8"),
+    (4096, 32, 14336, False, 40, False, False, "two_tok rows1 ipb8"), (4096, 32, 14336, False, 41, False, False, "two rows1 ipb8"),
+    (4096, 32, 14336, False, 82, False, False, "one rows1 ipb8"),
+    (4096, 32, 12288, True, 30, True, False, "two_late rows1 ipb4"), (4096, 32, 12288, True, 31, True, False, "two_late rows1 ipb8"),
+    (4096, 32, 12288, True, 100, True, False, "one_late rows1 ipb8"), (4096, 32, 12288, True, 117, True, False, "one rows1 ipb8"),
+    (4096, 32, 12288, True, 139, True, False, "one rows3 ipb8"),
+    (8192, 64, 28672, False, 1, True, False, "two_tok rows1 ipb4"), (8192, 64, 28672, False, 10, True, False, "two_late rows1 ipb4"),
+    (8192, 64, 28672, False, 11, True, False, "two_late rows1 ipb8"), (8192, 64, 28672, False, 28, True, False, "two rows1 ipb16"),
+    (8192, 64, 28672, False, 31, True, False, "one_late rows1 ipb16"), (8192, 64, 28672, False, 33, True, False, "wide_late rows1 ipb16"),
+    (8192, 64, 28672, False, 49, True, False, "wide_late rows3 ipb16"), (8192, 64, 28672, False, 56, True, False, "wide rows3 ipb16"),
+    (8192, 64, 28672, True, 25, True, False, "two_late rows1 ipb8"), (8192, 64, 28672, True, 26, True, False, "two_late rows1 ipb16"),
+    (8192, 64, 28672, True, 48, True, False, "wide_late rows1 ipb16"), (8192, 64, 28672, True, 49, True, False, "wide rows1 ipb16"),
+    (8192, 64, 28672, True, 83, True, False, "wide rows3 ipb16"),
+    (4096, 32, 14336, False, 4, True, True, "one_tok rows1 ipb4"), (4096, 32, 14336, False, 14, True, True, "one_late rows1 ipb4"),
+    (4096, 32, 14336, False, 100, True, True, "one_late rows3 ipb8"), (4096, 32, 14336, False, 130, True, True, "one rows3 ipb8"),
+    (8192, 64, 22016, True, 12, True, True, "one_late rows1 ipb4"), (8192, 64, 22016, True, 50, True, True, "wide_late rows1 ipb16"),
+    (8192, 64, 22016, True, 60, True, True, "wide rows1 ipb16"), (8192, 64, 22016, True, 100, True, True, "wide rows3 ipb16"),
 ]

@@ -44,8 +44,8 @@ ADDNORM_CASES = [
     (BF16, 4096, 13, "strided", 0, "row-strided views"),
     (BF16, 4096, 21, "rank3", 0, "[3, 7, H] flattened"),
     (BF16, 8192, 19, "contig", 0, "register row, H 8192"),
-    (BF16, 8192, 1500, "contig", 0, "H 8192 persistent grid: several rows per block"),
-    (FP16, 8192, 700, "strided", 0, "fp16 H 8192 persistent, row-strided"),
+    (BF16, 8192, 1500, "contig", 0, "H 8192, bulk copies"),
+    (FP16, 8192, 700, "strided", 0, "fp16 H 8192, four vectors per thread, row-strided"),
     (BF16, 2048, 5, "contig", 0, "register row, H 2048"),
     (BF16, 1000, 5, "contig", 0, "two-pass vector loop, ragged H"),
     (BF16, 100, 6, "contig", 0, "H*2 not a multiple of 16: generic"),
@@ -648,7 +648,9 @@ def chain_device(inp, dtype, qknorm, layout="fused"):
 
 def check_chain(ref, out, inp, dtype=BF16):
     hb = lambda n: P.host_bits(out[n], dtype)
-    assert np.array_equal(hb("r1"), ref["r1"]) and np.array_equal(hb("r2"), ref["r2"])
+    assert np.array_equal(hb("r2"), ref["r2"])
+    if out["r1"] is not None:  # in place, r2 has taken its place
+        assert np.array_equal(hb("r1"), ref["r1"])
     P.check_act(hb("x1"), ref["x1_ref"], ref["x1"], dtype, "x1", exact_frac=0.99)
     P.check_act(hb("x2"), ref["x2_ref"], ref["x2"], dtype, "x2", exact_frac=0.99)
     P.check_act(hb("q"), ref["q_ref"], ref["q"], dtype, "q", exact_frac=0.99)
@@ -665,15 +667,10 @@ def check_chain(ref, out, inp, dtype=BF16):
 @pytest.mark.parametrize("pdl", [False, True], ids=["plain", "pdl"])
 @pytest.mark.parametrize("cfg_name,T", [("LLAMA", 1), ("LLAMA", 4), ("LLAMA", 16), ("LLAMA", 64),
                                         ("QWEN3", 1), ("QWEN3", 8), ("QWEN3", 32), ("QWEN3", 128),
-                                        # without PDL, either side of the token-major /
-                                        # role-major boundary (two blocks per SM: 33 Llama
-                                        # tokens are 297 blocks, 34 are 306) and of the one-wave
-                                        # limit of two norm CTAs; under PDL 16, 33, 34 Llama and
-                                        # 8, 32, 40 Qwen3 tokens take the late-trigger entry,
-                                        # 1 and 4 the token-major grid, 64 and 67 neither
                                         ("LLAMA", 33), ("LLAMA", 34), ("LLAMA", 67), ("QWEN3", 40)])
 def test_layer_chain_fused_matches_oracle(S, cfg_name, T, pdl):
-    """The benchmarked layer configurations, with and without programmatic dependent launch
+    """The benchmarked layer configurations, with and without programmatic dependent launch (the
+    limits of the entries: test_layer_chain_entry_limits)
     (with it, as bench.py launches: token-major grids prefetch every block's lines, larger ones
     the norm blocks' rows and their tokens' RoPE head-rows, before the wait)."""
     cfg = getattr(synth, cfg_name)
@@ -693,9 +690,30 @@ def test_layer_chain_fused_matches_oracle(S, cfg_name, T, pdl):
     check_chain(ref, out, inp)
 
 
+@pytest.mark.parametrize("H,Hq,I,qk,T,pdl,inplace,plan", plans.CHAIN_LIMITS)
+def test_layer_chain_entry_limits(S, H, Hq, I, qk, T, pdl, inplace, plan):
+    """Both sides of each line of the layer chain's rule, every entry of it reached."""
+    assert plans.chain(qk, H, Hq, I, T, pdl, inplace) == plan
+    cfg = dict(H=H, Hq=Hq, Hkv=8, D=128, S=1024, I=I, theta=1e6, qknorm=qk, eps=1e-6)
+    dtype = FP16 if T % 2 else BF16
+    inp = synth.layer_inputs(np.random.default_rng(H + T), T, cfg, dtype=dtype)
+    ref = L.layer_chain(inp, cfg["theta"], cfg["eps"], dtype, qknorm=qk)
+    op = S.OP_LAYER_CHAIN_QKNORM if qk else S.OP_LAYER_CHAIN
+    s = one_version_scm(S, S.make_spec(op, dtype, [H, Hq, 8, 128, 1024, I], 1, 4096, layout=S.LAYOUT_ANY,
+                                       rope_theta=cfg["theta"]), flags=S.OPT_PDL if pdl else 0)
+    ts, out = chain_device(inp, dtype, qk, layout="separate" if inplace else "fused")
+    if inplace:  # x1 = h, r1 = r0, x2 = attn_out, r2 = r1, o = g
+        ts[3], ts[4], ts[13], ts[14], ts[17] = ts[0], ts[1], ts[11], ts[1], ts[15]
+        out.update(x1=ts[0], r1=None, x2=ts[11], r2=ts[1], o=ts[15])
+    invoke_ok(s, S, S.make_args(op, ts, eps=cfg["eps"], rope_theta=cfg["theta"]))
+    assert S.trident_scm_device_status(s.h, stream()) == (S.OK, 0)
+    s.close()
+    check_chain(ref, out, inp, dtype)
+
+
 def test_layer_chain_largest_bucket(S):
     """The largest token count the benchmark's chain versions accept (4096 Llama tokens: a grid
-    of 16,384 blocks several waves long -- one CTA per token for the norms, three head-rows per
+    several waves long -- one CTA per token for the norms, three head-rows per
     RoPE lane group, SwiGLU tiles of 4 x 256 vectors -- with the norm-row prefetch under PDL),
     every output against the oracle."""
     cfg = synth.LLAMA
@@ -716,11 +734,11 @@ def test_layer_chain_largest_bucket(S):
 
 @pytest.mark.parametrize("dtype,H,Hq,I,T,qk", [
     (FP16, 4096, 32, 14336, 4, False),     # fp16 chain
-    (BF16, 8192, 64, 28672, 3, False),     # H 8192 instantiation (4 vectors per thread)
+    (BF16, 8192, 64, 28672, 3, False),     # H 8192 instantiation (512 threads)
     (BF16, 8192, 64, 28672, 200, True),    # H 8192, grid beyond one wave: one block per token
     (FP16, 8192, 64, 28672, 5, True),
-    # several waves with 36 head-rows per token: three-row RoPE lane groups whose rows belong
-    # to two tokens (the H 8192 case above covers it with q/k norm, 80 head-rows per token)
+    # several waves with 36 head-rows per token: nine lane groups' rows, three items of three each
+    # (the H 8192 case above: 80 head-rows per token, with q/k norm)
     (BF16, 4096, 20, 14336, 300, False),
 ])
 @pytest.mark.parametrize("pdl", [False, True], ids=["plain", "pdl"])  # PDL: token-major / late trigger

@@ -14,3 +14,8 @@ def test_norm_entries(dtype, T, H, off, res, plain):
 @pytest.mark.parametrize("T,Hq,Hkv,D,qk,entry", plans.ROPE_LIMITS)
 def test_rope_entries(T, Hq, Hkv, D, qk, entry):
     assert plans.rope(T, Hq, Hkv, D, qk) == entry
+
+
+def test_chain_entries():
+    got = [plans.chain(qk, H, Hq, I, T, pdl, inplace) for H, Hq, I, qk, T, pdl, inplace, _ in plans.CHAIN_LIMITS]
+    assert got == [c[-1] for c in plans.CHAIN_LIMITS]
