@@ -137,6 +137,9 @@ constexpr int kStepMax = 48;
 // takes the wider tiles too: blocks queue for slots there, and a tile that moves twice the bytes
 // for the same fixed costs pays.
 constexpr int kChainRopeRows = 3;
+// RoPE items per block of small whole-step grids (blocks of 256 and of 512 threads).
+constexpr int kChainStepItems = 3;
+constexpr int kChainStepItemsWide = 4;
 constexpr int kChainTileVecs = 512;
 constexpr int kChainStepTileVecs = 1024;
 constexpr int kChainWideTileVecs = 1024;

@@ -1683,10 +1683,21 @@ int32_t step_chunk(trident_scm* scm, const trident_args* a, int32_t m, void* str
     }
     const int32_t split = (!inplace && two <= v0->step_wave_blocks) ? 2 : 1;
     const int32_t rope_k = split == 1 ? chain_rope_k(one, v0->step_wave_blocks, a[0].op == TRIDENT_OP_LAYER_CHAIN_QKNORM) : 1;
+    // Fewer RoPE items per block (kChainStepItems) while the grid with them is of more than 1.2 blocks
+    // per SM and still fits one wave: 36 layers with q/k norm at 1 / 2 tokens 3.45 / 3.70 -> 2.99 / 3.39
+    // us, 12 at 3 / 6 3.31 / 3.68 -> 2.92 / 3.46, 8 at 8 3.63 -> 3.45; smaller grids lose (4 layers of 4
+    // tokens without the norm 2.74 / 3.03).
+    int32_t ipb = v0->ke.threads / 32;
+    if (split == 2) {
+      const int32_t few = ipb > 8 ? kChainStepItemsWide : kChainStepItems;
+      int64_t spread = 0;
+      for (int32_t i = 0; i < m; ++i)
+        spread += (int64_t)2 * sig[i].T + (sig[i].T * P.c[i].rope.ipt + few - 1) / few + P.c[i].nC;
+      if (5 * spread > 6 * (int64_t)scm->sm_count && spread <= v0->step_wave_blocks) ipb = few;
+    }
     int64_t first = 0;
     for (int32_t i = 0; i < m; ++i) {
-      const int64_t blocks = set_chain_split(scm->versions[sel[i]], &P.c[i], sig[i].T, split, rope_k,
-                                             v0->ke.threads / 32);
+      const int64_t blocks = set_chain_split(scm->versions[sel[i]], &P.c[i], sig[i].T, split, rope_k, ipb);
       P.first[i] = (int32_t)first;
       first += blocks;
       if (first > 0x7fffffff)

@@ -82,6 +82,22 @@ def test_step_llama_layers_both_splits(S, T):
         check_chain(L.layer_chain(inp, cfg["theta"], cfg["eps"], BF16), out, inp)
 
 
+@pytest.mark.parametrize("H,qk,dtype,layers,T", [
+    (8192, False, BF16, 8, 1), (8192, True, FP16, 8, 3), (8192, False, BF16, 4, 20),  # one wave, several
+    (8192, True, BF16, 6, 9), (4096, True, BF16, 12, 3), (4096, False, FP16, 24, 1), (4096, False, BF16, 8, 7)])
+def test_step_other_sizes(S, H, qk, dtype, layers, T):
+    """Whole-step launches at H 8192 (blocks of 512 threads) and small grids with fewer RoPE items
+    per block, role-major ones included."""
+    cfg = dict(synth.LLAMA, H=H, Hq=H // 128, I=28672 if H == 8192 else 12288, S=256, qknorm=qk)
+    s, _ = step_scm(S, cfg, dtype, S.LAYOUT_ANY)
+    inps, outs, args = build_layers(S, cfg, T, layers, dtype=dtype, seed=H + T)
+    run_step(S, s, args)
+    assert s.stats().fused_launches == 1
+    s.close()
+    for inp, (_, out) in zip(inps, outs):
+        check_chain(L.layer_chain(inp, cfg["theta"], cfg["eps"], dtype, qknorm=qk), out, inp, dtype)
+
+
 def test_step_in_place_layers(S):
     cfg = synth.LLAMA
     T = 5
