@@ -195,7 +195,7 @@ struct KernelEntry {
   int32_t nm_threads[kNormEntries] = {};
   int32_t rows = 1;      // norms: rows per block of the NM_VEC entry
   int32_t edge_rows = 1;  // ... and of the NM_EDGE_MANY entry,
-  int64_t edge_many = 0;  // which calls of at least this many rows take
+  int64_t edge_many = 0;  // which calls of at least this many rows take (on 152 SMs)
 };
 
 enum KernelKind : int32_t {

@@ -73,8 +73,19 @@ constexpr float kNormRows2Vecs = 1024.f;
 constexpr int64_t kNormEdgeRows = 3072;
 // fp32 EDGE rows of more than 512 vectors take two vectors per thread from this many rows (more
 // rows resident): 4000 x 3001 25.4 -> 20.6 us, with the residual 34.8 -> 30.7; 8559 x 2222 35.7 ->
-// 29.6; at 300 rows 2.31 / 2.76. (16 bits: 3000 x 3999 12.5 / 13.7.)
+// 29.6; at 300 rows 2.31 / 2.76. (16 bits: 3000 x 3999 12.5 / 13.7.) Up to 768 vectors without the residual
+// from half as many: 1200 x 2222 5.55 / 4.57, 800 x 2222 4.20 / 4.89.
 constexpr int64_t kNormEdgeWideRows = 2048;
+// (Both on 152 SMs; norm_plan scales them.) EDGE rows of more than 1024 vectors without the residual:
+// two vectors per thread leave one block per SM, which long calls do not hide. In fp32 eight per thread
+// from one row per SM, six where two blocks fit (us, two / eight): 304 x 6001 5.5 / 4.8, 1200 17.8 / 13.9, 5000
+// 67.7 / 47.9 (scalar accesses 61.0); 800 x 5001 8.9 / 8.6, 3000 26.4 / 23.5. In 16 bits from two rows per SM
+// four up to 1280 vectors, eight up to 1536, as many as still give whole blocks an SM to share: 600 /
+// 9000 x 9501 10.1 / 142 -> 8.4 / 99.5 (scalar 108), x 11201 11.6 / 156 -> 11.0 / 120 (127); 9001, where two
+// blocks of two fit, 7.9 / 95 against 8.4 / 96. Above 1536 scalar accesses from 25 rows per SM: 4500 / 9000
+// x 12478 85.2 / 166 -> 79.3 / 140, 3000 57.5 / 60.4 (four per thread 176 at 9000).
+constexpr int kNormEdgeSms = 152;
+constexpr int64_t kNormEdgeNever = (int64_t)1 << 40;
 
 // Calls of few rows, in rows per SM. Rows of 33 to 128 vectors: norm_block_kernel, a vector per thread,
 // instead of two or four per lane one after the other (warp / block, us): 64 x 1024 bf16 1.87 / 1.19, 2200
@@ -94,7 +105,8 @@ static NormRange norm_few_range(bool res, int ve, int64_t nvec) {
 // (EDGE 2). With fewer, the branches' round trips hide in the launch; with more, the loads they save
 // count. Branches / none, at an odd offset: 600 x 333 2.05 / 2.87 us, 900 3.67 / 2.93; 300 x 1001 2.42 /
 // 3.29, 450 3.94 / 3.37, 900 4.08 / 3.34, 2000 4.56 / 4.67; 300 x 1537 3.81 / 3.42, 1333 4.26 / 4.42;
-// residual 450 x 333 1.94 / 2.86, 1333 3.59 / 2.97; 600 x 1001 3.60 / 3.40, 900 3.19 / 3.82. In fp32, with half the weights per vector, the branches are faster (600 x 1001 2.06 / 2.48).
+// residual 450 x 333 1.94 / 2.86, 1333 3.59 / 2.97; 600 x 1001 3.60 / 3.40, 900 3.19 / 3.82. With two
+// vectors per thread never (80 x 12478 3.50 / 3.68). In fp32, with half the weights per vector, the branches are faster (600 x 1001 2.06 / 2.48).
 static NormRange norm_edge_range(bool res) { return res ? NormRange{200.f, 570.f} : NormRange{300.f, 1280.f}; }
 
 template <int DT>
@@ -635,16 +647,17 @@ static void pick(int64_t H, KernelEntry* out) {
   }
   // rows that begin anywhere hold nvec or nvec - 1 whole vectors, and at least one
   out->edge_rows = 1;
-  out->edge_many = INT64_MAX;
+  out->edge_many = kNormEdgeNever;
   if (nvec >= 2 && nvec <= kNormBlockVecs) {
     out->nm_threads[NM_EDGE] = threads;
     if constexpr (VE == 8) {
-      const NormRange r = norm_edge_range(RES);
-      out->edge_lo = r.lo / (float)threads;
-      out->edge_hi = r.hi / (float)threads;
-      out->nm_threads[NM_EDGE_FLAT] = threads;
-      out->nm_fn[NM_EDGE_FLAT] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, 2, false>
-                                          : (const void*)norm_block_kernel<DT, RES, 2, 2, false>;
+      if (vpt == 1) {
+        const NormRange r = norm_edge_range(RES);
+        out->edge_lo = r.lo / (float)threads;
+        out->edge_hi = r.hi / (float)threads;
+        out->nm_threads[NM_EDGE_FLAT] = threads;
+        out->nm_fn[NM_EDGE_FLAT] = (const void*)norm_block_kernel<DT, RES, 1, 2, false>;
+      }
     }
     out->nm_fn[NM_EDGE] = vpt == 1 ? (const void*)norm_block_kernel<DT, RES, 1, 1, false>
                                    : (const void*)norm_block_kernel<DT, RES, 2, 1, false>;
@@ -655,9 +668,20 @@ static void pick(int64_t H, KernelEntry* out) {
       else if (nvec <= 64) out->nm_fn[NM_EDGE_MANY] = (const void*)norm_rows_edge_kernel<DT, RES, 2>;
       else if constexpr (!RES) out->nm_fn[NM_EDGE_MANY] = (const void*)norm_rows_edge_kernel<DT, RES, 4>;
     } else if (VE == 4 && vpt == 1 && nvec > 512) {
-      out->edge_many = kNormEdgeWideRows;
+      out->edge_many = RES || nvec > 768 ? kNormEdgeWideRows : kNormEdgeWideRows / 2;
       out->nm_threads[NM_EDGE_MANY] = norm_threads(nvec, 2);
       out->nm_fn[NM_EDGE_MANY] = (const void*)norm_block_kernel<DT, RES, 2, 1, false>;
+    } else if constexpr (!RES) {
+      const int ev = nvec <= (VE == 8 ? 1152 : 1024) ? 0 : VE == 8 && nvec <= 1280 ? 4 : VE == 8 && nvec > 1536 ? 1 : 8;
+      if (ev == 1) {
+        out->edge_many = (threads <= 832 ? 25 : 40) * kNormEdgeSms;
+        out->nm_fn[NM_EDGE_MANY] = out->nm_fn[NM_GENERIC];
+      } else if (ev) {
+        out->edge_many = (VE == 8 ? 2 : threads <= 640 ? 6 : 1) * kNormEdgeSms + 1;
+        out->nm_threads[NM_EDGE_MANY] = norm_threads(nvec, ev);
+        out->nm_fn[NM_EDGE_MANY] = ev == 4 ? (const void*)norm_block_kernel<DT, RES, 4, 1, false>
+                                           : (const void*)norm_block_kernel<DT, RES, 8, 1, false>;
+      }
     }
   }
   if (H % VE != 0) return;
@@ -751,7 +775,7 @@ NormEntry norm_plan(const KernelEntry& ke, NormParams* p, bool res, int32_t eb, 
         : ke.nm_fn[NM_MID] && rows_sm > ke.mid_lo && rows_sm <= ke.mid_hi ? NM_MID
         : ke.nm_fn[NM_LARGE] && rows_sm > ke.large_sm ? NM_LARGE : NM_VEC;
   else if (together && ke.nm_fn[NM_EDGE] && p->T <= INT32_MAX)
-    e = p->T >= ke.edge_many ? NM_EDGE_MANY
+    e = p->T >= ke.edge_many * sms / kNormEdgeSms ? NM_EDGE_MANY
         : ke.nm_fn[NM_EDGE_FLAT] && rows_sm > ke.edge_lo && rows_sm <= ke.edge_hi ? NM_EDGE_FLAT : NM_EDGE;
   *threads = ke.nm_threads[e];
   *smem = e == NM_LARGE ? ke.large_smem : 0;

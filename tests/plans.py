@@ -60,7 +60,13 @@ NORM_LIMITS = [
     (1, 475, 333, 1, "edge", "edge"), (2, 713, 333, 1, "edge_flat", "edge_flat"),       # rows at odd offsets
     (1, 1354, 333, 1, "edge", "edge_flat"), (2, 357, 1023, 1, "edge_flat", "edge_flat"),
     (1, 88, 4001, 1, "edge_flat", "edge"), (2, 91, 4095, 1, "edge_flat", "edge_flat"),
-    (1, 40, 9001, 1, "edge", "edge"), (2, 85, 9007, 1, "edge_flat", "edge_flat"),       # two vectors per thread
+    (2, 304, 9501, 1, "edge", "edge"), (2, 305, 9501, 1, "edge", "edge_many"),     # more per thread
+    (1, 305, 10241, 1, "edge", "edge_many"), (1, 306, 12287, 1, "edge", "edge_many"),
+    (1, 3799, 12299, 1, "edge", "edge"), (2, 3801, 12301, 1, "edge", "edge_many"),      # scalar accesses
+    (3, 152, 5601, 1, "edge", "edge"), (3, 153, 5601, 1, "edge", "edge_many"), (3, 157, 8191, 1, "edge", "edge_many"),
+    (3, 912, 4501, 1, "edge", "edge"), (3, 913, 4501, 1, "edge", "edge_many"),
+    (3, 1023, 2222, 1, "edge", "edge"), (3, 1025, 2222, 1, "edge", "edge_many"),
+    (1, 40, 9001, 1, "edge", "edge"), (2, 85, 9007, 1, "edge", "edge"),                 # two vectors per thread
 ]
 
 # RoPE calls at the limits of their entries: (T, Hq, Hkv, D, q/k norm, entry and block size).
