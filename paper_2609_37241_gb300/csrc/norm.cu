@@ -90,7 +90,7 @@ constexpr int64_t kNormEdgeNever = (int64_t)1 << 40;
 // Calls of few rows, in rows per SM. Rows of 33 to 128 vectors: norm_block_kernel, a vector per thread,
 // instead of two or four per lane one after the other (warp / block, us): 64 x 1024 bf16 1.87 / 1.19, 2200
 // 3.20 / 3.00, 3000 3.62 / 3.85; 1300 x 512 2.60 / 1.98, 2200 2.67 / 3.02; 1300 x 320 2.05 / 1.93, 1700
-// 2.06 / 2.25; residual 64 x 1024 2.06 / 1.11, 4500 7.33 / 6.91, 7000 10.2 / 10.2; 1300 x 320 2.25 / 2.10,
+// 2.06 / 2.25; residual 64 x 1024 2.06 / 1.11, 2200 4.43 / 3.40, 4331 in fp16 4.73 / 5.42; 1300 x 320 2.25 / 2.10,
 // 2200 2.65 / 3.22. Rows of 2048 vectors: eight per thread of 256 instead of two per thread of 1024, whose
 // one block per SM waits longest on itself: 64 / 152 x 16384 bf16 2.63 / 3.63 -> 2.34 / 3.13, residual 3.91
 // / 4.91 -> 3.42 / 4.17; fp32 only below half a row per SM (64 x 8192 3.04 -> 2.53, 100 3.40 / 3.97), with
@@ -98,7 +98,7 @@ constexpr int64_t kNormEdgeNever = (int64_t)1 << 40;
 static NormRange norm_few_range(bool res, int ve, int64_t nvec) {
   if (nvec == kNormBlockVecs) return ve == 8 ? NormRange{0.f, 1.f} : res ? NormRange{0.4f, 1.f} : NormRange{0.f, 0.5f};
   if (nvec > 32 && nvec <= 64) return {0.f, 9.f};
-  if (nvec > 64 && nvec <= 128) return {0.f, res ? 40.f : 14.f};
+  if (nvec > 64 && nvec <= 128) return {0.f, res ? 16.f : 14.f};
   return {0.f, 0.f};
 }
 // EDGE rows in 16 bits, a block per row: from lo to hi threads per SM the loads stand in no branch
@@ -402,8 +402,12 @@ __global__ void __launch_bounds__(kThreads) norm_rows_edge_kernel(const NormPara
 // (16384 x 5120 50.7 us against 52-61 with two). gamma loaded after the reduction instead cost
 // 2-3 us per call. The wait is bounded: if it runs out, the block sets TRIDENT_DEVERR_TIMEOUT,
 // waits again (bounded) for its copies and returns without writing.
-template <int DT, bool RES, int VPT, bool FULL>
-__global__ void __launch_bounds__(512, RES ? (VPT == 2 ? 3 : 2) : 1) norm_bulk_kernel(const NormParams p) {
+// NT, MB: at most NT threads, at least MB blocks per SM. Without the residual and its bound, 64 registers
+// left two blocks of 272 to 384 threads (rows of 1025 to 1536 vectors): 7000 x 10752 57.8 us, 49.4 with three,
+// the two-pass kernel before 52.5; wider rows, two blocks of up to 512 either way, take eight vectors per
+// thread of 256: 7000 x 12544 64.6 -> 59.3 (61.1), 4000 x 16384 44.4 -> 40.3.
+template <int DT, bool RES, int VPT, bool FULL, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) norm_bulk_kernel(const NormParams p) {
   constexpr int VE = Act<DT>::VE;
   constexpr int EB = Act<DT>::BYTES;
   extern __shared__ __align__(128) uint4 s_rows[];
@@ -621,6 +625,23 @@ static void pick_rows(int64_t nvec, KernelEntry* out) {
 }
 
 template <int DT, bool RES>
+static const void* norm_bulk(int64_t nvec, int vpt, bool full) {
+  if constexpr (RES) {
+    if (vpt == 2) return full ? (const void*)norm_bulk_kernel<DT, RES, 2, true, 512, 3>
+                              : (const void*)norm_bulk_kernel<DT, RES, 2, false, 512, 3>;
+    return full ? (const void*)norm_bulk_kernel<DT, RES, 4, true, 512, 2>
+                : (const void*)norm_bulk_kernel<DT, RES, 4, false, 512, 2>;
+  } else {
+    if (nvec <= 1024) return full ? (const void*)norm_bulk_kernel<DT, RES, 4, true, 512, 1>
+                                  : (const void*)norm_bulk_kernel<DT, RES, 4, false, 512, 1>;
+    if (vpt == 4) return full ? (const void*)norm_bulk_kernel<DT, RES, 4, true, 384, 3>
+                              : (const void*)norm_bulk_kernel<DT, RES, 4, false, 384, 3>;
+    return full ? (const void*)norm_bulk_kernel<DT, RES, 8, true, 256, 3>
+                : (const void*)norm_bulk_kernel<DT, RES, 8, false, 256, 3>;
+  }
+}
+
+template <int DT, bool RES>
 static void pick(int64_t H, KernelEntry* out) {
   constexpr int VE = Act<DT>::VE;
   const int64_t nvec = H / VE;
@@ -705,14 +726,11 @@ static void pick(int64_t H, KernelEntry* out) {
     out->large_sm = vpt == 2 ? wave : (!RES && nvec <= 256 ? 4 : 2) * wave;
     if constexpr (VE == 8) {
       if (RES || nvec >= 256) {
-        const int bv = RES && nvec <= 1024 ? 2 : 4;
+        const int bv = RES ? (nvec <= 1024 ? 2 : 4) : nvec <= 1536 ? 4 : 8;
         const int bt = norm_threads(nvec, bv);
         const bool bfull = bt * bv == nvec;
         out->nm_threads[NM_LARGE] = bt;
-        out->nm_fn[NM_LARGE] = bv == 2 ? (bfull ? (const void*)norm_bulk_kernel<DT, RES, 2, true>
-                                                : (const void*)norm_bulk_kernel<DT, RES, 2, false>)
-                                       : (bfull ? (const void*)norm_bulk_kernel<DT, RES, 4, true>
-                                                : (const void*)norm_bulk_kernel<DT, RES, 4, false>);
+        out->nm_fn[NM_LARGE] = norm_bulk<DT, RES>(nvec, bv, bfull);
         out->large_smem = (int32_t)(nvec * 16 * (RES ? 2 : 1));
       }
       const int rv = nvec % kThreads == 0 ? (int)(nvec / kThreads) : 0;

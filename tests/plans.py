@@ -48,13 +48,15 @@ def chain(qk, H, Hq, I, T, pdl=True, inplace=False, Hkv=8):
 NORM_LIMITS = [
     (1, 608, 6144, 0, "vec", "vec"), (1, 609, 6144, 0, "large_bulk", "large_bulk"),     # two waves of blocks
     (2, 152, 12296, 0, "vec", "vec"), (1, 153, 12288, 0, "large_bulk", "large_bulk"),   # one, two vectors each
+    (2, 311, 8448, 0, "large_bulk", "large_bulk"), (1, 157, 12288, 0, "large_bulk", "large_bulk"),
+    (2, 160, 12296, 0, "large_bulk", "large_bulk"), (1, 161, 16384, 0, "large_bulk", "large_bulk"),
     (1, 1217, 2048, 0, "mid", "vec"), (2, 690, 4096, 0, "mid", "mid"), (1, 608, 4096, 0, "vec", "vec"),
     (2, 1217, 4096, 0, "large_regs", "large_bulk"), (1, 609, 8192, 0, "mid", "large_bulk"),
     (2, 913, 8192, 0, "large_bulk", "large_bulk"),
     (3, 1217, 2048, 0, "vec", "large_regs"), (3, 457, 5000, 0, "vec", "large_regs"),    # four per thread
     (3, 305, 8192, 0, "vec", "large_regs"), (3, 305, 7000, 0, "vec", "large_regs"),     # eight
     (1, 1368, 264, 0, "few", "few"), (1, 1369, 264, 0, "vec", "vec"),  # few rows
-    (2, 2128, 1024, 0, "few", "few"), (2, 2129, 1024, 0, "few", "vec"), (3, 6081, 512, 0, "vec", "vec"),
+    (2, 2128, 1024, 0, "few", "few"), (2, 2129, 1024, 0, "few", "vec"), (2, 2432, 1024, 0, "few", "vec"), (3, 2433, 512, 0, "vec", "vec"),
     (3, 1, 148, 0, "few", "few"), (1, 152, 16384, 0, "few", "few"), (2, 153, 16384, 0, "large_bulk", "large_bulk"),
     (3, 61, 8192, 0, "few", "few"), (3, 77, 8192, 0, "few", "vec"), (3, 60, 8192, 0, "vec", "few"),
     (1, 475, 333, 1, "edge", "edge"), (2, 713, 333, 1, "edge_flat", "edge_flat"),       # rows at odd offsets
