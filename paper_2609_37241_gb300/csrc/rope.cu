@@ -5,8 +5,8 @@
 // of consecutive head-rows of one token (RopeGeom, rope_pair_rows in device_common.cuh): D / 16
 // lanes per head-row, each lane holding both halves of its rotated pairs, so that a rotation
 // needs no exchange between lanes and a token's angles are computed once per lane and item.
-// Four entries, by the call's size (rope_plan): one head-row per lane group, in small or larger
-// blocks, two where it pays, and for calls of many tokens three, staged in shared memory by
+// Four entries, by the call's size (rope_plan): one head-row per lane group, for heads of 64 also in
+// larger blocks, two where it pays, and for calls of many tokens three, staged in shared memory by
 // cp.async.bulk (rope_bulk_kernel). Other head sizes that are multiples of 16 take rope_any_kernel,
 // the same with lanes left over; the generic kernel gives each head-row one warp and scalar
 // accesses (any alignment, any even D). All compute (cos, sin) of pos * theta^(-2i/D) in the kernel
@@ -26,39 +26,47 @@
 
 namespace trident {
 
-// One head-row per lane group (small entry) in blocks of 64, 128 or 256 threads, or two rows (mid
-// entry) in blocks of 64, by the call's size in warp items per SM. Up to a few items the call is one
-// memory round trip: one row per group in the smallest blocks. A second row halves the warps that
-// fetch the same frequency and weight lines, which pays while their blocks stay few and again on long
-// calls; in between, one row in larger blocks. Where a form stops paying is measured, not derived:
-// launches back to back go in steps of about 0.8 us, one more where a grid no longer starts within
-// the one before, and each form steps at its own size. us per call at its lines (D 128 unless stated):
-//   without the norm, two rows up to 2.28 blocks per SM: 345 blocks (230 tokens of 32 + 8 + 8 heads of D
-//     64) 2.06, 360 (240 tokens) 2.85; one row in 64 threads up to 8 items, 128 in (10.9, 12] and 256 up to 24
-//     against two rows: 400 tokens of 16 + 4 + 4 of D 64 2.25 / 2.72; 300 of 32 + 8 + 8 of D 64 2.25 / 2.91, 260
-//     of 20 + 4 + 4 2.03 / 2.85; 250 of 32 + 8 + 8 of D 64 2.42 / 2.87, 220 of 32 + 8 + 8 2.75 / 2.96, 300 2.87 /
-//     3.07, 335 2.98 / 2.83, 400 3.65 / 3.33. (Two rows beat this by up to 14 % where their blocks come to
-//     400 or 800: 270 tokens of 32 + 8 + 8 2.73 / 2.39.)
-//   with it, two rows from 4.5 items to 1.72 blocks per SM: 60 tokens of 32 + 8 + 8 2.33, one row 2.32; 150 of D
-//     64 2.38 / 2.88; 260 of 16 + 4 + 4 of D 64 2.31 / 2.76, 270 3.19 / 1.94; one row in 128 threads up to one
-//     wave of them, 32 items, 64 threads / two rows beside it: 280 of 16 + 4 + 4 of D 64 2.79 / 2.91 / 3.19, 300
-//     of 32 + 8 + 8 of D 64 2.95 / 3.08 / 3.29, 105 of 16 + 8 + 8 of D 256 2.60 / 3.02 / 3.17, 335 of 32 + 8 + 8
-//     3.19 / 3.50 / 3.74, 400 3.99 / 4.45 / 4.12; beyond two rows: 440 5.02 / 4.91 / 4.36.
-constexpr int kRopeThreads = 64;     // block of the mid entry, and the smallest of the small one
+// One head-row per lane group (small entry) or two (mid), by the call's one-row items per SM. Up
+// to three the call is one memory round trip, and a second row only lengthens it; on long calls
+// two rows halve the warps that fetch the same frequency and weight lines (60 tokens of 32 + 8 + 8
+// heads, D 128, with q/k norm 2.33 us against 2.62, 500 tokens 4.67 / 5.51). In between the lines are
+// measured, not derived: launches of the same call back to back go in steps of about 0.8 us, one more
+// where a grid no longer starts within the one before it, and each form steps at sizes of its own.
+// Heads of 128 and 256, with q/k norm: two rows from 4.5 to 6 items per SM (75 tokens of 32 + 8 + 8 2.40 /
+// 2.66) and from 27 (400 tokens 4.36 / 4.59), one row elsewhere: 45 tokens 2.25 -> 2.05 us, 90 3.32 -> 2.73,
+// 140 3.39 -> 2.62, 225 3.66 -> 3.33, 28 + 4 + 4 heads at 150 3.77 -> 2.89. Without the norm one row from 10.5
+// to 12 and from 13 to 15 items: 28 head-rows (20 + 4 + 4) at 240 / 257 tokens 2.87 / 2.87 -> 2.33 / 2.35, 180
+// tokens of 48 2.87 -> 2.47, D 256 at 130 2.87 -> 2.46; between those, 28 head-rows at 264 tokens (12.2) 2.84 /
+// 3.31, and outside, 105 tokens of 48 (8.3) 2.04 / 2.80, 320 (25) 3.55 / 4.08. (As one of a layer's four
+// single-op launches two rows win there too, mean per launch 144 / 176 tokens of 32 + 8 + 8 2.37 / 2.56 us, one
+// row 2.77 / 2.99.)
+// Heads of 64, half the bytes per item, by the blocks of two-row items, and one row in larger blocks
+// beyond them: without the norm two rows up to 2.28 blocks per SM (230 / 240 tokens of 32 + 8 + 8 2.06 / 2.85),
+// then one in 64 threads up to 8 items (400 of 16 + 4 + 4 2.20 / 2.72), in 128 from 10.9 to 12 (300 of 32 + 8 + 8
+// 2.26, in 256 2.68, two rows 2.91) and in 256 up to 24 (250 / 320 / 400 of 32 + 8 + 8 2.42 / 2.59 / 2.32 against
+// 2.87 / 2.87 / 2.83); with it two rows from 4.5 items to 1.72 blocks per SM (150 of 32 + 8 + 8 2.38 / 2.88; 260
+// of 16 + 4 + 4 2.31 / 2.76, 280 3.19 / 2.79), then one in 128 threads up to one wave of them, 32 items (300 of
+// 32 + 8 + 8 2.95, in 64 threads 3.08, two rows 3.29).
+constexpr int kRopeThreads = 64;     // block of the small and mid entries (128: the same within 3 %)
 constexpr int kRopeMaxThreads = 256;
 struct RopeChoice { bool two; int32_t threads; };
-static RopeChoice rope_choice(int64_t one, int64_t two, bool qk, int64_t sms) {  // items with one and two rows
+static RopeChoice rope_choice(int64_t one, int64_t two, int32_t D, bool qk, int64_t sms) {  // items with one and two rows
+  const int64_t n = 2 * one;  // in half items
+  if (n <= 6 * sms) return {false, 64};
+  if (D > 64) {
+    const bool small = qk ? n <= 54 * sms && !(n > 9 * sms && n <= 12 * sms)
+                          : (n > 21 * sms && n <= 24 * sms) || (n > 26 * sms && n <= 30 * sms);
+    return {!small, 64};
+  }
   const int64_t blocks = (two + 1) / 2;
   if (qk) {
-    if (2 * one <= 9 * sms) return {false, 64};
-    if (100 * blocks <= 172 * sms) return {true, 64};
-    return one <= 32 * sms ? RopeChoice{false, 128} : RopeChoice{true, 64};
+    if (n <= 9 * sms) return {false, 64};
+    if (100 * blocks <= 172 * sms || one > 32 * sms) return {true, 64};
+    return {false, 128};
   }
-  if (one <= 3 * sms) return {false, 64};
-  if (100 * blocks <= 228 * sms) return {true, 64};
+  if (100 * blocks <= 228 * sms || one > 24 * sms) return {true, 64};
   if (one <= 8 * sms) return {false, 64};
-  if (10 * one > 109 * sms && one <= 12 * sms) return {false, 128};
-  return one <= 24 * sms ? RopeChoice{false, 256} : RopeChoice{true, 64};
+  return {false, 10 * one > 109 * sms && one <= 12 * sms ? 128 : 256};
 }
 // Calls of at least this many tokens and bulk items take the bulk-copy entry: 640 tokens (2560
 // items) with q/k norm 5.06 us against 5.80 with two register-held rows per group, 2048 tokens
@@ -68,9 +76,9 @@ static RopeChoice rope_choice(int64_t one, int64_t two, bool qk, int64_t sms) { 
 constexpr int32_t kRopeBulkTokens = 512;
 constexpr int64_t kRopeBulkItems = 2304;
 
-
 // Before the launch wait: the lane's frequencies (the version's table is written only at
-// registration; with p.freq_late the previous kernel writes it, and they are read after), and with p.prefetch the L2 prefetch of the item's row lines and position.
+// registration; with p.freq_late the previous kernel writes it, and they are read after), and with
+// p.prefetch the L2 prefetch of the item's row lines and position.
 // NT: the largest block; blocks of more than 64 threads at most four per SM of 256 (more resident ones
 // take the SM from the launch before: 300 tokens of 32 + 8 + 8 heads of D 64 2.26 us, without the limit 2.66).
 template <int DT, int D, bool QKNORM, int R, int NT>
@@ -78,7 +86,7 @@ __global__ void __launch_bounds__(NT, NT == kRopeThreads ? 0 : 4) rope_pair_kern
   pdl_trigger();
   int64_t t;
   int first, end;
-  const int64_t item = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  const int64_t item = (int64_t)blockIdx.x * ((NT == kRopeThreads ? NT : blockDim.x) / 32) + threadIdx.x / 32;
   const bool live = rope_item(p, item, &t, &first, &end);
   float4 fq[4];
   if (!p.freq_late) rope_pair_freqs(p.inv_freq, (threadIdx.x & 31) % RopeGeom<D>::LPG, fq);
@@ -309,7 +317,7 @@ RopeEntry rope_plan(const RopePlans& plans, RopeParams* p, int32_t* threads, int
   RopeEntry e = ROPE_BULK;
   *threads = kRopeBulkThreads;
   if (p->T < kRopeBulkTokens || p->T * plans.split[ROPE_BULK].ipt < kRopeBulkItems) {
-    const RopeChoice c = rope_choice(p->T * plans.split[ROPE_SMALL].ipt, p->T * plans.split[ROPE_MID].ipt,
+    const RopeChoice c = rope_choice(p->T * plans.split[ROPE_SMALL].ipt, p->T * plans.split[ROPE_MID].ipt, p->D,
                                      p->gamma_q != nullptr, sms);
     e = c.two ? ROPE_MID : c.threads > kRopeThreads ? ROPE_BLOCKS : ROPE_SMALL;
     *threads = c.threads;
@@ -361,7 +369,7 @@ static void pick_any(int32_t D, KernelEntry* out) {
 template <int DT, bool QK, int D>
 static void pick_d(KernelEntry* out) {
   out->fn = (const void*)rope_pair_kernel<DT, D, QK, 1, kRopeThreads>;
-  out->fn_blocks = (const void*)rope_pair_kernel<DT, D, QK, 1, kRopeMaxThreads>;
+  if constexpr (D == 64) out->fn_blocks = (const void*)rope_pair_kernel<DT, D, QK, 1, kRopeMaxThreads>;
   out->fn_mid = (const void*)rope_pair_kernel<DT, D, QK, 2, kRopeThreads>;
   out->fn_large = (const void*)rope_bulk_kernel<DT, D, QK>;
 }

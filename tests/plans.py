@@ -73,14 +73,17 @@ NORM_LIMITS = [
 
 # RoPE calls at the limits of their entries: (T, Hq, Hkv, D, q/k norm, entry and block size).
 ROPE_LIMITS = [
-    (38, 32, 8, 128, False, "one_64"), (39, 32, 8, 128, False, "two_64"), (115, 32, 8, 128, False, "two_64"),
-    (116, 32, 8, 128, False, "one_256"), (139, 32, 8, 128, False, "one_128"), (152, 32, 8, 128, False, "one_128"),
-    (153, 32, 8, 128, False, "one_256"), (304, 32, 8, 128, False, "one_256"), (305, 32, 8, 128, False, "two_64"),
-    (575, 32, 8, 128, False, "two_64"), (576, 32, 8, 128, False, "bulk_128"),
-    (57, 32, 8, 128, True, "one_64"), (58, 32, 8, 128, True, "two_64"), (87, 32, 8, 128, True, "two_64"),
-    (88, 32, 8, 128, True, "one_128"), (405, 32, 8, 128, True, "one_128"), (406, 32, 8, 128, True, "two_64"),
-    (347, 16, 4, 64, False, "one_64"), (405, 16, 4, 64, False, "one_64"), (406, 16, 4, 64, False, "one_256"),
-    (511, 5, 1, 128, True, "two_64"), (400, 3, 2, 256, False, "one_256"), (333, 3, 3, 256, True, "one_128"),
+    (38, 32, 8, 128, False, "one_64"), (39, 32, 8, 128, False, "two_64"), (133, 32, 8, 128, False, "two_64"),
+    (134, 32, 8, 128, False, "one_64"), (153, 32, 8, 128, False, "two_64"), (190, 32, 8, 128, False, "one_64"),
+    (191, 32, 8, 128, False, "two_64"), (575, 32, 8, 128, False, "two_64"), (576, 32, 8, 128, False, "bulk_128"),
+    (57, 32, 8, 128, True, "one_64"), (58, 32, 8, 128, True, "two_64"), (76, 32, 8, 128, True, "two_64"),
+    (77, 32, 8, 128, True, "one_64"), (342, 32, 8, 128, True, "one_64"), (343, 32, 8, 128, True, "two_64"),
+    (511, 5, 1, 128, True, "one_64"), (400, 3, 2, 256, False, "one_64"), (333, 3, 3, 256, True, "one_64"),
+    (230, 32, 8, 64, False, "two_64"), (231, 32, 8, 64, False, "one_256"), (280, 32, 8, 64, False, "one_128"),
+    (305, 32, 8, 64, False, "one_256"), (608, 32, 8, 64, False, "one_256"), (609, 32, 8, 64, False, "two_64"),
+    (347, 16, 4, 64, False, "one_64"), (406, 16, 4, 64, False, "one_256"), (1152, 32, 8, 64, False, "bulk_128"),
+    (114, 32, 8, 64, True, "one_64"), (115, 32, 8, 64, True, "two_64"), (174, 32, 8, 64, True, "two_64"),
+    (175, 32, 8, 64, True, "one_128"), (810, 32, 8, 64, True, "one_128"), (811, 32, 8, 64, True, "two_64"),
 ]
 
 # Layer-chain calls at the limits of their entries: (H, q heads, I, q/k norm, T, PDL, in place, plan);

@@ -528,7 +528,7 @@ def test_rope_kv_entry_limits(S, T, Hq, Hkv, D, qk, entry):
     """Both sides of each line of the RoPE kernels' rule."""
     assert plans.rope(T, Hq, Hkv, D, qk) == entry
     dtype = FP16 if T % 2 else BF16
-    ref, got, inp = run_rope(S, T, Hq, Hkv, D, 1024, 5e5, qk, dtype=dtype, layout="fused", seed=T + Hq)
+    ref, got, inp = run_rope(S, T, Hq, Hkv, D, 2048, 5e5, qk, dtype=dtype, layout="fused", seed=T + Hq)
     assert got["status"] == 0 and ref["bad"] == 0
     check_rope(ref, got, inp, dtype)
 
