@@ -156,7 +156,7 @@ struct ChainStepParams {
 enum PointwiseEntry : int32_t { PW_FLAT, PW_FLAT2, PW_ROWS, PW_ROWS2, PW_GENERIC, kPwEntries };
 // Picks the entry of a call (index into pw_fn) from its packed params, fills their vector
 // fields and sets the grid. eb: element size.
-int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks);
+int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks, int32_t sms);
 
 // Norm entries (norm_plan): 16-byte aligned rows, rows at any common offset (few or many rows),
 // scalar accesses, the entry of long aligned calls (bulk copies, more vectors per thread, or two
@@ -180,7 +180,7 @@ struct KernelEntry {
   const void* fn_large = nullptr;  // RoPE: the bulk-copy entry (rope_plan chooses)
   const void* any_fn[2] = {};      // RoPE versions of the generic kind: rope_any_kernel (or NULL)
   const void* fn_mid = nullptr;    // RoPE: two head-rows per lane group
-  const void* fn_blocks = nullptr;  // RoPE: fn for blocks of 128 or 256 threads
+  const void* fn_blocks = nullptr;  // RoPE, D 64: fn for blocks of 128 or 256 threads
   const void* pw_fn[kPwEntries] = {};  // elementwise, by PointwiseEntry
   float large_sm = 0;      // norms: calls of more rows per SM take the NM_LARGE entry
   float few_lo = 0, few_hi = 0;  // ... of rows per SM in (few_lo, few_hi] the NM_FEW entry
@@ -265,7 +265,7 @@ const void* empty_kernel_entry();  // the latency-floor probe's kernel (does not
 
 // Validation, guard-equivalent checks (sizes, layouts, 16-byte alignment, overlap) and
 // parameter packing of a ROPE_KV / QKNORM_ROPE_KV argument tuple without an SCM. Leaves
-// p->cs and p->err NULL. Returns a trident_status (message in trident_scm_last_error).
+// p->inv_freq and p->err NULL. Returns a trident_status (message in trident_scm_last_error).
 int32_t prepare_rope_args(const void* trident_args_ptr, RopeParams* p, int32_t* dtype,
                           bool* qknorm);
 

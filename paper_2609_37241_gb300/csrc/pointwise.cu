@@ -185,7 +185,7 @@ static void pick(int32_t dtype, KernelEntry* out) {
 // 2.00 / 2.40 / 3.51); with a single 16-byte load per thread a large one has too few bytes in
 // flight (silu 4096 / 8192 / 16384 x 1000 2.84 / 5.66 / 11.6 against 2.87 / 4.20 / 10.1 with two).
 // Cache hints (evict-first stores, no L1 allocation) changed nothing or lost 1-4 %.
-int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks) {
+int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks, int32_t sms) {
   const int64_t ve = 16 / eb, n = p->T * p->W;
   const bool binary = pw_binary(op), masked = op == PW_MASKED_FILL;
   const uintptr_t off = (uintptr_t)p->a & 15;
@@ -216,10 +216,10 @@ int pointwise_plan(PointwiseParams* p, int32_t op, int32_t eb, int64_t* blocks) 
     p->units = 0;
     p->mask_vec = 0;
     *blocks = (n + kThreads - 1) / kThreads;
-    if (*blocks > 152 * 64) *blocks = 152 * 64;
+    if (*blocks > (int64_t)sms * 64) *blocks = (int64_t)sms * 64;
     return PW_GENERIC;
   }
-  const bool two = !binary && p->units > 3 * 152 * 2048 / 2;
+  const bool two = !binary && p->units > 3 * (int64_t)sms * 2048 / 2;
   const int64_t per = (two ? 2 : 1) * kThreads;
   *blocks = (p->units + per - 1) / per;
   return rows ? (two ? PW_ROWS2 : PW_ROWS) : (two ? PW_FLAT2 : PW_FLAT);

@@ -831,7 +831,7 @@ int32_t do_launch(trident_scm* scm, const Version& v, const trident_args* a, con
     case TRIDENT_OP_MASKED_FILL: {
       pack_pointwise(a, s, &P.pw);
       int64_t blocks = 0;
-      pw_entry = pointwise_plan(&P.pw, op, elem_size(v.d.dtype), &blocks);
+      pw_entry = pointwise_plan(&P.pw, op, elem_size(v.d.dtype), &blocks, scm->sm_count);
       cfg.gridDimX = cap_grid(blocks);
       break;
     }
