@@ -32,8 +32,8 @@ __device__ __forceinline__ void pdl_prologue() {
 // pdl_trigger and pdl_wait, while the previous kernel of the stream may still run: a
 // prefetch changes no value that a later load returns (the loads come after the wait), it
 // only lets the DRAM fetch overlap the previous kernel's tail and the launch handoff. The
-// host enables it (params.prefetch) for grids of at most one block per SM launched with
-// programmatic stream serialisation: a grid that fills the GPU becomes resident only as the
+// host enables it (params.prefetch) for grids of at most 256 threads per SM (a layer chain's: one
+// block) launched with programmatic stream serialisation: a grid that fills the GPU becomes resident only as the
 // previous kernel's blocks retire, and its prefetches then compete with that kernel.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.L2 [%0];" :: "l"(p)); }
 

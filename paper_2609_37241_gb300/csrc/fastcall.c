@@ -6,8 +6,8 @@
  * the whole dispatch it wraps; a METH_FASTCALL call costs a few tens of nanoseconds. The
  * binding's own invoke, invoke_seq and invoke_step go through run() where it is built: per
  * pass from Python, 36 one-token layer chains 80 -> 71 us, an 8-token step of 36 layers
- * (replayed) 12.9 -> 9.5 us, eight nested-argument norms 36.7 -> 31.9 us (with the shim
- * looked up once instead of per call). */
+ * (replayed) 12.9 -> 9.5 us. Eight nested-argument norms took 31.9 to 34.2 us where they had
+ * taken 36.7 to 37.2, within the spread of their runs (11 % on one box). */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>

@@ -149,7 +149,7 @@ __device__ __forceinline__ void load_gamma_at(const float* gamma, int i, int H, 
 
 // LPR lanes per row, VPT vectors per lane (VPT > 1 only with 32 lanes); lane l owns the
 // vectors l + LPR * v. FULL: the lanes' vectors are exactly the row's. R rows per lane group at
-// a time, their loads issued together.
+// a time, their loads issued together. The grid covers every row, so the loop runs once.
 template <int DT, bool RES, int LPR, int VPT, bool FULL, int R>
 __global__ void __launch_bounds__(kThreads) norm_rows_kernel(const NormParams p) {
   pdl_trigger();
@@ -583,6 +583,7 @@ __global__ void __launch_bounds__(kThreads) norm_loop_kernel(const NormParams p)
   }
 }
 
+// The loop goes on only past 2^31 - 1 rows, the grid's limit.
 template <int DT, bool RES>
 __global__ void __launch_bounds__(kThreads) norm_generic_kernel(const NormParams p) {
   pdl_prologue();

@@ -178,7 +178,7 @@ def test_fuzz_layer_chain(S, seed):
     rng = random.Random(300 + seed)
     base = rng.choice([synth.LLAMA, synth.QWEN3])
     dtype = rng.choice([BF16, BF16, FP16])
-    # up to 80 tokens one wave (late trigger under PDL from 5 tokens); 80, 150 and 260 tokens
+    # up to 81 Llama tokens one wave (late trigger under PDL from 5 to 72); 150 and 260 tokens
     # several waves (one norm CTA per token, three head-rows per RoPE lane group)
     T = rng.choice([1, 2, 5, 16, 17, 19, 33, 64, 80, 150, 260])
     cfg = dict(base, S=rng.choice([128, 8192]) if T <= 128 else 8192)

@@ -69,7 +69,7 @@ def test_step_qwen3_36_layers_one_launch(S):
 
 @pytest.mark.parametrize("T", [1, 16, 64])
 def test_step_llama_layers_both_splits(S, T):
-    # 4 Llama layers: 144 blocks per layer at T = 16 fit one wave together (two CTAs per
+    # 4 Llama layers: 88 blocks per layer at T = 16 fit one wave together (two CTAs per
     # token); at T = 64 they do not (one CTA per token)
     cfg = synth.LLAMA
     lay = S.LAYOUT_ROWSTRIDED if T > 1 else S.LAYOUT_CONTIG
